@@ -24,8 +24,7 @@ GFD_HD int tab_off(int L) { return L - 2; }
 // Number of interpolation nodes for the regularisation-parameter equation
 // (Sec. 3.2, Eq. 11) evaluated per spectral pass.
 constexpr int KNODES = 12;
-constexpr int KNARROW = 8;  // nodes of the first pass from iteration NARROW_FROM on
-constexpr int NARROW_FROM = 5;
+constexpr int KMOM = 8;  // moments of a first pass that expands about an extrapolated lambda
 // Fallback passes launched after the fused pass of each iteration (default).
 constexpr int LAMBDA_FALLBACK_PASSES = 4;
 constexpr double LAMBDA_LO = 1e-14;
@@ -36,18 +35,22 @@ constexpr int ST_NONFINITE = 2;
 constexpr int ST_BAD_PSF = 4;
 constexpr int ST_BAD_RHO = 8;
 constexpr int ST_PASSES_EXHAUSTED = 16;
-constexpr int ST_COPY_TIMEOUT = 32;
 
-GFD_HD float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-GFD_HD float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
-GFD_HD float2 cmul(float2 a, float2 b) {
-  return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
+// Complex arithmetic on float2 as packed FP32 pairs: one add.f32x2 / fma.f32x2
+// instruction handles both components, and takes negated and duplicated
+// operands as they are.  The rate per component is that of the scalar
+// instructions, but half the issue slots are used, which is what the transform
+// kernels run out of.  Every component is rounded as in the scalar form.
+GFD_D float2 cadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+GFD_D float2 csub(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
+GFD_D float2 cmul(float2 a, float2 b) {
+  return __ffma2_rn(make_float2(a.x, a.x), b, make_float2(-a.y * b.y, a.y * b.x));
 }
-GFD_HD float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
-GFD_HD float2 cscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
+GFD_D float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
+GFD_D float2 cscale(float2 a, float s) { return __fmul2_rn(a, make_float2(s, s)); }
 // multiply by -i (forward) or +i (inverse)
 template <bool INV>
-GFD_HD float2 cmul_mi(float2 a) {
+GFD_D float2 cmul_mi(float2 a) {
   return INV ? make_float2(-a.y, a.x) : make_float2(a.y, -a.x);
 }
 
@@ -85,49 +88,6 @@ GFD_D void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
-// One-dimensional bulk copies (the TMA engine) completed on an mbarrier.
-// A block stages a contiguous tile with one instruction from one thread:
-//   mbar_init once; per tile, the issuing thread calls bulk_load (which arms
-//   the barrier with the byte count) and every thread waits with mbar_wait on
-//   the barrier's current phase parity, which then flips.
-// Addresses are 16-byte aligned and sizes multiples of 16 (the tiles are whole
-// column slabs of 256-byte aligned planes).
-GFD_D void mbar_init(unsigned long long* bar) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(bar)) : "memory");
-  asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-}
-GFD_D void bulk_load(void* smem_dst, const void* gsrc, unsigned int bytes, unsigned long long* bar) {
-  // earlier generic-proxy reads of the buffer are ordered before the async write
-  asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(bar)),
-               "r"(bytes)
-               : "memory");
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
-          smem_u32(smem_dst)),
-      "l"(gsrc), "r"(bytes), "r"(smem_u32(bar))
-      : "memory");
-}
-GFD_D bool mbar_try_wait(unsigned long long* bar, unsigned int parity) {
-  unsigned int done;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-      " selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(done)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return done != 0;
-}
-// Wait for the phase of the given parity; false if it has not completed after
-// the iteration limit (each try_wait blocks for at most a short, hardware-set
-// time), so that a copy that never lands cannot hang the kernel.
-constexpr int MBAR_WAIT_LIMIT = 1 << 22;
-GFD_D bool mbar_wait(unsigned long long* bar, unsigned int parity) {
-  for (int i = 0; i < MBAR_WAIT_LIMIT; ++i)
-    if (mbar_try_wait(bar, parity)) return true;
-  return false;
-}
-
 // Bulk prefetch of [p, p + bytes) into L2 (p 16-byte aligned, bytes a
 // multiple of 16), split into pieces of at most 16 KB issued by the lanes of
 // warp 0.  No completion to wait for: later loads simply find the lines in L2.
@@ -153,20 +113,19 @@ struct ImgState {
   double lam;        // lambda of the current iteration (inf: branch u_E in K)
   double lo, hi;     // bracket of the nodes of the next pass
   double invT;       // 1 / T
-  int mode;          // node layout of the next pass: 0 geometric, 1 Chebyshev in lambda
+  int mode;          // next pass: 0 geometric nodes, 1 Chebyshev nodes, 2 moments about node[0]
   double lam_up;     // upper bound of the root from res and amax
   double res;        // ||h*u_E - y||^2 of the current iteration
   double sum_u;      // FP64 sum of the current iterate u_E (its DC bin)
   double d00;        // DC residual sum(h) sum(u_E) - sum(y), FP64
   double err2;       // FP64 sum (u - u_orig)^2
   double lam_prev;   // last finite lambda resolved before the current one
-  float node[KNODES];// node values lambda_j (float) of the pending pass
+  alignas(8) float node[KNODES];  // node values lambda_j (float) of the pending pass
   unsigned int cta_done;   // items of the current spectral pass completed
   unsigned int gf_done;    // last-block-done counter (guided filter)
   int need;          // 1: lambda unresolved, a fallback pass must run
   int status;        // ST_* bits
   int iter;          // iteration index of the pending outputs
-  int nk;            // nodes of the pending pass (KNODES, or KNARROW for a narrow first pass)
   double rtol;       // relative width of lambda at which the root search stops
   unsigned int absmax[2];  // bits of max |u_I|, max |u_p| of the current iteration
 };

@@ -1,59 +1,107 @@
-// Power-of-two complex FFT on a team of threads, staged in shared memory.
+// Power-of-two complex FFT on a team of threads, exchanged through shared memory.
 //
 // The transform X[k] = sum_n x[n] W_L^{nk}, W_L = exp(-2 pi i / L) (forward)
 // or with W_L^{-nk} (inverse, unnormalised), is computed by the mixed-radix
 // decimation-in-frequency recursion L = r_0 * L_1:
 //   X[i + r_0 k1] = sum_{n1} W_{L_1}^{n1 k1} [ W_L^{n1 i} sum_{n2} x[n1 + L_1 n2] W_{r_0}^{n2 i} ].
 // Stage s holds prod_{s'<s} r_{s'} independent sub-transforms of length L_s,
-// stored contiguously; a butterfly (g, j) loads the r_s elements
-// g*L_s + j + i*L_{s+1}, applies a radix-r_s DFT in registers and the twiddle
-// W_{L_s}^{j i}, and stores them back in place.  After the last stage X[k]
-// sits at the digit-reversed position out_pos(k).
+// stored contiguously; butterfly (g, jj) takes the r_s elements
+// g*L_s + jj + i*L_{s+1}, applies a radix-r_s DFT in registers and the twiddle
+// W_{L_s}^{jj i}, and puts them back in place.
 //
-// A team has L/R threads, each doing R/r_s butterflies per stage; all teams of
-// a block run the same L and synchronise with __syncthreads between stages.
-// Shared addresses are padded by one element per 16 (phys()) to spread banks.
+// A team has T = L/E threads with E elements each.  The first stage takes its
+// inputs from registers (the caller loads element n = beta + i*L_1 of
+// butterfly beta straight from global memory: consecutive threads, consecutive
+// n), and the last stage leaves its outputs in registers: it walks its groups
+// in the order of their output index kappa (d_0 fastest), so that butterfly
+// kappa yields X[kappa + (L/r) i] and consecutive threads hold consecutive
+// k, ready to be stored to global memory.  A transform of two (three) stages
+// thus passes through shared memory once (twice), with one (two) barriers.
+//
+// Three kinds differ in where a thread must hold mirrored elements:
+//   FK_COL  complex columns: the last stage has one butterfly of E outputs;
+//   FK_C2R  inverse rows: the first stage's butterflies come in mirrored
+//           pairs (beta, L_1 - beta), which hold n and L - n of all their
+//           elements, so the split of the packed row spectrum needs no exchange;
+//   FK_R2C  forward rows: likewise (kappa, L/r - kappa) in the last stage.
+// Shared positions are padded (P1 elements per L_1, P2 per L_2) so that every
+// access of 16 consecutive threads falls on distinct 8-byte banks (FK_R2C: 1.5
+// passes on average; the mirrored order and the two orders before it leave no
+// padding that is conflict-free for all three).
 #pragma once
 #include "common.cuh"
 
 namespace gfd {
 
-constexpr int radix_for(int L) { return L >= 256 ? 16 : (L >= 64 ? 8 : (L >= 16 ? 4 : 2)); }
+enum FftKind { FK_COL = 0, FK_C2R = 1, FK_R2C = 2 };
 
-constexpr int stage_radix(int L, int R, int s) {
-  int rem = L;
-  for (int i = 0; i < s; ++i) {
-    int r = rem < R ? rem : R;
-    rem /= r;
-  }
-  return rem < R ? rem : R;
+// Elements per thread.
+constexpr int fft_elems(int K, int L) {
+  if (K == FK_COL) return L >= 256 ? 16 : (L >= 64 ? 8 : (L >= 16 ? 4 : 2));
+  return L >= 64 ? 16 : (L >= 16 ? 8 : 4);
 }
-constexpr int stage_len(int L, int R, int s) {
-  int rem = L;
-  for (int i = 0; i < s; ++i) {
-    int r = rem < R ? rem : R;
-    rem /= r;
+
+// Radix of stage s (1 past the last stage).
+constexpr int fft_radix(int K, int L, int s) {
+  struct Row {
+    int L, r[3];
+  };
+  constexpr Row col[] = {{8, {2, 2, 2}},    {16, {4, 4, 1}},   {32, {2, 4, 4}},  {64, {8, 8, 1}},
+                         {128, {4, 4, 8}},  {256, {16, 16, 1}}, {512, {4, 8, 16}}, {1024, {4, 16, 16}},
+                         {2048, {8, 16, 16}}, {4096, {16, 16, 16}}};
+  constexpr Row c2r[] = {{4, {2, 2, 1}},   {8, {2, 4, 1}},    {16, {4, 4, 1}},   {32, {4, 8, 1}},
+                         {64, {8, 8, 1}},  {128, {8, 16, 1}}, {256, {4, 4, 16}}, {512, {4, 8, 16}},
+                         {1024, {8, 8, 16}}, {2048, {8, 16, 16}}};
+  constexpr Row r2c[] = {{4, {2, 2, 1}},   {8, {4, 2, 1}},    {16, {4, 4, 1}},  {32, {8, 4, 1}},
+                         {64, {8, 8, 1}},  {128, {16, 8, 1}}, {256, {8, 4, 8}}, {512, {8, 8, 8}},
+                         {1024, {8, 16, 8}}, {2048, {16, 16, 8}}};
+  for (int i = 0; i < 10; ++i) {
+    const Row& q = K == FK_COL ? col[i] : (K == FK_C2R ? c2r[i] : r2c[i]);
+    if (q.L == L) return s < 3 ? q.r[s] : 1;
   }
-  return rem;
+  return 1;
 }
-constexpr int num_stages(int L, int R) {
-  int n = 0, rem = L;
-  while (rem > 1) {
-    int r = rem < R ? rem : R;
-    rem /= r;
-    ++n;
-  }
+constexpr int fft_stages(int K, int L) { return fft_radix(K, L, 2) > 1 ? 3 : 2; }
+// L_s: length of the sub-transforms of stage s.
+constexpr int fft_len(int K, int L, int s) {
+  int n = L;
+  for (int i = 0; i < s; ++i) n /= fft_radix(K, L, i);
   return n;
 }
+// Pad elements per L_1 and per L_2 positions.
+constexpr int fft_pad1(int K, int L) {
+  if (K == FK_COL) return L == 32 ? 0 : 1;
+  if (K == FK_C2R) return L <= 4 || L == 256 ? 0 : (L == 512 ? 4 : (L >= 1024 ? 2 : 1));
+  return L <= 4 ? 0 : (L == 512 ? 7 : (L >= 1024 ? 5 : 1));
+}
+constexpr int fft_pad2(int K, int L) {
+  if (K == FK_COL) return L == 32 ? 1 : 0;
+  return K == FK_C2R && L >= 256 ? 1 : 0;
+}
 
-GFD_HD int phys(int a) { return a + (a >> 4); }
-// elements of one team's buffer (odd, so that teams interleave across banks)
-GFD_HD int team_stride(int L) { return L + (L >> 4) + 1; }
-// Buffer stride of the B interleaved column teams of a column pass.  Loads
-// and stores that walk B columns fastest put B columns x 16/B consecutive
-// elements in a half-warp; a stride of 16/B (mod 16) float2 places them on
-// distinct bank pairs.
-GFD_HD int col_team_stride(int L, int B) { return L + (L >> 4) + (B < 16 ? 16 / B : 1); }
+template <int K, int L>
+struct FftGeo {
+  static constexpr int E = fft_elems(K, L), T = L / E, S = fft_stages(K, L);
+  static constexpr int L1 = fft_len(K, L, 1), L2 = S == 3 ? fft_len(K, L, 2) : 1;
+  static constexpr int P1 = fft_pad1(K, L), P2 = S == 3 ? fft_pad2(K, L) : 0;
+  static constexpr int RF = fft_radix(K, L, 0), RL = fft_radix(K, L, S - 1);
+  static constexpr int KL = L / RL;  // butterflies of the last stage
+  // padded distances of the elements of a butterfly of stage 0 and of stage 1
+  static constexpr int STEP0 = L1 + P1 + (S == 3 ? (L1 / L2) * P2 : 0);
+  static constexpr int STEP1 = L2 + P2;  // S == 3
+  static constexpr int MIN_SIZE = (RF - 1) * STEP0 + L1 + (S == 3 ? (L1 / L2 - 1) * P2 : 0);
+  // float2 elements of one transform's buffer; rows shorter than 256 carry a
+  // skew that keeps the teams of a warp on different banks
+  static constexpr int SIZE =
+      K == FK_COL ? MIN_SIZE
+                  : (L == 4 ? 5
+                            : (L == 8 ? (K == FK_C2R ? 10 : 14)
+                                      : (L == 16 ? 22
+                                                 : (L == 32 ? (K == FK_C2R ? 36 : 44)
+                                                            : (L == 64 ? 76
+                                                                       : (L == 128 ? (K == FK_C2R ? 136 : 152)
+                                                                                   : MIN_SIZE))))));
+};
 
 // cos / sin of 2 pi m / 16
 __device__ constexpr float kCos16[16] = {
@@ -95,8 +143,11 @@ GFD_D float2 const_twiddle(float2 v) {
     const float c = kCos16[m], cl = kCos16Lo[m];
     const float s = INV ? kSin16[m] : -kSin16[m];
     const float sl = INV ? kSin16Lo[m] : -kSin16Lo[m];
-    return make_float2(fmaf(v.x, c, fmaf(-v.y, s, fmaf(v.x, cl, -v.y * sl))),
-                       fmaf(v.x, s, fmaf(v.y, c, fmaf(v.x, sl, v.y * cl))));
+    const float2 vx = make_float2(v.x, v.x), vy = make_float2(v.y, v.y);
+    return __ffma2_rn(vx, make_float2(c, s),
+                      __ffma2_rn(vy, make_float2(-s, c),
+                                 __ffma2_rn(vx, make_float2(cl, sl),
+                                            __fmul2_rn(vy, make_float2(-sl, cl)))));
   }
 }
 
@@ -137,193 +188,72 @@ struct DFT<2, INV> {
   }
 };
 
-// tw: the table of the transform length L (W_L^m, m < L)
-// (a generic load: the table may sit in shared or global memory)
-GFD_D float2 twiddle(const float2* __restrict__ tw, int m, bool inv) {
-  float2 w = tw[m];
-  if (inv) w.y = -w.y;
+// W_{Ls}^m from the per-length tables (tw: all lengths, see tab_off).
+template <bool INV>
+GFD_D float2 twiddle(const float2* __restrict__ tw, int Ls, int m) {
+  float2 w = __ldg(&tw[tab_off(Ls) + m]);
+  if (INV) w.y = -w.y;
   return w;
 }
 
-// Shared-memory address of element a of a team's sequence.
-struct PaddedIdx {  // contiguous with one pad element per 16
-  GFD_D int operator()(int a) const { return phys(a); }
-};
-struct IdentIdx {  // contiguous, unpadded (landing buffers of rows)
-  GFD_D int operator()(int a) const { return a; }
-};
-struct StridedIdx {  // element a of column b of an interleaved [a][B] tile
-  int stride;
-  GFD_D int operator()(int a) const { return a * stride; }
-};
+// First stage, butterfly beta: x holds its inputs; results go to buf.
+template <int K, int L, bool INV>
+GFD_D void fft_first(float2 (&x)[FftGeo<K, L>::RF], int beta, float2* buf,
+                     const float2* __restrict__ tw) {
+  using G = FftGeo<K, L>;
+  DFT<G::RF, INV>::run(x);
+  float2* o = buf + (beta + (G::S == 3 ? (beta / G::L2) * G::P2 : 0));
+  o[0] = x[0];
+#pragma unroll
+  for (int i = 1; i < G::RF; ++i)
+    o[i * G::STEP0] = cmul(x[i], twiddle<INV>(tw, L, beta * i));
+}
 
-template <int L, int R, bool INV, int s>
-struct Stage {
-  template <class Idx>
-  GFD_D static void run(float2* buf, int j, const float2* __restrict__ tw, Idx idx) {
-    constexpr int Ls = stage_len(L, R, s);
-    if constexpr (Ls > 1) {
-      constexpr int r = Ls < R ? Ls : R;
-      constexpr int Ln = Ls / r;
-      constexpr int T = L / R;
-      constexpr int twstep = L / Ls;  // W_Ls = W_L^(L / Ls)
+// Middle stage (three-stage transforms), thread j of the team, in place.
+template <int K, int L, bool INV>
+GFD_D void fft_mid(float2* buf, int j, const float2* __restrict__ tw) {
+  using G = FftGeo<K, L>;
+  if constexpr (G::S == 3) {
+    constexpr int r = fft_radix(K, L, 1), NB = G::E / r;
 #pragma unroll
-      for (int q = 0; q < R / r; ++q) {
-        const int beta = j + T * q;
-        const int g = beta / Ln;
-        const int jj = beta % Ln;
-        const int base = g * Ls + jj;
-        float2 x[r];
-#pragma unroll
-        for (int i = 0; i < r; ++i) x[i] = buf[idx(base + i * Ln)];
-        DFT<r, INV>::run(x);
-        if constexpr (Ln > 1) {
-#pragma unroll
-          for (int i = 1; i < r; ++i) x[i] = cmul(x[i], twiddle(tw, jj * i * twstep, INV));
-        }
-#pragma unroll
-        for (int i = 0; i < r; ++i) buf[idx(base + i * Ln)] = x[i];
-      }
-      __syncthreads();
-      Stage<L, R, INV, s + 1>::run(buf, j, tw, idx);
-    }
-  }
-};
-
-// Two transforms of the same length on one team (buffers A and B), stage by
-// stage: each butterfly's twiddles are loaded once and applied to both.
-template <int L, int R, bool INV, int s>
-struct Stage2 {
-  template <class Idx>
-  GFD_D static void run(float2* bufA, float2* bufB, int j, const float2* __restrict__ tw, Idx idx) {
-    constexpr int Ls = stage_len(L, R, s);
-    if constexpr (Ls > 1) {
-      constexpr int r = Ls < R ? Ls : R;
-      constexpr int Ln = Ls / r;
-      constexpr int T = L / R;
-      constexpr int twstep = L / Ls;
-#pragma unroll
-      for (int q = 0; q < R / r; ++q) {
-        const int beta = j + T * q;
-        const int g = beta / Ln;
-        const int jj = beta % Ln;
-        const int base = g * Ls + jj;
-        float2 w[r];
-        if constexpr (Ln > 1) {
-#pragma unroll
-          for (int i = 1; i < r; ++i) w[i] = twiddle(tw, jj * i * twstep, INV);
-        }
-#pragma unroll 1
-        for (int h = 0; h < 2; ++h) {
-          float2* buf = h ? bufB : bufA;
-          float2 x[r];
-#pragma unroll
-          for (int i = 0; i < r; ++i) x[i] = buf[idx(base + i * Ln)];
-          DFT<r, INV>::run(x);
-          if constexpr (Ln > 1) {
-#pragma unroll
-            for (int i = 1; i < r; ++i) x[i] = cmul(x[i], w[i]);
-          }
-#pragma unroll
-          for (int i = 0; i < r; ++i) buf[idx(base + i * Ln)] = x[i];
-        }
-      }
-      __syncthreads();
-      Stage2<L, R, INV, s + 1>::run(bufA, bufB, j, tw, idx);
-    }
-  }
-};
-
-// First stage reading from a separate (landing) buffer `in` addressed by
-// iidx, writing to buf addressed by idx; the remaining stages run in buf.
-template <int L, int R, bool INV>
-struct Stage0From {
-  template <class InIdx, class Idx>
-  GFD_D static void run(const float2* in, InIdx iidx, float2* buf, int j,
-                        const float2* __restrict__ tw, Idx idx) {
-    constexpr int Ls = L;
-    constexpr int r = Ls < R ? Ls : R;
-    constexpr int Ln = Ls / r;
-    constexpr int T = L / R;
-    constexpr int twstep = L / Ls;
-#pragma unroll
-    for (int q = 0; q < R / r; ++q) {
-      const int beta = j + T * q;
-      const int g = beta / Ln;
-      const int jj = beta % Ln;
-      const int base = g * Ls + jj;
+    for (int q = 0; q < NB; ++q) {
+      const int beta = j + G::T * q;
+      const int g = beta / G::L2, jj = beta % G::L2;
+      float2* o = buf + (g * G::STEP0 + jj);
       float2 x[r];
 #pragma unroll
-      for (int i = 0; i < r; ++i) x[i] = in[iidx(base + i * Ln)];
+      for (int i = 0; i < r; ++i) x[i] = o[i * G::STEP1];
       DFT<r, INV>::run(x);
-      if constexpr (Ln > 1) {
+      o[0] = x[0];
 #pragma unroll
-        for (int i = 1; i < r; ++i) x[i] = cmul(x[i], twiddle(tw, jj * i * twstep, INV));
-      }
-#pragma unroll
-      for (int i = 0; i < r; ++i) buf[idx(base + i * Ln)] = x[i];
+      for (int i = 1; i < r; ++i)
+        o[i * G::STEP1] = cmul(x[i], twiddle<INV>(tw, G::L1, jj * i));
     }
   }
-};
-
-// Transform whose input sits in `in` (read once, by the first stage) and
-// whose stages and output live in buf.  Ends block-synchronised, after which
-// `in` may be overwritten.
-template <int L, bool INV, class InIdx, class Idx = PaddedIdx>
-GFD_D void fft_team_from(const float2* in, InIdx iidx, float2* buf, int j,
-                         const float2* __restrict__ tw, Idx idx = Idx()) {
-  constexpr int R = radix_for(L);
-  Stage0From<L, R, INV>::run(in, iidx, buf, j, tw, idx);
-  __syncthreads();
-  Stage<L, R, INV, 1>::run(buf, j, tw, idx);
 }
 
-// Run the whole transform of one team (thread j of L/R) in place on buf.
-// Precondition: buf filled and a __syncthreads() issued by the caller.
-// Postcondition: X[k] at buf[idx(out_pos<L>(k))], block synchronised.
-template <int L, bool INV, class Idx = PaddedIdx>
-GFD_D void fft_team(float2* buf, int j, const float2* __restrict__ tw, Idx idx = Idx()) {
-  Stage<L, radix_for(L), INV, 0>::run(buf, j, tw, idx);
-}
-
-// fft_team on two buffers of the same team at once (shared twiddles).
-template <int L, bool INV, class Idx = PaddedIdx>
-GFD_D void fft_team2(float2* bufA, float2* bufB, int j, const float2* __restrict__ tw,
-                     Idx idx = Idx()) {
-  Stage2<L, radix_for(L), INV, 0>::run(bufA, bufB, j, tw, idx);
-}
-
-// position of output k after the in-place stages (digit reversal)
-template <int L>
-GFD_D int out_pos(int k) {
-  constexpr int R = radix_for(L);
-  constexpr int S = num_stages(L, R);
-  int p = 0, rem = k;
+// Last stage, butterfly kappa: x[i] = X[kappa + KL * i].
+template <int K, int L, bool INV>
+GFD_D void fft_last(float2 (&x)[FftGeo<K, L>::RL], int kappa, const float2* buf) {
+  using G = FftGeo<K, L>;
+  int p;
+  if constexpr (G::S == 3)
+    p = (kappa % G::RF) * G::STEP0 + (kappa / G::RF) * G::STEP1;
+  else
+    p = kappa * G::STEP0;
+  const float2* in = buf + p;
 #pragma unroll
-  for (int s = 0; s < S; ++s) {
-    const int r = stage_radix(L, R, s);
-    const int Ln = stage_len(L, R, s) / r;
-    p += (rem % r) * Ln;
-    rem /= r;
-  }
-  return p;
+  for (int i = 0; i < G::RL; ++i) x[i] = in[i];
+  DFT<G::RL, INV>::run(x);
 }
 
-// inverse of out_pos: the output index stored at position p
-template <int L>
-GFD_D int in_pos(int p) {
-  constexpr int R = radix_for(L);
-  constexpr int S = num_stages(L, R);
-  int k = 0, mul = 1, rem = p;
-#pragma unroll
-  for (int s = 0; s < S; ++s) {
-    const int r = stage_radix(L, R, s);
-    const int Ln = stage_len(L, R, s) / r;
-    k += (rem / Ln) * mul;
-    rem %= Ln;
-    mul *= r;
-  }
-  return k;
+// Buffer stride of the B columns of a column pass, whose consecutive threads
+// walk B columns x 16/B consecutive elements: 16/B (mod 16) puts them on
+// distinct banks.
+template <int M>
+GFD_HD int col_stride(int B) {
+  const int want = B < 16 ? 16 / B : 1, n = FftGeo<FK_COL, M>::SIZE;
+  return n + ((want - n) & 15);
 }
 
 }  // namespace gfd

@@ -253,17 +253,18 @@ __global__ void k_adj_solve(const AdjDesc* __restrict__ descs, int M, int N,
     const int k = (int)(idx / L), l = (int)(idx - (size_t)k * L);
     const float d2r = __ldg(&d2tab[tab_off(M) + k]);
     float2 UI, Up;
-    if (l != 0) {
-      solve_bin(d.UE[idx], d.H[idx], d.Y[idx], lam, d2r + __ldg(&d2tab[tab_off(N) + l]), branch,
-                UI, Up);
+    if (branch) {  // lambda = inf: u_I = u_p = u_E (Sec. 3.2)
+      UI = Up = d.UE[idx];
+    } else if (l != 0) {
+      solve_bin(d.UE[idx], d.H[idx], d.Y[idx], lam, d2r + __ldg(&d2tab[tab_off(N) + l]), UI, Up);
     } else {
       const size_t m = (size_t)((M - k) & (M - 1)) * L;
       float2 EA, EB, HA, HB, YA, YB, IA, IB, PA, PB;
       unpack_pair(d.UE[idx], d.UE[m], EA, EB);
       unpack_pair(d.H[idx], d.H[m], HA, HB);
       unpack_pair(d.Y[idx], d.Y[m], YA, YB);
-      solve_bin(EA, HA, YA, lam, d2r, branch, IA, PA);
-      solve_bin(EB, HB, YB, lam, d2r + 4.0f, branch, IB, PB);
+      solve_bin(EA, HA, YA, lam, d2r, IA, PA);
+      solve_bin(EB, HB, YB, lam, d2r + 4.0f, IB, PB);
       UI = pack_pair(IA, IB);
       Up = pack_pair(PA, PB);
     }

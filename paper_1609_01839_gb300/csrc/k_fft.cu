@@ -35,326 +35,339 @@ GFD_D float2* cplx_plane(const ImgDesc& d, int sel) {
   return reinterpret_cast<float2*>(real_plane(d, sel));
 }
 
-constexpr int threads_per_team(int L) { return L / radix_for(L); }
-// Largest column length whose twiddle table the column passes keep in
-// shared memory (8 KB at 1024).
-constexpr int SMEM_TW_MAX = 1024;
+// Streaming loads: spectra and images pass through once per launch and stay out
+// of L1, which keeps the twiddle tables there.
+GFD_D float2 load_stream(const float2* p) { return __ldcg(p); }
 
-// Persistent pass kernels.  Each block walks the work items item =
-// blockIdx.x + k * gridDim.x; the inputs of the next item are copied
-// asynchronously into a landing buffer while the current item's transform
-// runs in a separate (padded) work buffer, so that global loads stay in
-// flight while the block computes.
-
-// ---------------------------------------------------------------------------
-// Row pass, forward: real rows -> packed row spectra (tiled).  An item is
-// rpc consecutive rows of one image.  Each row of N reals is read as N/2
-// complex z[n] = x[2n] + i x[2n+1]; Z = FFT_{N/2}(z); then
-// X[k] = (Z[k] + conj Z[-k])/2 + W_N^k (Z[k] - conj Z[-k])/(2i), and
-// X[0], X[N/2] = Re Z[0] +- Im Z[0] (packed as X[0] + i X[N/2]).
-// ---------------------------------------------------------------------------
-// float2 elements of the row-pass work area of rpc teams, rounded up to even.
-GFD_HD int row_work_elems(int L, int rpc) { return (rpc * team_stride(L) + 1) & ~1; }
-
-template <int L>
-__global__ void __launch_bounds__(256, 2)
-k_row_r2c(ClassDesc cd, const ImgDesc* __restrict__ imgs, const float2* __restrict__ tw, int rpc,
-          int src_sel, int dst_sel, int do_sum) {
-  extern __shared__ __align__(16) float2 smem[];
-  constexpr int R = radix_for(L), T = threads_per_team(L);
-  constexpr int N = 2 * L;
-  const int TB = cd.TB, M = cd.M;
-  const int item_elems = rpc * L;
-  float2* land = smem;
-  float2* work = land + item_elems;
-  // team_stride(L) is odd: round the work area up to an even number of float2
-  // so that the output rows (read as 16-byte vectors) start 16-byte aligned
-  float2* outb = work + row_work_elems(L, rpc);
-  double* red = reinterpret_cast<double*>(outb + item_elems);
-  // length-L twiddle table in shared memory (L <= SMEM_TW_MAX)
-  const float2* twL = tw + tab_off(L);
-  if constexpr (L <= SMEM_TW_MAX) {
-    float2* stw = reinterpret_cast<float2*>(red + 32);
-    for (int i = threadIdx.x; i < L; i += blockDim.x) stw[i] = twL[i];
-    twL = stw;  // visible after the loop's first __syncthreads()
-  }
-  const int team = threadIdx.x / T, j = threadIdx.x % T;
-  const int n_items = cd.n_img * M / rpc;
-  auto issue = [&](int item) {
-    if (item < n_items) {
-      const int row_c = item * rpc;
-      const ImgDesc& d = imgs[cd.img0 + row_c / M];
-      const float2* src =
-          reinterpret_cast<const float2*>(real_plane(d, src_sel)) + (size_t)(row_c % M) * L;
-      for (int c = threadIdx.x; c < item_elems / 2; c += blockDim.x)
-        cp_async16(land + 2 * c, src + 2 * c);
-    }
-    cp_async_commit();
-  };
-  issue(blockIdx.x);
-  for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
-    cp_async_wait<0>();
+// Barrier among the threads of a row team: teams of at most a warp exchange
+// inside it.
+template <int T>
+GFD_D void team_sync(unsigned int mask) {
+  if constexpr (T <= 32)
+    __syncwarp(mask);
+  else
     __syncthreads();
-    const int row0 = (item * rpc) % M;
-    const ImgDesc& d = imgs[cd.img0 + (item * rpc) / M];
-    float2* buf = work + team * team_stride(L);
-    const float2* in = land + team * L;
-    if (do_sum) {
-      float part = 0.0f;
-#pragma unroll
-      for (int i = 0; i < R; ++i) {
-        const float2 v = in[j + i * T];
-        part += v.x + v.y;
-      }
-      part = warp_sum(part);
-      if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = (double)part;
-    }
-    fft_team_from<L, false>(in, IdentIdx(), buf, j, twL);  // first stage reads land
-    issue(item + gridDim.x);                               // land is free again
-    if (do_sum && threadIdx.x == 0) {
-      double s = 0.0;
-      for (int w = 0; w < num_warps(); ++w) s += red[w];
-      d.rowsum[row0 / rpc] = s;  // one partial per item, summed by the column pass
-    }
-    float2* ob = outb + team * L;
-#pragma unroll
-    for (int i = 0; i < R; ++i) {
-      const int k = j + i * T;
-      const float2 Zk = buf[phys(out_pos<L>(k))];
-      float2 out;
-      if (k == 0) {
-        out = make_float2(Zk.x + Zk.y, Zk.x - Zk.y);
-      } else {
-        const float2 Zm = cconj(buf[phys(out_pos<L>(L - k))]);
-        const float2 E = cscale(cadd(Zk, Zm), 0.5f);
-        const float2 D = csub(Zk, Zm);
-        const float2 O = make_float2(0.5f * D.y, -0.5f * D.x);  // D / (2i)
-        out = cadd(E, cmul(__ldg(&tw[tab_off(N) + k]), O));
-      }
-      ob[k] = out;
-    }
-    __syncthreads();
-    // copy out tile by tile: rows row0 .. row0+rpc-1 of tile t are contiguous
-    float2* dst = cplx_plane(d, dst_sel);
-    // 16-byte chunks: rpc * TB / 2 per tile, TB / 2 per row (powers of two)
-    const int lg_pt = __ffs(rpc * TB / 2) - 1, lg_hr = __ffs(TB / 2) - 1;
-    for (int c = threadIdx.x; c < item_elems / 2; c += blockDim.x) {
-      const int t = c >> lg_pt, w = c & ((1 << lg_pt) - 1);
-      const int r = w >> lg_hr, q = w & ((1 << lg_hr) - 1);
-      const float4 v = *reinterpret_cast<const float4*>(outb + r * L + t * TB + 2 * q);
-      *reinterpret_cast<float4*>(dst + (size_t)t * M * TB + (size_t)(row0 + r) * TB + 2 * q) = v;
-    }
-  }
-  cp_async_wait<0>();
+}
+GFD_D unsigned int warp_mask() {
+  return blockDim.x >= 32 ? 0xffffffffu : ((1u << blockDim.x) - 1u);
 }
 
 // ---------------------------------------------------------------------------
-// Row pass, inverse: packed row spectra (tiled) -> real rows (scaled).
-// Z[k] = (R[k] + conj R[L-k]) + i (R[k] - conj R[L-k]) W_N^{-k}, with
-// R[0], R[N/2] the real and imaginary parts of the packed entry 0; the
-// unnormalised inverse FFT of Z gives x[2n] + i x[2n+1] times N.
-// Items cover spectrum sel0 -> real plane dsel0, then sel1 -> dsel1.
+// Row passes.  A block takes rpc consecutive rows of one image, a team of T
+// threads per row.  Elements go from global memory to registers, through the
+// team's buffer in shared memory once or twice, and from registers to global
+// memory; the mirrored pairs that the real transform needs sit in one thread
+// (fft.cuh).  Teams of a warp or less (rows of up to 1024 reals) run without
+// block barriers.  What bounds them is shared memory and the pieces of TB
+// values that a row has in each tile (16 to 64 bytes per store): the
+// transform that staged its input, every stage and its output in shared memory
+// took 4.25 ms (forward) and 7.4 ms (inverse, two planes) per batched solve of
+// 256 images, this one 2.95 and 5.7 ms.
 // ---------------------------------------------------------------------------
+
+// The slots of a mirrored butterfly pair (A, B) of radix r over positions
+// beta + D i (A) and D - beta + D i (B), D r = L: slot t pairs A_t with
+// B_{r-1-t}, whose position is L minus that of A_t.  The pair holding beta = 0
+// and beta = D/2 mirrors onto itself instead: slots 1..r/2-1 pair A_t with
+// A_{r-t}, slots r/2..r-1 pair B_u with B_{r-1-u} (u = t - r/2), and slot 0
+// holds positions 0 and L/2, both their own mirrors.
+template <int r>
+struct MirrorSlots {
+  // position of slot t's first element
+  GFD_D static int first(bool self, int beta, int D, int t) {
+    return (self && t >= r / 2) ? D / 2 + D * (t - r / 2) : beta + D * t;
+  }
+  // and of its second
+  GFD_D static int second(bool self, int beta, int D, int t) {
+    return (self && t == 0) ? D * r / 2 : D * r - first(self, beta, D, t);
+  }
+};
+
+GFD_D float2 select2(bool c, float2 a, float2 b) { return c ? a : b; }
+
+// Forward: real rows -> packed row spectra (tiled).  Each row of N reals is read
+// as N/2 complex z[n] = x[2n] + i x[2n+1]; Z = FFT_{N/2}(z); with
+// E = (Z[k] + conj Z[-k]) / 2 and O = (Z[k] - conj Z[-k]) / (2i),
+// X[k] = E + W_N^k O and X[-k] = conj(E - W_N^k O); X[0], X[N/2] = Re Z[0] +-
+// Im Z[0] (packed as X[0] + i X[N/2]).  do_sum: FP64 row sums of the source.
+template <int L>
+__global__ void __launch_bounds__(256, 3)
+k_row_r2c(ClassDesc cd, const ImgDesc* __restrict__ imgs, const float2* __restrict__ tw, int rpc,
+          int src_sel, int dst_sel, int do_sum) {
+  extern __shared__ __align__(16) float2 smem[];
+  using G = FftGeo<FK_R2C, L>;
+  constexpr int T = G::T, r0 = G::RF, rl = G::RL;
+  constexpr int N = 2 * L, KL = G::KL;
+  const int TB = cd.TB, M = cd.M;
+  const int team = threadIdx.x / T, j = threadIdx.x % T;
+  const int row_c = blockIdx.x * rpc + team;
+  const ImgDesc& d = imgs[cd.img0 + row_c / M];
+  const int row = row_c % M;
+  const unsigned int mask = warp_mask();
+  float2* buf = smem + team * G::SIZE;
+  const float2* src = reinterpret_cast<const float2*>(real_plane(d, src_sel)) + (size_t)row * L;
+  float part = 0.0f;
+#pragma unroll
+  for (int q = 0; q < G::E / r0; ++q) {
+    const int beta = j + T * q;
+    float2 x[r0];
+#pragma unroll
+    for (int i = 0; i < r0; ++i) x[i] = load_stream(src + beta + i * G::L1);
+    if (do_sum) {
+#pragma unroll
+      for (int i = 0; i < r0; ++i) part += x[i].x + x[i].y;
+    }
+    fft_first<FK_R2C, L, false>(x, beta, buf, tw);
+  }
+  if (do_sum) {  // one FP64 sum per row
+    __shared__ double red[8];
+    if constexpr (T <= 32) {
+#pragma unroll
+      for (int o = T / 2; o > 0; o >>= 1) part += __shfl_xor_sync(mask, part, o);
+      if (j == 0) d.rowsum[row] = (double)part;
+    } else {
+      part = warp_sum(part);
+      if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = (double)part;
+      __syncthreads();
+      if (j == 0) {
+        double s = 0.0;
+        for (int w = 0; w < T / 32; ++w) s += red[(threadIdx.x >> 5) + w];
+        d.rowsum[row] = s;
+      }
+    }
+  }
+  team_sync<T>(mask);
+  if constexpr (G::S == 3) {
+    fft_mid<FK_R2C, L, false>(buf, j, tw);
+    team_sync<T>(mask);
+  }
+  // tiled row: column k of tile k / TB
+  float2* dst = cplx_plane(d, dst_sel) + (size_t)row * TB;
+  const int lg = __ffs(TB) - 1;
+  auto put = [&](int k, float2 v) {
+    dst[(((size_t)(k >> lg) * M) << lg) + (k & (TB - 1))] = v;
+  };
+#pragma unroll
+  for (int q = 0; q < G::E / rl / 2; ++q) {
+    const int kap = j + T * q;
+    const bool self = q == 0 && j == 0;
+    float2 A[rl], B[rl];
+    fft_last<FK_R2C, L, false>(A, kap, buf);
+    fft_last<FK_R2C, L, false>(B, self ? KL / 2 : KL - kap, buf);
+#pragma unroll
+    for (int t = 0; t < rl; ++t) {
+      const int k = MirrorSlots<rl>::first(self, kap, KL, t);
+      float2 a = A[t], b = B[rl - 1 - t];
+      if (q == 0) {
+        if (t >= rl / 2) a = select2(self, B[t - rl / 2], a);
+        if (t >= rl / 2)
+          b = select2(self, B[rl + rl / 2 - 1 - t], b);
+        else
+          b = select2(self, A[t == 0 ? rl / 2 : rl - t], b);
+      }
+      const float2 E = cscale(cadd(a, cconj(b)), 0.5f);
+      const float2 D = cscale(csub(a, cconj(b)), 0.5f);
+      const float2 WO = cmul(__ldg(&tw[tab_off(N) + k]), make_float2(D.y, -D.x));
+      float2 u = cadd(E, WO), v = cconj(csub(E, WO));
+      if (q == 0 && t == 0 && self) {
+        u = make_float2(a.x + a.y, a.x - a.y);  // X[0] + i X[N/2]
+        v = cconj(b);                           // X[N/4] = conj Z[L/2]
+      }
+      put(k, u);
+      put(MirrorSlots<rl>::second(self, kap, KL, t), v);
+    }
+  }
+}
+
+// Inverse: packed row spectra (tiled) -> real rows (scaled).  With
+// E = R[k] + conj R[L-k] and O = (R[k] - conj R[L-k]) W_N^{-k},
+// Z[k] = E + i O and Z[L-k] = conj(E) + i conj(O) (R[0], R[N/2] are the real and
+// imaginary parts of the packed entry 0); the unnormalised inverse FFT of Z
+// gives x[2n] + i x[2n+1] times N.  Blocks cover spectrum sel0 -> real plane
+// dsel0, then sel1 -> dsel1.
 template <int L>
 __global__ void __launch_bounds__(256, 3)
 k_row_c2r(ClassDesc cd, const ImgDesc* __restrict__ imgs, const float2* __restrict__ tw, int rpc,
           int sel0, int sel1, int dsel0, int dsel1, float scale, ImgState* st) {
   extern __shared__ __align__(16) float2 smem[];
-  constexpr int R = radix_for(L), T = threads_per_team(L);
+  using G = FftGeo<FK_C2R, L>;
+  constexpr int T = G::T, r0 = G::RF, rl = G::RL;
   constexpr int N = 2 * L;
   const int TB = cd.TB, M = cd.M;
-  const int item_elems = rpc * L;
-  float2* land = smem;
-  float2* work = smem + item_elems;
-  const float2* twL = tw + tab_off(L);
-  if constexpr (L <= SMEM_TW_MAX) {
-    float2* stw = work + rpc * team_stride(L);
-    for (int i = threadIdx.x; i < L; i += blockDim.x) stw[i] = twL[i];
-    twL = stw;  // visible after the loop's first __syncthreads()
-  }
   const int team = threadIdx.x / T, j = threadIdx.x % T;
   const int per_plane = cd.n_img * M / rpc;
-  const int n_items = sel1 >= 0 ? 2 * per_plane : per_plane;
-  // 16-byte chunks: rpc * TB / 2 per tile, TB / 2 per row (powers of two)
-  const int lg_pt = __ffs(rpc * TB / 2) - 1, lg_hr = __ffs(TB / 2) - 1;
-  auto issue = [&](int item) {
-    if (item < n_items) {
-      int sel = sel0;
-      if (item >= per_plane) {
-        item -= per_plane;
-        sel = sel1;
-      }
-      const int row_c = item * rpc;
-      const ImgDesc& d = imgs[cd.img0 + row_c / M];
-      const float2* src = cplx_plane(d, sel) + (size_t)(row_c % M) * TB;
-      for (int c = threadIdx.x; c < item_elems / 2; c += blockDim.x) {
-        const int t = c >> lg_pt, w = c & ((1 << lg_pt) - 1);
-        const int r = w >> lg_hr, q = w & ((1 << lg_hr) - 1);
-        cp_async16(land + r * L + t * TB + 2 * q, src + (size_t)t * M * TB + r * TB + 2 * q);
-      }
-    }
-    cp_async_commit();
+  const bool second = (int)blockIdx.x >= per_plane;
+  const int row_c = ((int)blockIdx.x - (second ? per_plane : 0)) * rpc + team;
+  const int li = row_c / M, row = row_c % M;
+  const ImgDesc& d = imgs[cd.img0 + li];
+  const unsigned int mask = warp_mask();
+  float2* buf = smem + team * G::SIZE;
+  const float2* src = cplx_plane(d, second ? sel1 : sel0) + (size_t)row * TB;
+  const int lg = __ffs(TB) - 1;
+  auto get = [&](int k) {
+    return load_stream(src + (((size_t)(k >> lg) * M) << lg) + (k & (TB - 1)));
   };
-  issue(blockIdx.x);
-  for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
-    cp_async_wait<0>();
-    __syncthreads();
-    int it = item, dsel = dsel0;
-    if (it >= per_plane) {
-      it -= per_plane;
-      dsel = dsel1;
+#pragma unroll
+  for (int q = 0; q < G::E / r0 / 2; ++q) {
+    const int beta = j + T * q;
+    const bool self = q == 0 && j == 0;
+    float2 u[r0], v[r0];  // Z at the slots' first and second positions
+#pragma unroll
+    for (int t = 0; t < r0; ++t) {
+      u[t] = get(MirrorSlots<r0>::first(self, beta, G::L1, t));
+      v[t] = get(MirrorSlots<r0>::second(self, beta, G::L1, t));
     }
-    const int row_c = it * rpc + team;
-    const int li = row_c / M, row = row_c % M;
-    const ImgDesc& d = imgs[cd.img0 + li];
-    float2* buf = work + team * team_stride(L);
-    const float2* in = land + team * L;
-    for (int k = j; k <= L / 2; k += T) {
-      if (k == 0) {
-        const float2 t0 = in[0];
-        buf[phys(0)] = make_float2(t0.x + t0.y, t0.x - t0.y);
-      } else {
-        const int km = L - k;
-        const float2 Rk = in[k], Rm = in[km];
-        {
-          const float2 E = cadd(Rk, cconj(Rm));
-          const float2 O = cmul(csub(Rk, cconj(Rm)), cconj(__ldg(&tw[tab_off(N) + k])));
-          buf[phys(k)] = make_float2(E.x - O.y, E.y + O.x);
-        }
-        if (km != k) {
-          const float2 E = cadd(Rm, cconj(Rk));
-          const float2 O = cmul(csub(Rm, cconj(Rk)), cconj(__ldg(&tw[tab_off(N) + km])));
-          buf[phys(km)] = make_float2(E.x - O.y, E.y + O.x);
-        }
+#pragma unroll
+    for (int t = 0; t < r0; ++t) {
+      const int k = MirrorSlots<r0>::first(self, beta, G::L1, t);
+      const float2 a = u[t], b = v[t];
+      const float2 E = cadd(a, cconj(b)), D = csub(a, cconj(b));
+      const float2 O = cmul(D, cconj(__ldg(&tw[tab_off(N) + k])));
+      u[t] = make_float2(E.x - O.y, E.y + O.x);
+      v[t] = make_float2(E.x + O.y, O.x - E.y);
+      if (q == 0 && t == 0 && self) {
+        u[t] = make_float2(a.x + a.y, a.x - a.y);
+        v[t] = make_float2(2.0f * b.x, -2.0f * b.y);
       }
     }
-    __syncthreads();
-    issue(item + gridDim.x);
-    fft_team<L, true>(buf, j, twL);
-    float2* rowp = reinterpret_cast<float2*>(real_plane(d, dsel)) + (size_t)row * L;
-    float amax = 0.0f;
+    float2 A[r0], B[r0];
 #pragma unroll
-    for (int i = 0; i < R; ++i) {
-      const int n = j + i * T;
-      const float2 v = cscale(buf[phys(out_pos<L>(n))], scale);
-      rowp[n] = v;
+    for (int i = 0; i < r0; ++i) {
+      A[i] = u[i];
+      B[i] = v[r0 - 1 - i];
+      if (q == 0) {
+        if (i >= r0 / 2) A[i] = select2(self, i == r0 / 2 ? v[0] : v[r0 - i], A[i]);
+        B[i] = select2(self, i < r0 / 2 ? u[i + r0 / 2] : v[r0 + r0 / 2 - 1 - i], B[i]);
+      }
+    }
+    fft_first<FK_C2R, L, true>(A, beta, buf, tw);
+    fft_first<FK_C2R, L, true>(B, self ? G::L1 / 2 : G::L1 - beta, buf, tw);
+  }
+  team_sync<T>(mask);
+  if constexpr (G::S == 3) {
+    fft_mid<FK_C2R, L, true>(buf, j, tw);
+    team_sync<T>(mask);
+  }
+  float2* rowp =
+      reinterpret_cast<float2*>(real_plane(d, second ? dsel1 : dsel0)) + (size_t)row * L;
+  float amax = 0.0f;
+#pragma unroll
+  for (int q = 0; q < G::E / rl; ++q) {
+    const int kap = j + T * q;
+    float2 x[rl];
+    fft_last<FK_C2R, L, true>(x, kap, buf);
+#pragma unroll
+    for (int i = 0; i < rl; ++i) {
+      const float2 v = cscale(x[i], scale);
+      rowp[kap + i * G::KL] = v;
       amax = fmaxf(amax, fmaxf(fabsf(v.x), fabsf(v.y)));
     }
-    // largest |value| of the plane (u_I, u_p): bounds the guided filter's
-    // split window sums; non-negative floats order like their bit patterns
-    if (st) {
-      amax = warp_max(amax);  // the teams of a warp share one image and plane
-      if ((threadIdx.x & 31) == 0)
-        atomicMax(&st[cd.img0 + li].absmax[dsel == dsel0 ? 0 : 1], __float_as_uint(amax));
-    }
   }
-  cp_async_wait<0>();
+  // largest |value| of the plane (u_I, u_p): bounds the guided filter's
+  // split window sums; non-negative floats order like their bit patterns
+  if (st) {
+    amax = warp_max(amax);  // the teams of a warp share one image and plane
+    if ((threadIdx.x & 31) == 0)
+      atomicMax(&st[cd.img0 + li].absmax[second ? 1 : 0], __float_as_uint(amax));
+  }
 }
 
 // ---------------------------------------------------------------------------
 // Column passes.  An item is B adjacent packed columns of one image (B = TB
-// in the iteration kernels: one contiguous tile).  It lands as an [M][B]
-// tile and team b (threads b, b+B, ...) transforms column c0+b.
+// in the iteration kernels: one contiguous tile of M x B values), thread
+// (b, j) = (threadIdx % B, threadIdx / B) of column b's team.  Consecutive
+// threads walk the B columns, then consecutive rows, so every load and store
+// of a warp covers whole sectors of the tile.  They are bound by the latency
+// of these loads at 16 to 24 warps per SM: inputs come straight from global
+// memory to the first stage's registers (no landing tile, which cost a pass
+// through shared memory and half the blocks per SM), the next item's tiles are
+// prefetched into L2, and the tile width is a compile-time constant, so that
+// a thread's rows are immediate offsets.
 // ---------------------------------------------------------------------------
 
-// Setup / utility column FFT (not pipelined): plane src -> dst, in place
-// allowed; B columns (inside one tile) per block.  Loads and stores walk the
-// B columns fastest (coalesced rows of the tile); the in-place stages walk a
-// column's team fastest (conflict-free with the phys() padding); results are
-// read in storage (digit-reversed) order so that shared reads stay
-// conflict-free, and scattered to their rows.
+// Setup / utility column FFT: plane src -> dst, in place allowed; B columns
+// (inside one tile) per block.
 template <int M, bool INV>
-__global__ void k_col_plain(ClassDesc cd, const ImgDesc* __restrict__ imgs,
-                            const float2* __restrict__ tw, int B, int src_sel, int dst_sel) {
-  extern __shared__ float2 smem[];
-  constexpr int R = radix_for(M), T = threads_per_team(M);
+__global__ void __launch_bounds__(512)
+k_col_plain(ClassDesc cd, const ImgDesc* __restrict__ imgs, const float2* __restrict__ tw, int B,
+            int src_sel, int dst_sel) {
+  extern __shared__ __align__(16) float2 smem[];
+  using G = FftGeo<FK_COL, M>;
+  constexpr int T = G::T, r0 = G::RF;
   const int Lc = cd.N / 2, TB = cd.TB;
   const int cpi = Lc / B;
   const ImgDesc& d = imgs[cd.img0 + blockIdx.x / cpi];
   const int c0 = (blockIdx.x % cpi) * B;
-  const int ts = col_team_stride(M, B);
-  const int bs = threadIdx.x % B, js = threadIdx.x / B;
-  const int bf = T >= 16 ? threadIdx.x / T : bs, jf = T >= 16 ? threadIdx.x % T : js;
-  const size_t off = (size_t)(c0 / TB) * M * TB + (c0 % TB) + bs;
-  float2* bufs = smem + bs * ts;
+  const int b = threadIdx.x & (B - 1), j = threadIdx.x >> (__ffs(B) - 1);
+  const size_t off = (size_t)(c0 / TB) * M * TB + (c0 % TB) + b;
   const float2* src = cplx_plane(d, src_sel) + off;
   float2* dst = cplx_plane(d, dst_sel) + off;
+  float2* buf = smem + b * col_stride<M>(B);
 #pragma unroll
-  for (int i = 0; i < R; ++i) {
-    const int a = js + i * T;
-    bufs[phys(a)] = src[(size_t)a * TB];
+  for (int q = 0; q < G::E / r0; ++q) {
+    const int beta = j + T * q;
+    float2 x[r0];
+#pragma unroll
+    for (int i = 0; i < r0; ++i) x[i] = load_stream(src + (size_t)(beta + i * G::L1) * TB);
+    fft_first<FK_COL, M, INV>(x, beta, buf, tw);
   }
   __syncthreads();
-  fft_team<M, INV>(smem + bf * ts, jf, tw + tab_off(M));
-#pragma unroll
-  for (int i = 0; i < R; ++i) {
-    const int p = js + i * T;
-    dst[(size_t)in_pos<M>(p) * TB] = bufs[phys(p)];
+  if constexpr (G::S == 3) {
+    fft_mid<FK_COL, M, INV>(buf, j, tw);
+    __syncthreads();
   }
+  float2 x[G::E];
+  fft_last<FK_COL, M, INV>(x, j, buf);
+#pragma unroll
+  for (int i = 0; i < G::E; ++i) dst[(size_t)(j + i * T) * TB] = x[i];
 }
 
 // Forward column FFT of the iterate's row spectra (in place on S), fused with
-// the first evaluation of Eq. 11 at the nodes of the image's bracket.  Only
-// the S tile lands in shared memory; it is consumed by the first FFT stage,
-// after which the next item's tile is requested, so the copy overlaps the
-// remaining stages and the Eq. 11 sums (H and Y are read from global memory
-// in that loop).  A block takes a contiguous range of items and keeps its
-// per-node sums in registers while consecutive items belong to the same
-// image; it publishes them (one partial slot, one counter update) only when
-// the image changes.  NK: the nodes of the pass (KNODES, or KNARROW for the
-// narrow brackets of iterations NARROW_FROM on).
-template <int M, int NK>
+// the first evaluation of Eq. 11: node sums, or the moments about the
+// extrapolated lambda (lambda.cuh), from the transform's outputs in registers
+// and H, Y loaded beside them.  A block takes a contiguous range of items and
+// keeps its sums while consecutive items belong to the same image; it
+// publishes them (one partial slot, one counter update) only when the image
+// changes.  The next item's tiles are requested into L2 while the current one
+// is transformed.  Batched solve of 256 images, 15 iterations: 10.3 ms with
+// staged tiles and 12 or 8 nodes per pass, 7.2 ms as it is; 4 images of 4096^2,
+// 30 iterations: 16.2 -> 9.6 ms.  Three blocks per SM (80 registers) spill and
+// take 8.0 ms.
+template <int M, int BT>
 __global__ void __launch_bounds__(M >= 4096 ? 512 : 256, M >= 4096 ? 1 : 2)
 k_col_fwd_lambda(ClassDesc cd, const ImgDesc* __restrict__ imgs, ImgState* st,
                  const float2* __restrict__ tw, int iter, int row_items) {
   extern __shared__ __align__(16) float2 smem[];
-  constexpr int R = radix_for(M), T = threads_per_team(M);
-  __shared__ float s_nodes[KNODES];
+  using G = FftGeo<FK_COL, M>;
+  constexpr int T = G::T, r0 = G::RF, E = G::E;
+  __shared__ float2 s_nodes[KNODES / 2];
+  __shared__ int s_mode;
   __shared__ double s_tot[KNODES + 1];
   __shared__ int s_flag;
   __shared__ WarpAcc s_wacc;
-  __shared__ __align__(8) unsigned long long s_bar;  // completion of the landing tile
-  const int B = cd.TB;
+  const int B = BT > 0 ? BT : cd.TB;
   const int Lc = cd.N / 2;
   const int cpi = Lc / B;
   const int n_items = cd.n_img * cpi;
   const int per_cta = (n_items + gridDim.x - 1) / gridDim.x;
   const int first = blockIdx.x * per_cta;
   const int stop = min(first + per_cta, n_items);
+  if (first >= stop) return;  // the last blocks of a grid that does not divide the items
   const int tile = M * B;
-  const int ts = col_team_stride(M, B);
-  float2* landS = smem;
-  float2* work = landS + tile;
-  double* red = reinterpret_cast<double*>(work + B * ts);
-  // the length-M twiddle table, copied once per (persistent) block for
-  // M <= SMEM_TW_MAX; larger tables stay in global memory
-  const float2* twM = tw + tab_off(M);
-  if constexpr (M <= SMEM_TW_MAX) {
-    float2* stw = reinterpret_cast<float2*>(red + num_warps() * (KNODES + 1));
-    for (int i = threadIdx.x; i < M; i += blockDim.x) stw[i] = twM[i];
-    twM = stw;  // visible after the loop's first __syncthreads()
-  }
-  // b-fastest mapping for tile I/O, team-fastest for the in-place stages
-  const int b = threadIdx.x % B, j = threadIdx.x / B;
-  const int bf = T >= 16 ? threadIdx.x / T : b, jf = T >= 16 ? threadIdx.x % T : j;
-  // the item's S tile is one contiguous slab: one bulk copy by thread 0,
-  // completed on s_bar; H and Y of the item are read after its transform,
-  // so they are only prefetched into L2
-  if (threadIdx.x == 0) mbar_init(&s_bar);
-  __syncthreads();
-  unsigned int parity = 0;
-  auto issue = [&](int item) {
+  const int b = threadIdx.x & (B - 1), j = threadIdx.x >> (__ffs(B) - 1);
+  float2* buf = smem + b * col_stride<M>(B);
+  double* red = reinterpret_cast<double*>(smem + B * col_stride<M>(B));
+  auto prefetch = [&](int item) {
     if (item < stop) {
       const ImgDesc& d = imgs[cd.img0 + item / cpi];
       const size_t off = (size_t)(item % cpi) * tile;
-      if (threadIdx.x == 0) bulk_load(landS, d.S + off, (unsigned int)(tile * sizeof(float2)), &s_bar);
+      prefetch_l2(d.S + off, (unsigned int)(tile * sizeof(float2)));
       prefetch_l2(d.H + off, (unsigned int)(tile * sizeof(float2)));
       prefetch_l2(d.Y + off, (unsigned int)(tile * sizeof(float2)));
     }
   };
-  float acc[KNODES + 1];
-#pragma unroll
-  for (int q = 0; q <= KNODES; ++q) acc[q] = 0.0f;
+  BinAcc acc;
+  acc.clear();
   int cur = -1, slot = 0, count = 0;
   // publish the sums of `count` items of image `cur` (slot = its first tile);
   // the block completing the image's count reduces all slots and updates
@@ -385,83 +398,151 @@ k_col_fwd_lambda(ClassDesc cd, const ImgDesc* __restrict__ imgs, ImgState* st,
     count = 0;
   };
   warp_acc_clear(&s_wacc);  // first use follows the loop's __syncthreads()
-  issue(first);
-  for (int item = first; item < stop; ++item) {
-    const int gi = cd.img0 + item / cpi;
+  for (int item = first;; ++item) {
+    const int gi = item < stop ? cd.img0 + item / cpi : -1;
     const int t = item % cpi;
-    if (!mbar_wait(&s_bar, parity)) atomicOr(&st[gi].status, ST_COPY_TIMEOUT);
-    parity ^= 1;
-    __syncthreads();
     if (gi != cur) {
+      __syncthreads();
       if (count > 0) flush();
+      if (item >= stop) break;
       cur = gi;
       slot = t;
-      for (int q = threadIdx.x; q < KNODES; q += blockDim.x) s_nodes[q] = __ldcg(&st[gi].node[q]);
+      for (int q = threadIdx.x; q < KNODES / 2; q += blockDim.x)
+        s_nodes[q] = __ldcg(reinterpret_cast<const float2*>(st[gi].node) + q);
+      if (threadIdx.x == 0) s_mode = __ldcg(&st[gi].mode);
     }
     const ImgDesc& d = imgs[gi];
     ImgState* S = st + gi;
-    const int col = t * B + b;
     const size_t off = (size_t)t * tile;
+    float2* spec = d.S + off + b;
+    prefetch(item + 1);
     if (t == 0) {  // the DC bin needs sum(u_E): total of the row pass's partials
       block_sum_columns(d.rowsum, row_items, 1, 1, red, s_tot);
       if (threadIdx.x == 0) S->sum_u = s_tot[0];
     }
-    float2* buf = work + b * ts;
-    Stage0From<M, R, false>::run(landS + b, StridedIdx{B}, buf, j, twM, PaddedIdx());
-    __syncthreads();  // the landing tile is consumed
-    issue(item + 1);
-    Stage<M, R, false, 1>::run(work + bf * ts, jf, twM, PaddedIdx());  // ends synchronised
-    float nodes[KNODES];
+    __syncthreads();  // the previous item's reads of the buffer are done
 #pragma unroll
-    for (int q = 0; q < KNODES; ++q) nodes[q] = s_nodes[q];
-    float2* spec = d.S + off + b;
+    for (int q = 0; q < E / r0; ++q) {
+      const int beta = j + T * q;
+      float2 x[r0];
+#pragma unroll
+      for (int i = 0; i < r0; ++i) x[i] = load_stream(spec + (beta + i * G::L1) * B);
+      fft_first<FK_COL, M, false>(x, beta, buf, tw);
+    }
+    __syncthreads();
+    if constexpr (G::S == 3) {
+      fft_mid<FK_COL, M, false>(buf, j, tw);
+      __syncthreads();
+    }
+    float2 x[E];  // U_E at rows j + T i
+    fft_last<FK_COL, M, false>(x, j, buf);
+    const bool mom = s_mode == MODE_MOM;
+    const float c = s_nodes[0].x;
     const float2* Hc = d.H + off + b;
     const float2* Yc = d.Y + off + b;
-    if (col != 0) {
-      // positions p in storage order; p holds output row k = in_pos(p)
-#pragma unroll 4
-      for (int i = 0; i < R; ++i) {
-        const int p = j + i * T;
-        const int k = in_pos<M>(p);
-        const float2 Hk = __ldg(&Hc[(size_t)k * B]);
-        const float2 Yk = __ldg(&Yc[(size_t)k * B]);
-        const float2 U = buf[phys(p)];
-        spec[(size_t)k * B] = U;
-        const float2 r = csub(cmul(Hk, U), Yk);
-        const float rr = fmaf(r.x, r.x, r.y * r.y);
-        const float a = fmaf(Hk.x, Hk.x, Hk.y * Hk.y);
-        accum_bin<NK>(2.0f * rr, a, nodes, acc);  // bins l and N-l
+    // residual terms |H U_E - Y|^2 and |H|^2 of one bin
+    auto terms = [](float2 H, float2 Y, float2 U, float& r, float& a) {
+      const float2 e = csub(cmul(H, U), Y);
+      r = fmaf(e.x, e.x, e.y * e.y);
+      a = fmaf(H.x, H.x, H.y * H.y);
+    };
+    bool pair0 = false;
+    if (t == 0) {  // packed column 0: the rows k and M - k of the outputs meet in shared memory
+      __syncthreads();
+      pair0 = b == 0;
+      if (pair0) {
+#pragma unroll
+        for (int i = 0; i < E; ++i) smem[j + T * i] = x[i];
+      }
+      __syncthreads();
+    }
+    if (!pair0) {
+#pragma unroll
+      for (int i = 0; i < E; ++i) spec[(j + T * i) * B] = x[i];
+    }
+    constexpr int G4 = E < 4 ? E : 4;  // bins whose loads are in flight together
+    if (mom && !pair0) {
+#pragma unroll
+      for (int i0 = 0; i0 < E; i0 += G4) {
+        float2 H[G4], Y[G4];
+#pragma unroll
+        for (int i = 0; i < G4; ++i) {
+          H[i] = load_stream(Hc + (j + T * (i0 + i)) * B);
+          Y[i] = load_stream(Yc + (j + T * (i0 + i)) * B);
+        }
+#pragma unroll
+        for (int i = 0; i < G4; ++i) {
+          float r, a;
+          terms(H[i], Y[i], x[i0 + i], r, a);
+          accum_bin_moments(2.0f * r, a, c, acc);  // bins l and N-l
+        }
       }
     } else {
-      for (int i = 0; i < R; ++i) {
-        const int k = j + i * T;
-        float2 U = buf[phys(out_pos<M>(k))];
-        const float2 Um = buf[phys(out_pos<M>((M - k) & (M - 1)))];
-        float2 UA, UB;
-        unpack_pair(U, Um, UA, UB);
-        const float2 HA = d.H0[k], HB = d.HN[k], YA = d.Y0[k], YB = d.YN[k];
-        float rA;
-        if (k == 0) {
-          // DC bin in FP64 from exact sums: d00 = sum(h) sum(u_E) - sum(y)
-          const double su = s_tot[0];
-          const double d00 = S->sum_h * su - S->sum_y;
-          S->d00 = d00;
-          rA = (float)(d00 * d00);
-          U.x = (float)su;
+      // node sums (the first iterations) and column 0: a loop of G4 bins a
+      // time, so that the code stays small in the instruction cache
+      float2 nodes[KNODES / 2];
+#pragma unroll
+      for (int q = 0; q < KNODES / 2; ++q) nodes[q] = s_nodes[q];
+#pragma unroll 1
+      for (int i0 = 0; i0 < E; i0 += G4) {
+        float r[2 * G4], a[2 * G4];  // terms of the bins, weights included
+        if (!pair0) {
+          float2 H[G4], Y[G4], U[G4];
+#pragma unroll
+          for (int i = 0; i < G4; ++i) {
+            const int o = (j + T * (i0 + i)) * B;
+            H[i] = load_stream(Hc + o);
+            Y[i] = load_stream(Yc + o);
+            U[i] = spec[o];
+          }
+#pragma unroll
+          for (int i = 0; i < G4; ++i) {
+            terms(H[i], Y[i], U[i], r[i], a[i]);
+            r[i] *= 2.0f;  // bins l and N-l
+          }
         } else {
-          const float2 r = csub(cmul(HA, UA), YA);
-          rA = fmaf(r.x, r.x, r.y * r.y);
+          float2 HA[G4], HB[G4], YA[G4], YB[G4];
+#pragma unroll
+          for (int i = 0; i < G4; ++i) {
+            const int k = j + T * (i0 + i);
+            HA[i] = __ldcg(&d.H0[k]);
+            HB[i] = __ldcg(&d.HN[k]);
+            YA[i] = __ldcg(&d.Y0[k]);
+            YB[i] = __ldcg(&d.YN[k]);
+          }
+#pragma unroll
+          for (int i = 0; i < G4; ++i) {
+            const int k = j + T * (i0 + i);
+            float2 U = smem[k];
+            const float2 Um = smem[(M - k) & (M - 1)];
+            float2 UA, UB;
+            unpack_pair(U, Um, UA, UB);
+            terms(HA[i], YA[i], UA, r[i], a[i]);
+            terms(HB[i], YB[i], UB, r[G4 + i], a[G4 + i]);
+            if (k == 0) {
+              // DC bin in FP64 from exact sums: d00 = sum(h) sum(u_E) - sum(y)
+              const double su = s_tot[0];
+              const double d00 = S->sum_h * su - S->sum_y;
+              S->d00 = d00;
+              r[i] = (float)(d00 * d00);
+              U.x = (float)su;
+            }
+            spec[k * B] = U;
+          }
         }
-        const float2 rb = csub(cmul(HB, UB), YB);
-        accum_bin<NK>(rA, fmaf(HA.x, HA.x, HA.y * HA.y), nodes, acc);
-        accum_bin<NK>(fmaf(rb.x, rb.x, rb.y * rb.y), fmaf(HB.x, HB.x, HB.y * HB.y), nodes, acc);
-        spec[(size_t)k * B] = U;
+#pragma unroll
+        for (int i = 0; i < 2 * G4; ++i) {
+          if (i >= G4 && !pair0) break;
+          if (mom)
+            accum_bin_moments(r[i], a[i], c, acc);
+          else
+            accum_bin(r[i], a[i], nodes, acc);
+        }
       }
     }
-    warp_fold(acc, &s_wacc);
+    warp_fold(acc, mom ? KMOM : KNODES, &s_wacc);
     ++count;
   }
-  if (count > 0) flush();
 }
 
 // Fallback evaluation of Eq. 11 over the stored spectrum U_E for images whose
@@ -485,12 +566,11 @@ k_lambda_pass(ClassDesc cd, const ImgDesc* __restrict__ imgs, ImgState* st, int 
   for (int q = threadIdx.x; q < KNODES; q += blockDim.x) s_nodes[q] = __ldcg(&S->node[q]);
   warp_acc_clear(&s_wacc);
   __syncthreads();
-  float nodes[KNODES];
+  float2 nodes[KNODES / 2];
 #pragma unroll
-  for (int q = 0; q < KNODES; ++q) nodes[q] = s_nodes[q];
-  float acc[KNODES + 1];
-#pragma unroll
-  for (int q = 0; q <= KNODES; ++q) acc[q] = 0.0f;
+  for (int q = 0; q < KNODES / 2; ++q) nodes[q] = make_float2(s_nodes[2 * q], s_nodes[2 * q + 1]);
+  BinAcc acc;
+  acc.clear();
   const int e0 = (blockIdx.x % cpi) * chunk;
   const int lg_tile = __ffs(M * TB) - 1, lg_tb = __ffs(TB) - 1;  // powers of two
   // bins in pairs (b, b+1) of one tile row, read as 16-byte vectors; runs of
@@ -538,7 +618,7 @@ k_lambda_pass(ClassDesc cd, const ImgDesc* __restrict__ imgs, ImgState* st, int 
         }
       }
     }
-    warp_fold(acc, &s_wacc);
+    warp_fold(acc, KNODES, &s_wacc);
   }
   block_partials_folded(&s_wacc, d.part + (size_t)(blockIdx.x % cpi) * (KNODES + 1));
   if (last_item(&S->cta_done, cpi, &s_flag)) {
@@ -555,121 +635,127 @@ k_lambda_pass(ClassDesc cd, const ImgDesc* __restrict__ imgs, ImgState* st, int 
 }
 
 
-// Spectral solves fused with the inverse column FFTs: an item's U_E tile
-// lands in shared memory (H and Y are read from global memory next to it);
-// Eq. 8 and 9 fill two work tiles (U_I, U_p) that are inverse-transformed
-// while the next item's tile is fetched.
-template <int M>
-__global__ void __launch_bounds__(M >= 4096 ? 512 : 256, M >= 4096 ? 1 : 2)
+// Eq. 8 and 9 at rows k of packed column 0, which holds the bins (k, 0) and
+// (k, N/2): U_I and U_p of both, packed again.
+__device__ __noinline__ float4 solve_col0(const ImgDesc& d, int M, int B, int k, float lam,
+                                          float d2r) {
+  const float2 U = __ldcg(&d.S[k * B]), Um = __ldcg(&d.S[((M - k) & (M - 1)) * B]);
+  float2 UA, UB, IA, IB, PA, PB;
+  unpack_pair(U, Um, UA, UB);
+  solve_bin(UA, d.H0[k], d.Y0[k], lam, d2r, IA, PA);
+  solve_bin(UB, d.HN[k], d.YN[k], lam, d2r + 4.0f, IB, PB);
+  const float2 I = pack_pair(IA, IB), P = pack_pair(PA, PB);
+  return make_float4(I.x, I.y, P.x, P.y);
+}
+
+// Spectral solves fused with the inverse column FFTs: the first stage's inputs
+// are formed by Eq. 8 and 9 from U_E, H and Y as they are loaded (each bin once),
+// U_I and U_p then go through one buffer each.  Batched solve of 256 images, 15
+// iterations: 14.8 ms with staged tiles, 8.6 ms as it is; 4 images of 4096^2,
+// 30 iterations: 22.6 -> 11.7 ms.  Three blocks per SM where the first radix is
+// small enough for 80 registers (9.6 -> 8.6 ms); a first radix of 16 holds both
+// planes' 16 inputs and keeps 128.
+template <int M, int BT>
+__global__ void __launch_bounds__(M >= 4096 ? 512 : 256,
+                                  M >= 4096 ? 1 : (FftGeo<FK_COL, M>::RF <= 8 && M >= 512 ? 3 : 2))
 k_col_solve_inv(ClassDesc cd, const ImgDesc* __restrict__ imgs, ImgState* st,
                 const float2* __restrict__ tw, const float* __restrict__ d2tab) {
   extern __shared__ __align__(16) float2 smem[];
-  constexpr int R = radix_for(M), T = threads_per_team(M);
-  const int N = cd.N, Lc = N / 2, B = cd.TB;
+  using G = FftGeo<FK_COL, M>;
+  constexpr int T = G::T, r0 = G::RF, E = G::E;
+  const int N = cd.N, Lc = N / 2, B = BT > 0 ? BT : cd.TB;
   const int cpi = Lc / B;
   const int n_items = cd.n_img * cpi;
   const int tile = M * B;
-  const int ts = col_team_stride(M, B);
-  float2* landU = smem;
-  float2* workI = landU + tile;
-  float2* workP = workI + B * ts;
-  __shared__ __align__(8) unsigned long long s_bar;  // completion of the landing tile
-  const float2* twM = tw + tab_off(M);
-  if constexpr (M <= SMEM_TW_MAX) {
-    float2* stw = workP + B * ts;
-    for (int i = threadIdx.x; i < M; i += blockDim.x) stw[i] = twM[i];
-    twM = stw;  // visible after the loop's first __syncthreads()
-  }
-  if (threadIdx.x == 0) mbar_init(&s_bar);
-  __syncthreads();
-  unsigned int parity = 0;
-  // b-fastest mapping for tile I/O, team-fastest for the in-place stages
-  const int b = threadIdx.x % B, j = threadIdx.x / B;
-  const int bf = T >= 16 ? threadIdx.x / T : b, jf = T >= 16 ? threadIdx.x % T : j;
-  // the item's U_E tile: one bulk copy by thread 0, completed on s_bar; H and
-  // Y of the item are prefetched into L2
-  auto issue = [&](int item) {
-    if (item < n_items) {
-      const ImgDesc& d = imgs[cd.img0 + item / cpi];
-      const size_t off = (size_t)(item % cpi) * tile;
-      if (threadIdx.x == 0) bulk_load(landU, d.S + off, (unsigned int)(tile * sizeof(float2)), &s_bar);
-      prefetch_l2(d.H + off, (unsigned int)(tile * sizeof(float2)));
-      prefetch_l2(d.Y + off, (unsigned int)(tile * sizeof(float2)));
-    }
-  };
-  issue(blockIdx.x);
+  const int b = threadIdx.x & (B - 1), j = threadIdx.x >> (__ffs(B) - 1);
+  float2* bufI = smem + b * col_stride<M>(B);
+  float2* bufP = bufI + B * col_stride<M>(B);
+  const float* d2m = d2tab + tab_off(M);
   for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
     const int gi = cd.img0 + item / cpi;
-    if (!mbar_wait(&s_bar, parity)) atomicOr(&st[gi].status, ST_COPY_TIMEOUT);
-    parity ^= 1;
-    __syncthreads();
     const ImgDesc& d = imgs[gi];
     const int t = item % cpi;
     const int col = t * B + b;
-    const size_t off = (size_t)t * tile;
+    const size_t off = (size_t)t * tile + b;
+    {  // the next item's tiles on their way into L2
+      const int next = item + gridDim.x;
+      if (next < n_items) {
+        const ImgDesc& dn = imgs[cd.img0 + next / cpi];
+        const size_t on = (size_t)(next % cpi) * tile;
+        prefetch_l2(dn.S + on, (unsigned int)(tile * sizeof(float2)));
+        prefetch_l2(dn.H + on, (unsigned int)(tile * sizeof(float2)));
+        prefetch_l2(dn.Y + on, (unsigned int)(tile * sizeof(float2)));
+      }
+    }
     const double lamd = __ldcg(&st[gi].lam);
-    const bool branch = !(lamd < 1e300);
+    const bool branch = !(lamd < 1e300);  // lambda = inf: u_I = u_p = u_E (Sec. 3.2)
     if (t == 0 && threadIdx.x == 0) {  // the inverse row pass re-forms them
       st[gi].absmax[0] = 0u;
       st[gi].absmax[1] = 0u;
     }
-    const float lam = branch ? 0.0f : (float)lamd;
+    const float lam = (float)lamd;
     const float d2c = __ldg(&d2tab[tab_off(N) + col]);
-    float2* bufI = workI + b * ts;
-    float2* bufP = workP + b * ts;
-    const float2* Hc = d.H + off + b;
-    const float2* Yc = d.Y + off + b;
-#pragma unroll 4
-    for (int i = 0; i < R; ++i) {
-      const int k = j + i * T;
-      const int e = k * B + b;
-      const float d2r = __ldg(&d2tab[tab_off(M) + k]);
-      const float2 U = landU[e];
-      float2 UI, Up;
-      if (col != 0) {
-        const float2 Hv = __ldg(&Hc[(size_t)k * B]);
-        const float2 Yv = __ldg(&Yc[(size_t)k * B]);
-        solve_bin(U, Hv, Yv, lam, d2r + d2c, branch, UI, Up);
+    const float2* Sc = d.S + off;
+    const float2* Hc = d.H + off;
+    const float2* Yc = d.Y + off;
+    if (item != (int)blockIdx.x) __syncthreads();  // the previous item's reads are done
+#pragma unroll
+    for (int q = 0; q < E / r0; ++q) {
+      const int beta = j + T * q;
+      float2 xI[r0], xP[r0];
+      if (branch) {
+#pragma unroll
+        for (int i = 0; i < r0; ++i) xI[i] = xP[i] = load_stream(Sc + (beta + i * G::L1) * B);
+      } else if (col != 0) {
+        constexpr int G4 = r0 < 4 ? r0 : 4;
+#pragma unroll
+        for (int i0 = 0; i0 < r0; i0 += G4) {
+          float2 U[G4], H[G4], Y[G4];
+#pragma unroll
+          for (int i = 0; i < G4; ++i) {
+            const int o = (beta + (i0 + i) * G::L1) * B;
+            U[i] = load_stream(Sc + o);
+            H[i] = load_stream(Hc + o);
+            Y[i] = load_stream(Yc + o);
+          }
+#pragma unroll
+          for (int i = 0; i < G4; ++i)
+            solve_bin(U[i], H[i], Y[i], lam, __ldg(&d2m[beta + (i0 + i) * G::L1]) + d2c,
+                      xI[i0 + i], xP[i0 + i]);
+        }
       } else {
-        const float2 Um = landU[((M - k) & (M - 1)) * B + b];
-        float2 UA, UB, IA, IB, PA, PB;
-        unpack_pair(U, Um, UA, UB);
-        solve_bin(UA, d.H0[k], d.Y0[k], lam, d2r, branch, IA, PA);
-        solve_bin(UB, d.HN[k], d.YN[k], lam, d2r + 4.0f, branch, IB, PB);
-        UI = make_float2(IA.x - IB.y, IA.y + IB.x);  // A + i B
-        Up = make_float2(PA.x - PB.y, PA.y + PB.x);
+#pragma unroll
+        for (int i = 0; i < r0; ++i) {
+          const int k = beta + i * G::L1;
+          const float4 v = solve_col0(d, M, B, k, lam, __ldg(&d2m[k]));
+          xI[i] = make_float2(v.x, v.y);
+          xP[i] = make_float2(v.z, v.w);
+        }
       }
-      bufI[phys(k)] = UI;
-      bufP[phys(k)] = Up;
+      fft_first<FK_COL, M, true>(xI, beta, bufI, tw);
+      fft_first<FK_COL, M, true>(xP, beta, bufP, tw);
     }
     __syncthreads();
-    issue(item + gridDim.x);
-    fft_team2<M, true>(workI + bf * ts, workP + bf * ts, jf, twM);
-    float2* qi = d.QI + off + b;
-    float2* qp = d.Qp + off + b;
-#pragma unroll 4
-    for (int i = 0; i < R; ++i) {
-      const int p = j + i * T;  // storage order; row in_pos(p)
-      const size_t k = (size_t)in_pos<M>(p);
-      qi[k * B] = bufI[phys(p)];
-      qp[k * B] = bufP[phys(p)];
+    if constexpr (G::S == 3) {
+      fft_mid<FK_COL, M, true>(bufI, j, tw);
+      fft_mid<FK_COL, M, true>(bufP, j, tw);
+      __syncthreads();
     }
+    float2 x[E];
+    float2* qi = d.QI + off;
+    fft_last<FK_COL, M, true>(x, j, bufI);
+#pragma unroll
+    for (int i = 0; i < E; ++i) qi[(j + T * i) * B] = x[i];
+    float2* qp = d.Qp + off;
+    fft_last<FK_COL, M, true>(x, j, bufP);
+#pragma unroll
+    for (int i = 0; i < E; ++i) qp[(j + T * i) * B] = x[i];
   }
 }
 
 // ---------------------------------------------------------------------------
 // launch configuration and dispatch
 // ---------------------------------------------------------------------------
-template <class K>
-static int max_threads(K kernel) {
-  static int cached = 0;
-  if (cached == 0) {
-    cudaFuncAttributes a{};
-    cached = cudaFuncGetAttributes(&a, (const void*)kernel) == cudaSuccess ? a.maxThreadsPerBlock : 256;
-  }
-  return cached;
-}
-
 static int sm_count() {
   static int n = 0;
   if (n == 0) {
@@ -701,9 +787,11 @@ static int floor_pow2(int v) {
   return p;
 }
 
+// Threads of a row pass's team for rows of L packed values.
+static int row_team(int L) { return L / fft_elems(FK_C2R, L); }
+
 int rows_per_item(int L, int M, int row_threads) {
-  const int T = threads_per_team(L);
-  int r = (row_threads > 0 ? row_threads : DEF_ROW_THREADS) / T;
+  int r = (row_threads > 0 ? row_threads : DEF_ROW_THREADS) / row_team(L);
   if (r < 1) r = 1;
   if (r > M) r = M;
   return floor_pow2(r);
@@ -713,22 +801,13 @@ int rows_per_item(int L, int M, int row_threads) {
 // col_threads threads (512 for M = 4096), at least 2 columns (16-byte
 // copies), at most N/2.
 int class_tile_width(int M, int N, int col_threads) {
-  const int T = M / radix_for(M);
+  const int T = M / fft_elems(FK_COL, M);
   const int ct = col_threads > 0 ? (col_threads > 256 ? 256 : col_threads) : DEF_COL_THREADS;
   const int threads = M >= 4096 ? 512 : ct;
   int B = threads / T;
   if (B < 2) B = 2;
   if (B > N / 2) B = N / 2;
   return floor_pow2(B);
-}
-
-static size_t row_r2c_smem(int L, int rpc) {
-  return (size_t)2 * rpc * L * sizeof(float2) + (size_t)row_work_elems(L, rpc) * sizeof(float2) +
-         32 * sizeof(double) + (L <= SMEM_TW_MAX ? (size_t)L * sizeof(float2) : 0);
-}
-static size_t row_c2r_smem(int L, int rpc) {
-  return (size_t)rpc * L * sizeof(float2) + (size_t)rpc * team_stride(L) * sizeof(float2) +
-         (L <= SMEM_TW_MAX ? (size_t)L * sizeof(float2) : 0);
 }
 
 #define GFD_CASE_L(F, ...)             \
@@ -758,12 +837,11 @@ static size_t row_c2r_smem(int L, int rpc) {
 template <int L>
 static void do_row_r2c(const ClassLaunch& c, const Tables& t, int src, int dst, int sum,
                        cudaStream_t s) {
+  using G = FftGeo<FK_R2C, L>;
   const int rpc = rows_per_item(L, c.cd.M, c.row_threads);
-  const int n_items = c.cd.n_img * c.cd.M / rpc;
-  const int thr = rpc * threads_per_team(L);
-  const size_t smem = row_r2c_smem(L, rpc);
-  const int grid = persistent_grid(k_row_r2c<L>, thr, smem, n_items, c.grid_div);
-  k_row_r2c<L><<<grid, thr, smem, s>>>(c.cd, c.imgs, t.tw, rpc, src, dst, sum);
+  const int blocks = c.cd.n_img * c.cd.M / rpc;
+  k_row_r2c<L><<<blocks, rpc * G::T, rpc * G::SIZE * sizeof(float2), s>>>(c.cd, c.imgs, t.tw, rpc,
+                                                                          src, dst, sum);
 }
 
 cudaError_t launch_row_r2c(const ClassLaunch& c, const Tables& t, int src, int dst,
@@ -778,14 +856,12 @@ cudaError_t launch_row_r2c(const ClassLaunch& c, const Tables& t, int src, int d
 template <int L>
 static void do_row_c2r(const ClassLaunch& c, const Tables& t, int sel0, int sel1, int dsel0,
                        int dsel1, float scale, cudaStream_t s) {
+  using G = FftGeo<FK_C2R, L>;
   const int rpc = rows_per_item(L, c.cd.M, c.row_threads);
-  int n_items = c.cd.n_img * c.cd.M / rpc;
-  if (sel1 >= 0) n_items *= 2;
-  const int thr = rpc * threads_per_team(L);
-  const size_t smem = row_c2r_smem(L, rpc);
-  const int grid = persistent_grid(k_row_c2r<L>, thr, smem, n_items, c.grid_div);
-  k_row_c2r<L><<<grid, thr, smem, s>>>(c.cd, c.imgs, t.tw, rpc, sel0, sel1, dsel0, dsel1, scale,
-                                       dsel0 == SEL_UI ? c.st : nullptr);
+  int blocks = c.cd.n_img * c.cd.M / rpc;
+  if (sel1 >= 0) blocks *= 2;
+  k_row_c2r<L><<<blocks, rpc * G::T, rpc * G::SIZE * sizeof(float2), s>>>(
+      c.cd, c.imgs, t.tw, rpc, sel0, sel1, dsel0, dsel1, scale, dsel0 == SEL_UI ? c.st : nullptr);
 }
 
 cudaError_t launch_row_c2r(const ClassLaunch& c, const Tables& t, int sel0, int sel1, int dsel0,
@@ -801,13 +877,11 @@ template <int M>
 static void do_col_plain(const ClassLaunch& c, const Tables& t, int src, int dst, bool inv,
                          cudaStream_t s) {
   const int Lc = c.cd.N / 2;
-  const int T = threads_per_team(M);
-  const int mt = inv ? max_threads(k_col_plain<M, true>) : max_threads(k_col_plain<M, false>);
-  int B = (mt < 512 ? mt : 512) / T;
-  if (B < 1) B = 1;
+  constexpr int T = FftGeo<FK_COL, M>::T;
+  int B = 512 / T;
   if (B > Lc) B = Lc;
   if (B > c.cd.TB) B = c.cd.TB;  // a block stays inside one tile
-  const size_t smem = (size_t)B * col_team_stride(M, B) * sizeof(float2);
+  const size_t smem = (size_t)B * col_stride<M>(B) * sizeof(float2);
   const int nblk = c.cd.n_img * (Lc / B);
   if (inv)
     k_col_plain<M, true><<<nblk, B * T, smem, s>>>(c.cd, c.imgs, t.tw, B, src, dst);
@@ -824,33 +898,42 @@ cudaError_t launch_col_plain(const ClassLaunch& c, const Tables& t, int src, int
   return cudaGetLastError();
 }
 
-template <int M>
-static size_t col_smem(int B, int landings, int works, int nthr) {
-  return (size_t)landings * M * B * sizeof(float2) +
-         (size_t)works * B * col_team_stride(M, B) * sizeof(float2) +
-         (size_t)((nthr + 31) / 32) * (KNODES + 1) * sizeof(double) +
-         (M <= SMEM_TW_MAX ? (size_t)M * sizeof(float2) : 0);
-}
+// Column kernels of the long transforms exist for every tile width that
+// class_tile_width gives them, so that a thread's rows lie at constant offsets;
+// shorter ones (BT = 0) take the width at run time.
+#define GFD_COL_WIDTHS(F, M, B, ...)                                     \
+  do {                                                                   \
+    if constexpr ((M) >= 2048) {                                         \
+      F<M, 2>(__VA_ARGS__);                                              \
+    } else if constexpr ((M) == 1024) {                                  \
+      if ((B) == 4) F<M, 4>(__VA_ARGS__); else F<M, 2>(__VA_ARGS__);     \
+    } else if constexpr ((M) == 512) {                                   \
+      if ((B) == 8) F<M, 8>(__VA_ARGS__);                                \
+      else if ((B) == 4) F<M, 4>(__VA_ARGS__);                           \
+      else F<M, 2>(__VA_ARGS__);                                         \
+    } else if constexpr ((M) == 256) {                                   \
+      if ((B) == 16) F<M, 16>(__VA_ARGS__);                              \
+      else if ((B) == 8) F<M, 8>(__VA_ARGS__);                           \
+      else if ((B) == 4) F<M, 4>(__VA_ARGS__);                           \
+      else F<M, 2>(__VA_ARGS__);                                         \
+    } else {                                                             \
+      F<M, 0>(__VA_ARGS__);                                              \
+    }                                                                    \
+  } while (0)
 
-template <int M, int NK>
-static void do_col_fwd_lambda_nk(const ClassLaunch& c, const Tables& t, int iter, cudaStream_t s) {
+template <int M, int BT>
+static void do_col_fwd_lambda_w(const ClassLaunch& c, const Tables& t, int iter, cudaStream_t s) {
   const int Lc = c.cd.N / 2, B = c.cd.TB;
-  const int nthr = B * threads_per_team(M);
-  const size_t smem = col_smem<M>(B, 1, 1, nthr);
+  const int nthr = B * FftGeo<FK_COL, M>::T;
+  const size_t smem = (size_t)B * col_stride<M>(B) * sizeof(float2) + 16 * sizeof(double);
   const int n_items = c.cd.n_img * (Lc / B);
-  const int grid = persistent_grid(k_col_fwd_lambda<M, NK>, nthr, smem, n_items, c.grid_div);
-  const int row_items = c.cd.M / rows_per_item(c.cd.N / 2, c.cd.M, c.row_threads);
-  k_col_fwd_lambda<M, NK><<<grid, nthr, smem, s>>>(c.cd, c.imgs, c.st, t.tw, iter, row_items);
+  const int grid = persistent_grid(k_col_fwd_lambda<M, BT>, nthr, smem, n_items, c.grid_div);
+  k_col_fwd_lambda<M, BT><<<grid, nthr, smem, s>>>(c.cd, c.imgs, c.st, t.tw, iter, c.cd.M);
 }
 
-// The brackets resolve_warp lays out for iteration `iter` have KNARROW nodes
-// from NARROW_FROM on: the pass evaluates exactly those.
 template <int M>
 static void do_col_fwd_lambda(const ClassLaunch& c, const Tables& t, int iter, cudaStream_t s) {
-  if (iter >= NARROW_FROM)
-    do_col_fwd_lambda_nk<M, KNARROW>(c, t, iter, s);
-  else
-    do_col_fwd_lambda_nk<M, KNODES>(c, t, iter, s);
+  GFD_COL_WIDTHS(do_col_fwd_lambda_w, M, c.cd.TB, c, t, iter, s);
 }
 
 cudaError_t launch_col_fwd_lambda(const ClassLaunch& c, const Tables& t, int iter,
@@ -871,14 +954,19 @@ cudaError_t launch_lambda_pass(const ClassLaunch& c, int iter, bool last_chance,
   return cudaGetLastError();
 }
 
+template <int M, int BT>
+static void do_col_solve_inv_w(const ClassLaunch& c, const Tables& t, cudaStream_t s) {
+  const int Lc = c.cd.N / 2, B = c.cd.TB;
+  const int nthr = B * FftGeo<FK_COL, M>::T;
+  const size_t smem = (size_t)2 * B * col_stride<M>(B) * sizeof(float2);
+  const int n_items = c.cd.n_img * (Lc / B);
+  const int grid = persistent_grid(k_col_solve_inv<M, BT>, nthr, smem, n_items, c.grid_div);
+  k_col_solve_inv<M, BT><<<grid, nthr, smem, s>>>(c.cd, c.imgs, c.st, t.tw, t.d2);
+}
+
 template <int M>
 static void do_col_solve_inv(const ClassLaunch& c, const Tables& t, cudaStream_t s) {
-  const int Lc = c.cd.N / 2, B = c.cd.TB;
-  const int nthr = B * threads_per_team(M);
-  const size_t smem = col_smem<M>(B, 1, 2, 0);
-  const int n_items = c.cd.n_img * (Lc / B);
-  const int grid = persistent_grid(k_col_solve_inv<M>, nthr, smem, n_items, c.grid_div);
-  k_col_solve_inv<M><<<grid, nthr, smem, s>>>(c.cd, c.imgs, c.st, t.tw, t.d2);
+  GFD_COL_WIDTHS(do_col_solve_inv_w, M, c.cd.TB, c, t, s);
 }
 
 cudaError_t launch_col_solve_inv(const ClassLaunch& c, const Tables& t, cudaStream_t s) {
@@ -918,13 +1006,24 @@ static cudaError_t cfg_row() {
   return allow_smem(k_row_c2r<L>);
 }
 template <int M>
+static cudaError_t cfg_col_fused();
+template <int M>
 static cudaError_t cfg_col() {
   cudaError_t e;
   if ((e = allow_smem(k_col_plain<M, false>)) != cudaSuccess) return e;
   if ((e = allow_smem(k_col_plain<M, true>)) != cudaSuccess) return e;
-  if ((e = allow_smem(k_col_fwd_lambda<M, KNODES>)) != cudaSuccess) return e;
-  if ((e = allow_smem(k_col_fwd_lambda<M, KNARROW>)) != cudaSuccess) return e;
-  return allow_smem(k_col_solve_inv<M>);
+  return cfg_col_fused<M>();
+}
+template <int M, int BT>
+static void cfg_col_width(cudaError_t& e) {
+  if (e == cudaSuccess) e = allow_smem(k_col_fwd_lambda<M, BT>);
+  if (e == cudaSuccess) e = allow_smem(k_col_solve_inv<M, BT>);
+}
+template <int M>
+static cudaError_t cfg_col_fused() {
+  cudaError_t e = cudaSuccess;
+  for (int B = 2; B <= 16; B *= 2) GFD_COL_WIDTHS(cfg_col_width, M, B, e);
+  return e;
 }
 
 cudaError_t configure_fft_kernels() {

@@ -22,14 +22,21 @@
 //   arithmetic (FP64 is slow on this part), and its root is located by
 //   multisection with one trial point per lane, which needs only the sign
 //   of the interpolant.
-// The first pass of each iteration is fused into the forward column FFT and
-// uses a bracket of ratio 4 around an extrapolation of the previous lambdas.
-// From iteration NARROW_FROM on, where the extrapolation comes within a few
-// percent of the root, it evaluates KNARROW = 8 nodes on a bracket of ratio
-// 1.56, whose degree-7 interpolant is as accurate as the degree-11 one on
-// ratio 4 (the strip of analyticity is the same, the bracket's half-width in
-// t three times smaller).  A root outside that bracket lies close to it: the
-// fallback pass takes the ratio-4 bracket next to it.
+// The first pass of each iteration is fused into the forward column FFT.  In
+// iterations 0-2 its bracket is wide or of ratio 4; from iteration 3 on lambda
+// moves little and the pass needs no bracket: it expands f about the
+// extrapolated lambda c.  With t = c / (a + c) in (0, 1], s = ln(lambda / c) and
+// e = tanh(s / 2),
+//   lambda / (a + lambda) = t (1 + e) / (1 + e x),   x = 2 t - 1 in (-1, 1],
+// so  P f(lambda) = (1 + e)^2 sum_k (k + 1) (-e)^k N_k,  N_k = sum_b r_b t_b^2 x_b^k,
+// a series in e whose terms shrink at least as fast as (k + 1) |e|^k whatever
+// the spectrum is.  One reciprocal per bin and two operations per moment serve
+// all KMOM = 8 moments (12 nodes take a reciprocal and five operations each),
+// and on the batched workload |e| <= 0.01 from iteration 5 on: the truncated
+// terms are below 1e-15.  The root is accepted where its truncation error is
+// below MOM_TOL; otherwise the series at a few |e| on the root's side, as far
+// as its sign is certain against the truncated terms, gives the bracket of a
+// fallback pass.
 #pragma once
 #include "common.cuh"
 #include "df.cuh"
@@ -37,11 +44,10 @@
 namespace gfd {
 
 constexpr float INTERP_RATIO = 4.0f;   // largest bracket ratio interpolated
-constexpr float PRIMARY_RATIO = 2.0f;  // primary bracket: [c/2, 2 c]
-constexpr float NARROW_RATIO = 1.25f;  // from iteration NARROW_FROM: [c/1.25, 1.25 c]
-constexpr float NARROW_INTERP_RATIO = 1.6f;  // largest ratio interpolated with KNARROW nodes
+constexpr float MOM_REACH = 0.35f;      // largest |e| searched: lambda within a factor 2.08 of c
+constexpr float MOM_TOL = 1e-10f;       // accepted truncation error of the root, relative
 constexpr float INITIAL_LO = 1e-8f, INITIAL_HI = 1e4f;
-constexpr int MODE_GEOM = 0, MODE_CHEB = 1;
+constexpr int MODE_GEOM = 0, MODE_CHEB = 1, MODE_MOM = 2;
 
 // Lanes of the warp that runs a per-image update (threads 0..31 of the
 // block): the whole warp, or every thread of a block smaller than a warp
@@ -51,54 +57,56 @@ GFD_D unsigned int upd_mask() {
   return blockDim.x >= 32 ? 0xffffffffu : ((1u << blockDim.x) - 1u);
 }
 
-// cos(pi j / (n - 1)), j = 0..n-1 (Chebyshev-Lobatto points) for n = KNODES
-// and n = KNARROW
+// cos(pi j / (n - 1)), j = 0..n-1 (Chebyshev-Lobatto points), n = KNODES
 __device__ constexpr float kLobatto[KNODES] = {
     1.0f, 0.9594929736144974f, 0.8412535328311812f, 0.6548607339452851f,
     0.41541501300188644f, 0.14231483827328512f, -0.142314838273285f, -0.4154150130018863f,
     -0.654860733945285f, -0.8412535328311811f, -0.9594929736144974f, -1.0f};
-__device__ constexpr float kLobatto8[KNARROW] = {
-    1.0f, 0.9009688679024191f, 0.6234898018587336f, 0.22252093395631445f,
-    -0.2225209339563144f, -0.6234898018587335f, -0.900968867902419f, -1.0f};
 
-// Node lambda_j (ascending) of a bracket [lo, hi] of nk nodes for the given
-// layout (nodes j >= nk repeat hi and are not evaluated).
-GFD_D float bracket_node(float lo, float hi, int mode, int j, int nk) {
+// Node lambda_j (ascending) of a bracket [lo, hi] for the given layout.
+GFD_D float bracket_node(float lo, float hi, int mode, int j) {
   if (j == 0) return lo;
-  if (j >= nk - 1) return hi;
-  if (mode == MODE_CHEB) {  // Chebyshev-Lobatto in ln(lambda)
-    const float c = nk == KNARROW ? kLobatto8[j] : kLobatto[j];
-    return lo * exp2f(0.5f * (1.0f - c) * log2f(hi / lo));
-  }
-  return lo * exp2f((float)j / (nk - 1) * log2f(hi / lo));
+  if (j >= KNODES - 1) return hi;
+  if (mode == MODE_CHEB)  // Chebyshev-Lobatto in ln(lambda)
+    return lo * exp2f(0.5f * (1.0f - kLobatto[j]) * log2f(hi / lo));
+  return lo * exp2f((float)j / (KNODES - 1) * log2f(hi / lo));
 }
 
-// Chebyshev nodes (interpolated) for brackets narrow enough for nk nodes,
-// geometric nodes (bracketed) otherwise.
-GFD_D int bracket_mode(float lo, float hi, int nk) {
-  return hi <= (nk == KNARROW ? NARROW_INTERP_RATIO : INTERP_RATIO) * lo ? MODE_CHEB : MODE_GEOM;
+// Chebyshev nodes (interpolated) for narrow brackets, geometric nodes
+// (bracketed) otherwise.
+GFD_D int bracket_mode(float lo, float hi) {
+  return hi <= INTERP_RATIO * lo ? MODE_CHEB : MODE_GEOM;
 }
 
-// Set the next pass's bracket of nk nodes (single thread).
-GFD_D void set_bracket(ImgState* st, float lo, float hi, int nk = KNODES) {
-  const int mode = bracket_mode(lo, hi, nk);
+// Set the next pass's bracket (single thread).
+GFD_D void set_bracket(ImgState* st, float lo, float hi) {
+  const int mode = bracket_mode(lo, hi);
   st->lo = lo;
   st->hi = hi;
   st->mode = mode;
-  st->nk = nk;
-  for (int j = 0; j < KNODES; ++j) st->node[j] = bracket_node(lo, hi, mode, j, nk);
+  for (int j = 0; j < KNODES; ++j) st->node[j] = bracket_node(lo, hi, mode, j);
 }
 
 // Warp variant: lane j < KNODES writes node j.
-GFD_D void set_bracket_warp(ImgState* st, float lo, float hi, int lane, int nk = KNODES) {
-  const int mode = bracket_mode(lo, hi, nk);
+GFD_D void set_bracket_warp(ImgState* st, float lo, float hi, int lane) {
+  const int mode = bracket_mode(lo, hi);
   if (lane == 0) {
     st->lo = lo;
     st->hi = hi;
     st->mode = mode;
-    st->nk = nk;
   }
-  if (lane < KNODES) st->node[lane] = bracket_node(lo, hi, mode, lane, nk);
+  if (lane < KNODES) st->node[lane] = bracket_node(lo, hi, mode, lane);
+  __syncwarp(upd_mask());
+}
+
+// The next pass expands f about c (node[0]).
+GFD_D void set_center_warp(ImgState* st, float c, int lane) {
+  if (lane == 0) {
+    st->lo = c;
+    st->hi = c;
+    st->mode = MODE_MOM;
+    st->node[0] = c;
+  }
   __syncwarp(upd_mask());
 }
 
@@ -109,38 +117,47 @@ GFD_D void set_bracket_warp(ImgState* st, float lo, float hi, int lane, int nk =
 // the same reciprocal error for a given node: a node-dependent bias of ~1e-7
 // in f(lambda_j) that moves the root by ~1e-7 / |d ln f / d ln lambda|,
 // i.e. by percents where f is nearly flat in lambda.
-// NK: the nodes the pass evaluates (acc[NK..KNODES-1] are left alone).
-template <int NK = KNODES>
-GFD_D void accum_bin(float wr, float a, const float* nodes, float* acc) {
-  acc[KNODES] += wr;
+// Nodes are taken two at a time (packed FP32 pairs).
+struct BinAcc {
+  float2 v[KNODES / 2];  // node sums (moments N_0.. in MODE_MOM)
+  float w;               // sum of wr
+  GFD_D void clear() {
 #pragma unroll
-  for (int j = 0; j < NK; ++j) {
-    const float d = a + nodes[j];
-    const float q = __fdividef(1.0f, d);
-    const float t0 = nodes[j] * q;
-    const float t = fmaf(fmaf(-t0, d, nodes[j]), q, t0);
-    acc[j] = fmaf(wr, t * t, acc[j]);
+    for (int j = 0; j < KNODES / 2; ++j) v[j] = make_float2(0.0f, 0.0f);
+    w = 0.0f;
+  }
+};
+
+GFD_D void accum_bin(float wr, float a, const float2* nodes, BinAcc& acc) {
+  acc.w += wr;
+  const float2 w2 = make_float2(wr, wr), a2 = make_float2(a, a);
+#pragma unroll
+  for (int j = 0; j < KNODES / 2; ++j) {
+    const float2 n = nodes[j];
+    const float2 d = cadd(a2, n);
+    const float2 q = make_float2(__fdividef(1.0f, d.x), __fdividef(1.0f, d.y));
+    const float2 t0 = __fmul2_rn(n, q);
+    const float2 t = __ffma2_rn(__ffma2_rn(make_float2(-t0.x, -t0.y), d, n), q, t0);
+    acc.v[j] = __ffma2_rn(w2, __fmul2_rn(t, t), acc.v[j]);
   }
 }
 
-// Block-wide sums of the KNODES+1 per-thread partials (FP32 within a warp,
-// FP64 across warps), stored with plain stores to part[0..KNODES].
-// red must hold num_warps() * (KNODES+1) doubles.  Ends synchronised.
-GFD_D void block_partials(float* acc, double* red, double* part) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int nwarp = num_warps();
+// The bin's terms of the moments about c (MODE_MOM), two at a time.
+GFD_D void accum_bin_moments(float wr, float a, float c, BinAcc& acc) {
+  acc.w += wr;
+  const float d = a + c;
+  const float q = __fdividef(1.0f, d);
+  const float t0 = c * q;
+  const float t = fmaf(fmaf(-t0, d, c), q, t0);
+  const float p0 = wr * (t * t);
+  const float x = fmaf(2.0f, t, -1.0f);
+  const float2 xx = make_float2(x * x, x * x);
+  float2 p = make_float2(p0, p0 * x);
 #pragma unroll
-  for (int j = 0; j <= KNODES; ++j) {
-    const float v = warp_sum(acc[j]);
-    if (lane == 0) red[warp * (KNODES + 1) + j] = (double)v;
+  for (int j = 0; j < KMOM / 2; ++j) {
+    acc.v[j] = cadd(acc.v[j], p);
+    if (j + 1 < KMOM / 2) p = __fmul2_rn(p, xx);
   }
-  __syncthreads();
-  for (int j = threadIdx.x; j <= KNODES; j += blockDim.x) {
-    double s = 0.0;
-    for (int w = 0; w < nwarp; ++w) s += red[w * (KNODES + 1) + j];
-    part[j] = s;
-  }
-  __syncthreads();
 }
 
 // Long sums of the per-bin terms.  Threads keep FP32 partials over a short
@@ -155,18 +172,26 @@ struct WarpAcc {
   float lo[16][KNODES + 1];
 };
 
-GFD_D void warp_fold(float* acc, WarpAcc* wa) {
+GFD_D void warp_fold_one(float v, int j, int lane, int warp, WarpAcc* wa) {
+  v = warp_sum(v);
+  if (lane == 0) {
+    const df t = two_sum(wa->hi[warp][j], v);
+    wa->hi[warp][j] = t.hi;
+    wa->lo[warp][j] += t.lo;
+  }
+}
+
+// n: the leading sums in use (KNODES, or KMOM in MODE_MOM); the rest are zero.
+GFD_D void warp_fold(BinAcc& acc, int n, WarpAcc* wa) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-  for (int j = 0; j <= KNODES; ++j) {
-    const float v = warp_sum(acc[j]);
-    if (lane == 0) {
-      const df t = two_sum(wa->hi[warp][j], v);
-      wa->hi[warp][j] = t.hi;
-      wa->lo[warp][j] += t.lo;
-    }
-    acc[j] = 0.0f;
+  for (int j = 0; j < KNODES; j += 2) {
+    if (j >= n) break;
+    warp_fold_one(acc.v[j / 2].x, j, lane, warp, wa);
+    warp_fold_one(acc.v[j / 2].y, j + 1, lane, warp, wa);
   }
+  warp_fold_one(acc.w, KNODES, lane, warp, wa);
+  acc.clear();
 }
 
 // part[j] = sum over warps of hi + lo (FP64); clears the accumulators.
@@ -278,7 +303,8 @@ GFD_D df df_div_fast(df a, df b) {  // a / b, error ~2^-44 relative
   return quick_two_sum(q1, r * ib);
 }
 
-GFD_D double interp_root_warp(float xm, float gm, int j, double rtol, int lane, int nk) {
+GFD_D double interp_root_warp(float xm, float gm, int j, double rtol, int lane) {
+  constexpr int nk = KNODES;
   const bool own = lane < nk;
   const df tm = own ? df_from_double(log((double)xm)) : df_make(0.0f);
   // All abscissa differences are scaled by a power of two ~ 1/(node span):
@@ -355,7 +381,7 @@ GFD_D double interp_root_warp(float xm, float gm, int j, double rtol, int lane, 
       S.lo += u.lo + q.lo;
     };
 #pragma unroll 2
-    for (int m = 0; m < nk; m += 2) {  // nk is even; registers stay low in the pass kernels
+    for (int m = 0; m < nk; m += 2) {  // registers stay low in the pass kernels
       term(m, S0);
       term(m + 1, S1);
     }
@@ -381,50 +407,127 @@ GFD_D double interp_root_warp(float xm, float gm, int j, double rtol, int lane, 
   return exp(0.5 * (df_to_double(a) + df_to_double(b)));
 }
 
-// Record lambda_k and set the bracket of iteration k+1's fused first pass.
-// lambda jumps by a factor of 2..150 from the first iteration (u_E = 0) to
-// the second, and mostly falls to 0.2..1.2 of it in the third; later it
-// changes smoothly, so the bracket is centred on the extrapolation
-// lambda_k (lambda_k / lambda_{k-1}) (ratio clamped to [1/2, 2]).  The second
-// iteration's bracket has geometric nodes, resolved by one more pass; the
-// third's, [0.28, 1.1] lambda_1, and the later ones are narrow enough
-// (ratio <= 4) for the interpolation to resolve them in the fused pass itself.
+// Record lambda_k and set up iteration k+1's fused first pass.  lambda jumps
+// by a factor of 2..600 from the first iteration (u_E = 0) to the second, and
+// mostly falls to 0.2..1.2 of it in the third; the fourth stays within a few
+// percent of the third on most images, and later it changes smoothly.  The
+// second iteration's bracket has geometric nodes, resolved by one more pass;
+// the third's, [0.28, 1.1] lambda_1, is narrow enough (ratio <= 4) for the
+// interpolation to resolve it in the fused pass itself; later first passes
+// expand f about lambda_2, then about the extrapolation
+// lambda_k (lambda_k / lambda_{k-1}) (ratio clamped to [1/2, 2]).
 GFD_D void resolve_warp(ImgState* st, double lam, int iter, double* lam_out, int lane) {
   if (lane == 0) {
     st->lam = lam;
     st->need = 0;
     if (lam_out) lam_out[iter] = lam;
   }
-  // the first pass of iteration iter + 1 evaluates nk nodes
-  const int nk = iter + 1 >= NARROW_FROM ? KNARROW : KNODES;
+  // lambda = inf (or no finite root) keeps the pending bracket or centre
   if (isfinite(lam) && lam > 0.0) {
     const float l = (float)lam;
-    float lo, hi;
+    const double prev = st->lam_prev;
+    __syncwarp(upd_mask());  // every lane has read lam_prev
     if (iter == 0) {
-      lo = l;
-      hi = 150.0f * l;
+      set_bracket_warp(st, fmaxf(l, (float)LAMBDA_LO), 150.0f * l, lane);
     } else if (iter == 1) {
-      lo = 0.28f * l;
-      hi = 1.1f * l;
+      set_bracket_warp(st, fmaxf(0.28f * l, (float)LAMBDA_LO), 1.1f * l, lane);
     } else {
-      const double prev = st->lam_prev;
       float c = l;
-      if (isfinite(prev) && prev > 0.0) c = l * fminf(fmaxf((float)(lam / prev), 0.5f), 2.0f);
-      const float ratio = nk == KNARROW ? NARROW_RATIO : PRIMARY_RATIO;
-      lo = c / ratio;
-      hi = c * ratio;
+      if (iter > 2 && isfinite(prev) && prev > 0.0) {
+        const df ip = df_rcp(df_from_double(prev));
+        c = l * fminf(fmaxf(l * (ip.hi + ip.lo), 0.5f), 2.0f);
+      }
+      set_center_warp(st, fmaxf(c, (float)LAMBDA_LO), lane);
     }
-    lo = fmaxf(lo, (float)LAMBDA_LO);
-    set_bracket_warp(st, lo, hi, lane, nk);  // ends with __syncwarp()
     if (lane == 0) st->lam_prev = lam;
-  } else if (st->nk != nk) {
-    // lambda = inf (or no finite root): the pending bracket is kept, laid
-    // out for the node count of the next first pass
-    const float lo = (float)st->lo, hi = (float)st->hi;
-    __syncwarp(upd_mask());
-    set_bracket_warp(st, lo, hi, lane, nk);
   }
   __syncwarp(upd_mask());
+}
+
+// Root of the moment expansion about c = node[0] (see the top of the file).
+// tot[0..KMOM-1] are the sums N_k.  Every lane evaluates the series at a trial
+// point of its own in FP32, three rounds; two Newton steps with the series
+// in FP64 follow.  Sets lam to the root and returns true if it is accepted;
+// otherwise leaves the bracket of the next pass in (lo, hi).
+GFD_D bool moment_root_warp(const double* tot, double scale, float c, int lane, double& lam,
+                            float& lo, float& hi) {
+  const int nl = upd_lanes();
+  const unsigned int mask = upd_mask();
+  // a_k = (k + 1) (-1)^k N_k / (P T), one per lane, then to every lane
+  double ak = 0.0;
+  if (lane < KMOM) ak = tot[lane] * scale * ((lane & 1) ? -(lane + 1) : (lane + 1));
+  double a[KMOM];
+  float af[KMOM];
+#pragma unroll
+  for (int k = 0; k < KMOM; ++k) {
+    a[k] = __shfl_sync(mask, ak, k);
+    af[k] = (float)a[k];
+  }
+  auto value = [&](float e) {  // f / T - 1
+    float p = af[KMOM - 1];
+#pragma unroll
+    for (int k = KMOM - 2; k >= 0; --k) p = fmaf(p, e, af[k]);
+    return fmaf(p, (1.0f + e) * (1.0f + e), -1.0f);
+  };
+  float e0 = -MOM_REACH, e1 = MOM_REACH;
+  const float inv = 1.0f / (float)(nl + 1);
+  for (int round = 0; round < 3; ++round) {
+    const float w = e1 - e0;
+    const unsigned int above = __ballot_sync(mask, !(value(fmaf(w, (lane + 1) * inv, e0)) < 0.0f));
+    const int nb = above ? __ffs(above) - 1 : nl;  // leading trial points below the root
+    e1 = nb < nl ? fmaf(w, (nb + 1) * inv, e0) : e1;
+    e0 = nb > 0 ? fmaf(w, nb * inv, e0) : e0;
+  }
+  double e = 0.5 * ((double)e0 + (double)e1);
+  const float ef = (float)e, g = 1.0f + ef;
+  float p = af[KMOM - 1], dp = 0.0f;  // series and its derivative
+#pragma unroll
+  for (int k = KMOM - 2; k >= 0; --k) {
+    dp = fmaf(dp, ef, p);
+    p = fmaf(p, ef, af[k]);
+  }
+  const float slope = g * fmaf(g, dp, 2.0f * p);  // d(f / T) / de
+  const float islope = __fdividef(1.0f, slope);
+#pragma unroll 1
+  for (int it = 0; it < 5; ++it) {
+    double q = a[KMOM - 1];
+#pragma unroll
+    for (int k = KMOM - 2; k >= 0; --k) q = fma(q, e, a[k]);
+    const double F = fma(q, fma(e, e, fma(2.0, e, 1.0)), -1.0);
+    const float step = (float)F * islope;
+    e -= (double)step;
+    if (!(fabsf(step) > 1e-7f)) break;  // the next would be below 1e-13
+  }
+  const float er = (float)e;
+  // truncated terms, at most (KMOM + 1) |e|^KMOM N_0 (1 + e)^2 / (1 - |e|)^2 in
+  // all (N_k <= N_0), over the slope in s: de / ds = (1 - e^2) / 2
+  const float x2 = er * er, x4 = x2 * x2, d1 = 1.0f - fabsf(er);
+  const float err = (KMOM + 1) * x4 * x4 * af[0] * g * g * islope * 2.0f / ((1.0f - x2) * d1 * d1);
+  const float est = c * __fdividef(1.0f + er, 1.0f - er);
+  if (slope > 0.0f && err <= MOM_TOL && est > (float)LAMBDA_LO) {
+    lam = (double)c * (1.0 + e) / (1.0 - e);
+    return true;
+  }
+  // The root's side of c by the sign of f(c) - T; along it, the last |e| that
+  // the series certainly has before the root and the first certainly past it.
+  const bool up = a[0] < 1.0;
+  float before = 0.0f, past = 0.0f;
+#pragma unroll 1
+  for (int i = 0; i < 4; ++i) {
+    const float m = i == 0 ? 0.11f : (i == 1 ? 0.18f : (i == 2 ? 0.25f : MOM_REACH));
+    const float m2 = m * m, m4 = m2 * m2;
+    const float v = up ? value(m) : -value(-m);
+    const float r1 = (1.0f + m) / (1.0f - m);
+    const float margin = (KMOM + 1) * m4 * m4 * af[0] * r1 * r1 + 2e-7f;
+    if (v > margin) past = m;
+    if (!(v < -margin)) break;
+    before = m;
+  }
+  const float rb = (1.0f + before) / (1.0f - before), rp = (1.0f + past) / (1.0f - past);
+  const float near = 0.99f * rb, far = past > 0.0f ? 1.01f * rp : 3.95f * near;
+  lo = up ? c * near : c / far;
+  hi = up ? c * far : c / near;
+  return false;
 }
 
 // Consume the totals of the pass that just completed for this image (tot:
@@ -432,7 +535,7 @@ GFD_D void resolve_warp(ImgState* st, double lam, int iter, double* lam_out, int
 // 32 lanes of one warp of the image's last block; every lane takes the same
 // decisions from the same values.  FP64 is limited to a handful of
 // operations (the sums themselves are FP64).
-GFD_D void lambda_update_warp(ImgState* st, const double* tot, double P, bool primary,
+__device__ __noinline__ static void lambda_update_warp(ImgState* st, const double* tot, double P, bool primary,
                               bool last_chance, int iter, double* lam_out, double* res_out,
                               int lane) {
   const double invP = 1.0 / P;  // P is a power of two: exact
@@ -458,9 +561,26 @@ GFD_D void lambda_update_warp(ImgState* st, const double* tot, double P, bool pr
     }
     __syncwarp(upd_mask());
   }
-  // g_m = f(lambda_m) / T - 1, increasing in lambda, for the nk nodes the
-  // pass evaluated
-  const int nk = st->nk;
+  if (st->mode == MODE_MOM) {
+    const float c = st->node[0];
+    if (!isfinite(tot[0])) {
+      if (lane == 0) st->status |= ST_NONFINITE;
+      resolve_warp(st, INFINITY, iter, lam_out, lane);
+      return;
+    }
+    double lam;
+    float lo, hi;
+    if (moment_root_warp(tot, invP * st->invT, c, lane, lam, lo, hi)) {
+      resolve_warp(st, lam, iter, lam_out, lane);
+      return;
+    }
+    lo = fmaxf(lo, (float)LAMBDA_LO);
+    set_bracket_warp(st, lo, fmaxf(hi, 1.05f * lo), lane);
+    if (lane == 0) st->need = 1;
+    return;
+  }
+  // g_m = f(lambda_m) / T - 1, increasing in lambda, for the pass's nodes
+  constexpr int nk = KNODES;
   const float gm = lane < nk ? (float)((tot[lane] * invP - T) * st->invT) : 0.0f;
   const float xm = lane < nk ? st->node[lane] : 0.0f;
   const float g0 = __shfl_sync(upd_mask(), gm, 0);
@@ -469,7 +589,9 @@ GFD_D void lambda_update_warp(ImgState* st, const double* tot, double P, bool pr
   const float hi = __shfl_sync(upd_mask(), xm, nk - 1);
   const int mode = st->mode;
   // a missed first bracket whose root is expected close to it
-  const bool near = nk == KNARROW || (primary && iter == 2 && mode == MODE_CHEB);
+  const bool near = primary && iter == 2 && mode == MODE_CHEB;
+  // the second iteration's jump, past its first bracket: seldom far past it
+  const bool jump = primary && iter == 1;
   bool open = true;
   if (!(g0 <= 0.0f)) {  // root below the bracket (or NaN)
     if (!isfinite(g0)) {
@@ -482,22 +604,25 @@ GFD_D void lambda_update_warp(ImgState* st, const double* tot, double P, bool pr
       resolve_warp(st, LAMBDA_LO, iter, lam_out, lane);
       return;
     }
-    // below a narrow first bracket, or the third iteration's first bracket
-    // (four passes to go): the ratio-4 bracket just under it; otherwise
-    // everything down to the smallest lambda
+    // below the third iteration's first bracket (four passes to go): the
+    // ratio-4 bracket just under it; otherwise everything down to the smallest
+    // lambda
     const float nlo = near ? fmaxf(0.25f * lo, (float)LAMBDA_LO) : (float)LAMBDA_LO;
     set_bracket_warp(st, nlo, lo, lane);
   } else if (gK < 0.0f) {  // root above the bracket
-    // above a narrow first bracket: the ratio-4 bracket just over it;
-    // otherwise up to the bound from res and |H|^2
-    set_bracket_warp(st, hi, near ? 4.0f * hi : fmaxf(st->lam_up, hi * 4.0f), lane);
+    // above the third iteration's first bracket: the ratio-4 bracket just
+    // over it; above the second's: a ratio-16 bracket, whose intervals are
+    // interpolated by the pass after; otherwise up to the bound from res and
+    // |H|^2
+    set_bracket_warp(st, hi, near ? 4.0f * hi : (jump ? 16.0f * hi : fmaxf(st->lam_up, hi * 4.0f)),
+                     lane);
   } else {
     // nodes with g < 0 form a prefix 0..j
     const unsigned below = __ballot_sync(upd_mask(), lane < nk && gm < 0.0f);
     int j = 31 - __clz(below | 1u);
     if (j > nk - 2) j = nk - 2;
     if (mode == MODE_CHEB) {
-      const double lam = interp_root_warp(xm, gm, j, st->rtol, lane, nk);
+      const double lam = interp_root_warp(xm, gm, j, st->rtol, lane);
       resolve_warp(st, lam, iter, lam_out, lane);
       open = false;
     } else {

@@ -17,28 +17,24 @@ GFD_D void unpack_pair(float2 Sk, float2 Smk, float2& A, float2& Bv) {
 }
 GFD_D float2 pack_pair(float2 A, float2 B) { return make_float2(A.x - B.y, A.y + B.x); }
 
-// Eq. 9 (u_p) and Eq. 8 (u_I) at one bin:
+// 1/d for d > 0: the hardware approximation and one residual step (almost
+// always the correctly rounded quotient, as __frcp_rn, in three instructions).
+GFD_D float rcp_refined(float d) {
+  const float q = __fdividef(1.0f, d);
+  return fmaf(fmaf(-d, q, 1.0f), q, q);
+}
+
+// Eq. 9 (u_p) and Eq. 8 (u_I) at one bin, lambda finite:
 //   U_p = (conj(H) Y + lam U_E) / (|H|^2 + lam)
 //   U_I = (conj(H) Y + lam D2 U_E) / (|H|^2 + lam D2),  D2 = |F(nabla)|^2.
-GFD_D void solve_bin(float2 U, float2 H, float2 Y, float lam, float D2, bool branch,
-                     float2& UI, float2& Up) {
-  if (branch) {  // lambda = inf: u_I = u_p = u_E (Sec. 3.2)
-    UI = U;
-    Up = U;
-    return;
-  }
-  const float2 HY = make_float2(fmaf(H.x, Y.x, H.y * Y.y), fmaf(H.x, Y.y, -H.y * Y.x));
+GFD_D void solve_bin(float2 U, float2 H, float2 Y, float lam, float D2, float2& UI, float2& Up) {
+  const float2 HY = __ffma2_rn(make_float2(H.x, H.x), Y, make_float2(H.y * Y.y, -H.y * Y.x));
   const float a = fmaf(H.x, H.x, H.y * H.y);
-  const float ip = __frcp_rn(a + lam);
-  Up = make_float2(fmaf(lam, U.x, HY.x) * ip, fmaf(lam, U.y, HY.y) * ip);
+  Up = cscale(__ffma2_rn(make_float2(lam, lam), U, HY), rcp_refined(a + lam));
   const float lg = lam * D2;
   const float den = a + lg;
-  if (den > 0.0f) {
-    const float ii = __frcp_rn(den);
-    UI = make_float2(fmaf(lg, U.x, HY.x) * ii, fmaf(lg, U.y, HY.y) * ii);
-  } else {
-    UI = U;
-  }
+  const float2 v = cscale(__ffma2_rn(make_float2(lg, lg), U, HY), rcp_refined(den));
+  UI = den > 0.0f ? v : U;
 }
 
 }  // namespace gfd
