@@ -282,7 +282,11 @@ k_row_c2r(ClassDesc cd, const ImgDesc* __restrict__ imgs, const float2* __restri
 // memory to the first stage's registers (no landing tile, which cost a pass
 // through shared memory and half the blocks per SM), the next item's tiles are
 // prefetched into L2, and the tile width is a compile-time constant, so that
-// a thread's rows are immediate offsets.
+// a thread's rows are immediate offsets.  The prefetch is issued just before the
+// last stage: at the start of an item it comes so early that on a batch larger
+// than L2 its lines are gone before use (ncu: 329 MB read for 201 MB of
+// tiles; the solve pass took 8.6 ms per batched solve, 6.8 ms with the late
+// prefetch, 7.1 ms with none).
 // ---------------------------------------------------------------------------
 
 // Setup / utility column FFT: plane src -> dst, in place allowed; B columns
@@ -328,11 +332,11 @@ k_col_plain(ClassDesc cd, const ImgDesc* __restrict__ imgs, const float2* __rest
 // and H, Y loaded beside them.  A block takes a contiguous range of items and
 // keeps its sums while consecutive items belong to the same image; it
 // publishes them (one partial slot, one counter update) only when the image
-// changes.  The next item's tiles are requested into L2 while the current one
-// is transformed.  Batched solve of 256 images, 15 iterations: 10.3 ms with
-// staged tiles and 12 or 8 nodes per pass, 7.2 ms as it is; 4 images of 4096^2,
-// 30 iterations: 16.2 -> 9.6 ms.  Three blocks per SM (80 registers) spill and
-// take 8.0 ms.
+// changes.  Batched solve of 256 images, 15 iterations: 10.3 ms with staged
+// tiles and 12 or 8 nodes per pass, 7.0 ms as it is; 4 images of 4096^2, 30
+// iterations: 16.2 -> 9.5 ms (without prefetch, which takes 10.8 ms there: one
+// block per SM loads and computes in turn).  Three blocks per SM (80 registers)
+// spill and take 8.0 ms.
 template <int M, int BT>
 __global__ void __launch_bounds__(M >= 4096 ? 512 : 256, M >= 4096 ? 1 : 2)
 k_col_fwd_lambda(ClassDesc cd, const ImgDesc* __restrict__ imgs, ImgState* st,
@@ -415,7 +419,6 @@ k_col_fwd_lambda(ClassDesc cd, const ImgDesc* __restrict__ imgs, ImgState* st,
     ImgState* S = st + gi;
     const size_t off = (size_t)t * tile;
     float2* spec = d.S + off + b;
-    prefetch(item + 1);
     if (t == 0) {  // the DC bin needs sum(u_E): total of the row pass's partials
       block_sum_columns(d.rowsum, row_items, 1, 1, red, s_tot);
       if (threadIdx.x == 0) S->sum_u = s_tot[0];
@@ -434,6 +437,7 @@ k_col_fwd_lambda(ClassDesc cd, const ImgDesc* __restrict__ imgs, ImgState* st,
       fft_mid<FK_COL, M, false>(buf, j, tw);
       __syncthreads();
     }
+    if (M < 4096) prefetch(item + 1);
     float2 x[E];  // U_E at rows j + T i
     fft_last<FK_COL, M, false>(x, j, buf);
     const bool mom = s_mode == MODE_MOM;
@@ -651,8 +655,8 @@ __device__ __noinline__ float4 solve_col0(const ImgDesc& d, int M, int B, int k,
 // Spectral solves fused with the inverse column FFTs: the first stage's inputs
 // are formed by Eq. 8 and 9 from U_E, H and Y as they are loaded (each bin once),
 // U_I and U_p then go through one buffer each.  Batched solve of 256 images, 15
-// iterations: 14.8 ms with staged tiles, 8.6 ms as it is; 4 images of 4096^2,
-// 30 iterations: 22.6 -> 11.7 ms.  Three blocks per SM where the first radix is
+// iterations: 14.8 ms with staged tiles, 6.8 ms as it is; 4 images of 4096^2,
+// 30 iterations: 22.6 -> 9.4 ms.  Three blocks per SM where the first radix is
 // small enough for 80 registers (9.6 -> 8.6 ms); a first radix of 16 holds both
 // planes' 16 inputs and keeps 128.
 template <int M, int BT>
@@ -677,7 +681,7 @@ k_col_solve_inv(ClassDesc cd, const ImgDesc* __restrict__ imgs, ImgState* st,
     const int t = item % cpi;
     const int col = t * B + b;
     const size_t off = (size_t)t * tile + b;
-    {  // the next item's tiles on their way into L2
+    auto prefetch_next = [&]() {
       const int next = item + gridDim.x;
       if (next < n_items) {
         const ImgDesc& dn = imgs[cd.img0 + next / cpi];
@@ -686,7 +690,7 @@ k_col_solve_inv(ClassDesc cd, const ImgDesc* __restrict__ imgs, ImgState* st,
         prefetch_l2(dn.H + on, (unsigned int)(tile * sizeof(float2)));
         prefetch_l2(dn.Y + on, (unsigned int)(tile * sizeof(float2)));
       }
-    }
+    };
     const double lamd = __ldcg(&st[gi].lam);
     const bool branch = !(lamd < 1e300);  // lambda = inf: u_I = u_p = u_E (Sec. 3.2)
     if (t == 0 && threadIdx.x == 0) {  // the inverse row pass re-forms them
@@ -741,6 +745,7 @@ k_col_solve_inv(ClassDesc cd, const ImgDesc* __restrict__ imgs, ImgState* st,
       fft_mid<FK_COL, M, true>(bufP, j, tw);
       __syncthreads();
     }
+    prefetch_next();
     float2 x[E];
     float2* qi = d.QI + off;
     fft_last<FK_COL, M, true>(x, j, bufI);
