@@ -67,10 +67,10 @@ typedef enum {
  * window sums of I, p, I^2 and I p).  Every variant takes the statistics about
  * a per-strip reference value (a_k and b_k do not depend on it). */
 #define GFD_VAR_COMPENSATED 0  /* split sums (default): each deviation is split on a
-                                  power-of-two grid from a bound on |u_I|, |u_p| into
-                                  an integer leading part (window sums exact in int32,
-                                  n S_II - S_I^2 exact in int64) and an FP32 remainder
-                                  (its sums compensate the leading part's truncation) */
+                                  grid from a bound on |u_I|, |u_p| into an integer
+                                  leading part (window sums, squares included, exact
+                                  in FP32) and an FP32 remainder (its sums compensate
+                                  the leading part's truncation) */
 #define GFD_VAR_FP64 1         /* FP64 accumulators (reference point; slow on this part) */
 #define GFD_VAR_FP32 2         /* plain FP32 sums about the reference (precision study) */
 #define GFD_VAR_FP32_RAW 3     /* plain FP32 sums of the raw values, no reference shift */

@@ -75,19 +75,6 @@ GFD_D float warp_max(float v) {
 }
 GFD_D int num_warps() { return (int)((blockDim.x + 31) >> 5); }
 
-// Asynchronous global -> shared copies (16-byte chunks, L2 only) with
-// commit groups; waits are hardware waits on the thread's own groups.
-GFD_D unsigned int smem_u32(const void* p) { return (unsigned int)__cvta_generic_to_shared(p); }
-GFD_D void cp_async16(void* smem_dst, const void* gsrc) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_u32(smem_dst)), "l"(gsrc)
-               : "memory");
-}
-GFD_D void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-GFD_D void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
-
 // Bulk prefetch of [p, p + bytes) into L2 (p 16-byte aligned, bytes a
 // multiple of 16), split into pieces of at most 16 KB issued by the lanes of
 // warp 0.  No completion to wait for: later loads simply find the lines in L2.

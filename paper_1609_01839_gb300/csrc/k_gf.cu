@@ -3,10 +3,11 @@
 // at the canvas edge (every mean divided by the number of pixels it covers).
 //
 // Every warp works alone, down a strip of GFW_COLS input columns (4 per
-// lane): no block barriers.  Input rows enter a per-warp ring in shared
-// memory by 16-byte asynchronous copies GFW_AHEAD rows ahead of use; each lane
-// copies and reads only its own 4 columns.  For the item's rows the warp
-// forms, row by row,
+// lane): no block barriers.  Input rows are loaded to registers one row ahead
+// of use (and requested into L2 a few rows ahead); their deviations from the
+// reference enter a per-warp ring in shared memory, where the row that leaves
+// the windows finds them again.  Each lane touches only its own 4 columns.
+// For the item's rows the warp forms, row by row,
 //   1. window sums down its columns of J = I - c_I, Q = p - c_p, J^2, J Q
 //      (in registers; slid from row to row, and for plain FP32 sums re-formed
 //      directly every 4 rows),
@@ -41,23 +42,21 @@ namespace gfd {
 
 constexpr int GFW_COLS = 128;   // input columns per strip (4 per lane)
 constexpr int GFW_SUB = 4;      // rows between direct re-formations of FP32 column sums
-constexpr int GFW_WARPS = 4;    // warps per block
-constexpr int GFW_AHEAD = 2;    // input rows requested ahead of use
+constexpr int GFW_WARPS = 4;    // most warps per block
+constexpr int GFW_AHEAD = 4;    // input rows requested into L2 ahead of use
 constexpr int GF_RMAX = 8;      // w <= 17
 constexpr unsigned FULL = 0xffffffffu;
 
 template <int RAD>
 struct GfwGeom {
   static constexpr int WIN = 2 * RAD + 1;
-  static constexpr int RI = WIN + 1 + GFW_AHEAD;  // input ring rows: window, the row leaving, ahead
+  static constexpr int RI = WIN + 1;  // rows of the ring of deviations: the window, the row leaving
   static constexpr int HALO = 4 * ((RAD + 1) / 2);  // >= 2r, multiple of 4
   static constexpr int WOUT = GFW_COLS - 2 * HALO;  // output columns per strip
 };
 
-// per-warp shared memory: (a, b) ring of 2r+1 rows, (I, p) ring of 2r+2+GFW_AHEAD rows
-GFD_HD int gfw_ring_floats(int rad) {
-  return (2 * (2 * rad + 1) + 2 * (2 * rad + 2 + GFW_AHEAD)) * GFW_COLS;
-}
+// per-warp shared memory: (a, b) ring of 2r+1 rows, (J, Q) ring of 2r+2 rows
+GFD_HD int gfw_ring_floats(int rad) { return 2 * ((2 * rad + 1) + (2 * rad + 2)) * GFW_COLS; }
 static int gfw_wout(int rad) { return GFW_COLS - 8 * ((rad + 1) / 2); }
 
 // ---------------------------------------------------------------------------
@@ -100,64 +99,55 @@ struct SumDF {
   }
 };
 
-// Split sums.  Every deviation x (J or Q) is split on a power-of-two grid g
-// chosen per item from a bound on |x| (g >= 2^-b max |x|): x = g m + x_l with
-// m = round(x / g), |m| <= 2^b, and x_l = x - g m (exact).  Window sums of m,
-// m_J^2 and m_J m_Q are exact in int32 on the integer pipe, and so are
-// n S_mm - S_m^2 and n S_mJ mQ - S_mJ S_mQ: b = split_bits(r) is the largest
-// with n^2 2^(2b) < 2^31 for windows of n = (2r+1)^2 pixels (11 at most).
-// The remainders' parts, x_l, J^2 - (g_J m_J)^2 = J_l (J + g_J m_J) and
-// J Q - g_J m_J g_Q m_Q = g_J m_J Q_l + J_l Q, are summed in FP32, where
-// their rounding is 2^-b of that of plain sums.
+// Split sums.  Every deviation x (J or Q) is split on a grid g chosen per item
+// from a bound on |x|: x = g m + x_l with m = round(x / g), |m| <= split_max(r),
+// and x_l = x - g m, both exact in FP32 (g has a 3-bit mantissa).  split_max
+// keeps the window sums of m_J^2 and m_J m_Q below 2^24, so the sums of m,
+// m_J^2 and m_J m_Q are exact in FP32; n S_mm - S_m^2 and n S_mJmQ - S_mJ S_mQ
+// follow with one rounding (the square's error comes from an FMA).  The
+// remainders' parts, x_l, J^2 - (g_J m_J)^2 = J J_l + J_l g_J m_J and
+// J Q - g_J m_J g_Q m_Q = J Q_l + J_l g_Q m_Q, are summed in FP32, where
+// their rounding is about 1 / (2 split_max) of that of plain sums.
+// Everything comes in pairs (J, Q), one packed FP32 instruction per pair, in
+// the register pairs that the ring's rows load; mixing int32 and FP32 halves
+// cost 10 % more instructions.  What bounds the kernel now: the FP32 pipe, the
+// shuffles (0.93 per cycle and SM) and issue are each about half busy, with 12
+// warps per SM (registers and rings) to overlap them; DRAM is at 15 %.  Per
+// batched solve of 256 images 14.7 -> 12.1 ms, of which 1.3 by the choice of
+// rows per item (gfw_rows).  Fewer registers (128: spills) took 15.3 ms; leaving
+// rows re-read through L1 instead of the ring 16.7 ms.
 struct SumIG {
   static constexpr int kSub = 1 << 30;
-  int h;
-  float l;
 };
 
-// The grids of one item: g, 1/g and g * kMagic for J and for Q.
+// The grids of one item: g and 1/g for (J, Q).
 struct IGGrid {
-  float gJ, igJ, mgJ, gQ, igQ, mgQ;
+  float2 g, ig;
 };
 
 constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23: adding it rounds |v| < 2^22 to an integer
 
-// Bits of the split's integer part for windows of radius r: the largest b
-// <= 11 with ((2r+1)^2)^2 2^(2b) < 2^31 (r = 2: 10, r = 3, 4: 9, r = 8: 7).
-constexpr int split_bits(int rad) {
+// Largest |m| of the split for windows of radius r: (2r+1)^2 m^2 <= 2^24.
+constexpr int split_max(int rad) {
   const long long n = (long long)(2 * rad + 1) * (2 * rad + 1);
-  int b = 11;
-  while (b > 0 && n * n * (1LL << (2 * b)) >= (1LL << 31)) --b;
-  return b;
+  int m = 2048;
+  while (n * m * m > (1LL << 24)) --m;
+  return m;
 }
 
-static_assert(split_bits(2) == 10 && split_bits(3) == 9 && split_bits(4) == 9 &&
-                  split_bits(8) == 7 && split_bits(0) == 11,
-              "split bits per window radius");
+static_assert(split_max(2) == 819 && split_max(3) == 585 && split_max(4) == 455 &&
+                  split_max(8) == 240 && split_max(0) == 2048,
+              "split range per window radius");
 
+// The smallest g with a 3-bit mantissa and bound / g <= split_max - 1.
 template <int RAD>
-GFD_D void ig_grid(float bound, float& g, float& ig, float& mg) {
-  constexpr int B = split_bits(RAD);
+GFD_D void ig_grid(float bound, float& g, float& ig) {
   int e = 0;
-  if (bound > 0.0f && bound < 3e38f) frexpf(bound, &e);  // bound <= 2^e
+  float f = 0.5f;
+  if (bound > 0.0f && bound < 1e37f) f = frexpf(bound * (1.0f / (split_max(RAD) - 1)), &e);
   if (e < -100) e = -100;
-  g = ldexpf(1.0f, e - B);
-  ig = ldexpf(1.0f, B - e);
-  mg = kMagic * g;
-}
-
-// x = g m + xl: m = round(x / g) (kMagic + x / g rounds to an integer-valued
-// float whose low bits are m), g m exact, xl = x - g m exact.
-GFD_D void ig_split(float x, float ig, float g, float mg, int& m, float& xh, float& xl) {
-  const float t = fmaf(x, ig, kMagic);
-  m = __float_as_int(t) - __float_as_int(kMagic);
-  xh = fmaf(t, g, -mg);
-  xl = x - xh;
-}
-
-// int32 |v| < 2^22 to float, exactly, without a conversion instruction
-GFD_D float small_int_to_float(int v) {
-  return __int_as_float(__float_as_int(kMagic) + v) - kMagic;
+  g = ldexpf(ceilf(8.0f * f) * 0.125f, e);
+  ig = 1.0f / g;
 }
 
 // Value of lane (lane + off) (compile-time offset after unrolling).
@@ -185,9 +175,7 @@ GFD_D void gather_row(const T (&v)[4], T (&e)[2 * RAD + 4]) {
 // Window sums of radius RAD along the strip: s[k] = sum of columns
 // 4*lane + k - RAD .. 4*lane + k + RAD.
 template <int RAD, class T>
-GFD_D void hsum4_scalar(const T (&v)[4], T (&s)[4]) {
-  T e[2 * RAD + 4];
-  gather_row<RAD>(v, e);
+GFD_D void row_sums(const T (&e)[2 * RAD + 4], T (&s)[4]) {
   T acc = e[0];
 #pragma unroll
   for (int q = 1; q <= 2 * RAD; ++q) acc += e[q];
@@ -199,9 +187,11 @@ GFD_D void hsum4_scalar(const T (&v)[4], T (&s)[4]) {
   }
 }
 
-template <int RAD>
-GFD_D void hsum4(const float (&v)[4], float (&s)[4]) {
-  hsum4_scalar<RAD>(v, s);
+template <int RAD, class T>
+GFD_D void hsum4_scalar(const T (&v)[4], T (&s)[4]) {
+  T e[2 * RAD + 4];
+  gather_row<RAD>(v, e);
+  row_sums<RAD>(e, s);
 }
 
 template <int RAD>
@@ -255,21 +245,6 @@ GFD_D void hsum4(const SumDF (&v)[4], SumDF (&s)[4]) {
   }
 }
 
-template <int RAD>
-GFD_D void hsum4(const SumIG (&v)[4], SumIG (&s)[4]) {
-  const int ih[4] = {v[0].h, v[1].h, v[2].h, v[3].h};
-  const float il[4] = {v[0].l, v[1].l, v[2].l, v[3].l};
-  int oh[4];
-  float ol[4];
-  hsum4_scalar<RAD>(ih, oh);
-  hsum4_scalar<RAD>(il, ol);
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    s[k].h = oh[k];
-    s[k].l = ol[k];
-  }
-}
-
 // Means and (co)variance of a window of n pixels from S = (sum J, sum Q,
 // sum J^2, sum J Q):  var = (n S_JJ - S_J^2) / n^2 (sigma_k^2, the
 // population variance), cov = (n S_JQ - S_J S_Q) / n^2.
@@ -307,27 +282,6 @@ GFD_D void window_stats(const SumDF& s0, const SumDF& s1, const SumDF& s2, const
   cov = (c.hi + c.lo) * inv2;
 }
 
-// Split sums: the integer parts of n S_JJ - S_J^2 and n S_JQ - S_J S_Q are
-// exact in int32 (the split's bits keep every product below 2^31, and E by
-// Cauchy-Schwarz; the differences are formed in modular unsigned arithmetic);
-// the remainders' parts are added in FP32.
-GFD_D void window_stats(const SumIG& s0, const SumIG& s1, const SumIG& s2, const SumIG& s3,
-                        float n, float inv_n, const IGGrid& G, float& mJ, float& mQ, float& var,
-                        float& cov) {
-  const unsigned ni = (unsigned)(int)n;
-  const int D = (int)(ni * (unsigned)s2.h - (unsigned)s0.h * (unsigned)s0.h);
-  const int E = (int)(ni * (unsigned)s3.h - (unsigned)s0.h * (unsigned)s1.h);
-  const float hJ = G.gJ * small_int_to_float(s0.h);  // g_J sum m_J (exact)
-  const float hQ = G.gQ * small_int_to_float(s1.h);
-  const float lv = fmaf(n, s2.l, -fmaf(2.0f * hJ + s0.l, s0.l, 0.0f));
-  const float lc = fmaf(n, s3.l, -fmaf(hJ, s1.l, fmaf(hQ + s1.l, s0.l, 0.0f)));
-  const float inv2 = inv_n * inv_n;
-  mJ = (hJ + s0.l) * inv_n;
-  mQ = (hQ + s1.l) * inv_n;
-  var = fmaf(G.gJ * G.gJ, __int2float_rn(D), lv) * inv2;
-  cov = fmaf(G.gJ * G.gQ, __int2float_rn(E), lc) * inv2;
-}
-
 // Column-sum update by one input row's deviations (sign +1: the row enters,
 // -1: it leaves).
 template <class ACC>
@@ -342,28 +296,6 @@ GFD_D void col_update(ACC (&V)[4][4], const float (&J)[4], const float (&Q)[4], 
   }
 }
 
-GFD_D void col_update(SumIG (&V)[4][4], const float (&J)[4], const float (&Q)[4], float sgn,
-                      const IGGrid& G) {
-  const int si = sgn > 0.0f ? 1 : -1;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    int mJ, mQ;
-    float Jh, Jl, Qh, Ql;
-    ig_split(J[k], G.igJ, G.gJ, G.mgJ, mJ, Jh, Jl);
-    ig_split(Q[k], G.igQ, G.gQ, G.mgQ, mQ, Qh, Ql);
-    const int smJ = si * mJ;
-    V[0][k].h += smJ;
-    V[1][k].h += si * mQ;
-    V[2][k].h += smJ * mJ;
-    V[3][k].h += smJ * mQ;
-    const float sJl = sgn * Jl;
-    V[0][k].l += sJl;
-    V[1][k].l += sgn * Ql;
-    V[2][k].l = fmaf(sJl, J[k] + Jh, V[2][k].l);
-    V[3][k].l = fmaf(sgn * Jh, Ql, fmaf(sJl, Q[k], V[3][k].l));
-  }
-}
-
 template <class ACC>
 GFD_D void col_clear(ACC (&V)[4][4]) {
 #pragma unroll
@@ -371,15 +303,104 @@ GFD_D void col_clear(ACC (&V)[4][4]) {
 #pragma unroll
     for (int k = 0; k < 4; ++k) V[q][k].clear();
 }
-GFD_D void col_clear(SumIG (&V)[4][4]) {
+// Row window sums of a pair of quantities (single shuffles, packed additions).
+template <int RAD>
+GFD_D void hsum4_pair(const float2 (&v)[4], float2 (&s)[4]) {
+  float2 e[2 * RAD + 4];
 #pragma unroll
-  for (int q = 0; q < 4; ++q)
+  for (int q = 0; q < 2 * RAD + 4; ++q) {
+    const int c = q - RAD;
+    const int lo = c >= 0 ? c / 4 : -((3 - c) / 4);
+    e[q] = make_float2(lane_shift(v[c - 4 * lo].x, lo), lane_shift(v[c - 4 * lo].y, lo));
+  }
+  float2 acc = e[0];
+#pragma unroll
+  for (int q = 1; q <= 2 * RAD; ++q) acc = cadd(acc, e[q]);
+  s[0] = acc;
+#pragma unroll
+  for (int k = 1; k < 4; ++k) {
+    acc = cadd(acc, csub(e[k + 2 * RAD], e[k - 1]));
+    s[k] = acc;
+  }
+}
+
+// The window sums down the strip's columns of one lane and what a row needs of
+// them: the means of J and Q, sigma_k^2 and the covariance of the lane's four
+// windows.
+template <int RAD, class ACC>
+struct GfwCols {  // one accumulator per quantity and column
+  ACC V[4][4];    // [J, Q, J^2, J Q][column]
+  GFD_D void clear() { col_clear(V); }
+  GFD_D void update(const float2 (&x)[4], float sgn, const IGGrid& G) {
+    const float j[4] = {x[0].x, x[1].x, x[2].x, x[3].x};
+    const float q[4] = {x[0].y, x[1].y, x[2].y, x[3].y};
+    col_update(V, j, q, sgn, G);
+  }
+  template <class F>
+  GFD_D void windows(const float (&n)[4], const float (&inv_n)[4], const IGGrid& G, F out) const {
+    ACC S0[4], S1[4], S2[4], S3[4];
+    hsum4<RAD>(V[0], S0);
+    hsum4<RAD>(V[1], S1);
+    hsum4<RAD>(V[2], S2);
+    hsum4<RAD>(V[3], S3);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      V[q][k].h = 0;
-      V[q][k].l = 0.0f;
+      float mJ, mQ, var, cov;
+      window_stats(S0[k], S1[k], S2[k], S3[k], n[k], inv_n[k], G, mJ, mQ, var, cov);
+      out(k, mJ, mQ, var, cov);
     }
-}
+  }
+};
+
+// Split sums, in pairs.
+template <int RAD>
+struct GfwCols<RAD, SumIG> {
+  float2 h01[4], h23[4];  // (m_J, m_Q), (m_J^2, m_J m_Q) per column, exact
+  float2 l01[4], l23[4];  // the remainders' parts
+  GFD_D void clear() {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) h01[k] = h23[k] = l01[k] = l23[k] = make_float2(0.0f, 0.0f);
+  }
+  // one input row's deviations enter (sgn 1) or leave (sgn -1; a constant)
+  GFD_D void update(const float2 (&x)[4], float sgn, const IGGrid& G) {
+    const float2 mag = make_float2(kMagic, kMagic);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float2 m = csub(__ffma2_rn(x[k], G.ig, mag), mag);
+      const float2 xh = __fmul2_rn(m, G.g);
+      const float2 xl = csub(x[k], xh);
+      const float sm = sgn * m.x, sx = sgn * x[k].x, sl = sgn * xl.x;
+      h01[k] = sgn > 0.0f ? cadd(h01[k], m) : csub(h01[k], m);
+      h23[k] = __ffma2_rn(make_float2(sm, sm), m, h23[k]);
+      l01[k] = sgn > 0.0f ? cadd(l01[k], xl) : csub(l01[k], xl);
+      l23[k] = __ffma2_rn(make_float2(sx, sx), xl, __ffma2_rn(make_float2(sl, sl), xh, l23[k]));
+    }
+  }
+  template <class F>
+  GFD_D void windows(const float (&n)[4], const float (&inv_n)[4], const IGGrid& G, F out) const {
+    float2 S01[4], S23[4], L01[4], L23[4];
+    hsum4_pair<RAD>(h01, S01);
+    hsum4_pair<RAD>(h23, S23);
+    hsum4_pair<RAD>(l01, L01);
+    hsum4_pair<RAD>(l23, L23);
+    const float2 gg = make_float2(G.g.x * G.g.x, G.g.x * G.g.y);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float2 sJ = make_float2(S01[k].x, S01[k].x), n2 = make_float2(n[k], n[k]);
+      // (n S_mm - S_m^2, n S_mJmQ - S_mJ S_mQ): p + e the exact products
+      const float2 p = __fmul2_rn(sJ, S01[k]), pn = make_float2(-p.x, -p.y);
+      const float2 e = __ffma2_rn(sJ, S01[k], pn);
+      const float2 D = csub(__ffma2_rn(n2, S23[k], pn), e);
+      const float2 hh = __fmul2_rn(G.g, S01[k]);  // (g_J sum m_J, g_Q sum m_Q)
+      const float2 t = __ffma2_rn(hh, make_float2(2.0f, 1.0f), L01[k]);  // 2 h_J + l_J, h_Q + l_Q
+      const float2 c = __fmul2_rn(t, make_float2(L01[k].x, L01[k].x));
+      const float2 lo = __ffma2_rn(n2, L23[k], make_float2(-c.x, -fmaf(hh.x, L01[k].y, c.y)));
+      const float2 m = cscale(cadd(hh, L01[k]), inv_n[k]);
+      const float2 vc = cscale(__ffma2_rn(gg, D, lo), inv_n[k] * inv_n[k]);
+      out(k, m.x, m.y, vc.x, vc.y);
+    }
+  }
+};
 
 // Pixels of the window of radius RAD about position x in [0, L) that lie in
 // [0, L) (truncated windows).
@@ -389,28 +410,36 @@ GFD_D int window_count(int x, int L, int RAD) {
   return b - a + 1;
 }
 
+// 1/n for small integers n as floats, the correctly rounded quotient.
+GFD_D float rcp_count(float n) {
+  const float q = __fdividef(1.0f, n);
+  return fmaf(fmaf(-n, q, 1.0f), q, q);
+}
+
 template <int RAD, class ACC, bool TRUNC>
 GFD_D void gfw_items(const ClassDesc& cd, const ImgDesc* __restrict__ imgs, ImgState* st,
-                     int iter, bool shifted, int H, float* ring, int gwarp, int nwarps) {
+                     int iter, bool shifted, int rows, float* ring, int gwarp, int nwarps) {
   using G = GfwGeom<RAD>;
   constexpr int WIN = G::WIN, HALO = G::HALO, WOUT = G::WOUT, RI = G::RI;
   const int lane = threadIdx.x & 31;
   const int M = cd.M, N = cd.N;
   const int strips = (N + WOUT - 1) / WOUT;
-  const int per_img = strips * (M / H);
+  const int per_img = strips * ((M + rows - 1) / rows);
   const int n_items = cd.n_img * per_img;
   const float n_full = (float)(WIN * WIN);
   const float inv_full = 1.0f / n_full;
-  float* const ra = ring;                   // [WIN][GFW_COLS] a
-  float* const rb = ra + WIN * GFW_COLS;    // [WIN][GFW_COLS] b
-  float* const rI = rb + WIN * GFW_COLS;    // [RI][GFW_COLS] I
-  float* const rP = rI + RI * GFW_COLS;     // [RI][GFW_COLS] p
+  // rings of rows of (a, b) and of (J, Q): this lane's columns 0, 1 of a row at
+  // [row], columns 2, 3 half a row on, as (x0, y0, x1, y1)
+  float4* const rab = reinterpret_cast<float4*>(ring) + lane;
+  constexpr int ROW = GFW_COLS / 2, HALF = ROW / 2;  // float4 per ring row
+  float4* const rjq = rab + WIN * ROW;
   // this lane's columns lie in the strip's output part
   const bool out_lane = 4 * lane >= HALO && 4 * lane < HALO + WOUT;
 
   for (int item = gwarp; item < n_items; item += nwarps) {
     const int li = item / per_img, rem = item - li * per_img;
-    const int y0 = (rem / strips) * H, x0 = (rem % strips) * WOUT;
+    const int y0 = (rem / strips) * rows, x0 = (rem % strips) * WOUT;
+    const int H = rows < M - y0 ? rows : M - y0;
     const int gi = cd.img0 + li;
     const ImgDesc& d = imgs[gi];
     const float* __restrict__ I = d.uI;
@@ -443,96 +472,112 @@ GFD_D void gfw_items(const ClassDesc& cd, const ImgDesc* __restrict__ imgs, ImgS
     if constexpr (std::is_same<ACC, SumIG>::value) {
       // |J| <= max |u_I| + |c_I| (the bound the inverse row pass recorded)
       const ImgState* S = st + gi;
-      ig_grid<RAD>(__uint_as_float(__ldcg(&S->absmax[0])) + fabsf(cI), G.gJ, G.igJ, G.mgJ);
-      ig_grid<RAD>(__uint_as_float(__ldcg(&S->absmax[1])) + fabsf(cP), G.gQ, G.igQ, G.mgQ);
+      ig_grid<RAD>(__uint_as_float(__ldcg(&S->absmax[0])) + fabsf(cI), G.g.x, G.ig.x);
+      ig_grid<RAD>(__uint_as_float(__ldcg(&S->absmax[1])) + fabsf(cP), G.g.y, G.ig.y);
     }
-    // input row j of the item is image row y0 - 2r + j, ring slot j % RI
+    // input row j of the item is image row y0 - 2r + j; it stays in ring slot
+    // j % RI until row j + RI enters
     const int nin = H + 4 * RAD;
-    auto fetch = [&](int j) {
-      if (j < nin) {
-        const size_t off = (size_t)((y0 - 2 * RAD + j) & (M - 1)) * N + gx;
-        cp_async16(rI + (j % RI) * GFW_COLS + 4 * lane, I + off);
-        cp_async16(rP + (j % RI) * GFW_COLS + 4 * lane, P + off);
-      }
+    auto row_off = [&](int j) { return (unsigned)((y0 - 2 * RAD + j) & (M - 1)) * N + gx; };
+    auto load = [&](int j, float4& vi, float4& vp) {
+      const unsigned off = row_off(j);
+      vi = __ldcg(reinterpret_cast<const float4*>(I + off));
+      vp = __ldcg(reinterpret_cast<const float4*>(P + off));
     };
-    auto ring4 = [&](const float* r, int j) {
-      return reinterpret_cast<const float4*>(r + (j % RI) * GFW_COLS)[lane];
-    };
-    // deviations of input row j about the references (zero outside the
-    // canvas for truncated windows)
-    auto devs = [&](int j, float (&J)[4], float (&Q)[4]) {
-      const float4 iv = ring4(rI, j), pv = ring4(rP, j);
-      J[0] = iv.x - cI; J[1] = iv.y - cI; J[2] = iv.z - cI; J[3] = iv.w - cI;
-      Q[0] = pv.x - cP; Q[1] = pv.y - cP; Q[2] = pv.z - cP; Q[3] = pv.w - cP;
+    const float2 cc = make_float2(cI, cP);
+    // deviations of input row j about the references (zero outside the canvas
+    // for truncated windows), also put into ring slot `slot`
+    auto enter = [&](int j, int slot, const float4& vi, const float4& vp, float2 (&x)[4]) {
+      x[0] = csub(make_float2(vi.x, vp.x), cc);
+      x[1] = csub(make_float2(vi.y, vp.y), cc);
+      x[2] = csub(make_float2(vi.z, vp.z), cc);
+      x[3] = csub(make_float2(vi.w, vp.w), cc);
       if constexpr (TRUNC) {
         const int yy = y0 - 2 * RAD + j;
         const float rm = (yy >= 0 && yy < M) ? 1.0f : 0.0f;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          J[k] *= rm * cmask[k];
-          Q[k] *= rm * cmask[k];
-        }
+        for (int k = 0; k < 4; ++k) x[k] = cscale(x[k], rm * cmask[k]);
       }
+      rjq[slot * ROW] = make_float4(x[0].x, x[0].y, x[1].x, x[1].y);
+      rjq[slot * ROW + HALF] = make_float4(x[2].x, x[2].y, x[3].x, x[3].y);
     };
-    for (int j = 0; j <= 2 * RAD; ++j) fetch(j);
-    cp_async_commit();
+    auto ring_row = [&](int slot, float2 (&x)[4]) {
+      const float4 u = rjq[slot * ROW], v = rjq[slot * ROW + HALF];
+      x[0] = make_float2(u.x, u.y);
+      x[1] = make_float2(u.z, u.w);
+      x[2] = make_float2(v.x, v.y);
+      x[3] = make_float2(v.z, v.w);
+    };
+    GfwCols<RAD, ACC> V;
+    float2 VA[4];  // (a, b) per column: window sums down the columns
 #pragma unroll
-    for (int a = 1; a < GFW_AHEAD; ++a) {
-      fetch(2 * RAD + a);
-      cp_async_commit();
-    }
-    ACC V[4][4];     // [J, Q, J^2, J Q][column]: window sums down the columns
-    float VA[2][4];  // [a, b][column]
+    for (int k = 0; k < 4; ++k) VA[k] = make_float2(0.0f, 0.0f);
     float err = 0.0f;
+    // the first window's rows but one go to the ring; the next row waits in
+    // registers
+    float4 nI, nP;
+    load(0, nI, nP);
+    for (int j = 0; j < 2 * RAD; ++j) {
+      float2 x[4];
+      const float4 vi = nI, vp = nP;
+      load(j + 1, nI, nP);
+      enter(j, j, vi, vp, x);
+    }
+    float2 old[4];  // row s - 1: the guidance of output row s - 1 - 2r, leaving at step s
+    // ring slots of input rows s and s + 2r and of stats row s
+    int s_cur = 0, s_new = 2 * RAD, s_ab = 0;
     // stats row s (image row y0 - r + s) has its column window on input rows
     // j = s .. s + 2r; output row t = s - 2r needs stats rows t .. t + 2r
     for (int s = 0; s < H + 2 * RAD; ++s) {
-      fetch(s + 2 * RAD + GFW_AHEAD);  // its slot held row s - 2, no longer needed
-      cp_async_commit();
-      cp_async_wait<GFW_AHEAD>();      // rows up to s + 2r have landed
       const int t = s - 2 * RAD;  // output row (if >= 0)
       // the reference row of the ISNR sums is requested early (used last)
       float4 g = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
       if (uo && store && t >= 0)
         g = __ldg(reinterpret_cast<const float4*>(uo + (size_t)((y0 + t) & (M - 1)) * N + gx));
+      float2 x[4];
+      enter(s + 2 * RAD, s_new, nI, nP, x);
+      if (s + 1 < H + 2 * RAD) load(s + 2 * RAD + 1, nI, nP);
+      if (s + 2 * RAD + GFW_AHEAD < nin && (lane & 7) == 0) {  // one request per 128 bytes
+        const unsigned off = row_off(s + 2 * RAD + GFW_AHEAD);
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(I + off));
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(P + off));
+      }
       if (s % ACC::kSub == 0) {
-        col_clear(V);
-#pragma unroll
+        V.clear();
+        int slot = s_cur;
+#pragma unroll(ACC::kSub < 1000 ? WIN : 1)
         for (int dd = 0; dd < WIN; ++dd) {
-          float J[4], Q[4];
-          devs(s + dd, J, Q);
-          col_update(V, J, Q, 1.0f, G);
+          float2 y[4];
+          ring_row(slot, y);
+          V.update(y, 1.0f, G);
+          slot = slot + 1 == RI ? 0 : slot + 1;
         }
       } else {
-        float Jn[4], Qn[4], Jo[4], Qo[4];
-        devs(s + 2 * RAD, Jn, Qn);
-        devs(s - 1, Jo, Qo);
-        col_update(V, Jn, Qn, 1.0f, G);
-        col_update(V, Jo, Qo, -1.0f, G);
+        V.update(x, 1.0f, G);
+        V.update(old, -1.0f, G);
       }
+      ring_row(s_cur, old);
       // 2. row window sums -> a_k (Eq. 3), b_k (Eq. 4)
-      ACC S0[4], S1[4], S2[4], S3[4];
-      hsum4<RAD>(V[0], S0);
-      hsum4<RAD>(V[1], S1);
-      hsum4<RAD>(V[2], S2);
-      hsum4<RAD>(V[3], S3);
-      float A[4], B[4];
-      float nrow = 0.0f, srow_mask = 1.0f;
+      float n[4], inv_n[4];
+      float srow_mask = 1.0f;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        n[k] = n_full;
+        inv_n[k] = inv_full;
+      }
       if constexpr (TRUNC) {
         const int ys = y0 - RAD + s;
         const bool in = ys >= 0 && ys < M;
         srow_mask = in ? 1.0f : 0.0f;
-        nrow = in ? (float)window_count(ys, M, RAD) : 1.0f;
-      }
+        const float nrow = in ? (float)window_count(ys, M, RAD) : 1.0f;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        float n = n_full, inv_n = inv_full;
-        if constexpr (TRUNC) {
-          n = nrow * ncol[k];
-          inv_n = __frcp_rn(n);
+        for (int k = 0; k < 4; ++k) {
+          n[k] = nrow * ncol[k];
+          inv_n[k] = rcp_count(n[k]);
         }
-        float mJ, mQ, var, cov;
-        window_stats(S0[k], S1[k], S2[k], S3[k], n, inv_n, G, mJ, mQ, var, cov);
+      }
+      float A[4], B[4];
+      V.windows(n, inv_n, G, [&](int k, float mJ, float mQ, float var, float cov) {
         A[k] = __fdividef(cov, var + eps);  // var + eps >= eps > 0
         // b_k about the references: b_k = B_k + c_p - a_k c_I (Eq. 4), and the
         // constant parts are restored in the output below
@@ -542,59 +587,48 @@ GFD_D void gfw_items(const ClassDesc& cd, const ImgDesc* __restrict__ imgs, ImgS
           A[k] *= m;
           B[k] *= m;
         }
-      }
+      });
       // 3. ring slot s % WIN holds stats row s - WIN until overwritten here
-      float4* const sa = reinterpret_cast<float4*>(ra + (s % WIN) * GFW_COLS) + lane;
-      float4* const sb = reinterpret_cast<float4*>(rb + (s % WIN) * GFW_COLS) + lane;
       const bool slide = t > 0 && t % GFW_SUB != 0;
       if (slide) {
-        const float4 oa = *sa, ob = *sb;
-        VA[0][0] += A[0] - oa.x;
-        VA[0][1] += A[1] - oa.y;
-        VA[0][2] += A[2] - oa.z;
-        VA[0][3] += A[3] - oa.w;
-        VA[1][0] += B[0] - ob.x;
-        VA[1][1] += B[1] - ob.y;
-        VA[1][2] += B[2] - ob.z;
-        VA[1][3] += B[3] - ob.w;
+        const float4 u = rab[s_ab * ROW], v = rab[s_ab * ROW + HALF];
+        VA[0] = cadd(VA[0], csub(make_float2(A[0], B[0]), make_float2(u.x, u.y)));
+        VA[1] = cadd(VA[1], csub(make_float2(A[1], B[1]), make_float2(u.z, u.w)));
+        VA[2] = cadd(VA[2], csub(make_float2(A[2], B[2]), make_float2(v.x, v.y)));
+        VA[3] = cadd(VA[3], csub(make_float2(A[3], B[3]), make_float2(v.z, v.w)));
       }
-      *sa = make_float4(A[0], A[1], A[2], A[3]);
-      *sb = make_float4(B[0], B[1], B[2], B[3]);
+      rab[s_ab * ROW] = make_float4(A[0], B[0], A[1], B[1]);
+      rab[s_ab * ROW + HALF] = make_float4(A[2], B[2], A[3], B[3]);
+      s_cur = s_cur + 1 == RI ? 0 : s_cur + 1;
+      s_new = s_new + 1 == RI ? 0 : s_new + 1;
+      s_ab = s_ab + 1 == WIN ? 0 : s_ab + 1;
       if (t < 0) continue;
       if (!slide) {  // direct: the ring holds stats rows t .. t + 2r
 #pragma unroll
-        for (int k = 0; k < 4; ++k) VA[0][k] = VA[1][k] = 0.0f;
+        for (int k = 0; k < 4; ++k) VA[k] = make_float2(0.0f, 0.0f);
 #pragma unroll
         for (int q = 0; q < WIN; ++q) {
-          const float4 a4 = reinterpret_cast<const float4*>(ra + q * GFW_COLS)[lane];
-          const float4 b4 = reinterpret_cast<const float4*>(rb + q * GFW_COLS)[lane];
-          VA[0][0] += a4.x;
-          VA[0][1] += a4.y;
-          VA[0][2] += a4.z;
-          VA[0][3] += a4.w;
-          VA[1][0] += b4.x;
-          VA[1][1] += b4.y;
-          VA[1][2] += b4.z;
-          VA[1][3] += b4.w;
+          const float4 u = rab[q * ROW], v = rab[q * ROW + HALF];
+          VA[0] = cadd(VA[0], make_float2(u.x, u.y));
+          VA[1] = cadd(VA[1], make_float2(u.z, u.w));
+          VA[2] = cadd(VA[2], make_float2(v.x, v.y));
+          VA[3] = cadd(VA[3], make_float2(v.z, v.w));
         }
       }
       // 4. row window sums of a, b -> u = abar I + bbar (Eq. 5); the guidance
       //    at output row t is input row j = t + 2r = s.  With b_k = B_k + c_p
       //    - a_k c_I, u = abar (I - c_I) + Bbar + c_p: no large terms cancel
       //    where I and p are large (small lambda amplifies noise in them)
-      float SA[4], SB[4];
-      hsum4<RAD>(VA[0], SA);
-      hsum4<RAD>(VA[1], SB);
-      const float4 iv = ring4(rI, s);
-      const float ic[4] = {iv.x - cI, iv.y - cI, iv.z - cI, iv.w - cI};
+      float2 SAB[4];
+      hsum4_pair<RAD>(VA, SAB);
       float nout = 0.0f;
       if constexpr (TRUNC) nout = (float)window_count(y0 + t, M, RAD);
       float o[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        float inv_n = inv_full;
-        if constexpr (TRUNC) inv_n = __frcp_rn(nout * ncol[k]);
-        o[k] = fmaf(fmaf(SA[k], ic[k], SB[k]), inv_n, cP);
+        float in = inv_full;
+        if constexpr (TRUNC) in = rcp_count(nout * ncol[k]);
+        o[k] = fmaf(fmaf(SAB[k].x, old[k].x, SAB[k].y), in, cP);
       }
       if (store) {
         const size_t off = (size_t)((y0 + t) & (M - 1)) * N + gx;
@@ -605,7 +639,6 @@ GFD_D void gfw_items(const ClassDesc& cd, const ImgDesc* __restrict__ imgs, ImgS
         }
       }
     }
-    cp_async_wait<0>();  // the ring is reused by the next item
     if (uo) {
       // ||u - u_orig||^2 of this item: FP32 in the warp, FP64 across items
       err = warp_sum(err);
@@ -628,24 +661,16 @@ GFD_D void gfw_items(const ClassDesc& cd, const ImgDesc* __restrict__ imgs, ImgS
   }
 }
 
-template <class ACC, bool TRUNC>
+// One kernel per window radius: its registers and code are those of the radius.
+template <int RAD, class ACC, bool TRUNC>
 __global__ void __launch_bounds__(GFW_WARPS * 32)
 k_guided_filter(ClassDesc cd, const ImgDesc* __restrict__ imgs, ImgState* st, int iter,
-                int shifted_i, int rad, int H) {
+                int shifted, int H) {
   extern __shared__ __align__(16) float gsm[];
-  const int warp = threadIdx.x >> 5;
-  const int gwarp = blockIdx.x * GFW_WARPS + warp;
-  const int nwarps = gridDim.x * GFW_WARPS;
-  float* ring = gsm + (size_t)warp * gfw_ring_floats(rad);
-  const bool shifted = shifted_i != 0;
-#define GFD_GF_CASE(R) \
-  case R: gfw_items<R, ACC, TRUNC>(cd, imgs, st, iter, shifted, H, ring, gwarp, nwarps); break;
-  switch (rad) {
-    GFD_GF_CASE(0) GFD_GF_CASE(1) GFD_GF_CASE(2) GFD_GF_CASE(3) GFD_GF_CASE(4)
-    GFD_GF_CASE(5) GFD_GF_CASE(6) GFD_GF_CASE(7)
-    default: gfw_items<8, ACC, TRUNC>(cd, imgs, st, iter, shifted, H, ring, gwarp, nwarps); break;
-  }
-#undef GFD_GF_CASE
+  const int warp = threadIdx.x >> 5, W = blockDim.x >> 5;
+  gfw_items<RAD, ACC, TRUNC>(cd, imgs, st, iter, shifted != 0, H,
+                             gsm + (size_t)warp * gfw_ring_floats(RAD), blockIdx.x * W + warp,
+                             gridDim.x * W);
 }
 
 static int gf_sm_count() {
@@ -658,17 +683,34 @@ static int gf_sm_count() {
   return n;
 }
 
-using GfKernel = void (*)(ClassDesc, const ImgDesc*, ImgState*, int, int, int, int);
+using GfKernel = void (*)(ClassDesc, const ImgDesc*, ImgState*, int, int, int);
 
-static GfKernel gf_kernel(int var_mode, int boundary) {
-  const bool tr = boundary == GFD_BOUNDARY_TRUNCATED;
+template <int RAD>
+static GfKernel gf_kernel_rad(int var_mode, bool tr) {
   switch (var_mode) {
-    case GFD_VAR_FP64: return tr ? k_guided_filter<SumF64, true> : k_guided_filter<SumF64, false>;
+    case GFD_VAR_FP64:
+      return tr ? k_guided_filter<RAD, SumF64, true> : k_guided_filter<RAD, SumF64, false>;
     case GFD_VAR_FP32:
-    case GFD_VAR_FP32_RAW: return tr ? k_guided_filter<SumF32, true> : k_guided_filter<SumF32, false>;
+    case GFD_VAR_FP32_RAW:
+      return tr ? k_guided_filter<RAD, SumF32, true> : k_guided_filter<RAD, SumF32, false>;
     case GFD_VAR_DOUBLE_FLOAT:
-      return tr ? k_guided_filter<SumDF, true> : k_guided_filter<SumDF, false>;
-    default: return tr ? k_guided_filter<SumIG, true> : k_guided_filter<SumIG, false>;
+      return tr ? k_guided_filter<RAD, SumDF, true> : k_guided_filter<RAD, SumDF, false>;
+    default: return tr ? k_guided_filter<RAD, SumIG, true> : k_guided_filter<RAD, SumIG, false>;
+  }
+}
+
+static GfKernel gf_kernel(int var_mode, int boundary, int rad) {
+  const bool tr = boundary == GFD_BOUNDARY_TRUNCATED;
+  switch (rad) {
+    case 0: return gf_kernel_rad<0>(var_mode, tr);
+    case 1: return gf_kernel_rad<1>(var_mode, tr);
+    case 2: return gf_kernel_rad<2>(var_mode, tr);
+    case 3: return gf_kernel_rad<3>(var_mode, tr);
+    case 4: return gf_kernel_rad<4>(var_mode, tr);
+    case 5: return gf_kernel_rad<5>(var_mode, tr);
+    case 6: return gf_kernel_rad<6>(var_mode, tr);
+    case 7: return gf_kernel_rad<7>(var_mode, tr);
+    default: return gf_kernel_rad<GF_RMAX>(var_mode, tr);
   }
 }
 
@@ -700,51 +742,91 @@ cudaError_t launch_plane_absmax(const ClassLaunch& c, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// Rows per item (any number; the last item of a strip may have fewer).  A warp
+// takes H + 2r + a few row steps for its H output rows; alone on its scheduler a
+// step takes about twice its issue time (dependent latencies), so warps up to
+// two per scheduler are free and more share it.  Candidates fill one, two, ...
+// warps per scheduler and then whole waves of the resident warps, so that no
+// wave is left nearly empty: one 4096 x 4096 image, w = 9, has 37 strips, whose
+// 64-row items make 1.3 waves.  Few items are cut down to 4 rows to spread over
+// the GPU (one 256 x 256 image, w = 7: 20 us with 16 rows, 12 us).
+static int gfw_rows(int M, int hmax, int rad, int images, int strips, int resident, int scheds) {
+  const long long per_row = (long long)images * strips;
+  int best = 0;
+  double best_t = 0.0;
+  for (int c = 1; c <= 12; ++c) {
+    const int per_sched = resident / scheds < 1 ? 1 : resident / scheds;
+    const long long target = c < per_sched ? (long long)c * scheds
+                                           : (long long)(c - per_sched + 1) * resident;
+    long long nb = target / per_row;
+    if (nb < 1) nb = 1;
+    if (nb > M / 4) nb = M / 4;
+    int H = (int)((M + nb - 1) / nb);
+    if (H > hmax) H = hmax;
+    nb = (M + H - 1) / H;
+    const long long items = per_row * nb, active = items < resident ? items : resident;
+    const double waves = (double)((items + resident - 1) / resident);
+    const double share = (double)((active + scheds - 1) / scheds);
+    const double t = waves * (H + 2 * rad + 2 + 0.5 * rad) * (share > 2.0 ? share : 2.0);
+    if (best == 0 || t < best_t) {
+      best = H;
+      best_t = t;
+    }
+  }
+  return best;
+}
+
 // One launch per window radius present in the class (the images of a class
 // are ordered by radius, so each group is a contiguous range).  Items are
-// (image, strip, block of H rows); H is halved (down to 16) while there are
-// fewer items than resident warps.
+// (image, strip, block of H rows).  Wide windows' rings leave room for fewer
+// warps per SM than whole blocks of GFW_WARPS would use: blocks shrink to the
+// size that keeps most warps resident (w = 17: 6 instead of 4).
 cudaError_t launch_guided_filter(const ClassLaunch& c, int iter, int var_mode, int boundary,
                                  cudaStream_t s) {
-  const GfKernel kern = gf_kernel(var_mode, boundary);
   const int shifted = var_mode == GFD_VAR_FP32_RAW ? 0 : 1;
   for (int g = 0; g < c.n_rad_groups; ++g) {
     const RadGroup& rg = c.rad_groups[g];
+    const GfKernel kern = gf_kernel(var_mode, boundary, rg.rad);
     ClassDesc cd = c.cd;
     cd.img0 = rg.img0;
     cd.n_img = rg.n_img;
-    const size_t smem = (size_t)GFW_WARPS * gfw_ring_floats(rg.rad) * sizeof(float);
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, GFW_WARPS * 32, smem) !=
-            cudaSuccess ||
-        per_sm < 1)
-      per_sm = 1;
+    int W = GFW_WARPS, per_sm = 0;
+    for (int w = GFW_WARPS; w >= 1; w /= 2) {
+      int n = 0;
+      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+              &n, kern, w * 32, (size_t)w * gfw_ring_floats(rg.rad) * sizeof(float)) != cudaSuccess)
+        n = 0;
+      if (n * w > per_sm * W) {
+        W = w;
+        per_sm = n;
+      }
+    }
+    if (per_sm < 1) per_sm = 1;
+    const size_t smem = (size_t)W * gfw_ring_floats(rg.rad) * sizeof(float);
     const int div = c.grid_div > 1 ? c.grid_div : 1;
-    const int warps = (per_sm * gf_sm_count() + div - 1) / div * GFW_WARPS;
+    const int blocks = (per_sm * gf_sm_count() + div - 1) / div;
     const int strips = (cd.N + gfw_wout(rg.rad) - 1) / gfw_wout(rg.rad);
-    const int hmax = c.gf_rows > 0 ? c.gf_rows : DEF_GF_ROWS;
-    int H = cd.M < hmax ? cd.M : hmax;
-    while (H > 16 && cd.n_img * strips * (cd.M / H) < warps) H /= 2;
-    const int n_items = cd.n_img * strips * (cd.M / H);
-    int grid = (per_sm * gf_sm_count() + div - 1) / div;
-    const int need = (n_items + GFW_WARPS - 1) / GFW_WARPS;
-    if (grid > need) grid = need;
-    kern<<<grid, GFW_WARPS * 32, smem, s>>>(cd, c.imgs, c.st, iter, shifted, rg.rad, H);
+    // the default leaves the choice to the rule; a tuned shape bounds it
+    const int hmax = c.gf_rows > 0 && c.gf_rows != DEF_GF_ROWS ? c.gf_rows : 2 * DEF_GF_ROWS;
+    const int H = gfw_rows(cd.M, hmax, rg.rad, cd.n_img, strips, blocks * W,
+                           (4 * gf_sm_count() + div - 1) / div);
+    const int n_items = cd.n_img * strips * ((cd.M + H - 1) / H);
+    const int need = (n_items + W - 1) / W;
+    kern<<<blocks < need ? blocks : need, W * 32, smem, s>>>(cd, c.imgs, c.st, iter, shifted, H);
   }
   return cudaGetLastError();
 }
 
 cudaError_t configure_gf_kernel() {
-  const int bytes = (int)(GFW_WARPS * gfw_ring_floats(GF_RMAX) * sizeof(float));
-  const GfKernel ks[8] = {k_guided_filter<SumIG, false>,  k_guided_filter<SumIG, true>,
-                          k_guided_filter<SumDF, false>,  k_guided_filter<SumDF, true>,
-                          k_guided_filter<SumF64, false>, k_guided_filter<SumF64, true>,
-                          k_guided_filter<SumF32, false>, k_guided_filter<SumF32, true>};
-  for (GfKernel k : ks) {
-    const cudaError_t e =
-        cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e != cudaSuccess) return e;
-  }
+  const int modes[4] = {GFD_VAR_COMPENSATED, GFD_VAR_DOUBLE_FLOAT, GFD_VAR_FP64, GFD_VAR_FP32};
+  for (int mode : modes)
+    for (int b : {GFD_BOUNDARY_PERIODIC, GFD_BOUNDARY_TRUNCATED})
+      for (int rad = 0; rad <= GF_RMAX; ++rad) {
+        const cudaError_t e = cudaFuncSetAttribute(
+            (const void*)gf_kernel(mode, b, rad), cudaFuncAttributeMaxDynamicSharedMemorySize,
+            (int)(GFW_WARPS * gfw_ring_floats(rad) * sizeof(float)));
+        if (e != cudaSuccess) return e;
+      }
   return cudaSuccess;
 }
 
