@@ -25,7 +25,6 @@ constexpr int AUX_SLOTS = 8;
 // Fallback lambda passes launched per iteration from the fourth iteration on.
 constexpr int LATE_LAMBDA_PASSES = 2;
 constexpr int CHAINS = GFD_CHAINS;
-
 // A host <-> device copy that the host entry point asks a solve to issue.
 struct HostCopy {
   void* dst;
@@ -296,7 +295,8 @@ cudaError_t build_plan(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs, int i
     cl.cd.n_img = (int)members[ci].size();
     cl.cd.img0 = (int)pl.order.size();
     const ClassTune tn = c->tune.get(cl.cd.M, cl.cd.N);
-    cl.cd.TB = class_tile_width(cl.cd.M, cl.cd.N, tn.col_threads);
+    cl.short_cols = short_columns(cl.cd.M, cl.cd.N, cl.cd.n_img);
+    cl.cd.TB = class_tile_width(cl.cd.M, cl.cd.N, tn.col_threads, cl.short_cols);
     cl.row_threads = tn.row_threads;
     cl.gf_rows = tn.gf_rows;
     cl.class_id = (int)ci;
@@ -401,6 +401,12 @@ cudaError_t build_plan(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs, int i
     if (tm) GFD_CK(tm->end(s));                          \
   } while (0)
 
+// Classes whose fallback passes run as one launch: small canvases, and few
+// enough images that their clusters are resident together.
+bool lambda_loop(const ClassLaunch& cl) {
+  return cl.cd.M * cl.cd.N <= LAMBDA_LOOP_PIXELS && cl.cd.n_img <= 32;
+}
+
 cudaError_t record(gfdeconv_ctx* c, Plan& pl, cudaStream_t s, Timer* tm = nullptr,
                    bool chains = false) {
   long long L = 0;
@@ -465,8 +471,15 @@ cudaError_t record(gfdeconv_ctx* c, Plan& pl, cudaStream_t s, Timer* tm = nullpt
       // iterations 0-2 start from wide brackets; later ones from the
       // extrapolated root, which the fused pass almost always resolves
       const int npass = k < 3 ? passes : std::min(passes, LATE_LAMBDA_PASSES);
+      for (auto& cl : classes)
+        if (lambda_loop(cl)) {
+          if (tm) tm->cur_cls = cl.class_id;
+          GFD_T(GFD_PHASE_LAMBDA_PASS, launch_lambda_loop(cl, k, npass, s));
+          ++L;
+        }
       for (int p = 1; p <= npass; ++p)
         for (auto& cl : classes) {
+          if (lambda_loop(cl)) continue;
           if (tm) tm->cur_cls = cl.class_id;
           GFD_T(GFD_PHASE_LAMBDA_PASS, launch_lambda_pass(cl, k, p == npass, s));
           ++L;

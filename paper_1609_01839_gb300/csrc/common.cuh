@@ -100,6 +100,7 @@ struct ImgState {
   double lam;        // lambda of the current iteration (inf: branch u_E in K)
   double lo, hi;     // bracket of the nodes of the next pass
   double invT;       // 1 / T
+  double invP;       // 1 / (M N)
   int mode;          // next pass: 0 geometric nodes, 1 Chebyshev nodes, 2 moments about node[0]
   double lam_up;     // upper bound of the root from res and amax
   double res;        // ||h*u_E - y||^2 of the current iteration

@@ -247,6 +247,83 @@ GFD_D void fft_last(float2 (&x)[FftGeo<K, L>::RL], int kappa, const float2* buf)
   DFT<G::RL, INV>::run(x);
 }
 
+// ---------------------------------------------------------------------------
+// Short transforms of few columns (column passes of small problems): 4 elements
+// per thread, radix 4 with a last radix-2 stage where log2 M is odd, lengths at
+// run time.  A lone 256 x 256 image leaves the chip idle, so what counts is one
+// warp's path: its instruction count (a radix-16 pass runs some 2000 a thread,
+// this about 400) and its code, which is fetched anew by every launch.
+// ---------------------------------------------------------------------------
+GFD_HD int short_pos(int p) { return p + (p >> 3); }
+
+// Position of output group kappa of `bits` index bits (an even number): base-4
+// digits reversed.
+GFD_D int rev4(int kappa, int bits) {
+  if (bits == 0) return 0;
+  const unsigned r = __brev((unsigned)kappa) >> (32 - bits);
+  return (int)(((r & 0x55555555u) << 1) | ((r >> 1) & 0x55555555u));
+}
+
+// One butterfly of a stage of length Ls with its twiddles, offset jj.
+template <bool INV>
+GFD_D void short_butterfly(float2 (&x)[4], int Ls, int jj, const float2* __restrict__ tw) {
+  DFT<4, INV>::run(x);
+#pragma unroll
+  for (int i = 1; i < 4; ++i) x[i] = cmul(x[i], twiddle<INV>(tw, Ls, jj * i));
+}
+
+// NS transforms of length M = 2^lg >= 8 side by side: x[n][i] = element j + i M/4
+// on entry, X[j + i M/4] on return (thread j of M/4).  buf[n]: their buffers.
+// Contains block barriers; the buffers must be free on entry.
+template <int NS, bool INV>
+GFD_D void short_fft(float2 (&x)[NS][4], float2* const (&buf)[NS], int lg, int j,
+                     const float2* __restrict__ tw) {
+  int Ln = 1 << (lg - 2), Ls = 4 * Ln;
+#pragma unroll
+  for (int n = 0; n < NS; ++n) {
+    short_butterfly<INV>(x[n], Ls, j, tw);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) buf[n][short_pos(j + i * Ln)] = x[n][i];
+  }
+  Ls = Ln;
+#pragma unroll 1
+  while (Ls > 4) {
+    __syncthreads();
+    Ln = Ls >> 2;
+    const int jj = j & (Ln - 1), base = ((j - jj) << 2) + jj;
+#pragma unroll
+    for (int n = 0; n < NS; ++n) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) x[n][i] = buf[n][short_pos(base + i * Ln)];
+      short_butterfly<INV>(x[n], Ls, jj, tw);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) buf[n][short_pos(base + i * Ln)] = x[n][i];
+    }
+    Ls = Ln;
+  }
+  __syncthreads();
+  if (Ls == 4) {
+    const int base = rev4(j, lg - 2) * 4;
+#pragma unroll
+    for (int n = 0; n < NS; ++n) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) x[n][i] = buf[n][short_pos(base + i)];
+      DFT<4, INV>::run(x[n]);
+    }
+  } else {  // two radix-2 butterflies: kappa = j and j + M/4
+    const int b0 = rev4(j, lg - 1) * 2, b1 = rev4(j + (1 << (lg - 2)), lg - 1) * 2;
+#pragma unroll
+    for (int n = 0; n < NS; ++n) {
+      const float2 a0 = buf[n][short_pos(b0)], a1 = buf[n][short_pos(b0 + 1)];
+      const float2 c0 = buf[n][short_pos(b1)], c1 = buf[n][short_pos(b1 + 1)];
+      x[n][0] = cadd(a0, a1);
+      x[n][2] = csub(a0, a1);
+      x[n][1] = cadd(c0, c1);
+      x[n][3] = csub(c0, c1);
+    }
+  }
+}
+
 // Buffer stride of the B columns of a column pass, whose consecutive threads
 // walk B columns x 16/B consecutive elements: 16/B (mod 16) puts them on
 // distinct banks.

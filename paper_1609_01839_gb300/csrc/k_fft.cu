@@ -11,6 +11,8 @@
 // l % TB, TB the class's tile width.  A column item (TB columns, all M rows)
 // is then one contiguous block of memory, and a row item (rpc rows) writes a
 // contiguous run of rpc * TB values per tile.  TB = N/2 is plain row-major.
+#include <cooperative_groups.h>
+
 #include "fft.cuh"
 #include "lambda.cuh"
 #include "spectral.cuh"
@@ -392,7 +394,7 @@ k_col_fwd_lambda(ClassDesc cd, const ImgDesc* __restrict__ imgs, ImgState* st,
       block_sum_columns(d.part, cpi, KNODES + 1, KNODES + 1, red, s_tot);
       for (int q = threadIdx.x; q < cpi * (KNODES + 1); q += blockDim.x) d.part[q] = 0.0;
       if (threadIdx.x < 32)
-        lambda_update_warp(S, s_tot, (double)cd.M * cd.N, true, false, iter, d.lam_out, d.res_out,
+        lambda_update_warp(S, s_tot, true, false, iter, d.lam_out, d.res_out,
                            threadIdx.x);
       if (threadIdx.x == 0) {
         S->cta_done = 0;
@@ -549,62 +551,42 @@ k_col_fwd_lambda(ClassDesc cd, const ImgDesc* __restrict__ imgs, ImgState* st,
   }
 }
 
-// Fallback evaluation of Eq. 11 over the stored spectrum U_E for images whose
-// root is still open; a block covers `chunk` elements (in tiled order) of one
-// image.
-__global__ void __launch_bounds__(256)
-k_lambda_pass(ClassDesc cd, const ImgDesc* __restrict__ imgs, ImgState* st, int chunk, int iter,
-              int last_chance) {
-  __shared__ float s_nodes[KNODES];
-  __shared__ double red[32 * (KNODES + 1)];
-  __shared__ double s_tot[KNODES + 1];
-  __shared__ int s_flag;
-  __shared__ WarpAcc s_wacc;
-  const int Lc = cd.N / 2, TB = cd.TB, M = cd.M;
-  const int per_img = M * Lc;
-  const int cpi = per_img / chunk;
-  const int gi = cd.img0 + blockIdx.x / cpi;
-  ImgState* S = st + gi;
-  if (__ldcg(&S->need) == 0) return;
-  const ImgDesc& d = imgs[gi];
-  for (int q = threadIdx.x; q < KNODES; q += blockDim.x) s_nodes[q] = __ldcg(&S->node[q]);
-  warp_acc_clear(&s_wacc);
-  __syncthreads();
-  float2 nodes[KNODES / 2];
-#pragma unroll
-  for (int q = 0; q < KNODES / 2; ++q) nodes[q] = make_float2(s_nodes[2 * q], s_nodes[2 * q + 1]);
-  BinAcc acc;
-  acc.clear();
-  const int e0 = (blockIdx.x % cpi) * chunk;
+// The node sums of Eq. 11 over `pairs` bin pairs (in tiled order) from pair p0
+// on, by nt threads of which this is thread t, folded into wa.  Bins in pairs
+// (b, b+1) of one tile row, read as 16-byte vectors; runs of 8 pairs per
+// thread between folds (uniform control flow).
+GFD_D void pass_bins(const ClassDesc& cd, const ImgDesc& d, const ImgState* S,
+                     const float2 (&nodes)[KNODES / 2], int p0, int pairs, int t, int nt,
+                     WarpAcc* wa) {
+  const int TB = cd.TB, M = cd.M;
   const int lg_tile = __ffs(M * TB) - 1, lg_tb = __ffs(TB) - 1;  // powers of two
-  // bins in pairs (b, b+1) of one tile row, read as 16-byte vectors; runs of
-  // 8 pairs per thread between folds (uniform control flow)
   const float4* S4 = reinterpret_cast<const float4*>(d.S);
   const float4* H4 = reinterpret_cast<const float4*>(d.H);
   const float4* Y4 = reinterpret_cast<const float4*>(d.Y);
-  const int pairs = chunk / 2, p0 = e0 / 2;
-  for (int base = 0; base < pairs; base += 8 * blockDim.x) {
+  BinAcc acc;
+  acc.clear();
+  for (int base = 0; base < pairs; base += 8 * nt) {
 #pragma unroll 4
     for (int q = 0; q < 8; ++q) {
-      const int pi = base + q * blockDim.x + threadIdx.x;
+      const int pi = base + q * nt + t;
       if (pi < pairs) {
         const int e = 2 * (p0 + pi);
-        const int t = e >> lg_tile, rem = e & ((1 << lg_tile) - 1);
+        const int tl = e >> lg_tile, rem = e & ((1 << lg_tile) - 1);
         const int k = rem >> lg_tb, b = rem & (TB - 1);  // b even
-        const float4 U2 = __ldcs(&S4[p0 + pi]);
-        const float4 H2 = __ldg(&H4[p0 + pi]), Y2 = __ldg(&Y4[p0 + pi]);
+        const float4 U2 = __ldcg(&S4[p0 + pi]);
+        const float4 H2 = __ldcg(&H4[p0 + pi]), Y2 = __ldcg(&Y4[p0 + pi]);
         {  // bin b + 1 (never column 0)
           const float2 H = make_float2(H2.z, H2.w);
           const float2 r = csub(cmul(H, make_float2(U2.z, U2.w)), make_float2(Y2.z, Y2.w));
           accum_bin(2.0f * fmaf(r.x, r.x, r.y * r.y), fmaf(H.x, H.x, H.y * H.y), nodes, acc);
         }
-        if (t != 0 || b != 0) {
+        if (tl != 0 || b != 0) {
           const float2 H = make_float2(H2.x, H2.y);
           const float2 r = csub(cmul(H, make_float2(U2.x, U2.y)), make_float2(Y2.x, Y2.y));
           accum_bin(2.0f * fmaf(r.x, r.x, r.y * r.y), fmaf(H.x, H.x, H.y * H.y), nodes, acc);
         } else {  // packed column 0: bins (k, 0) and (k, N/2)
           const float2 U = make_float2(U2.x, U2.y);
-          const float2 Um = d.S[(size_t)((M - k) & (M - 1)) * TB];
+          const float2 Um = __ldcg(&d.S[(size_t)((M - k) & (M - 1)) * TB]);
           float2 UA, UB;
           unpack_pair(U, Um, UA, UB);
           const float2 HA = d.H0[k], HB = d.HN[k], YA = d.Y0[k], YB = d.YN[k];
@@ -622,14 +604,41 @@ k_lambda_pass(ClassDesc cd, const ImgDesc* __restrict__ imgs, ImgState* st, int 
         }
       }
     }
-    warp_fold(acc, KNODES, &s_wacc);
+    warp_fold(acc, KNODES, wa);
   }
+}
+
+// Fallback evaluation of Eq. 11 over the stored spectrum U_E for images whose
+// root is still open; a block covers `chunk` elements (in tiled order) of one
+// image.
+__global__ void __launch_bounds__(256)
+k_lambda_pass(ClassDesc cd, const ImgDesc* __restrict__ imgs, ImgState* st, int chunk, int iter,
+              int last_chance) {
+  __shared__ float s_nodes[KNODES];
+  __shared__ double red[32 * (KNODES + 1)];
+  __shared__ double s_tot[KNODES + 1];
+  __shared__ int s_flag;
+  __shared__ WarpAcc s_wacc;
+  const int per_img = cd.M * (cd.N / 2);
+  const int cpi = per_img / chunk;
+  const int gi = cd.img0 + blockIdx.x / cpi;
+  ImgState* S = st + gi;
+  if (__ldcg(&S->need) == 0) return;
+  const ImgDesc& d = imgs[gi];
+  for (int q = threadIdx.x; q < KNODES; q += blockDim.x) s_nodes[q] = __ldcg(&S->node[q]);
+  warp_acc_clear(&s_wacc);
+  __syncthreads();
+  float2 nodes[KNODES / 2];
+#pragma unroll
+  for (int q = 0; q < KNODES / 2; ++q) nodes[q] = make_float2(s_nodes[2 * q], s_nodes[2 * q + 1]);
+  pass_bins(cd, d, S, nodes, (blockIdx.x % cpi) * (chunk / 2), chunk / 2, threadIdx.x, blockDim.x,
+            &s_wacc);
   block_partials_folded(&s_wacc, d.part + (size_t)(blockIdx.x % cpi) * (KNODES + 1));
   if (last_item(&S->cta_done, cpi, &s_flag)) {
     block_sum_columns(d.part, cpi, KNODES + 1, KNODES + 1, red, s_tot);
     for (int q = threadIdx.x; q < cpi * (KNODES + 1); q += blockDim.x) d.part[q] = 0.0;
     if (threadIdx.x < 32)
-      lambda_update_warp(S, s_tot, (double)cd.M * cd.N, false, last_chance != 0, iter,
+      lambda_update_warp(S, s_tot, false, last_chance != 0, iter,
                          d.lam_out, d.res_out, threadIdx.x);
     if (threadIdx.x == 0) {
       S->cta_done = 0;
@@ -638,6 +647,59 @@ k_lambda_pass(ClassDesc cd, const ImgDesc* __restrict__ imgs, ImgState* st, int 
   }
 }
 
+
+// All fallback passes of an iteration for small canvases: a cluster of
+// LOOP_BLOCKS blocks per image repeats the pass until the image's root is
+// resolved (npass at most), its blocks' sums meeting in the first block's
+// shared memory.  One launch instead of npass, most of which find nothing to
+// do and cost 2.5 to 4 us each on the chain of a small solve.
+constexpr int LOOP_BLOCKS = 8, LOOP_THREADS = 512;
+
+__global__ void __cluster_dims__(LOOP_BLOCKS, 1, 1) __launch_bounds__(LOOP_THREADS)
+k_lambda_loop(ClassDesc cd, const ImgDesc* __restrict__ imgs, ImgState* st, int iter, int npass) {
+  namespace cg = cooperative_groups;
+  __shared__ double s_part[LOOP_BLOCKS][KNODES + 1];  // of the cluster's first block
+  __shared__ double s_tot[KNODES + 1];
+  __shared__ WarpAcc s_wacc;
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = blockIdx.x % LOOP_BLOCKS;
+  const int gi = cd.img0 + blockIdx.x / LOOP_BLOCKS;
+  ImgState* S = st + gi;
+  // read by every block before the first cluster barrier, changed after it
+  if (__ldcg(&S->need) == 0) return;
+  const ImgDesc& d = imgs[gi];
+  const int pairs = cd.M * (cd.N / 2) / 2;
+  double* part = cl.map_shared_rank(&s_part[0][0], 0) + rank * (KNODES + 1);
+  for (int p = 1; p <= npass; ++p) {
+    float2 nodes[KNODES / 2];
+#pragma unroll
+    for (int q = 0; q < KNODES / 2; ++q)
+      nodes[q] = __ldcg(reinterpret_cast<const float2*>(S->node) + q);
+    warp_acc_clear(&s_wacc);
+    __syncthreads();
+    pass_bins(cd, d, S, nodes, 0, pairs, rank * LOOP_THREADS + threadIdx.x,
+              LOOP_BLOCKS * LOOP_THREADS, &s_wacc);
+    block_partials_folded(&s_wacc, part);
+    cl.sync();
+    if (rank == 0 && threadIdx.x < 32) {
+      if (threadIdx.x <= KNODES) {
+        double v[LOOP_BLOCKS];
+#pragma unroll
+        for (int r = 0; r < LOOP_BLOCKS; ++r) v[r] = s_part[r][threadIdx.x];
+#pragma unroll
+        for (int o = LOOP_BLOCKS / 2; o > 0; o /= 2)
+#pragma unroll
+          for (int r = 0; r < o; ++r) v[r] += v[r + o];
+        s_tot[threadIdx.x] = v[0];
+      }
+      __syncwarp();
+      lambda_update_warp(S, s_tot, false, p == npass, iter, d.lam_out, d.res_out, threadIdx.x);
+      __threadfence();
+    }
+    cl.sync();
+    if (__ldcg(&S->need) == 0) break;  // the same for the whole cluster
+  }
+}
 
 // Eq. 8 and 9 at rows k of packed column 0, which holds the bins (k, 0) and
 // (k, N/2): U_I and U_p of both, packed again.
@@ -759,6 +821,160 @@ k_col_solve_inv(ClassDesc cd, const ImgDesc* __restrict__ imgs, ImgState* st,
 }
 
 // ---------------------------------------------------------------------------
+// Column passes of small problems: one item per block, 4 rows per thread
+// (short_fft), every global load requested before the transform.  Tiles of
+// class_tile_width.  One 256 x 256 image: forward pass 25 us as the persistent
+// radix-16 kernel (8 blocks of 256 threads), 15 us here, more than half of it
+// the reductions and the root of lambda behind the transform; solve pass 11 ->
+// 6 us.
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(512, 2)
+k_col_fwd_lambda_short(ClassDesc cd, const ImgDesc* __restrict__ imgs, ImgState* st,
+                       const float2* __restrict__ tw, int lg, int iter) {
+  extern __shared__ __align__(16) float2 smem[];
+  __shared__ double s_tot[KNODES + 1];
+  __shared__ int s_flag;
+  __shared__ WarpAcc s_wacc;
+  const int M = cd.M, B = cd.TB, Lc = cd.N / 2, cpi = Lc / B;
+  const int b = threadIdx.x & (B - 1), j = threadIdx.x >> (__ffs(B) - 1);
+  const int Q = M / 4;  // rows j + i Q
+  const int cs = short_pos(M) + 1;
+  double* red = reinterpret_cast<double*>(smem + ((B * cs + 1) & ~1));
+  const int gi = cd.img0 + blockIdx.x / cpi, t = blockIdx.x % cpi;
+  const ImgDesc& d = imgs[gi];
+  ImgState* S = st + gi;
+  const size_t off = (size_t)t * M * B + b;
+  float2* spec = d.S + off;
+  float2 x[1][4], H[4], Y[4];
+  const bool pair0 = t == 0 && b == 0;  // packed column 0: bins (k, 0) and (k, N/2)
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int k = j + i * Q;
+    x[0][i] = load_stream(spec + k * B);
+    H[i] = pair0 ? __ldcg(&d.H0[k]) : load_stream(d.H + off + k * B);
+    Y[i] = pair0 ? __ldcg(&d.Y0[k]) : load_stream(d.Y + off + k * B);
+  }
+  __shared__ float2 s_nodes[KNODES / 2];
+  for (int q = threadIdx.x; q < KNODES / 2; q += blockDim.x)
+    s_nodes[q] = __ldcg(reinterpret_cast<const float2*>(S->node) + q);
+  const bool mom = __ldcg(&S->mode) == MODE_MOM;
+  warp_acc_clear(&s_wacc);  // first use follows the transform's barriers
+  if (t == 0) {  // the DC bin needs sum(u_E): total of the row pass's sums
+    block_sum_columns(d.rowsum, M, 1, 1, red, s_tot);
+    if (threadIdx.x == 0) S->sum_u = s_tot[0];
+  }
+  float2* const bufs[1] = {smem + b * cs};
+  short_fft<1, false>(x, bufs, lg, j, tw);
+  if (t == 0) {  // rows k and M - k of column 0 meet in shared memory
+    __syncthreads();
+    if (pair0) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) smem[j + i * Q] = x[0][i];
+    }
+    __syncthreads();
+  }
+  BinAcc acc;
+  acc.clear();
+  auto bin = [&](float2 h, float2 y, float2 u, float w, bool dc) {
+    const float2 e = csub(cmul(h, u), y);
+    float r = w * fmaf(e.x, e.x, e.y * e.y);
+    if (dc) {
+      // DC bin in FP64 from exact sums: d00 = sum(h) sum(u_E) - sum(y)
+      const double d00 = S->sum_h * s_tot[0] - S->sum_y;
+      S->d00 = d00;
+      r = (float)(d00 * d00);
+    }
+    const float a = fmaf(h.x, h.x, h.y * h.y);
+    if (mom)
+      accum_bin_moments(r, a, s_nodes[0].x, acc);
+    else
+      accum_bin(r, a, s_nodes, acc);
+  };
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int k = j + i * Q;
+    float2 U = x[0][i];
+    if (pair0) {
+      float2 UA, UB;
+      unpack_pair(smem[k], smem[(M - k) & (M - 1)], UA, UB);
+      bin(H[i], Y[i], UA, 1.0f, k == 0);
+      bin(__ldcg(&d.HN[k]), __ldcg(&d.YN[k]), UB, 1.0f, false);
+      if (k == 0) U.x = (float)s_tot[0];
+    } else {
+      bin(H[i], Y[i], U, 2.0f, false);  // bins l and N-l
+    }
+    spec[k * B] = U;
+  }
+  warp_fold(acc, mom ? KMOM : KNODES, &s_wacc);
+  block_partials_folded(&s_wacc, d.part + (size_t)t * (KNODES + 1));
+  if (last_item(&S->cta_done, cpi, &s_flag)) {
+    block_sum_columns(d.part, cpi, KNODES + 1, KNODES + 1, red, s_tot);
+    for (int q = threadIdx.x; q < cpi * (KNODES + 1); q += blockDim.x) d.part[q] = 0.0;
+    if (threadIdx.x < 32)
+      lambda_update_warp(S, s_tot, true, false, iter, d.lam_out, d.res_out,
+                         threadIdx.x);
+    if (threadIdx.x == 0) {
+      S->cta_done = 0;
+      __threadfence();
+    }
+  }
+}
+
+__global__ void __launch_bounds__(512)
+k_col_solve_inv_short(ClassDesc cd, const ImgDesc* __restrict__ imgs, ImgState* st,
+                      const float2* __restrict__ tw, const float* __restrict__ d2tab, int lg) {
+  extern __shared__ __align__(16) float2 smem[];
+  const int M = cd.M, B = cd.TB, Lc = cd.N / 2, cpi = Lc / B;
+  const int b = threadIdx.x & (B - 1), j = threadIdx.x >> (__ffs(B) - 1);
+  const int Q = M / 4, cs = short_pos(M) + 1;
+  const int gi = cd.img0 + blockIdx.x / cpi, t = blockIdx.x % cpi;
+  const ImgDesc& d = imgs[gi];
+  const int col = t * B + b;
+  const size_t off = (size_t)t * M * B + b;
+  const double lamd = __ldcg(&st[gi].lam);
+  const bool branch = !(lamd < 1e300);  // lambda = inf: u_I = u_p = u_E (Sec. 3.2)
+  const float lam = (float)lamd;
+  if (t == 0 && threadIdx.x == 0) {  // the inverse row pass re-forms them
+    st[gi].absmax[0] = 0u;
+    st[gi].absmax[1] = 0u;
+  }
+  const float d2c = __ldg(&d2tab[tab_off(cd.N) + col]);
+  float2 x[2][4];
+  if (branch) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) x[0][i] = x[1][i] = load_stream(d.S + off + (j + i * Q) * B);
+  } else if (col != 0) {
+    float2 U[4], H[4], Y[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int o = (j + i * Q) * B;
+      U[i] = load_stream(d.S + off + o);
+      H[i] = load_stream(d.H + off + o);
+      Y[i] = load_stream(d.Y + off + o);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      solve_bin(U[i], H[i], Y[i], lam, __ldg(&d2tab[tab_off(M) + j + i * Q]) + d2c, x[0][i],
+                x[1][i]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int k = j + i * Q;
+      const float4 v = solve_col0(d, M, B, k, lam, __ldg(&d2tab[tab_off(M) + k]));
+      x[0][i] = make_float2(v.x, v.y);
+      x[1][i] = make_float2(v.z, v.w);
+    }
+  }
+  float2* const bufs[2] = {smem + b * cs, smem + (B + b) * cs};
+  short_fft<2, true>(x, bufs, lg, j, tw);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    d.QI[off + (j + i * Q) * B] = x[0][i];
+    d.Qp[off + (j + i * Q) * B] = x[1][i];
+  }
+}
+
+// ---------------------------------------------------------------------------
 // launch configuration and dispatch
 // ---------------------------------------------------------------------------
 static int sm_count() {
@@ -805,7 +1021,12 @@ int rows_per_item(int L, int M, int row_threads) {
 // Tile width of a class's spectra = columns per column item: a block of about
 // col_threads threads (512 for M = 4096), at least 2 columns (16-byte
 // copies), at most N/2.
-int class_tile_width(int M, int N, int col_threads) {
+int class_tile_width(int M, int N, int col_threads, bool short_cols) {
+  if (short_cols) {
+    int B = M >= 1024 ? 2 : 4;  // M/4 threads per column: 512 per block at most
+    while (B * M / 4 < 32 && B < N / 2) B *= 2;
+    return B < N / 2 ? B : N / 2;
+  }
   const int T = M / fft_elems(FK_COL, M);
   const int ct = col_threads > 0 ? (col_threads > 256 ? 256 : col_threads) : DEF_COL_THREADS;
   const int threads = M >= 4096 ? 512 : ct;
@@ -941,8 +1162,31 @@ static void do_col_fwd_lambda(const ClassLaunch& c, const Tables& t, int iter, c
   GFD_COL_WIDTHS(do_col_fwd_lambda_w, M, c.cd.TB, c, t, iter, s);
 }
 
+// Small problems (all images of a class together): the short column passes.
+// Above SHORT_PIXELS the persistent ones, which pass fewer times through shared
+// memory, take over.  Whole solves of 15 iterations, short against persistent
+// passes: one 256^2 image 0.79 / 1.03 ms, one 512^2 1.00 / 1.06, one 1024^2 1.25 /
+// 1.25 (the forward pass loses what the solve pass gains).
+bool short_columns(int M, int N, int n_img) {
+  // (a block holds at least the 16 threads that a lambda update needs)
+  return M <= 1024 && M * N >= 128 && (long long)M * N * n_img <= SHORT_PIXELS;
+}
+
+static void do_col_fwd_lambda_short(const ClassLaunch& c, const Tables& t, int iter,
+                                    cudaStream_t s) {
+  const int M = c.cd.M, B = c.cd.TB, lg = __builtin_ctz(M);
+  const size_t smem = (size_t)((B * (short_pos(M) + 1) + 1) & ~1) * sizeof(float2) +
+                      16 * sizeof(double);
+  k_col_fwd_lambda_short<<<c.cd.n_img * (c.cd.N / 2 / B), B * M / 4, smem, s>>>(c.cd, c.imgs, c.st,
+                                                                               t.tw, lg, iter);
+}
+
 cudaError_t launch_col_fwd_lambda(const ClassLaunch& c, const Tables& t, int iter,
                                   cudaStream_t s) {
+  if (c.short_cols) {
+    do_col_fwd_lambda_short(c, t, iter, s);
+    return cudaGetLastError();
+  }
   switch (c.cd.M) {
     GFD_CASE_M(do_col_fwd_lambda, c, t, iter, s)
     default: return cudaErrorInvalidValue;
@@ -956,6 +1200,11 @@ cudaError_t launch_lambda_pass(const ClassLaunch& c, int iter, bool last_chance,
   const int chunk = per_img < 16384 ? per_img : 16384;
   const int nblk = c.cd.n_img * (per_img / chunk);
   k_lambda_pass<<<nblk, 256, 0, s>>>(c.cd, c.imgs, c.st, chunk, iter, last_chance ? 1 : 0);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_lambda_loop(const ClassLaunch& c, int iter, int npass, cudaStream_t s) {
+  k_lambda_loop<<<c.cd.n_img * LOOP_BLOCKS, LOOP_THREADS, 0, s>>>(c.cd, c.imgs, c.st, iter, npass);
   return cudaGetLastError();
 }
 
@@ -975,6 +1224,13 @@ static void do_col_solve_inv(const ClassLaunch& c, const Tables& t, cudaStream_t
 }
 
 cudaError_t launch_col_solve_inv(const ClassLaunch& c, const Tables& t, cudaStream_t s) {
+  if (c.short_cols) {
+    const int M = c.cd.M, B = c.cd.TB;
+    k_col_solve_inv_short<<<c.cd.n_img * (c.cd.N / 2 / B), B * M / 4,
+                            (size_t)2 * B * (short_pos(M) + 1) * sizeof(float2), s>>>(
+        c.cd, c.imgs, c.st, t.tw, t.d2, __builtin_ctz(M));
+    return cudaGetLastError();
+  }
   switch (c.cd.M) {
     GFD_CASE_M(do_col_solve_inv, c, t, s)
     default: return cudaErrorInvalidValue;

@@ -194,19 +194,29 @@ GFD_D void warp_fold(BinAcc& acc, int n, WarpAcc* wa) {
   acc.clear();
 }
 
+// Sum over groups of n consecutive lanes (n a power of two <= 32), FP64.  An
+// FP64 addition takes 70 cycles here: a tree instead of one thread's chain.
+GFD_D double group_sum_dbl(double v, int n) {
+  const unsigned int mask = upd_mask();
+  for (int o = n >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o);
+  return v;
+}
+
 // part[j] = sum over warps of hi + lo (FP64); clears the accumulators.
 // Synchronises before and after.
 GFD_D void block_partials_folded(WarpAcc* wa, double* part) {
   __syncthreads();
-  const int nwarp = num_warps();
-  for (int j = threadIdx.x; j <= KNODES; j += blockDim.x) {
-    double s = 0.0;
-    for (int w = 0; w < nwarp; ++w) {
-      s += (double)wa->hi[w][j] + (double)wa->lo[w][j];
+  const int nwarp = num_warps();  // a power of two <= 16: one thread per (sum, warp)
+  for (int e = threadIdx.x; e < 16 * nwarp; e += blockDim.x) {
+    const int j = e / nwarp, w = e - j * nwarp;
+    double v = 0.0;
+    if (j <= KNODES) {
+      v = (double)wa->hi[w][j] + (double)wa->lo[w][j];
       wa->hi[w][j] = 0.0f;
       wa->lo[w][j] = 0.0f;
     }
-    part[j] = s;
+    v = group_sum_dbl(v, nwarp);
+    if (j <= KNODES && w == 0) part[j] = v;
   }
   __syncthreads();
 }
@@ -236,12 +246,22 @@ GFD_D void block_sum_columns(const double* vals, int n, int stride, int m, doubl
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nwarp = num_warps();
   if (m > 1 && (blockDim.x & 31) == 0) {  // whole warps
-    for (int j = warp; j < m; j += nwarp) {
-      double s = 0.0;
-      for (int i = lane; i < n; i += 32) s += __ldcg(&vals[(size_t)i * stride + j]);
+    for (int j = warp; j < m; j += 2 * nwarp) {  // two columns' chains side by side
+      const int j2 = j + nwarp;
+      double s = 0.0, t = 0.0;
+      for (int i = lane; i < n; i += 32) {
+        s += __ldcg(&vals[(size_t)i * stride + j]);
+        if (j2 < m) t += __ldcg(&vals[(size_t)i * stride + j2]);
+      }
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (lane == 0) sums[j] = s;
+      for (int o = 16; o > 0; o >>= 1) {
+        s += __shfl_xor_sync(0xffffffffu, s, o);
+        t += __shfl_xor_sync(0xffffffffu, t, o);
+      }
+      if (lane == 0) {
+        sums[j] = s;
+        if (j2 < m) sums[j2] = t;
+      }
     }
     __syncthreads();
     return;
@@ -252,10 +272,10 @@ GFD_D void block_sum_columns(const double* vals, int n, int stride, int m, doubl
     s = warp_sum_dbl(s);
     if (lane == 0) red[warp] = s;
     __syncthreads();
-    if (threadIdx.x == 0) {
-      double t = 0.0;
-      for (int w = 0; w < nwarp; ++w) t += red[w];
-      sums[j] = t;
+    if (warp == 0) {
+      double t = lane < nwarp ? red[lane] : 0.0;
+      if (nwarp > 1) t = group_sum_dbl(t, nwarp);
+      if (lane == 0) sums[j] = t;
     }
     __syncthreads();
   }
@@ -407,7 +427,8 @@ GFD_D double interp_root_warp(float xm, float gm, int j, double rtol, int lane) 
   return exp(0.5 * (df_to_double(a) + df_to_double(b)));
 }
 
-// Record lambda_k and set up iteration k+1's fused first pass.  lambda jumps
+// Record lambda_k and set up iteration k+1's fused first pass (prev: the last
+// finite lambda before it).  lambda jumps
 // by a factor of 2..600 from the first iteration (u_E = 0) to the second, and
 // mostly falls to 0.2..1.2 of it in the third; the fourth stays within a few
 // percent of the third on most images, and later it changes smoothly.  The
@@ -416,7 +437,8 @@ GFD_D double interp_root_warp(float xm, float gm, int j, double rtol, int lane) 
 // interpolation to resolve it in the fused pass itself; later first passes
 // expand f about lambda_2, then about the extrapolation
 // lambda_k (lambda_k / lambda_{k-1}) (ratio clamped to [1/2, 2]).
-GFD_D void resolve_warp(ImgState* st, double lam, int iter, double* lam_out, int lane) {
+GFD_D void resolve_warp(ImgState* st, double lam, double prev, int iter, double* lam_out,
+                        int lane) {
   if (lane == 0) {
     st->lam = lam;
     st->need = 0;
@@ -425,8 +447,6 @@ GFD_D void resolve_warp(ImgState* st, double lam, int iter, double* lam_out, int
   // lambda = inf (or no finite root) keeps the pending bracket or centre
   if (isfinite(lam) && lam > 0.0) {
     const float l = (float)lam;
-    const double prev = st->lam_prev;
-    __syncwarp(upd_mask());  // every lane has read lam_prev
     if (iter == 0) {
       set_bracket_warp(st, fmaxf(l, (float)LAMBDA_LO), 150.0f * l, lane);
     } else if (iter == 1) {
@@ -451,6 +471,7 @@ GFD_D void resolve_warp(ImgState* st, double lam, int iter, double* lam_out, int
 // otherwise leaves the bracket of the next pass in (lo, hi).
 GFD_D bool moment_root_warp(const double* tot, double scale, float c, int lane, double& lam,
                             float& lo, float& hi) {
+  static_assert(KMOM == 8, "the series is evaluated by halves of four terms");
   const int nl = upd_lanes();
   const unsigned int mask = upd_mask();
   // a_k = (k + 1) (-1)^k N_k / (P T), one per lane, then to every lane
@@ -490,10 +511,12 @@ GFD_D bool moment_root_warp(const double* tot, double scale, float c, int lane, 
   const float islope = __fdividef(1.0f, slope);
 #pragma unroll 1
   for (int it = 0; it < 5; ++it) {
-    double q = a[KMOM - 1];
-#pragma unroll
-    for (int k = KMOM - 2; k >= 0; --k) q = fma(q, e, a[k]);
-    const double F = fma(q, fma(e, e, fma(2.0, e, 1.0)), -1.0);
+    // the series by halves: four dependent FP64 operations (70 cycles each)
+    // instead of seven
+    const double e2 = e * e;
+    const double q0 = fma(fma(a[3], e, a[2]), e2, fma(a[1], e, a[0]));
+    const double q1 = fma(fma(a[7], e, a[6]), e2, fma(a[5], e, a[4]));
+    const double F = fma(fma(q1, e2 * e2, q0), fma(2.0, e, e2 + 1.0), -1.0);
     const float step = (float)F * islope;
     e -= (double)step;
     if (!(fabsf(step) > 1e-7f)) break;  // the next would be below 1e-13
@@ -505,7 +528,12 @@ GFD_D bool moment_root_warp(const double* tot, double scale, float c, int lane, 
   const float err = (KMOM + 1) * x4 * x4 * af[0] * g * g * islope * 2.0f / ((1.0f - x2) * d1 * d1);
   const float est = c * __fdividef(1.0f + er, 1.0f - er);
   if (slope > 0.0f && err <= MOM_TOL && est > (float)LAMBDA_LO) {
-    lam = (double)c * (1.0 + e) / (1.0 - e);
+    // c (1 + e) / (1 - e), the reciprocal by two Newton steps from FP32
+    const double d = 1.0 - e;
+    double q = (double)__fdividef(1.0f, (float)d);
+    q = fma(fma(-d, q, 1.0), q, q);
+    q = fma(fma(-d, q, 1.0), q, q);
+    lam = fma((double)c, e, (double)c) * q;
     return true;
   }
   // The root's side of c by the sign of f(c) - T; along it, the last |e| that
@@ -535,11 +563,13 @@ GFD_D bool moment_root_warp(const double* tot, double scale, float c, int lane, 
 // 32 lanes of one warp of the image's last block; every lane takes the same
 // decisions from the same values.  FP64 is limited to a handful of
 // operations (the sums themselves are FP64).
-__device__ __noinline__ static void lambda_update_warp(ImgState* st, const double* tot, double P, bool primary,
+__device__ __noinline__ static void lambda_update_warp(ImgState* st, const double* tot, bool primary,
                               bool last_chance, int iter, double* lam_out, double* res_out,
                               int lane) {
-  const double invP = 1.0 / P;  // P is a power of two: exact
-  const double T = st->T;
+  // the state's fields are requested together: they come from L2, one trip
+  const double invP = st->invP, T = st->T, invT = st->invT, prev = st->lam_prev;
+  const int mode = st->mode;
+  const float amax = (float)st->amax, node = lane < KNODES ? st->node[lane] : 0.0f;
   const double resinf = tot[KNODES] * invP;
   if (primary) {
     if (lane == 0) {
@@ -548,30 +578,30 @@ __device__ __noinline__ static void lambda_update_warp(ImgState* st, const doubl
     }
     if (!isfinite(resinf)) {
       if (lane == 0) st->status |= ST_NONFINITE;
-      resolve_warp(st, INFINITY, iter, lam_out, lane);
+      resolve_warp(st, INFINITY, prev, iter, lam_out, lane);
       return;
     }
     if (resinf <= T) {  // u_E in K (Sec. 3.2): lambda = inf, u_I = u_p = u_E
-      resolve_warp(st, INFINITY, iter, lam_out, lane);
+      resolve_warp(st, INFINITY, prev, iter, lam_out, lane);
       return;
     }
     if (lane == 0) {
       const float t = sqrtf((float)T / (float)resinf);
-      st->lam_up = fminf(1e30f, (float)st->amax * t / (1.0f - t));
+      st->lam_up = fminf(1e30f, amax * t / (1.0f - t));
     }
     __syncwarp(upd_mask());
   }
-  if (st->mode == MODE_MOM) {
-    const float c = st->node[0];
+  if (mode == MODE_MOM) {
+    const float c = __shfl_sync(upd_mask(), node, 0);
     if (!isfinite(tot[0])) {
       if (lane == 0) st->status |= ST_NONFINITE;
-      resolve_warp(st, INFINITY, iter, lam_out, lane);
+      resolve_warp(st, INFINITY, prev, iter, lam_out, lane);
       return;
     }
     double lam;
     float lo, hi;
-    if (moment_root_warp(tot, invP * st->invT, c, lane, lam, lo, hi)) {
-      resolve_warp(st, lam, iter, lam_out, lane);
+    if (moment_root_warp(tot, invP * invT, c, lane, lam, lo, hi)) {
+      resolve_warp(st, lam, prev, iter, lam_out, lane);
       return;
     }
     lo = fmaxf(lo, (float)LAMBDA_LO);
@@ -581,13 +611,12 @@ __device__ __noinline__ static void lambda_update_warp(ImgState* st, const doubl
   }
   // g_m = f(lambda_m) / T - 1, increasing in lambda, for the pass's nodes
   constexpr int nk = KNODES;
-  const float gm = lane < nk ? (float)((tot[lane] * invP - T) * st->invT) : 0.0f;
-  const float xm = lane < nk ? st->node[lane] : 0.0f;
+  const float gm = lane < nk ? (float)((tot[lane] * invP - T) * invT) : 0.0f;
+  const float xm = node;
   const float g0 = __shfl_sync(upd_mask(), gm, 0);
   const float gK = __shfl_sync(upd_mask(), gm, nk - 1);
   const float lo = __shfl_sync(upd_mask(), xm, 0);
   const float hi = __shfl_sync(upd_mask(), xm, nk - 1);
-  const int mode = st->mode;
   // a missed first bracket whose root is expected close to it
   const bool near = primary && iter == 2 && mode == MODE_CHEB;
   // the second iteration's jump, past its first bracket: seldom far past it
@@ -596,12 +625,12 @@ __device__ __noinline__ static void lambda_update_warp(ImgState* st, const doubl
   if (!(g0 <= 0.0f)) {  // root below the bracket (or NaN)
     if (!isfinite(g0)) {
       if (lane == 0) st->status |= ST_NONFINITE;
-      resolve_warp(st, INFINITY, iter, lam_out, lane);
+      resolve_warp(st, INFINITY, prev, iter, lam_out, lane);
       return;
     }
     if (lo <= (float)LAMBDA_LO * 1.000001f) {
       if (lane == 0) st->status |= ST_NONCONVERGED;
-      resolve_warp(st, LAMBDA_LO, iter, lam_out, lane);
+      resolve_warp(st, LAMBDA_LO, prev, iter, lam_out, lane);
       return;
     }
     // below the third iteration's first bracket (four passes to go): the
@@ -623,7 +652,7 @@ __device__ __noinline__ static void lambda_update_warp(ImgState* st, const doubl
     if (j > nk - 2) j = nk - 2;
     if (mode == MODE_CHEB) {
       const double lam = interp_root_warp(xm, gm, j, st->rtol, lane);
-      resolve_warp(st, lam, iter, lam_out, lane);
+      resolve_warp(st, lam, prev, iter, lam_out, lane);
       open = false;
     } else {
       const float nlo = __shfl_sync(upd_mask(), xm, j), nhi = __shfl_sync(upd_mask(), xm, j + 1);
@@ -636,7 +665,7 @@ __device__ __noinline__ static void lambda_update_warp(ImgState* st, const doubl
       if (lane == 0) st->status |= ST_PASSES_EXHAUSTED;
       const double mid = sqrt((double)st->lo * (double)st->hi);
       __syncwarp(upd_mask());
-      resolve_warp(st, mid, iter, lam_out, lane);
+      resolve_warp(st, mid, prev, iter, lam_out, lane);
     }
   }
 }

@@ -25,6 +25,9 @@ constexpr int DEF_ROW_THREADS = 256;
 constexpr int DEF_COL_THREADS = 256;
 constexpr int DEF_GF_ROWS = 64;
 
+// Most pixels of a class (all its images) that take the short column passes.
+constexpr long long SHORT_PIXELS = 1 << 20;
+
 struct Tables {
   const float2* tw;    // W_L^m for every L = 2..4096, size L at offset tab_off(L)
   const float* d2;     // 4 sin^2(pi m / L), same layout
@@ -48,6 +51,7 @@ struct ClassLaunch {
   int row_threads;      // threads per row-pass block (0 = DEF_ROW_THREADS)
   int gf_rows;          // largest rows per guided-filter item (0 = DEF_GF_ROWS)
   int class_id;         // index of the class in its plan (instrumentation)
+  bool short_cols;      // small problem: the short column passes (and their tile width)
 };
 
 // Row pass of the 2-D real DFT: real plane src -> packed rows dst.
@@ -60,7 +64,9 @@ cudaError_t launch_row_c2r(const ClassLaunch& c, const Tables& t, int sel0, int 
                            int dsel1, float scale, cudaStream_t s);
 // Tile width (columns per tile) of the spectra of an M x N class whose
 // column passes run col_threads threads per block (0 = default).
-int class_tile_width(int M, int N, int col_threads);
+int class_tile_width(int M, int N, int col_threads, bool short_cols);
+// Whether the column passes of n_img images of M x N are the short ones.
+bool short_columns(int M, int N, int n_img);
 // Rows per item of a row pass of length-L transforms on an M-row class.
 int rows_per_item(int L, int M, int row_threads);
 // Plain column FFT src -> dst (in place allowed), forward or inverse.
@@ -72,6 +78,10 @@ cudaError_t launch_col_fwd_lambda(const ClassLaunch& c, const Tables& t, int ite
 // Fallback lambda pass over the stored spectrum (exits early where resolved).
 cudaError_t launch_lambda_pass(const ClassLaunch& c, int iter, bool last_chance,
                                cudaStream_t s);
+// All fallback passes of an iteration (at most npass) in one launch, a cluster
+// of blocks per image; for canvases up to LAMBDA_LOOP_PIXELS.
+constexpr int LAMBDA_LOOP_PIXELS = 512 * 512;
+cudaError_t launch_lambda_loop(const ClassLaunch& c, int iter, int npass, cudaStream_t s);
 // Spectral solves (Eq. 8, 9) fused with the inverse column FFTs: S -> QI, Qp.
 cudaError_t launch_col_solve_inv(const ClassLaunch& c, const Tables& t, cudaStream_t s);
 // Guided filter (Eq. 3-5): real planes (uI, up) -> u.  iter < 0: no ISNR.
