@@ -44,6 +44,7 @@ struct HostCopies {
 
 struct Plan {
   std::vector<unsigned char> key;
+  std::vector<int> shape;  // what the captured graph depends on (plan_shape); empty: the key
   const HostCopies* copies = nullptr;  // set for the duration of a capture / record
   int n = 0, iters = 0;
   std::vector<int> order;                // internal index -> user index
@@ -136,6 +137,7 @@ struct gfdeconv_ctx {
   cudaStream_t cap = nullptr;
   cudaStream_t side[CHAINS - 1] = {};  // further chains of a captured solve
   cudaEvent_t ev_fork = nullptr;
+  cudaEvent_t ev_done = nullptr;      // the last solve's end
   cudaEvent_t ev_join[CHAINS - 1] = {};
   cudaEvent_t ev_in[CHAINS - 1] = {};  // a chain's host inputs have landed
   char* ws = nullptr;
@@ -255,6 +257,47 @@ std::vector<unsigned char> make_key(const gfdeconv_ctx* c, int n, const gfdeconv
   return k;
 }
 
+// What the captured graph of a solve depends on besides the context's options:
+// the images' sizes and windows in order, the iterations, whether checkpoints
+// are kept.  Pointers, PSF sizes, sigma and eps live in the descriptors that the
+// kernels read.  Empty where the graph itself holds caller pointers (copies of
+// u_I, u_p): such a plan serves its exact key only.
+std::vector<int> plan_shape(int n, const gfdeconv_image* imgs, int iters) {
+  std::vector<int> v;
+  v.reserve(3 * (size_t)n + 2);
+  v.push_back(iters);
+  int ckpt = 0;
+  for (int i = 0; i < n; ++i) {
+    if (imgs[i].uI_out || imgs[i].up_out) return {};
+    if (imgs[i].u_iters) ckpt = 1;
+    v.push_back(imgs[i].M);
+    v.push_back(imgs[i].N);
+    v.push_back(imgs[i].w);
+  }
+  v.push_back(ckpt);
+  return v;
+}
+
+// The caller's part of a descriptor.
+void fill_desc(const gfdeconv_ctx* c, const gfdeconv_image& im, ImgDesc& d) {
+  d.y = im.y;
+  d.h = im.h;
+  d.u = im.u_out;
+  d.uo = im.u_orig;
+  d.u0 = im.u_init;
+  d.u_iters = im.u_iters;
+  d.lam_out = im.lambda_out;
+  d.isnr_out = im.isnr_out;
+  d.res_out = im.res_out;
+  d.kh = im.kh;
+  d.kw = im.kw;
+  d.w = im.w;
+  d.sigma = im.sigma;
+  d.eps = im.eps;
+  d.rho_fixed = c->opts.rho;
+  d.lam_rtol = c->opts.lambda_rtol;
+}
+
 void drop_plan(gfdeconv_ctx* c) {
   if (c->plan.exec) cudaGraphExecDestroy(c->plan.exec);
   c->plan = Plan();
@@ -315,22 +358,7 @@ cudaError_t build_plan(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs, int i
       const gfdeconv_image& im = imgs[ui];
       const size_t P = (size_t)im.M * im.N;
       ImgDesc d{};
-      d.y = im.y;
-      d.h = im.h;
-      d.u = im.u_out;
-      d.uo = im.u_orig;
-      d.u0 = im.u_init;
-      d.u_iters = im.u_iters;
-      d.lam_out = im.lambda_out;
-      d.isnr_out = im.isnr_out;
-      d.res_out = im.res_out;
-      d.kh = im.kh;
-      d.kw = im.kw;
-      d.w = im.w;
-      d.sigma = im.sigma;
-      d.eps = im.eps;
-      d.rho_fixed = c->opts.rho;
-      d.lam_rtol = c->opts.lambda_rtol;
+      fill_desc(c, im, d);
       float2** planes[5] = {&d.S, &d.QI, &d.Qp, &d.H, &d.Y};
       for (float2** pp : planes) {
         *pp = reinterpret_cast<float2*>(cur);
@@ -401,10 +429,13 @@ cudaError_t build_plan(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs, int i
     if (tm) GFD_CK(tm->end(s));                          \
   } while (0)
 
-// Classes whose fallback passes run as one launch: small canvases, and few
-// enough images that their clusters are resident together.
-bool lambda_loop(const ClassLaunch& cl) {
-  return cl.cd.M * cl.cd.N <= LAMBDA_LOOP_PIXELS && cl.cd.n_img <= 32;
+// Classes whose fallback passes of iteration k run as one launch: small
+// canvases, and few enough images that their clusters are resident together.
+// A pass over a canvas of 1024 x 1024 takes 8 blocks three times as long as the
+// ordinary pass, so there only the later iterations do, where most images need
+// none.
+bool lambda_loop(const ClassLaunch& cl, int k) {
+  return cl.cd.M * cl.cd.N <= (k < 3 ? 1 : 4) * LAMBDA_LOOP_PIXELS && cl.cd.n_img <= 32;
 }
 
 cudaError_t record(gfdeconv_ctx* c, Plan& pl, cudaStream_t s, Timer* tm = nullptr,
@@ -472,14 +503,14 @@ cudaError_t record(gfdeconv_ctx* c, Plan& pl, cudaStream_t s, Timer* tm = nullpt
       // extrapolated root, which the fused pass almost always resolves
       const int npass = k < 3 ? passes : std::min(passes, LATE_LAMBDA_PASSES);
       for (auto& cl : classes)
-        if (lambda_loop(cl)) {
+        if (lambda_loop(cl, k)) {
           if (tm) tm->cur_cls = cl.class_id;
           GFD_T(GFD_PHASE_LAMBDA_PASS, launch_lambda_loop(cl, k, npass, s));
           ++L;
         }
       for (int p = 1; p <= npass; ++p)
         for (auto& cl : classes) {
-          if (lambda_loop(cl)) continue;
+          if (lambda_loop(cl, k)) continue;
           if (tm) tm->cur_cls = cl.class_id;
           GFD_T(GFD_PHASE_LAMBDA_PASS, launch_lambda_pass(cl, k, p == npass, s));
           ++L;
@@ -569,13 +600,24 @@ cudaError_t aux_slot(gfdeconv_ctx* c, size_t ws_bytes, AuxSlot** out) {
   return cudaSuccess;
 }
 
-cudaError_t aux_upload(AuxSlot* a, const ImgDesc& d, cudaStream_t s) {
-  return cudaMemcpyAsync(a->d_img, &d, sizeof(ImgDesc), cudaMemcpyHostToDevice, s);
+// The descriptor travels as a kernel argument: a small copy from pageable host
+// memory costs the host about twice a launch.  st: also clear its absmax.
+cudaError_t aux_upload(AuxSlot* a, const ImgDesc& d, cudaStream_t s, ImgState* st = nullptr) {
+  return launch_store_desc(d, a->d_img, st, s);
 }
 
 cudaError_t aux_finish(AuxSlot* a, cudaStream_t s) {
   a->used = true;
   return cudaEventRecord(a->done, s);
+}
+
+// Marks the end of a solve for a later one on another stream (a launch that the
+// caller captures into a graph of its own is left alone, as before).
+cudaError_t record_done(gfdeconv_ctx* c, cudaStream_t s) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)
+    return cudaSuccess;
+  return cudaEventRecord(c->ev_done, s);
 }
 
 int solve_batched_dev(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs, int iters,
@@ -604,7 +646,35 @@ int solve_batched_dev(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs, int it
     for (const auto& v : hc->out) put(v);
   }
   c->plan.copies = nullptr;
-  if (!(c->have_plan && c->plan.key == key)) {
+  std::vector<int> shape;
+  bool same = c->have_plan && c->plan.key == key;
+  if (!same && !hc && c->opts.use_graphs) shape = plan_shape(n, imgs, iters);
+  if (!same && !shape.empty() && c->have_plan && c->plan.exec && c->plan.shape == shape) {
+    // Other buffers or parameters in a solve of the same shape (the next image
+    // of a stream): the graph stays, only the descriptors are sent, in stream
+    // order behind the last solve.  Not while the caller captures the stream:
+    // the copy's source is this call's.
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
+      Plan& pl = c->plan;
+      for (int i = 0; i < n; ++i) {
+        fill_desc(c, imgs[pl.order[i]], pl.h_imgs[i]);
+        pl.user[i] = imgs[pl.order[i]];
+      }
+      cudaError_t e = cudaSuccess;
+      if (s != c->last_stream) e = cudaStreamWaitEvent(s, c->ev_done, 0);
+      if (e == cudaSuccess)
+        e = cudaMemcpyAsync(c->d_imgs, pl.h_imgs.data(), sizeof(ImgDesc) * n, cudaMemcpyHostToDevice,
+                            s);
+      if (e != cudaSuccess) {
+        drop_plan(c);
+        return map_err(e);
+      }
+      pl.key.swap(key);
+      same = true;
+    }
+  }
+  if (!same) {
     cudaError_t e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return map_err(e);
     drop_plan(c);
@@ -624,11 +694,13 @@ int solve_batched_dev(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs, int it
       }
     }
     c->plan.key.swap(key);
+    c->plan.shape.swap(shape);
     c->have_plan = true;
   }
   cudaError_t e;
   if (c->opts.use_graphs) {
     e = cudaGraphLaunch(c->plan.exec, s);
+    if (e == cudaSuccess && !c->plan.shape.empty()) e = record_done(c, s);
   } else {
     c->plan.copies = hc;
     e = record(c, c->plan, s);
@@ -791,6 +863,7 @@ int gfdeconv_create(gfdeconv_ctx** out, int cuda_device, const gfdeconv_opts* op
       (e = cudaMalloc(&c->aux_st, sizeof(ImgState))) != cudaSuccess ||
       (e = cudaMemset(c->aux_st, 0, sizeof(ImgState))) != cudaSuccess ||
       (e = cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking)) != cudaSuccess ||
+      (e = cudaEventCreateWithFlags(&c->ev_done, cudaEventDisableTiming)) != cudaSuccess ||
       (e = cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming)) != cudaSuccess) {
     gfdeconv_destroy(c);
     return map_err(e);
@@ -835,6 +908,7 @@ void gfdeconv_destroy(gfdeconv_ctx* c) {
     if (c->ev_in[q]) cudaEventDestroy(c->ev_in[q]);
   }
   if (c->ev_fork) cudaEventDestroy(c->ev_fork);
+  if (c->ev_done) cudaEventDestroy(c->ev_done);
   delete c;
 }
 
@@ -1508,7 +1582,7 @@ int gfdeconv_guidfilter(gfdeconv_ctx* c, const float* I, const float* p, int M, 
   d.u = u_out;
   d.w = w;
   d.eps = eps;
-  if ((e = aux_upload(a, d, s)) != cudaSuccess) return map_err(e);
+  if ((e = aux_upload(a, d, s, c->aux_st)) != cudaSuccess) return map_err(e);
   ClassLaunch cl{};
   cl.cd = ClassDesc{M, N, 1, 0, N / 2};
   cl.imgs = a->d_img;
@@ -1517,9 +1591,7 @@ int gfdeconv_guidfilter(gfdeconv_ctx* c, const float* I, const float* p, int M, 
   cl.n_rad_groups = 1;
   cl.rad_groups[0] = RadGroup{0, 1, (w - 1) / 2};
   if (c->opts.var_precision == GFD_VAR_COMPENSATED) {  // the split sums' bound
-    if ((e = cudaMemsetAsync(c->aux_st->absmax, 0, sizeof(c->aux_st->absmax), s)) != cudaSuccess ||
-        (e = launch_plane_absmax(cl, s)) != cudaSuccess)
-      return map_err(e);
+    if ((e = launch_plane_absmax(cl, s)) != cudaSuccess) return map_err(e);
   }
   if ((e = launch_guided_filter(cl, -1, c->opts.var_precision, c->opts.boundary, s)) != cudaSuccess)
     return map_err(e);
@@ -1656,8 +1728,6 @@ constexpr int NOALLOC_MAX_DEVICES = 64;
 // both look the address up and store the same value.
 std::atomic<void*> g_noalloc_addr[NOALLOC_MAX_DEVICES];
 
-__global__ void k_store_desc(ImgDesc d, ImgDesc* dst) { *dst = d; }
-
 }  // namespace
 }  // namespace gfd
 
@@ -1683,8 +1753,7 @@ int gfdeconv_fft2_r2c_noalloc(gfdeconv_ctx* c, const float* x, int M, int N, flo
   d.S = reinterpret_cast<float2*>(base + 256);
   d.Y = reinterpret_cast<float2*>(X);
   ImgDesc* d_desc = reinterpret_cast<ImgDesc*>(base);
-  k_store_desc<<<1, 1, 0, s>>>(d, d_desc);
-  if ((e = cudaGetLastError()) != cudaSuccess) return map_err(e);
+  if ((e = launch_store_desc(d, d_desc, nullptr, s)) != cudaSuccess) return map_err(e);
   ClassLaunch cl{};
   cl.cd = ClassDesc{M, N, 1, 0, N / 2};
   cl.imgs = d_desc;
@@ -1700,7 +1769,7 @@ int gfdeconv_device_arch(int cuda_device, int* binary_version, int* device_cc) {
   cudaError_t e = cudaSetDevice(cuda_device);
   if (e != cudaSuccess) return map_err(e);
   cudaFuncAttributes a{};
-  if ((e = cudaFuncGetAttributes(&a, (const void*)k_store_desc)) != cudaSuccess) return map_err(e);
+  if ((e = cudaFuncGetAttributes(&a, store_desc_kernel())) != cudaSuccess) return map_err(e);
   int major = 0, minor = 0;
   if ((e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, cuda_device)) !=
           cudaSuccess ||

@@ -32,6 +32,7 @@
 // accumulators, or plain FP32.  sigma_k^2 and the covariance are then formed
 // as (n S_JJ - S_J^2) / n^2 and (n S_JQ - S_J S_Q) / n^2 in that arithmetic
 // and rounded to FP32 once.
+#include <atomic>
 #include <type_traits>
 
 #include "common.cuh"
@@ -776,11 +777,37 @@ static int gfw_rows(int M, int hmax, int rad, int images, int strips, int reside
   return best;
 }
 
+// Warps per block and resident blocks per SM of a kernel.  Wide windows' rings
+// leave room for fewer warps per SM than whole blocks of GFW_WARPS would use:
+// blocks shrink to the size that keeps most warps resident (w = 17: 6 instead
+// of 4).  The answer is a property of the kernel, looked up once (threads that
+// race on the first call store the same value).
+static void gfw_block(GfKernel kern, int var_mode, int boundary, int rad, int& W, int& per_sm) {
+  static std::atomic<int> known[5][2][GF_RMAX + 1];
+  std::atomic<int>& k = known[var_mode][boundary][rad];
+  int v = k.load(std::memory_order_relaxed);
+  if (v == 0) {
+    int bw = GFW_WARPS, bn = 0;
+    for (int w = GFW_WARPS; w >= 1; w /= 2) {
+      int n = 0;
+      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+              &n, kern, w * 32, (size_t)w * gfw_ring_floats(rad) * sizeof(float)) != cudaSuccess)
+        n = 0;
+      if (n * w > bn * bw) {
+        bw = w;
+        bn = n;
+      }
+    }
+    v = bw * 256 + (bn < 1 ? 1 : bn);
+    if (bn >= 1) k.store(v, std::memory_order_relaxed);
+  }
+  W = v >> 8;
+  per_sm = v & 255;
+}
+
 // One launch per window radius present in the class (the images of a class
 // are ordered by radius, so each group is a contiguous range).  Items are
-// (image, strip, block of H rows).  Wide windows' rings leave room for fewer
-// warps per SM than whole blocks of GFW_WARPS would use: blocks shrink to the
-// size that keeps most warps resident (w = 17: 6 instead of 4).
+// (image, strip, block of H rows).
 cudaError_t launch_guided_filter(const ClassLaunch& c, int iter, int var_mode, int boundary,
                                  cudaStream_t s) {
   const int shifted = var_mode == GFD_VAR_FP32_RAW ? 0 : 1;
@@ -790,18 +817,8 @@ cudaError_t launch_guided_filter(const ClassLaunch& c, int iter, int var_mode, i
     ClassDesc cd = c.cd;
     cd.img0 = rg.img0;
     cd.n_img = rg.n_img;
-    int W = GFW_WARPS, per_sm = 0;
-    for (int w = GFW_WARPS; w >= 1; w /= 2) {
-      int n = 0;
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-              &n, kern, w * 32, (size_t)w * gfw_ring_floats(rg.rad) * sizeof(float)) != cudaSuccess)
-        n = 0;
-      if (n * w > per_sm * W) {
-        W = w;
-        per_sm = n;
-      }
-    }
-    if (per_sm < 1) per_sm = 1;
+    int W, per_sm;
+    gfw_block(kern, var_mode, boundary, rg.rad, W, per_sm);
     const size_t smem = (size_t)W * gfw_ring_floats(rg.rad) * sizeof(float);
     const int div = c.grid_div > 1 ? c.grid_div : 1;
     const int blocks = (per_sm * gf_sm_count() + div - 1) / div;

@@ -79,7 +79,7 @@ cudaError_t launch_col_fwd_lambda(const ClassLaunch& c, const Tables& t, int ite
 cudaError_t launch_lambda_pass(const ClassLaunch& c, int iter, bool last_chance,
                                cudaStream_t s);
 // All fallback passes of an iteration (at most npass) in one launch, a cluster
-// of blocks per image; for canvases up to LAMBDA_LOOP_PIXELS.
+// of blocks per image.
 constexpr int LAMBDA_LOOP_PIXELS = 512 * 512;
 cudaError_t launch_lambda_loop(const ClassLaunch& c, int iter, int npass, cudaStream_t s);
 // Spectral solves (Eq. 8, 9) fused with the inverse column FFTs: S -> QI, Qp.
@@ -93,6 +93,9 @@ cudaError_t launch_guided_filter(const ClassLaunch& c, int iter, int var_mode, i
 cudaError_t launch_guided_filter_color(const float* I, const float* p, int M, int N, int w,
                                        double eps, int boundary, float* ab, float* u,
                                        cudaStream_t s);
+// *dst = d (a descriptor for the utility calls); st: clear its absmax.
+cudaError_t launch_store_desc(const ImgDesc& d, ImgDesc* dst, ImgState* st, cudaStream_t s);
+const void* store_desc_kernel();
 // Largest |u_I|, |u_p| of every image into ImgState::absmax (which must be
 // zero before), for guided-filter calls outside a solve.
 cudaError_t launch_plane_absmax(const ClassLaunch& c, cudaStream_t s);
