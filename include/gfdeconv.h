@@ -207,7 +207,7 @@ int gfdeconv_fft2_r2c(gfdeconv_ctx* ctx, const float* x, int M, int N, float* X,
  *
  * Same arguments, result and layout as gfdeconv_fft2_r2c, but the call makes
  * no cudaMalloc / cudaFree and calls no allocating library: its intermediate
- * row-pass plane and its kernel descriptor live in one file-scope
+ * row-pass plane lives in one file-scope
  * `static __device__ __align__(256)` array of GFD_NOALLOC_SCRATCH_BYTES,
  * allocated when the library's device code is loaded.  It serves callers that
  * must not allocate on the device: code running under a memory budget that a
@@ -223,8 +223,7 @@ int gfdeconv_fft2_r2c(gfdeconv_ctx* ctx, const float* x, int M, int N, float* X,
  * call outside any stream capture.  The cached address belongs to the
  * device's current context; after cudaDeviceReset on that device, create a
  * new gfdeconv context and do not use this entry point again in the process.  Nothing in the scratch has to start
- * at zero: every call writes the descriptor and the whole intermediate plane
- * before reading them.  The scratch is shared by every call on a device, so
+ * at zero: every call writes the whole intermediate plane before reading it.  The scratch is shared by every call on a device, so
  * calls whose stream work overlaps (different streams, or different host
  * threads without ordering between them) race on it: order them on one stream
  * or synchronise between them.  ctx must be a live context (its twiddle table

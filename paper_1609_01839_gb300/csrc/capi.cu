@@ -119,7 +119,6 @@ struct TuneTable {
 };
 
 struct AuxSlot {
-  ImgDesc* d_img = nullptr;
   char* ws = nullptr;
   size_t ws_bytes = 0;
   cudaEvent_t done = nullptr;
@@ -149,7 +148,11 @@ struct gfdeconv_ctx {
   bool have_plan = false;
   cudaStream_t last_stream = nullptr;
   long long last_launches = 0;
+  // per-image state and launch_plane_absmax's scratch of the utility calls,
+  // AUX_SLOTS of each in turn: calls in flight on several streams do not meet
   ImgState* aux_st = nullptr;
+  unsigned int* aux_max = nullptr;
+  int aux_turn = 0;
   AuxSlot aux[AUX_SLOTS];
   int aux_next = 0;
   char* stage = nullptr;
@@ -582,12 +585,12 @@ cudaError_t capture(gfdeconv_ctx* c, Plan& pl) {
   return e3;
 }
 
-// Reserve an aux slot (descriptor + workspace) for a single-image utility call.
+// Reserve an aux slot (workspace) for a single-image utility call.  Descriptors
+// of these calls travel as kernel arguments: no copy, no launch for them.
 cudaError_t aux_slot(gfdeconv_ctx* c, size_t ws_bytes, AuxSlot** out) {
   AuxSlot& a = c->aux[c->aux_next];
   c->aux_next = (c->aux_next + 1) % AUX_SLOTS;
   if (a.used) GFD_CK(cudaEventSynchronize(a.done));
-  if (!a.d_img) GFD_CK(cudaMalloc(&a.d_img, sizeof(ImgDesc)));
   if (!a.done) GFD_CK(cudaEventCreateWithFlags(&a.done, cudaEventDisableTiming));
   if (ws_bytes > a.ws_bytes) {
     if (a.ws) cudaFree(a.ws);
@@ -598,12 +601,6 @@ cudaError_t aux_slot(gfdeconv_ctx* c, size_t ws_bytes, AuxSlot** out) {
   }
   *out = &a;
   return cudaSuccess;
-}
-
-// The descriptor travels as a kernel argument: a small copy from pageable host
-// memory costs the host about twice a launch.  st: also clear its absmax.
-cudaError_t aux_upload(AuxSlot* a, const ImgDesc& d, cudaStream_t s, ImgState* st = nullptr) {
-  return launch_store_desc(d, a->d_img, st, s);
 }
 
 cudaError_t aux_finish(AuxSlot* a, cudaStream_t s) {
@@ -860,8 +857,10 @@ int gfdeconv_create(gfdeconv_ctx** out, int cuda_device, const gfdeconv_opts* op
       (e = cudaMalloc(&c->d2, sizeof(float) * TAB_ENTRIES)) != cudaSuccess ||
       (e = cudaMemcpy(c->tw, tw.data(), sizeof(float2) * TAB_ENTRIES, cudaMemcpyHostToDevice)) != cudaSuccess ||
       (e = cudaMemcpy(c->d2, d2.data(), sizeof(float) * TAB_ENTRIES, cudaMemcpyHostToDevice)) != cudaSuccess ||
-      (e = cudaMalloc(&c->aux_st, sizeof(ImgState))) != cudaSuccess ||
-      (e = cudaMemset(c->aux_st, 0, sizeof(ImgState))) != cudaSuccess ||
+      (e = cudaMalloc(&c->aux_st, AUX_SLOTS * sizeof(ImgState))) != cudaSuccess ||
+      (e = cudaMemset(c->aux_st, 0, AUX_SLOTS * sizeof(ImgState))) != cudaSuccess ||
+      (e = cudaMalloc(&c->aux_max, AUX_SLOTS * ABSMAX_SCRATCH * sizeof(unsigned int))) != cudaSuccess ||
+      (e = cudaMemset(c->aux_max, 0, AUX_SLOTS * ABSMAX_SCRATCH * sizeof(unsigned int))) != cudaSuccess ||
       (e = cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking)) != cudaSuccess ||
       (e = cudaEventCreateWithFlags(&c->ev_done, cudaEventDisableTiming)) != cudaSuccess ||
       (e = cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming)) != cudaSuccess) {
@@ -887,7 +886,6 @@ void gfdeconv_destroy(gfdeconv_ctx* c) {
   cudaDeviceSynchronize();
   drop_plan(c);
   for (AuxSlot& a : c->aux) {
-    if (a.d_img) cudaFree(a.d_img);
     if (a.ws) cudaFree(a.ws);
     if (a.done) cudaEventDestroy(a.done);
   }
@@ -898,6 +896,7 @@ void gfdeconv_destroy(gfdeconv_ctx* c) {
   if (c->d_imgs) cudaFree(c->d_imgs);
   if (c->d_st) cudaFree(c->d_st);
   if (c->aux_st) cudaFree(c->aux_st);
+  if (c->aux_max) cudaFree(c->aux_max);
   if (c->stage) cudaFree(c->stage);
   if (c->adj_ws) cudaFree(c->adj_ws);
   if (c->hstage) cudaFreeHost(c->hstage);
@@ -1573,29 +1572,26 @@ int gfdeconv_guidfilter(gfdeconv_ctx* c, const float* I, const float* p, int M, 
   if (!(eps > 0.0) || w < 1 || w > 17 || !(w & 1)) return GFD_ERR_INVALID_ARG;
   if (cudaSetDevice(c->device) != cudaSuccess) return GFD_ERR_CUDA;
   cudaStream_t s = (cudaStream_t)stream;
-  AuxSlot* a = nullptr;
-  cudaError_t e = aux_slot(c, 0, &a);
-  if (e != cudaSuccess) return map_err(e);
+  cudaError_t e;
   ImgDesc d{};
   d.uI = const_cast<float*>(I);
   d.up = const_cast<float*>(p);
   d.u = u_out;
   d.w = w;
   d.eps = eps;
-  if ((e = aux_upload(a, d, s, c->aux_st)) != cudaSuccess) return map_err(e);
+  const int turn = c->aux_turn;
+  c->aux_turn = (turn + 1) % AUX_SLOTS;
   ClassLaunch cl{};
   cl.cd = ClassDesc{M, N, 1, 0, N / 2};
-  cl.imgs = a->d_img;
-  cl.st = c->aux_st;
+  cl.one = &d;
+  cl.st = c->aux_st + turn;
   cl.max_rad = (w - 1) / 2;
   cl.n_rad_groups = 1;
   cl.rad_groups[0] = RadGroup{0, 1, (w - 1) / 2};
   if (c->opts.var_precision == GFD_VAR_COMPENSATED) {  // the split sums' bound
-    if ((e = launch_plane_absmax(cl, s)) != cudaSuccess) return map_err(e);
+    if ((e = launch_plane_absmax(cl, c->aux_max + turn * ABSMAX_SCRATCH, s)) != cudaSuccess) return map_err(e);
   }
-  if ((e = launch_guided_filter(cl, -1, c->opts.var_precision, c->opts.boundary, s)) != cudaSuccess)
-    return map_err(e);
-  return map_err(aux_finish(a, s));
+  return map_err(launch_guided_filter(cl, -1, c->opts.var_precision, c->opts.boundary, s));
 }
 
 int gfdeconv_pad_symmetric(gfdeconv_ctx* c, const float* y, int m, int n, float* y_canvas, int M,
@@ -1648,10 +1644,9 @@ int gfdeconv_fft2_r2c(gfdeconv_ctx* c, const float* x, int M, int N, float* X, v
   d.u = const_cast<float*>(x);
   d.S = reinterpret_cast<float2*>(a->ws);
   d.Y = reinterpret_cast<float2*>(X);
-  if ((e = aux_upload(a, d, s)) != cudaSuccess) return map_err(e);
   ClassLaunch cl{};
   cl.cd = ClassDesc{M, N, 1, 0, N / 2};
-  cl.imgs = a->d_img;
+  cl.one = &d;
   cl.st = c->aux_st;
   const Tables t{c->tw, c->d2, c->twdf};
   if ((e = launch_row_r2c(cl, t, SEL_U, SEL_S, false, s)) != cudaSuccess) return map_err(e);
@@ -1670,17 +1665,15 @@ int gfdeconv_fft2_c2r(gfdeconv_ctx* c, const float* X, int M, int N, float* x, v
   cudaError_t e = aux_slot(c, P * sizeof(float), &a);
   if (e != cudaSuccess) return map_err(e);
   ImgDesc d{};
+  d.Qp = reinterpret_cast<float2*>(const_cast<float*>(X));  // read only
   d.QI = reinterpret_cast<float2*>(a->ws);
   d.uI = x;
-  if ((e = aux_upload(a, d, s)) != cudaSuccess) return map_err(e);
-  if ((e = cudaMemcpyAsync(a->ws, X, P * sizeof(float), cudaMemcpyDeviceToDevice, s)) != cudaSuccess)
-    return map_err(e);
   ClassLaunch cl{};
   cl.cd = ClassDesc{M, N, 1, 0, N / 2};
-  cl.imgs = a->d_img;
+  cl.one = &d;
   cl.st = c->aux_st;
   const Tables t{c->tw, c->d2, c->twdf};
-  if ((e = launch_col_plain(cl, t, SEL_QI, SEL_QI, true, s)) != cudaSuccess) return map_err(e);
+  if ((e = launch_col_plain(cl, t, SEL_QP, SEL_QI, true, s)) != cudaSuccess) return map_err(e);
   if ((e = launch_row_c2r(cl, t, SEL_QI, -1, SEL_UI, -1, 1.0f / ((float)M * (float)N), s)) !=
       cudaSuccess)
     return map_err(e);
@@ -1712,14 +1705,12 @@ const char* gfdeconv_last_cuda_error(void) {
 }  // extern "C"
 
 // ---------------------------------------------------------------------------
-// Allocation-free 2-D real DFT (no counterpart in the paper).  The descriptor
-// and the packed row-pass plane live in a static device array; the descriptor
-// is written by a one-thread kernel from its by-value argument, so no host
-// buffer is involved either.
+// Allocation-free 2-D real DFT (no counterpart in the paper).  The packed
+// row-pass plane lives in a static device array, the descriptor in the kernels'
+// arguments, so no host buffer is involved either.
 namespace gfd {
 namespace {
 
-static_assert(sizeof(ImgDesc) <= 256, "descriptor slot");
 static __device__ __align__(256) unsigned char g_noalloc_scratch[GFD_NOALLOC_SCRATCH_BYTES];
 
 constexpr int NOALLOC_MAX_DEVICES = 64;
@@ -1752,11 +1743,9 @@ int gfdeconv_fft2_r2c_noalloc(gfdeconv_ctx* c, const float* x, int M, int N, flo
   d.u = const_cast<float*>(x);
   d.S = reinterpret_cast<float2*>(base + 256);
   d.Y = reinterpret_cast<float2*>(X);
-  ImgDesc* d_desc = reinterpret_cast<ImgDesc*>(base);
-  if ((e = launch_store_desc(d, d_desc, nullptr, s)) != cudaSuccess) return map_err(e);
   ClassLaunch cl{};
   cl.cd = ClassDesc{M, N, 1, 0, N / 2};
-  cl.imgs = d_desc;
+  cl.one = &d;
   cl.st = nullptr;  // the plain passes keep no per-image state
   const Tables t{c->tw, c->d2, c->twdf};
   if ((e = launch_row_r2c(cl, t, SEL_U, SEL_S, false, s)) != cudaSuccess) return map_err(e);
@@ -1769,7 +1758,7 @@ int gfdeconv_device_arch(int cuda_device, int* binary_version, int* device_cc) {
   cudaError_t e = cudaSetDevice(cuda_device);
   if (e != cudaSuccess) return map_err(e);
   cudaFuncAttributes a{};
-  if ((e = cudaFuncGetAttributes(&a, store_desc_kernel())) != cudaSuccess) return map_err(e);
+  if ((e = cudaFuncGetAttributes(&a, some_kernel())) != cudaSuccess) return map_err(e);
   int major = 0, minor = 0;
   if ((e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, cuda_device)) !=
           cudaSuccess ||

@@ -94,8 +94,8 @@ GFD_D float2 select2(bool c, float2 a, float2 b) { return c ? a : b; }
 // Im Z[0] (packed as X[0] + i X[N/2]).  do_sum: FP64 row sums of the source.
 template <int L>
 __global__ void __launch_bounds__(256, 3)
-k_row_r2c(ClassDesc cd, const ImgDesc* __restrict__ imgs, const float2* __restrict__ tw, int rpc,
-          int src_sel, int dst_sel, int do_sum) {
+k_row_r2c(ClassDesc cd, const ImgDesc* __restrict__ imgs, const __grid_constant__ ImgDesc one,
+          const float2* __restrict__ tw, int rpc, int src_sel, int dst_sel, int do_sum) {
   extern __shared__ __align__(16) float2 smem[];
   using G = FftGeo<FK_R2C, L>;
   constexpr int T = G::T, r0 = G::RF, rl = G::RL;
@@ -103,7 +103,7 @@ k_row_r2c(ClassDesc cd, const ImgDesc* __restrict__ imgs, const float2* __restri
   const int TB = cd.TB, M = cd.M;
   const int team = threadIdx.x / T, j = threadIdx.x % T;
   const int row_c = blockIdx.x * rpc + team;
-  const ImgDesc& d = imgs[cd.img0 + row_c / M];
+  const ImgDesc& d = imgs ? imgs[cd.img0 + row_c / M] : one;
   const int row = row_c % M;
   const unsigned int mask = warp_mask();
   float2* buf = smem + team * G::SIZE;
@@ -189,8 +189,8 @@ k_row_r2c(ClassDesc cd, const ImgDesc* __restrict__ imgs, const float2* __restri
 // dsel0, then sel1 -> dsel1.
 template <int L>
 __global__ void __launch_bounds__(256, 3)
-k_row_c2r(ClassDesc cd, const ImgDesc* __restrict__ imgs, const float2* __restrict__ tw, int rpc,
-          int sel0, int sel1, int dsel0, int dsel1, float scale, ImgState* st) {
+k_row_c2r(ClassDesc cd, const ImgDesc* __restrict__ imgs, const __grid_constant__ ImgDesc one,
+          const float2* __restrict__ tw, int rpc, int sel0, int sel1, int dsel0, int dsel1, float scale, ImgState* st) {
   extern __shared__ __align__(16) float2 smem[];
   using G = FftGeo<FK_C2R, L>;
   constexpr int T = G::T, r0 = G::RF, rl = G::RL;
@@ -201,7 +201,7 @@ k_row_c2r(ClassDesc cd, const ImgDesc* __restrict__ imgs, const float2* __restri
   const bool second = (int)blockIdx.x >= per_plane;
   const int row_c = ((int)blockIdx.x - (second ? per_plane : 0)) * rpc + team;
   const int li = row_c / M, row = row_c % M;
-  const ImgDesc& d = imgs[cd.img0 + li];
+  const ImgDesc& d = imgs ? imgs[cd.img0 + li] : one;
   const unsigned int mask = warp_mask();
   float2* buf = smem + team * G::SIZE;
   const float2* src = cplx_plane(d, second ? sel1 : sel0) + (size_t)row * TB;
@@ -295,14 +295,14 @@ k_row_c2r(ClassDesc cd, const ImgDesc* __restrict__ imgs, const float2* __restri
 // (inside one tile) per block.
 template <int M, bool INV>
 __global__ void __launch_bounds__(512)
-k_col_plain(ClassDesc cd, const ImgDesc* __restrict__ imgs, const float2* __restrict__ tw, int B,
-            int src_sel, int dst_sel) {
+k_col_plain(ClassDesc cd, const ImgDesc* __restrict__ imgs, const __grid_constant__ ImgDesc one,
+            const float2* __restrict__ tw, int B, int src_sel, int dst_sel) {
   extern __shared__ __align__(16) float2 smem[];
   using G = FftGeo<FK_COL, M>;
   constexpr int T = G::T, r0 = G::RF;
   const int Lc = cd.N / 2, TB = cd.TB;
   const int cpi = Lc / B;
-  const ImgDesc& d = imgs[cd.img0 + blockIdx.x / cpi];
+  const ImgDesc& d = imgs ? imgs[cd.img0 + blockIdx.x / cpi] : one;
   const int c0 = (blockIdx.x % cpi) * B;
   const int b = threadIdx.x & (B - 1), j = threadIdx.x >> (__ffs(B) - 1);
   const size_t off = (size_t)(c0 / TB) * M * TB + (c0 % TB) + b;
@@ -1066,8 +1066,8 @@ static void do_row_r2c(const ClassLaunch& c, const Tables& t, int src, int dst, 
   using G = FftGeo<FK_R2C, L>;
   const int rpc = rows_per_item(L, c.cd.M, c.row_threads);
   const int blocks = c.cd.n_img * c.cd.M / rpc;
-  k_row_r2c<L><<<blocks, rpc * G::T, rpc * G::SIZE * sizeof(float2), s>>>(c.cd, c.imgs, t.tw, rpc,
-                                                                          src, dst, sum);
+  k_row_r2c<L><<<blocks, rpc * G::T, rpc * G::SIZE * sizeof(float2), s>>>(
+      c.cd, c.imgs, one_desc(c), t.tw, rpc, src, dst, sum);
 }
 
 cudaError_t launch_row_r2c(const ClassLaunch& c, const Tables& t, int src, int dst,
@@ -1087,7 +1087,8 @@ static void do_row_c2r(const ClassLaunch& c, const Tables& t, int sel0, int sel1
   int blocks = c.cd.n_img * c.cd.M / rpc;
   if (sel1 >= 0) blocks *= 2;
   k_row_c2r<L><<<blocks, rpc * G::T, rpc * G::SIZE * sizeof(float2), s>>>(
-      c.cd, c.imgs, t.tw, rpc, sel0, sel1, dsel0, dsel1, scale, dsel0 == SEL_UI ? c.st : nullptr);
+      c.cd, c.imgs, one_desc(c), t.tw, rpc, sel0, sel1, dsel0, dsel1, scale,
+      dsel0 == SEL_UI ? c.st : nullptr);
 }
 
 cudaError_t launch_row_c2r(const ClassLaunch& c, const Tables& t, int sel0, int sel1, int dsel0,
@@ -1110,9 +1111,9 @@ static void do_col_plain(const ClassLaunch& c, const Tables& t, int src, int dst
   const size_t smem = (size_t)B * col_stride<M>(B) * sizeof(float2);
   const int nblk = c.cd.n_img * (Lc / B);
   if (inv)
-    k_col_plain<M, true><<<nblk, B * T, smem, s>>>(c.cd, c.imgs, t.tw, B, src, dst);
+    k_col_plain<M, true><<<nblk, B * T, smem, s>>>(c.cd, c.imgs, one_desc(c), t.tw, B, src, dst);
   else
-    k_col_plain<M, false><<<nblk, B * T, smem, s>>>(c.cd, c.imgs, t.tw, B, src, dst);
+    k_col_plain<M, false><<<nblk, B * T, smem, s>>>(c.cd, c.imgs, one_desc(c), t.tw, B, src, dst);
 }
 
 cudaError_t launch_col_plain(const ClassLaunch& c, const Tables& t, int src, int dst,

@@ -665,11 +665,11 @@ GFD_D void gfw_items(const ClassDesc& cd, const ImgDesc* __restrict__ imgs, ImgS
 // One kernel per window radius: its registers and code are those of the radius.
 template <int RAD, class ACC, bool TRUNC>
 __global__ void __launch_bounds__(GFW_WARPS * 32)
-k_guided_filter(ClassDesc cd, const ImgDesc* __restrict__ imgs, ImgState* st, int iter,
-                int shifted, int H) {
+k_guided_filter(ClassDesc cd, const ImgDesc* __restrict__ imgs, const __grid_constant__ ImgDesc one,
+                ImgState* st, int iter, int shifted, int H) {
   extern __shared__ __align__(16) float gsm[];
   const int warp = threadIdx.x >> 5, W = blockDim.x >> 5;
-  gfw_items<RAD, ACC, TRUNC>(cd, imgs, st, iter, shifted != 0, H,
+  gfw_items<RAD, ACC, TRUNC>(cd, imgs ? imgs : &one, st, iter, shifted != 0, H,
                              gsm + (size_t)warp * gfw_ring_floats(RAD), blockIdx.x * W + warp,
                              gridDim.x * W);
 }
@@ -684,7 +684,7 @@ static int gf_sm_count() {
   return n;
 }
 
-using GfKernel = void (*)(ClassDesc, const ImgDesc*, ImgState*, int, int, int);
+using GfKernel = void (*)(ClassDesc, const ImgDesc*, const ImgDesc, ImgState*, int, int, int);
 
 template <int RAD>
 static GfKernel gf_kernel_rad(int var_mode, bool tr) {
@@ -715,31 +715,81 @@ static GfKernel gf_kernel(int var_mode, int boundary, int rad) {
   }
 }
 
-// Largest |I| and |p| of each image of a class into ImgState::absmax (the
-// bound of the split sums when no inverse row pass has recorded it).
-__global__ void k_plane_absmax(ClassDesc cd, const ImgDesc* __restrict__ imgs, ImgState* st) {
-  const int gi = cd.img0 + blockIdx.y;
-  const ImgDesc& d = imgs[gi];
-  const size_t P = (size_t)cd.M * cd.N;
+// Largest |I| and |p| of one image into ImgState::absmax (the bound of the
+// split sums when no inverse row pass has recorded it).  Every block leaves its
+// maxima in the scratch; the last one to finish (a counter, reset for the next
+// call) reduces them, so no launch has to clear anything first.  Bound by DRAM:
+// each thread keeps 8 independent 16-byte loads in flight.
+__global__ void __launch_bounds__(512)
+k_plane_absmax(const float* __restrict__ I, const float* __restrict__ p, int P4, ImgState* st,
+               unsigned int* __restrict__ scratch) {
+  __shared__ float s_m[2][16];
+  __shared__ bool s_last;
+  const float4* I4 = reinterpret_cast<const float4*>(I);
+  const float4* p4 = reinterpret_cast<const float4*>(p);
+  auto top = [](float m, float4 v) {
+    return fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
+  };
   float mi = 0.0f, mp = 0.0f;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < P;
-       i += (size_t)gridDim.x * blockDim.x) {
-    mi = fmaxf(mi, fabsf(__ldg(&d.uI[i])));
-    mp = fmaxf(mp, fabsf(__ldg(&d.up[i])));
+  const int step = gridDim.x * blockDim.x;
+  int i = blockIdx.x * blockDim.x + threadIdx.x;
+  for (; i + 3 * step < P4; i += 4 * step) {
+    float4 a[4], b[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      a[k] = __ldg(&I4[i + k * step]);
+      b[k] = __ldg(&p4[i + k * step]);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      mi = top(mi, a[k]);
+      mp = top(mp, b[k]);
+    }
+  }
+  for (; i < P4; i += step) {
+    mi = top(mi, __ldg(&I4[i]));
+    mp = top(mp, __ldg(&p4[i]));
   }
   mi = warp_max(mi);
   mp = warp_max(mp);
-  if ((threadIdx.x & 31) == 0) {
-    atomicMax(&st[gi].absmax[0], __float_as_uint(mi));
-    atomicMax(&st[gi].absmax[1], __float_as_uint(mp));
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (lane == 0) {
+    s_m[0][warp] = mi;
+    s_m[1][warp] = mp;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < num_warps(); ++w) {
+      mi = fmaxf(mi, s_m[0][w]);
+      mp = fmaxf(mp, s_m[1][w]);
+    }
+    scratch[2 * blockIdx.x] = __float_as_uint(mi);
+    scratch[2 * blockIdx.x + 1] = __float_as_uint(mp);
+    __threadfence();
+    s_last = atomicAdd(&scratch[2 * ABSMAX_BLOCKS], 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last || threadIdx.x >= 32) return;
+  __threadfence();
+  float m[2] = {0.0f, 0.0f};
+  for (int q = lane; q < (int)gridDim.x; q += 32) {
+    m[0] = fmaxf(m[0], __uint_as_float(__ldcg(&scratch[2 * q])));
+    m[1] = fmaxf(m[1], __uint_as_float(__ldcg(&scratch[2 * q + 1])));
+  }
+  m[0] = warp_max(m[0]);
+  m[1] = warp_max(m[1]);
+  if (lane == 0) {
+    st->absmax[0] = __float_as_uint(m[0]);
+    st->absmax[1] = __float_as_uint(m[1]);
+    scratch[2 * ABSMAX_BLOCKS] = 0u;
   }
 }
 
-cudaError_t launch_plane_absmax(const ClassLaunch& c, cudaStream_t s) {
-  const size_t P = (size_t)c.cd.M * c.cd.N;
-  int chunks = (int)((P + 256 * 8 - 1) / (256 * 8));
-  if (chunks > 128) chunks = 128;
-  k_plane_absmax<<<dim3(chunks, c.cd.n_img), 256, 0, s>>>(c.cd, c.imgs, c.st);
+cudaError_t launch_plane_absmax(const ClassLaunch& c, unsigned int* scratch, cudaStream_t s) {
+  const int P4 = c.cd.M * c.cd.N / 4;
+  int blocks = (P4 + 512 * 4 - 1) / (512 * 4);
+  if (blocks > ABSMAX_BLOCKS) blocks = ABSMAX_BLOCKS;
+  k_plane_absmax<<<blocks, 512, 0, s>>>(c.one->uI, c.one->up, P4, c.st, scratch);
   return cudaGetLastError();
 }
 
@@ -829,7 +879,8 @@ cudaError_t launch_guided_filter(const ClassLaunch& c, int iter, int var_mode, i
                            (4 * gf_sm_count() + div - 1) / div);
     const int n_items = cd.n_img * strips * ((cd.M + H - 1) / H);
     const int need = (n_items + W - 1) / W;
-    kern<<<blocks < need ? blocks : need, W * 32, smem, s>>>(cd, c.imgs, c.st, iter, shifted, H);
+    kern<<<blocks < need ? blocks : need, W * 32, smem, s>>>(cd, c.imgs, one_desc(c), c.st,
+                                                             iter, shifted, H);
   }
   return cudaGetLastError();
 }

@@ -238,17 +238,7 @@ __global__ void k_crop(const float* __restrict__ src, int N, float* __restrict__
   }
 }
 
-__global__ void k_store_desc(ImgDesc d, ImgDesc* dst, ImgState* st) {
-  if (threadIdx.x == 0) *dst = d;
-  if (st && threadIdx.x < 2) st->absmax[threadIdx.x] = 0u;
-}
-
-cudaError_t launch_store_desc(const ImgDesc& d, ImgDesc* dst, ImgState* st, cudaStream_t s) {
-  k_store_desc<<<1, 32, 0, s>>>(d, dst, st);
-  return cudaGetLastError();
-}
-
-const void* store_desc_kernel() { return (const void*)k_store_desc; }
+const void* some_kernel() { return (const void*)k_crop; }
 
 static unsigned plane_blocks(size_t total) {
   size_t nb = (total + 255) / 256;

@@ -44,6 +44,7 @@ struct ClassLaunch {
   ClassDesc cd;
   const ImgDesc* imgs;  // device array (whole batch)
   ImgState* st;         // device array (whole batch)
+  const ImgDesc* one;   // host: the descriptor of a utility call's one image (imgs is then null)
   int max_rad;          // largest guided-filter radius in the class
   int n_rad_groups;
   RadGroup rad_groups[9];
@@ -53,6 +54,9 @@ struct ClassLaunch {
   int class_id;         // index of the class in its plan (instrumentation)
   bool short_cols;      // small problem: the short column passes (and their tile width)
 };
+
+// The descriptor that a kernel takes as an argument beside `imgs`.
+inline ImgDesc one_desc(const ClassLaunch& c) { return c.one ? *c.one : ImgDesc{}; }
 
 // Row pass of the 2-D real DFT: real plane src -> packed rows dst.
 // do_sum: accumulate the FP64 sum of src into st.sum_u.
@@ -93,12 +97,13 @@ cudaError_t launch_guided_filter(const ClassLaunch& c, int iter, int var_mode, i
 cudaError_t launch_guided_filter_color(const float* I, const float* p, int M, int N, int w,
                                        double eps, int boundary, float* ab, float* u,
                                        cudaStream_t s);
-// *dst = d (a descriptor for the utility calls); st: clear its absmax.
-cudaError_t launch_store_desc(const ImgDesc& d, ImgDesc* dst, ImgState* st, cudaStream_t s);
-const void* store_desc_kernel();
-// Largest |u_I|, |u_p| of every image into ImgState::absmax (which must be
-// zero before), for guided-filter calls outside a solve.
-cudaError_t launch_plane_absmax(const ClassLaunch& c, cudaStream_t s);
+// Largest |u_I|, |u_p| of a utility call's image into ImgState::absmax, for
+// guided-filter calls outside a solve.  scratch: ABSMAX_SCRATCH words, zero
+// before the first call, left ready for the next.
+constexpr int ABSMAX_BLOCKS = 152;
+constexpr int ABSMAX_SCRATCH = 2 * ABSMAX_BLOCKS + 1;
+cudaError_t launch_plane_absmax(const ClassLaunch& c, unsigned int* scratch, cudaStream_t s);
+const void* some_kernel();  // any kernel of the library (its attributes)
 // Double-float 2-D real DFT of real plane src into spectrum plane dst
 // (SEL_H or SEL_YS); uses the S and Q_I planes as scratch.
 cudaError_t launch_fft2_r2c_df(const ClassLaunch& c, const float4* twdf, int src, int dst,
