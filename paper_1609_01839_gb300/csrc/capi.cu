@@ -102,6 +102,7 @@ struct ClassTune {
 
 struct TuneTable {
   int chains = CHAINS;  // concurrent chains of a captured solve (1..CHAINS)
+  bool tuned_chains = false;  // measured or from a file, not the default
   std::vector<ClassTune> cls;
   ClassTune get(int M, int N) const {
     for (const ClassTune& t : cls)
@@ -307,7 +308,21 @@ void drop_plan(gfdeconv_ctx* c) {
   c->have_plan = false;
 }
 
-cudaError_t build_plan(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs, int iters) {
+// Chains of an untuned solve.  Concurrent chains fill the tails of each other's
+// kernels; where a kernel runs for many waves they only cut its launches into
+// pieces.  Whole solves with 1, 2 and 4 chains: 4 images of 4096^2 58.4, 60.0,
+// 63.3 ms; 256 uneven images (107 Mpixel, three sizes) 40.0, 37.5, 38.6; 64
+// (27 Mpixel) 12.7, 11.3, 10.9.  (With host copies the chains also spread
+// the transfers: four there.)
+int default_chains(const std::vector<ClassLaunch>& classes) {
+  long long px = 0;
+  for (const ClassLaunch& cl : classes) px += (long long)cl.cd.M * cl.cd.N * cl.cd.n_img;
+  if (px < (1LL << 26)) return CHAINS;
+  return classes.size() == 1 ? 1 : 2;
+}
+
+cudaError_t build_plan(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs, int iters,
+                       bool host_copies = false) {
   Plan& pl = c->plan;
   pl.n = n;
   pl.iters = iters;
@@ -392,7 +407,8 @@ cudaError_t build_plan(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs, int i
   // parts: CHAINS consecutive runs of the images of every class, with their
   // window-radius groups cut to the range
   for (auto& v : pl.parts) v.clear();
-  const int nparts = std::max(1, std::min(CHAINS, c->tune.chains));
+  int nparts = std::max(1, std::min(CHAINS, c->tune.chains));
+  if (!c->tune.tuned_chains && !host_copies) nparts = std::min(nparts, default_chains(pl.classes));
   pl.nparts = nparts;
   for (const ClassLaunch& cl : pl.classes) {
     for (int part = 0; part < nparts; ++part) {
@@ -475,7 +491,7 @@ cudaError_t record(gfdeconv_ctx* c, Plan& pl, cudaStream_t s, Timer* tm = nullpt
     for (auto& cl : classes) {
       if (tm) tm->cur_cls = cl.class_id;
       GFD_T(GFD_PHASE_SETUP, launch_setup_init(cl, c->opts.rho, s));
-      L += 2;  // k_setup_init, k_zero_parts
+      ++L;
     }
     for (auto& cl : classes) {
       if (tm) tm->cur_cls = cl.class_id;
@@ -675,7 +691,7 @@ int solve_batched_dev(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs, int it
     cudaError_t e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return map_err(e);
     drop_plan(c);
-    e = build_plan(c, n, imgs, iters);
+    e = build_plan(c, n, imgs, iters, hc != nullptr);
     if (e != cudaSuccess) {
       drop_plan(c);
       return map_err(e);
@@ -735,7 +751,10 @@ bool load_tune(const char* path, TuneTable* out) {
     if (!std::strcmp(word, "chains")) {
       int q = 0;
       ok = std::sscanf(line, "%*s %d", &q) == 1 && q >= 1 && q <= CHAINS;
-      if (ok) t.chains = q;
+      if (ok) {
+        t.chains = q;
+        t.tuned_chains = true;
+      }
     } else if (!std::strcmp(word, "class")) {
       ClassTune c{};
       ok = std::sscanf(line, "%*s %d %d col_threads %d row_threads %d gf_rows %d", &c.M, &c.N,
@@ -1025,6 +1044,7 @@ int gfdeconv_autotune(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs, int it
     int pick = cur.chains;
     for (int q = 1; q <= CHAINS && e == cudaSuccess; ++q) {
       cur.chains = q;
+      cur.tuned_chains = true;
       c->tune = cur;
       drop_plan(c);
       const int r = solve_batched_dev(c, n, imgs, iters, s);  // builds and captures
@@ -1047,6 +1067,7 @@ int gfdeconv_autotune(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs, int it
     if (e1) cudaEventDestroy(e1);
     if (e != cudaSuccess) return fail(e);
     cur.chains = pick;
+    cur.tuned_chains = true;
   }
   c->tune = cur;
   drop_plan(c);

@@ -525,10 +525,10 @@ __global__ void k_adj_stats(const AdjDesc* __restrict__ descs, int M, int N) {
     atomicAdd(&d.acc[4], sy);
     atomicAdd(&d.acc[5], syy);
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    double s = 0.0;
-    for (int i = 0; i < d.kh * d.kw; ++i) s += fabs((double)d.h[i]);
-    d.acc[6] = s;
+  if (blockIdx.x == gridDim.x - 1) {
+    double s, a;
+    psf_sums(d.h, d.kh * d.kw, s, a);
+    if (threadIdx.x == 0) d.acc[6] = a;
   }
 }
 

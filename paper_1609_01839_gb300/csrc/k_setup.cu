@@ -85,22 +85,27 @@ __global__ void k_setup_stats(ClassDesc cd, const ImgDesc* __restrict__ imgs, Im
     atomicAdd(&st[gi].sum_yy, df_to_double(b));
     if (d.uo) atomicAdd(&st[gi].den_isnr, df_to_double(c));
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    double sh = 0.0, sa = 0.0;
-    for (int i = 0; i < d.kh * d.kw; ++i) {
-      const double v = (double)d.h[i];
-      sh += v;
-      sa += fabs(v);
+  if (blockIdx.x == gridDim.x - 1) {  // sum h, sum |h|
+    double sh, sa;
+    psf_sums(d.h, d.kh * d.kw, sh, sa);
+    if (threadIdx.x == 0) {
+      st[gi].sum_h = sh;
+      st[gi].amax = sa;  // squared in k_setup_init
     }
-    st[gi].sum_h = sh;
-    st[gi].amax = sa;  // squared in k_setup_init
   }
 }
 
-// Starting iterate of every image of a class: u_E = u_init, or 0 (Step 0).
-// Images are M*N floats, 16-byte aligned, M*N a multiple of 4 for every
-// supported canvas; grid-stride over float4 groups of all images.
-__global__ void k_init_u(ClassDesc cd, const ImgDesc* __restrict__ imgs) {
+// Starting iterate of every image of a class: u_E = u_init, or 0 (Step 0), and
+// zeroed partial slots of the spectral passes (each pass leaves them zeroed
+// again after reducing them).  Images are M*N floats, 16-byte aligned, M*N a
+// multiple of 4 for every supported canvas; grid-stride over float4 groups of
+// all images.
+__global__ void k_init_u(ClassDesc cd, const ImgDesc* __restrict__ imgs, int n_slots) {
+  for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < (size_t)n_slots * cd.n_img;
+       idx += (size_t)gridDim.x * blockDim.x) {
+    const size_t li = idx / n_slots;
+    imgs[cd.img0 + li].part[idx - li * n_slots] = 0.0;
+  }
   const size_t P4 = (size_t)cd.M * cd.N / 4;
   const size_t total = P4 * cd.n_img;
   for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
@@ -149,14 +154,6 @@ __global__ void k_setup_init(ClassDesc cd, const ImgDesc* __restrict__ imgs, Img
   S->need = 0;
   S->rtol = d.lam_rtol;
   set_bracket(S, INITIAL_LO, INITIAL_HI);
-}
-
-// Zero the per-item partial slots of the spectral passes (each pass leaves
-// them zeroed again after reducing them).
-__global__ void k_zero_parts(ClassDesc cd, const ImgDesc* __restrict__ imgs, int n_slots) {
-  const ImgDesc& d = imgs[cd.img0 + blockIdx.y];
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_slots; i += gridDim.x * blockDim.x)
-    d.part[i] = 0.0;
 }
 
 // Circular PSF embedding: offset (a - kh/2, b - kw/2) -> canvas index mod (M, N).
@@ -290,16 +287,15 @@ cudaError_t launch_init_u(const ClassLaunch& c, cudaStream_t s) {
   size_t nb = (total + 255) / 256;
   if (nb > 152 * 16) nb = 152 * 16;
   if (nb < 1) nb = 1;
-  k_init_u<<<(unsigned)nb, 256, 0, s>>>(c.cd, c.imgs);
+  const size_t Lc = c.cd.N / 2;
+  const size_t col_items = Lc / 2, pass_items = (size_t)c.cd.M * Lc / 4096 + 1;
+  const int n_slots = (int)((KNODES + 1) * (col_items > pass_items ? col_items : pass_items));
+  k_init_u<<<(unsigned)nb, 256, 0, s>>>(c.cd, c.imgs, n_slots);
   return cudaGetLastError();
 }
 
 cudaError_t launch_setup_init(const ClassLaunch& c, double rho_fixed, cudaStream_t s) {
   k_setup_init<<<(c.cd.n_img + 127) / 128, 128, 0, s>>>(c.cd, c.imgs, c.st, rho_fixed);
-  const size_t Lc = c.cd.N / 2;
-  const size_t col_items = Lc / 2, pass_items = (size_t)c.cd.M * Lc / 4096 + 1;
-  const int n_slots = (int)((KNODES + 1) * (col_items > pass_items ? col_items : pass_items));
-  k_zero_parts<<<dim3((n_slots + 255) / 256, c.cd.n_img), 256, 0, s>>>(c.cd, c.imgs, n_slots);
   return cudaGetLastError();
 }
 
