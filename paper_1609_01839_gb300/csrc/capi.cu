@@ -1163,10 +1163,9 @@ int gfdeconv_backward_batched(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs
   if (cudaSetDevice(c->device) != cudaSuccess) return GFD_ERR_CUDA;
   cudaStream_t s = (cudaStream_t)stream;
   const size_t P = (size_t)M * N;
-  // per image: 17 real planes (16 of the adjoint, u_E^k) and 11 spectra (10
-  // of the adjoint, the FFT scratch) of P floats each, 12 doubles (lambda,
-  // g_eps, the sums)
-  const int n_real = 17, n_spec = 11, n_dbl = 12;
+  // per image: 16 real planes and 11 spectra (10 of the adjoint, the FFT
+  // scratch) of P floats each, 12 doubles (lambda, g_eps, the sums)
+  const int n_real = 16, n_spec = 11, n_dbl = 12;
   const size_t plane = align256(P * sizeof(float));
   const size_t per_img = (n_real + n_spec) * plane + align256(n_dbl * sizeof(double));
   const size_t descs_bytes = align256(sizeof(AdjDesc) * n);
@@ -1191,7 +1190,7 @@ int gfdeconv_backward_batched(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs
   const size_t fft_stride = align256(sizeof(ImgDesc) * 2 * n) / sizeof(ImgDesc);
   cur += fft_bytes;
   std::vector<AdjDesc> ad(n);
-  std::vector<float*> uEcur(n), hc(n), scratch(n);
+  std::vector<float*> hc(n), scratch(n);
   std::vector<std::vector<ImgDesc>> fd(n_fft, std::vector<ImgDesc>(n));
   for (int i = 0; i < n; ++i) {
     char* b = cur + per_img * i;
@@ -1225,7 +1224,6 @@ int gfdeconv_backward_batched(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs
     a.gup = realp(13);
     a.gtmp = realp(14);
     a.gtmp2 = realp(15);
-    uEcur[i] = realp(16);
     a.H = specp(0);
     a.Y = specp(1);
     a.UE = specp(2);
@@ -1260,7 +1258,8 @@ int gfdeconv_backward_batched(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs
       q.QI = src;
       q.uI = dst;
     };
-    r2c(0, uEcur[i], a.UE, scr);
+    r2c(0, nullptr, a.UE, scr);  // from the checkpoints
+    fd[0][i].u_iters = imgs[i].u_iters;
     c2r(1, a.UI, uIp);  // the recomputed step: U_I, U_p -> u_I, u_p
     c2r(2, a.Up, upp);
     // g_uI, g_up are transformed in one launch (op 12), each through its own
@@ -1270,7 +1269,7 @@ int gfdeconv_backward_batched(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs
     r2c(4, a.gup, a.GUp, a.Up);
     r2c(5, hc[i], a.H, scr);
     r2c(6, imgs[i].y, a.Y, scr);
-    c2r(7, a.gUE, a.gtmp);
+    c2r(7, a.gUE, a.gu);
     c2r(8, a.gY, a.gtmp);
     c2r(9, a.gH, a.gtmp2);
     ImgDesc& q = fd[10][i];  // the PSF embedding writes q.uI
@@ -1280,18 +1279,19 @@ int gfdeconv_backward_batched(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs
     q.kw = imgs[i].kw;
     q.uI = hc[i];
   }
-  if ((e = cudaMemcpyAsync(d_desc, ad.data(), sizeof(AdjDesc) * n, cudaMemcpyHostToDevice, s)) !=
-      cudaSuccess)
-    return map_err(e);
   // paired transforms: u_I and u_p (inverse), g_uI and g_up (forward)
   fd[11] = fd[1];
   fd[11].insert(fd[11].end(), fd[2].begin(), fd[2].end());
   fd[12] = fd[3];
   fd[12].insert(fd[12].end(), fd[4].begin(), fd[4].end());
+  // all descriptors in one copy: the adjoint's, then the transforms'
+  std::vector<char> up(descs_bytes + fft_bytes);
+  std::memcpy(up.data(), ad.data(), sizeof(AdjDesc) * n);
   for (int op = 0; op < n_fft; ++op)
-    if ((e = cudaMemcpyAsync(d_fft + fft_stride * op, fd[op].data(), sizeof(ImgDesc) * fd[op].size(),
-                             cudaMemcpyHostToDevice, s)) != cudaSuccess)
-      return map_err(e);
+    std::memcpy(up.data() + descs_bytes + fft_stride * sizeof(ImgDesc) * op, fd[op].data(),
+                sizeof(ImgDesc) * fd[op].size());
+  if ((e = cudaMemcpyAsync(d_desc, up.data(), up.size(), cudaMemcpyHostToDevice, s)) != cudaSuccess)
+    return map_err(e);
   const Tables t{c->tw, c->d2, c->twdf};
   auto cls = [&](int op) {
     ClassLaunch cl{};
@@ -1300,9 +1300,9 @@ int gfdeconv_backward_batched(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs
     cl.st = nullptr;
     return cl;
   };
-  auto fwd = [&](int op) -> cudaError_t {
+  auto fwd = [&](int op, int src = SEL_U) -> cudaError_t {
     const ClassLaunch cl = cls(op);
-    cudaError_t r = launch_row_r2c(cl, t, SEL_U, SEL_S, false, s);
+    cudaError_t r = launch_row_r2c(cl, t, src, SEL_S, false, s);
     if (r == cudaSuccess) r = launch_col_plain(cl, t, SEL_S, SEL_YS, false, s);
     return r;
   };
@@ -1335,10 +1335,7 @@ int gfdeconv_backward_batched(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs
   for (int k = iters - 1; k >= 0; --k) {
     // recompute the step from u_E^k and the forward's lambda_k: U_E, then
     // U_I, U_p (Eq. 8-9) and u_I, u_p
-    for (int i = 0; i < n; ++i)
-      GFD_ADJ_CK(cudaMemcpyAsync(uEcur[i], imgs[i].u_iters + (size_t)k * P, P * sizeof(float),
-                                 cudaMemcpyDeviceToDevice, s));
-    GFD_ADJ_CK(fwd(0));
+    GFD_ADJ_CK(fwd(0, SEL_ITER0 + k));
     GFD_ADJ_CK(launch_adj_recompute(d_desc, n, M, N, k, c->d2, s));
     GFD_ADJ_CK(adj(11, invP));  // u_I and u_p
     for (int i0 = 0; i0 < n;) {  // guided-filter adjoint, one launch per run of equal w

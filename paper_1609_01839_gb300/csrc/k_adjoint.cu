@@ -38,89 +38,136 @@
 
 namespace gfd {
 
-constexpr int ADJ_TILE = 16;
+constexpr int ADJ_TX = 32, ADJ_TY = 16;   // output pixels of a block
+constexpr int ADJ_THREADS = 256;
+constexpr int ADJ_ROW = 4, ADJ_COL = 2;   // outputs per thread along a row, down a column
 
-// A compensated sum: hi is the FP32 running sum, lo the sum of the exact
-// rounding errors of its additions (and of the low parts of added
-// double-float terms).  hi + lo carries about 2^-48 relative error per term.
-struct CSum {
-  float hi, lo;
+// Compensated sums of two quantities, packed: hi the FP32 running sums, lo the
+// sums of the exact rounding errors of their additions (and of the low parts of
+// added double-float terms).  hi + lo carries about 2^-48 relative error per
+// term; taking a term away again is one more addition.
+struct CSum2 {
+  float2 hi, lo;
 };
-GFD_D void csum_add(CSum& s, df x) {
-  const df t = two_sum(s.hi, x.hi);
-  s.hi = t.hi;
-  s.lo += t.lo + x.lo;
+GFD_D void csum_add(CSum2& s, float2 v, float2 vlo) {
+  const float2 t = cadd(s.hi, v), bb = csub(t, s.hi);
+  const float2 e = cadd(csub(s.hi, csub(t, bb)), csub(v, bb));
+  s.hi = t;
+  s.lo = cadd(s.lo, cadd(e, vlo));
 }
-GFD_D df csum_df(CSum s) { return quick_two_sum(s.hi, s.lo); }  // |lo| <= |hi| in practice
 GFD_D df val_df(float v) { return df{v, 0.0f}; }
 
+// One compensated FP32 sum (a thread's share of a sum over bins or pixels).
+struct CSum {
+  float hi = 0.0f, lo = 0.0f;
+  GFD_D void add(float v) {
+    const df t = two_sum(hi, v);
+    hi = t.hi;
+    lo += t.lo;
+  }
+  GFD_D void add(df v) {
+    const df t = two_sum(hi, v.hi);
+    hi = t.hi;
+    lo += t.lo + v.lo;
+  }
+  GFD_D double get() const { return (double)hi + (double)lo; }
+};
+
 // ---------------------------------------------------------------------------
-// Tiled window sums: OP stages NS planes of a TILE x TILE tile plus an r halo
-// in shared memory, maps every staged pixel to NQ double-float quantities,
-// and gets their compensated window sums (periodic windows) at each output
-// pixel: along the tile's rows into shared memory, then down its columns.
+// Tiled window sums: OP stages NS planes of a TX x TY tile plus an r halo in
+// shared memory, maps every staged pixel to NQ double-float quantities, and
+// gets their compensated window sums (periodic windows) at each output pixel:
+// along the tile's rows into shared memory (four outputs per thread, slid), then
+// down its columns (two, slid).  Bound by FP32 instructions: a term is one
+// compensated addition per quantity, 3.3 along a row and 4.5 down a column per
+// output at r = 3 (7 and 7 with a sum of its own per output, in 16 x 16 tiles).
+// 16 images of 512^2, w = 7: 128, 122, 136 us for the three passes so, TODO_BOX now.
 // ---------------------------------------------------------------------------
 template <class OP>
-__global__ void __launch_bounds__(ADJ_TILE * ADJ_TILE)
+__global__ void __launch_bounds__(ADJ_THREADS)
 k_adj_box(const AdjDesc* __restrict__ descs, int M, int N, int rad) {
   extern __shared__ __align__(16) unsigned char adj_sm[];
-  constexpr int NS = OP::NS, NQ = OP::NQ;
+  constexpr int NS = OP::NS, NQ = OP::NQ, NP = (NQ + 1) / 2;  // NP pairs
   const AdjDesc& d = descs[blockIdx.z];
-  const int E = ADJ_TILE + 2 * rad;
-  float2* rows = reinterpret_cast<float2*>(adj_sm);                           // [E][T][NQ]
-  float* tile = reinterpret_cast<float*>(rows + (size_t)E * ADJ_TILE * NQ);   // [NS][E][E]
-  const int x0 = blockIdx.x * ADJ_TILE, y0 = blockIdx.y * ADJ_TILE;
-  for (int e = threadIdx.x; e < E * E; e += blockDim.x) {
-    const int ty = e / E, tx = e - ty * E;
+  const int EX = ADJ_TX + 2 * rad, EY = ADJ_TY + 2 * rad;
+  float4* rows = reinterpret_cast<float4*>(adj_sm);                       // [NP][EY][TX]: hi, lo
+  float* tile = reinterpret_cast<float*>(rows + (size_t)NP * EY * ADJ_TX);  // [NS][EY][EX]
+  const int x0 = blockIdx.x * ADJ_TX, y0 = blockIdx.y * ADJ_TY;
+  for (int e = threadIdx.x; e < EY * EX; e += blockDim.x) {
+    const int ty = e / EX, tx = e - ty * EX;
     const size_t off = (size_t)((y0 - rad + ty) & (M - 1)) * N + ((x0 - rad + tx) & (N - 1));
 #pragma unroll
-    for (int c = 0; c < NS; ++c) tile[c * E * E + e] = __ldg(&OP::plane(d, c)[off]);
+    for (int c = 0; c < NS; ++c) tile[c * EY * EX + e] = __ldg(&OP::plane(d, c)[off]);
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < E * ADJ_TILE; e += blockDim.x) {
-    const int ty = e / ADJ_TILE, tx = e - ty * ADJ_TILE;
-    CSum s[NQ];
+  for (int e = threadIdx.x; e < EY * (ADJ_TX / ADJ_ROW); e += blockDim.x) {
+    const int ty = e / (ADJ_TX / ADJ_ROW), tx = (e - ty * (ADJ_TX / ADJ_ROW)) * ADJ_ROW;
+    CSum2 s[NP];
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) s[q] = CSum{0.0f, 0.0f};
-    for (int dx = 0; dx <= 2 * rad; ++dx) {
-      const int o = ty * E + tx + dx;
+    for (int q = 0; q < NP; ++q) s[q].hi = s[q].lo = make_float2(0.0f, 0.0f);
+    auto term = [&](int dx, float sg) {
+      const int o = ty * EX + tx + dx;
       float v[NS];
 #pragma unroll
-      for (int c = 0; c < NS; ++c) v[c] = tile[c * E * E + o];
-      df q[NQ];
+      for (int c = 0; c < NS; ++c) v[c] = tile[c * EY * EX + o];
+      df q[2 * NP];
+      q[2 * NP - 1] = val_df(0.0f);
       OP::quantities(v, q);
 #pragma unroll
-      for (int k = 0; k < NQ; ++k) csum_add(s[k], q[k]);
-    }
+      for (int k = 0; k < NP; ++k)
+        csum_add(s[k], make_float2(sg * q[2 * k].hi, sg * q[2 * k + 1].hi),
+                 make_float2(sg * q[2 * k].lo, sg * q[2 * k + 1].lo));
+    };
+#pragma unroll 1
+    for (int dx = 0; dx < 2 * rad; ++dx) term(dx, 1.0f);
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) rows[(size_t)e * NQ + q] = make_float2(s[q].hi, s[q].lo);
+    for (int k = 0; k < ADJ_ROW; ++k) {
+      term(k + 2 * rad, 1.0f);
+#pragma unroll
+      for (int q = 0; q < NP; ++q)
+        rows[(q * EY + ty) * ADJ_TX + tx + k] =
+            make_float4(s[q].hi.x, s[q].hi.y, s[q].lo.x, s[q].lo.y);
+      if (k + 1 < ADJ_ROW) term(k, -1.0f);
+    }
   }
   __syncthreads();
-  const int tx = threadIdx.x % ADJ_TILE, ty = threadIdx.x / ADJ_TILE;
-  const int gy = y0 + ty, gx = x0 + tx;
-  CSum S[NQ];
+  const int tx = threadIdx.x % ADJ_TX, ty0 = (threadIdx.x / ADJ_TX) * ADJ_COL;
+  CSum2 S[NP];
 #pragma unroll
-  for (int q = 0; q < NQ; ++q) S[q] = CSum{0.0f, 0.0f};
-  for (int dy = 0; dy <= 2 * rad; ++dy) {
-    const float2* rr = rows + ((size_t)(ty + dy) * ADJ_TILE + tx) * NQ;
+  for (int q = 0; q < NP; ++q) S[q].hi = S[q].lo = make_float2(0.0f, 0.0f);
+  auto row = [&](int ty, float sg) {
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) csum_add(S[q], df{rr[q].x, rr[q].y});
-  }
-  df W[NQ];
-#pragma unroll
-  for (int q = 0; q < NQ; ++q) W[q] = csum_df(S[q]);  // window sums
+    for (int q = 0; q < NP; ++q) {
+      const float4 v = rows[(q * EY + ty) * ADJ_TX + tx];
+      csum_add(S[q], make_float2(sg * v.x, sg * v.y), make_float2(sg * v.z, sg * v.w));
+    }
+  };
+#pragma unroll 1
+  for (int dy = 0; dy < 2 * rad; ++dy) row(ty0 + dy, 1.0f);
   const float n = (float)((2 * rad + 1) * (2 * rad + 1));
   float eps_part = 0.0f;
-  if (gy < M && gx < N) eps_part = OP::output(d, (size_t)gy * N + gx, W, n);
+#pragma unroll
+  for (int k = 0; k < ADJ_COL; ++k) {
+    const int gy = y0 + ty0 + k, gx = x0 + tx;
+    row(ty0 + k + 2 * rad, 1.0f);
+    df W[2 * NP];
+#pragma unroll
+    for (int q = 0; q < NP; ++q) {  // window sums (|lo| <= |hi| in practice)
+      W[2 * q] = quick_two_sum(S[q].hi.x, S[q].lo.x);
+      W[2 * q + 1] = quick_two_sum(S[q].hi.y, S[q].lo.y);
+    }
+    if (gy < M && gx < N) eps_part += OP::output(d, (size_t)gy * N + gx, W, n);
+    if (k + 1 < ADJ_COL) row(ty0 + k, -1.0f);
+  }
   if (OP::kEps) {  // sum of the pass's eps adjoint over the block (FP64), one atomic
-    __shared__ double red[ADJ_TILE * ADJ_TILE / 32];
+    __shared__ double red[ADJ_THREADS / 32];
     double v = eps_part;
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     __syncthreads();
     if (threadIdx.x == 0) {
       double t = 0.0;
-      for (int w = 0; w < ADJ_TILE * ADJ_TILE / 32; ++w) t += red[w];
+      for (int w = 0; w < ADJ_THREADS / 32; ++w) t += red[w];
       atomicAdd(d.g_eps, t);
     }
   }
@@ -134,13 +181,13 @@ struct AdjStats {
   static constexpr int NS = 2, NQ = 4;
   static constexpr bool kEps = false;
   GFD_D static const float* plane(const AdjDesc& d, int c) { return c == 0 ? d.uI : d.up; }
-  GFD_D static void quantities(const float (&v)[NS], df (&q)[NQ]) {
+  GFD_D static void quantities(const float (&v)[NS], df* q) {
     q[0] = val_df(v[0]);
     q[1] = val_df(v[1]);
     q[2] = two_prod(v[0], v[1]);
     q[3] = two_prod(v[0], v[0]);
   }
-  GFD_D static float output(const AdjDesc& d, size_t o, const df (&S)[NQ], float n) {
+  GFD_D static float output(const AdjDesc& d, size_t o, const df* S, float n) {
     const float inv_n = 1.0f / n, inv2 = inv_n * inv_n;
     const float mu = df_float(S[0]) * inv_n, pb = df_float(S[1]) * inv_n;
     const float var = df_float(df_sub(df_mul_f(S[3], n), df_mul(S[0], S[0]))) * inv2;
@@ -162,12 +209,12 @@ struct AdjPoint {
   GFD_D static const float* plane(const AdjDesc& d, int c) {
     return c == 0 ? d.A : (c == 1 ? d.gu : d.uI);
   }
-  GFD_D static void quantities(const float (&v)[NS], df (&q)[NQ]) {
+  GFD_D static void quantities(const float (&v)[NS], df* q) {
     q[0] = val_df(v[0]);
     q[1] = two_prod(v[1], v[2]);
     q[2] = val_df(v[1]);
   }
-  GFD_D static float output(const AdjDesc& d, size_t o, const df (&S)[NQ], float n) {
+  GFD_D static float output(const AdjDesc& d, size_t o, const df* S, float n) {
     const float inv_n = 1.0f / n;
     const float a = d.A[o], mu = d.MU[o], pb = d.PB[o], ve = d.VE[o];
     const float abar = df_float(S[0]) * inv_n, g_b = df_float(S[2]) * inv_n;
@@ -194,11 +241,11 @@ struct AdjInputs {
   GFD_D static const float* plane(const AdjDesc& d, int c) {
     return c == 0 ? d.GCOV : (c == 1 ? d.GVAR : (c == 2 ? d.GMU : d.GPB));
   }
-  GFD_D static void quantities(const float (&v)[NS], df (&q)[NQ]) {
+  GFD_D static void quantities(const float (&v)[NS], df* q) {
 #pragma unroll
     for (int k = 0; k < NQ; ++k) q[k] = val_df(v[k]);
   }
-  GFD_D static float output(const AdjDesc& d, size_t o, const df (&S)[NQ], float n) {
+  GFD_D static float output(const AdjDesc& d, size_t o, const df* S, float n) {
     const float inv_n = 1.0f / n;
     const float I = d.uI[o], p = d.up[o];
     // m_Ip, m_II and mu terms: p box(g_cov) + 2 I box(g_var) + box(g_mu)
@@ -211,13 +258,16 @@ struct AdjInputs {
 };
 
 template <class OP>
+static size_t adj_box_smem(int rad) {
+  const size_t EX = ADJ_TX + 2 * rad, EY = ADJ_TY + 2 * rad;
+  return (OP::NQ + 1) / 2 * EY * ADJ_TX * sizeof(float4) + OP::NS * EY * EX * sizeof(float);
+}
+
+template <class OP>
 static cudaError_t launch_adj_box(const AdjDesc* descs, int n, int M, int N, int rad,
                                   cudaStream_t s) {
-  const int E = ADJ_TILE + 2 * rad;
-  const size_t smem = (size_t)E * ADJ_TILE * OP::NQ * sizeof(float2) +
-                      (size_t)OP::NS * E * E * sizeof(float);
-  const dim3 grid((N + ADJ_TILE - 1) / ADJ_TILE, (M + ADJ_TILE - 1) / ADJ_TILE, n);
-  k_adj_box<OP><<<grid, ADJ_TILE * ADJ_TILE, smem, s>>>(descs, M, N, rad);
+  const dim3 grid((N + ADJ_TX - 1) / ADJ_TX, (M + ADJ_TY - 1) / ADJ_TY, n);
+  k_adj_box<OP><<<grid, ADJ_THREADS, adj_box_smem<OP>(rad), s>>>(descs, M, N, rad);
   return cudaGetLastError();
 }
 
@@ -246,11 +296,11 @@ __global__ void k_adj_solve(const AdjDesc* __restrict__ descs, int M, int N,
   const double lamd = __ldcg(d.lam);
   const bool branch = !(lamd < 1e300);
   const float lam = branch ? 0.0f : (float)lamd;
-  const int L = N / 2;
-  const size_t total = (size_t)M * L;
-  for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-       idx += (size_t)gridDim.x * blockDim.x) {
-    const int k = (int)(idx / L), l = (int)(idx - (size_t)k * L);
+  const int L = N / 2, lg = __ffs(L) - 1;  // powers of two
+  const int total = M * L;
+  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total;
+       idx += gridDim.x * blockDim.x) {
+    const int k = idx >> lg, l = idx & (L - 1);
     const float d2r = __ldg(&d2tab[tab_off(M) + k]);
     float2 UI, Up;
     if (branch) {  // lambda = inf: u_I = u_p = u_E (Sec. 3.2)
@@ -364,17 +414,17 @@ __global__ void k_adj_spec_a(const AdjDesc* __restrict__ descs, int M, int N,
   const double lamd = __ldcg(d.lam);
   const bool branch = !(lamd < 1e300);
   const float lam = branch ? 0.0f : (float)lamd;
-  const int L = N / 2;
-  const size_t total = (size_t)M * L;
+  const int L = N / 2, lg = __ffs(L) - 1;  // powers of two
+  const int total = M * L;
   const float invP = 1.0f / ((float)M * (float)N);
-  double sl = 0.0, sf = 0.0;
-  for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-       idx += (size_t)gridDim.x * blockDim.x) {
+  CSum cl, cf;
+  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total;
+       idx += gridDim.x * blockDim.x) {
     if (branch) {
       d.gUE[idx] = make_float2(0.0f, 0.0f);
       continue;
     }
-    const int k = (int)(idx / L), l = (int)(idx - (size_t)k * L);
+    const int k = idx >> lg, l = idx & (L - 1);
     const float d2r = __ldg(&d2tab[tab_off(M) + k]);
     if (l != 0) {
       const BinA o = adj_bin_a(d.H[idx], d.Y[idx], d.UE[idx], cscale(d.GUI[idx], invP),
@@ -383,8 +433,8 @@ __global__ void k_adj_spec_a(const AdjDesc* __restrict__ descs, int M, int N,
       d.gUE[idx] = o.gUE;
       d.gH[idx] = cadd(d.gH[idx], o.gH);
       d.gY[idx] = cadd(d.gY[idx], o.gY);
-      sl += 2.0 * (double)o.glam;  // the bin and its mirror
-      sf += 2.0 * (double)o.fprime;
+      cl.add(2.0f * o.glam);  // the bin and its mirror
+      cf.add(2.0f * o.fprime);
     } else {
       const size_t m = (size_t)((M - k) & (M - 1)) * L;
       float2 HA, HB, YA, YB, EA, EB, GIA, GIB, GPA, GPB;
@@ -398,10 +448,13 @@ __global__ void k_adj_spec_a(const AdjDesc* __restrict__ descs, int M, int N,
       d.gUE[idx] = pack_pair(oa.gUE, ob.gUE);
       d.gH[idx] = cadd(d.gH[idx], pack_pair(oa.gH, ob.gH));
       d.gY[idx] = cadd(d.gY[idx], pack_pair(oa.gY, ob.gY));
-      sl += (double)oa.glam + (double)ob.glam;
-      sf += (double)oa.fprime + (double)ob.fprime;
+      cl.add(oa.glam);
+      cl.add(ob.glam);
+      cf.add(oa.fprime);
+      cf.add(ob.fprime);
     }
   }
+  double sl = cl.get(), sf = cf.get();
   __shared__ double red[2][32];
   for (int o = 16; o > 0; o >>= 1) {
     sl += __shfl_xor_sync(0xffffffffu, sl, o);
@@ -448,11 +501,11 @@ __global__ void k_adj_spec_b(const AdjDesc* __restrict__ descs, int M, int N) {
   if (!(lamd < 1e300)) return;
   const float lam = (float)lamd;
   const float cP = (float)(__ldcg(&d.acc[2]) / ((double)M * N));
-  const int L = N / 2;
-  const size_t total = (size_t)M * L;
-  for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-       idx += (size_t)gridDim.x * blockDim.x) {
-    const int k = (int)(idx / L), l = (int)(idx - (size_t)k * L);
+  const int L = N / 2, lg = __ffs(L) - 1;  // powers of two
+  const int total = M * L;
+  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total;
+       idx += gridDim.x * blockDim.x) {
+    const int k = idx >> lg, l = idx & (L - 1);
     float2 gUE, gH, gY;
     if (l != 0) {
       adj_bin_b(d.H[idx], d.Y[idx], d.UE[idx], lam, cP, gUE, gH, gY);
@@ -474,15 +527,15 @@ __global__ void k_adj_spec_b(const AdjDesc* __restrict__ descs, int M, int N) {
   }
 }
 
-// g_u of the previous step: the adjoint DFT of g_UE (in gtmp, scale 1), or
-// g_uI + g_up where lambda = inf (u_I = u_p = u_E).
+// g_u of the previous step is the adjoint DFT of g_UE, written by the inverse
+// transform; where lambda = inf (u_I = u_p = u_E) it is g_uI + g_up instead.
 __global__ void k_adj_next(const AdjDesc* __restrict__ descs, int M, int N) {
   const AdjDesc& d = descs[blockIdx.y];
-  const bool branch = !(__ldcg(d.lam) < 1e300);
+  if (__ldcg(d.lam) < 1e300) return;
   const size_t P = (size_t)M * N;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < P;
        i += (size_t)gridDim.x * blockDim.x)
-    d.gu[i] = branch ? d.guI[i] + d.gup[i] : d.gtmp[i];
+    d.gu[i] = d.guI[i] + d.gup[i];
 }
 
 cudaError_t launch_adj_spectral(const AdjDesc* descs, int n, int M, int N, const float* d2tab,
@@ -510,13 +563,14 @@ cudaError_t launch_adj_next(const AdjDesc* descs, int n, int M, int N, cudaStrea
 __global__ void k_adj_stats(const AdjDesc* __restrict__ descs, int M, int N) {
   const AdjDesc& d = descs[blockIdx.y];
   const size_t P = (size_t)M * N;
-  double sy = 0.0, syy = 0.0;
+  CSum cy, cyy;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < P;
        i += (size_t)gridDim.x * blockDim.x) {
-    const double v = d.y[i];
-    sy += v;
-    syy += v * v;
+    const float v = __ldg(&d.y[i]);
+    cy.add(v);
+    cyy.add(two_prod(v, v));
   }
+  double sy = cy.get(), syy = cyy.get();
   for (int o = 16; o > 0; o >>= 1) {
     sy += __shfl_xor_sync(0xffffffffu, sy, o);
     syy += __shfl_xor_sync(0xffffffffu, syy, o);
@@ -558,12 +612,14 @@ __global__ void k_adj_rho(const AdjDesc* __restrict__ descs, int n, double P) {
 __global__ void k_adj_final_y(const AdjDesc* __restrict__ descs, int M, int N) {
   const AdjDesc& d = descs[blockIdx.y];
   const size_t P = (size_t)M * N;
+  // g_num (2 y - 2 Sy / P) + g_den h1^2 2 y = a y + b, a in double-float
   const double g_num = d.acc[7], g_den = d.acc[8], Sy = d.acc[4], h1 = d.acc[6];
+  const df a = df_from_double(2.0 * (g_num + g_den * h1 * h1));
+  const df b = df_from_double(-2.0 * g_num * Sy / (double)P);
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < P;
        i += (size_t)gridDim.x * blockDim.x) {
-    const double y = d.y[i];
-    d.gy_out[i] = (float)((double)d.gtmp[i] + g_num * (2.0 * y - 2.0 * Sy / (double)P) +
-                          g_den * h1 * h1 * 2.0 * y);
+    const df v = df_add(df_add(df_mul_f(a, __ldg(&d.y[i])), b), df_make(__ldg(&d.gtmp[i])));
+    d.gy_out[i] = v.hi + v.lo;
   }
 }
 
@@ -601,17 +657,16 @@ cudaError_t launch_adj_final(const AdjDesc* descs, int n, int M, int N, int max_
   return cudaGetLastError();
 }
 
+template <class OP>
+static cudaError_t configure_adj_box() {
+  return cudaFuncSetAttribute(k_adj_box<OP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)adj_box_smem<OP>(8));
+}
+
 cudaError_t configure_adj_kernels() {
-  const int rmax = 8, E = ADJ_TILE + 2 * rmax;  // shared bytes of launch_adj_box at r = 8
-  const int b1 = E * ADJ_TILE * AdjStats::NQ * 8 + AdjStats::NS * E * E * 4;
-  const int b2 = E * ADJ_TILE * AdjPoint::NQ * 8 + AdjPoint::NS * E * E * 4;
-  const int b3 = E * ADJ_TILE * AdjInputs::NQ * 8 + AdjInputs::NS * E * E * 4;
-  cudaError_t e = cudaFuncSetAttribute(k_adj_box<AdjStats>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, b1);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_adj_box<AdjPoint>, cudaFuncAttributeMaxDynamicSharedMemorySize, b2);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_adj_box<AdjInputs>, cudaFuncAttributeMaxDynamicSharedMemorySize, b3);
+  cudaError_t e = configure_adj_box<AdjStats>();
+  if (e == cudaSuccess) e = configure_adj_box<AdjPoint>();
+  if (e == cudaSuccess) e = configure_adj_box<AdjInputs>();
   return e;
 }
 

@@ -107,7 +107,9 @@ k_row_r2c(ClassDesc cd, const ImgDesc* __restrict__ imgs, const __grid_constant_
   const int row = row_c % M;
   const unsigned int mask = warp_mask();
   float2* buf = smem + team * G::SIZE;
-  const float2* src = reinterpret_cast<const float2*>(real_plane(d, src_sel)) + (size_t)row * L;
+  const float* plane = src_sel >= SEL_ITER0 ? d.u_iters + (size_t)(src_sel - SEL_ITER0) * M * N
+                                            : real_plane(d, src_sel);
+  const float2* src = reinterpret_cast<const float2*>(plane) + (size_t)row * L;
   float part = 0.0f;
 #pragma unroll
   for (int q = 0; q < G::E / r0; ++q) {

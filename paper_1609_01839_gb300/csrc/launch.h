@@ -16,6 +16,7 @@ enum PlaneSel : int {
   SEL_YS = 6,  // observation spectrum
   SEL_UI = 7,  // u_I (real)
   SEL_UP = 8,  // u_p (real)
+  SEL_ITER0 = 16,  // checkpoint k (real, forward row pass only): SEL_ITER0 + k
 };
 
 // Tile shapes of one size class (threads per block of the row passes, which
