@@ -90,26 +90,29 @@ k_adj_box(const AdjDesc* __restrict__ descs, int M, int N, int rad) {
   constexpr int NS = OP::NS, NQ = OP::NQ, NP = (NQ + 1) / 2;  // NP pairs
   const AdjDesc& d = descs[blockIdx.z];
   const int EX = ADJ_TX + 2 * rad, EY = ADJ_TY + 2 * rad;
-  float4* rows = reinterpret_cast<float4*>(adj_sm);                       // [NP][EY][TX]: hi, lo
-  float* tile = reinterpret_cast<float*>(rows + (size_t)NP * EY * ADJ_TX);  // [NS][EY][EX]
+  // consecutive threads of the row sums take consecutive rows: odd pitches keep
+  // them on different banks
+  constexpr int RP = ADJ_TX + 1;
+  const int TP = EX | 1;
+  float4* rows = reinterpret_cast<float4*>(adj_sm);                   // [NP][EY][RP]: hi, lo
+  float* tile = reinterpret_cast<float*>(rows + (size_t)NP * EY * RP);  // [NS][EY][TP]
   const int x0 = blockIdx.x * ADJ_TX, y0 = blockIdx.y * ADJ_TY;
   for (int e = threadIdx.x; e < EY * EX; e += blockDim.x) {
     const int ty = e / EX, tx = e - ty * EX;
     const size_t off = (size_t)((y0 - rad + ty) & (M - 1)) * N + ((x0 - rad + tx) & (N - 1));
 #pragma unroll
-    for (int c = 0; c < NS; ++c) tile[c * EY * EX + e] = __ldg(&OP::plane(d, c)[off]);
+    for (int c = 0; c < NS; ++c) tile[(c * EY + ty) * TP + tx] = __ldg(&OP::plane(d, c)[off]);
   }
   __syncthreads();
   for (int e = threadIdx.x; e < EY * (ADJ_TX / ADJ_ROW); e += blockDim.x) {
-    const int ty = e / (ADJ_TX / ADJ_ROW), tx = (e - ty * (ADJ_TX / ADJ_ROW)) * ADJ_ROW;
+    const int ty = e % EY, tx = (e / EY) * ADJ_ROW;
     CSum2 s[NP];
 #pragma unroll
     for (int q = 0; q < NP; ++q) s[q].hi = s[q].lo = make_float2(0.0f, 0.0f);
     auto term = [&](int dx, float sg) {
-      const int o = ty * EX + tx + dx;
       float v[NS];
 #pragma unroll
-      for (int c = 0; c < NS; ++c) v[c] = tile[c * EY * EX + o];
+      for (int c = 0; c < NS; ++c) v[c] = tile[(c * EY + ty) * TP + tx + dx];
       df q[2 * NP];
       q[2 * NP - 1] = val_df(0.0f);
       OP::quantities(v, q);
@@ -125,7 +128,7 @@ k_adj_box(const AdjDesc* __restrict__ descs, int M, int N, int rad) {
       term(k + 2 * rad, 1.0f);
 #pragma unroll
       for (int q = 0; q < NP; ++q)
-        rows[(q * EY + ty) * ADJ_TX + tx + k] =
+        rows[(q * EY + ty) * RP + tx + k] =
             make_float4(s[q].hi.x, s[q].hi.y, s[q].lo.x, s[q].lo.y);
       if (k + 1 < ADJ_ROW) term(k, -1.0f);
     }
@@ -138,7 +141,7 @@ k_adj_box(const AdjDesc* __restrict__ descs, int M, int N, int rad) {
   auto row = [&](int ty, float sg) {
 #pragma unroll
     for (int q = 0; q < NP; ++q) {
-      const float4 v = rows[(q * EY + ty) * ADJ_TX + tx];
+      const float4 v = rows[(q * EY + ty) * RP + tx];
       csum_add(S[q], make_float2(sg * v.x, sg * v.y), make_float2(sg * v.z, sg * v.w));
     }
   };
@@ -260,7 +263,8 @@ struct AdjInputs {
 template <class OP>
 static size_t adj_box_smem(int rad) {
   const size_t EX = ADJ_TX + 2 * rad, EY = ADJ_TY + 2 * rad;
-  return (OP::NQ + 1) / 2 * EY * ADJ_TX * sizeof(float4) + OP::NS * EY * EX * sizeof(float);
+  return (OP::NQ + 1) / 2 * EY * (ADJ_TX + 1) * sizeof(float4) +
+         OP::NS * EY * (EX | 1) * sizeof(float);
 }
 
 template <class OP>

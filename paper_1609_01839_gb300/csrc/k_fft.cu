@@ -87,6 +87,19 @@ struct MirrorSlots {
 
 GFD_D float2 select2(bool c, float2 a, float2 b) { return c ? a : b; }
 
+// Which row of the block (of rpc) and which thread of its team a thread is on
+// the side of the tiled spectra: TB threads for the columns of a tile's row,
+// then the block's rows, whose pieces of TB values lie side by side, so that a
+// warp's access is one run of up to rpc * TB values instead of 32 / TB pieces.
+// On the side of the image a team is T consecutive threads.
+template <int T>
+GFD_D void tiled_thread(int TB, int rpc, int& row, int& j) {
+  const int w = TB < T ? TB : T, lw = __ffs(w) - 1, lr = __ffs(rpc) - 1;
+  const int tid = threadIdx.x;
+  row = (tid >> lw) & (rpc - 1);
+  j = ((tid >> (lw + lr)) << lw) + (tid & (w - 1));
+}
+
 // Forward: real rows -> packed row spectra (tiled).  Each row of N reals is read
 // as N/2 complex z[n] = x[2n] + i x[2n+1]; Z = FFT_{N/2}(z); with
 // E = (Z[k] + conj Z[-k]) / 2 and O = (Z[k] - conj Z[-k]) / (2i),
@@ -140,24 +153,27 @@ k_row_r2c(ClassDesc cd, const ImgDesc* __restrict__ imgs, const __grid_constant_
       }
     }
   }
-  team_sync<T>(mask);
   if constexpr (G::S == 3) {
-    fft_mid<FK_R2C, L, false>(buf, j, tw);
     team_sync<T>(mask);
+    fft_mid<FK_R2C, L, false>(buf, j, tw);
   }
-  // tiled row: column k of tile k / TB
-  float2* dst = cplx_plane(d, dst_sel) + (size_t)row * TB;
+  __syncthreads();  // the last stage's threads are spread over the block's rows
+  int trow, tj;
+  tiled_thread<T>(TB, rpc, trow, tj);
+  const float2* tbuf = smem + trow * G::SIZE;
+  // tiled row: column k of tile k / TB (the block's rows are of one image)
+  float2* dst = cplx_plane(d, dst_sel) + (size_t)(row - team + trow) * TB;
   const int lg = __ffs(TB) - 1;
   auto put = [&](int k, float2 v) {
     dst[(((size_t)(k >> lg) * M) << lg) + (k & (TB - 1))] = v;
   };
 #pragma unroll
   for (int q = 0; q < G::E / rl / 2; ++q) {
-    const int kap = j + T * q;
-    const bool self = q == 0 && j == 0;
+    const int kap = tj + T * q;
+    const bool self = q == 0 && tj == 0;
     float2 A[rl], B[rl];
-    fft_last<FK_R2C, L, false>(A, kap, buf);
-    fft_last<FK_R2C, L, false>(B, self ? KL / 2 : KL - kap, buf);
+    fft_last<FK_R2C, L, false>(A, kap, tbuf);
+    fft_last<FK_R2C, L, false>(B, self ? KL / 2 : KL - kap, tbuf);
 #pragma unroll
     for (int t = 0; t < rl; ++t) {
       const int k = MirrorSlots<rl>::first(self, kap, KL, t);
@@ -206,15 +222,18 @@ k_row_c2r(ClassDesc cd, const ImgDesc* __restrict__ imgs, const __grid_constant_
   const ImgDesc& d = imgs ? imgs[cd.img0 + li] : one;
   const unsigned int mask = warp_mask();
   float2* buf = smem + team * G::SIZE;
-  const float2* src = cplx_plane(d, second ? sel1 : sel0) + (size_t)row * TB;
+  int trow, tj;
+  tiled_thread<T>(TB, rpc, trow, tj);
+  float2* tbuf = smem + trow * G::SIZE;
+  const float2* src = cplx_plane(d, second ? sel1 : sel0) + (size_t)(row - team + trow) * TB;
   const int lg = __ffs(TB) - 1;
   auto get = [&](int k) {
     return load_stream(src + (((size_t)(k >> lg) * M) << lg) + (k & (TB - 1)));
   };
 #pragma unroll
   for (int q = 0; q < G::E / r0 / 2; ++q) {
-    const int beta = j + T * q;
-    const bool self = q == 0 && j == 0;
+    const int beta = tj + T * q;
+    const bool self = q == 0 && tj == 0;
     float2 u[r0], v[r0];  // Z at the slots' first and second positions
 #pragma unroll
     for (int t = 0; t < r0; ++t) {
@@ -244,10 +263,10 @@ k_row_c2r(ClassDesc cd, const ImgDesc* __restrict__ imgs, const __grid_constant_
         B[i] = select2(self, i < r0 / 2 ? u[i + r0 / 2] : v[r0 + r0 / 2 - 1 - i], B[i]);
       }
     }
-    fft_first<FK_C2R, L, true>(A, beta, buf, tw);
-    fft_first<FK_C2R, L, true>(B, self ? G::L1 / 2 : G::L1 - beta, buf, tw);
+    fft_first<FK_C2R, L, true>(A, beta, tbuf, tw);
+    fft_first<FK_C2R, L, true>(B, self ? G::L1 / 2 : G::L1 - beta, tbuf, tw);
   }
-  team_sync<T>(mask);
+  __syncthreads();  // back to a team per row
   if constexpr (G::S == 3) {
     fft_mid<FK_C2R, L, true>(buf, j, tw);
     team_sync<T>(mask);

@@ -37,15 +37,19 @@ constexpr int CGF_RMAX = 8;
 constexpr int CGF_ROW = 4, CGF_COL = 2;  // outputs per thread along a row, down a column
 constexpr int CGF_Q = 13;                // window sums, each a leading and a remainder part
 
-// Row sums [CGF_Q][rows][TX] float2 and the input tile [rows][cols] float4.
+// Row sums [CGF_Q][rows][CGF_RP] float2 and the input tile [rows][pitch] float4.
+// Consecutive threads of the row sums take consecutive rows: odd pitches keep
+// them on different banks.
+constexpr int CGF_RP = CGF_TX + 1;
+GFD_HD int cgf_pitch(int rad) { return (CGF_TX + 2 * rad) | 1; }
 GFD_HD size_t cgf_smem1(int rad) {
-  const int EX = CGF_TX + 2 * rad, EY = CGF_TY + 2 * rad;
-  return (size_t)CGF_Q * EY * CGF_TX * sizeof(float2) + (size_t)EX * EY * sizeof(float4);
+  const int EY = CGF_TY + 2 * rad;
+  return (size_t)cgf_pitch(rad) * EY * sizeof(float4) + (size_t)CGF_Q * EY * CGF_RP * sizeof(float2);
 }
-// pass 2: row sums [4][rows][TX] float2, the tile [rows][cols] float4
+// pass 2: row sums [2][rows][CGF_RP] float4, the tile [rows][pitch] float4
 GFD_HD size_t cgf_smem2(int rad) {
-  const int EX = CGF_TX + 2 * rad, EY = CGF_TY + 2 * rad;
-  return (size_t)4 * EY * CGF_TX * sizeof(float2) + (size_t)EX * EY * sizeof(float4);
+  const int EY = CGF_TY + 2 * rad;
+  return (size_t)(cgf_pitch(rad) + 2 * CGF_RP) * EY * sizeof(float4);
 }
 
 // Canvas index of tile coordinate v (may lie outside [0, L)); -1 when the
@@ -75,7 +79,7 @@ GFD_D void cgf_stage(float4* s, const float* p0, const float* p1, const float* p
       v = make_float4(__ldg(p0 + off) - c.x, __ldg(p1 + off) - c.y, __ldg(p2 + off) - c.z,
                       __ldg(p3 + off) - c.w);
     }
-    s[e] = v;
+    s[ty * cgf_pitch(rad) + tx] = v;
   }
 }
 
@@ -133,9 +137,9 @@ k_cgf_ab(const float* __restrict__ I, const float* __restrict__ p, int M, int N,
   extern __shared__ __align__(16) unsigned char cgf_sm[];
   __shared__ float s_max[4][CGF_THREADS / 32];
   const bool trunc = trunc_i != 0;
-  const int EX = CGF_TX + 2 * rad, EY = CGF_TY + 2 * rad;
-  float4* tile = reinterpret_cast<float4*>(cgf_sm);           // [EY][EX]
-  float2* rows = reinterpret_cast<float2*>(tile + EX * EY);   // [13][EY][TX]
+  const int EX = CGF_TX + 2 * rad, EY = CGF_TY + 2 * rad, TP = cgf_pitch(rad);
+  float4* tile = reinterpret_cast<float4*>(cgf_sm);           // [EY][TP]
+  float2* rows = reinterpret_cast<float2*>(tile + TP * EY);   // [13][EY][CGF_RP]
   const size_t P = (size_t)M * N;
   const int x0 = blockIdx.x * CGF_TX, y0 = blockIdx.y * CGF_TY;
   float4 c;
@@ -148,7 +152,7 @@ k_cgf_ab(const float* __restrict__ I, const float* __restrict__ p, int M, int N,
   // the tile's largest |deviation| of each plane fixes the grids
   float4 mx = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   for (int e = threadIdx.x; e < EX * EY; e += blockDim.x) {
-    const float4 v = tile[e];
+    const float4 v = tile[(e / EX) * TP + e % EX];
     mx = make_float4(fmaxf(mx.x, fabsf(v.x)), fmaxf(mx.y, fabsf(v.y)), fmaxf(mx.z, fabsf(v.z)),
                      fmaxf(mx.w, fabsf(v.w)));
   }
@@ -182,8 +186,8 @@ k_cgf_ab(const float* __restrict__ I, const float* __restrict__ p, int M, int N,
   }
   // row sums: CGF_ROW neighbouring outputs of a tile row, slid
   for (int e = threadIdx.x; e < EY * (CGF_TX / CGF_ROW); e += blockDim.x) {
-    const int ty = e / (CGF_TX / CGF_ROW), tx = (e - ty * (CGF_TX / CGF_ROW)) * CGF_ROW;
-    const float4* in = tile + ty * EX + tx;
+    const int ty = e % EY, tx = (e / EY) * CGF_ROW;
+    const float4* in = tile + ty * TP + tx;
     CgfSums s;
     s.clear();
 #pragma unroll 1
@@ -193,7 +197,7 @@ k_cgf_ab(const float* __restrict__ I, const float* __restrict__ p, int M, int N,
       s.update(in[k + 2 * rad], g, ig, 1.0f);
 #pragma unroll
       for (int q = 0; q < CGF_Q; ++q)
-        rows[(q * EY + ty) * CGF_TX + tx + k] = make_float2(s.h[q], s.l[q]);
+        rows[(q * EY + ty) * CGF_RP + tx + k] = make_float2(s.h[q], s.l[q]);
       if (k + 1 < CGF_ROW) s.update(in[k], g, ig, -1.0f);
     }
   }
@@ -204,15 +208,15 @@ k_cgf_ab(const float* __restrict__ I, const float* __restrict__ p, int M, int N,
 #pragma unroll
   for (int q = 0; q < CGF_Q; ++q) {
     S[q] = make_float2(0.0f, 0.0f);
-    const float2* rr = rows + (q * EY + ty0) * CGF_TX + tx;
-    for (int dy = 0; dy < 2 * rad; ++dy) S[q] = cadd(S[q], rr[dy * CGF_TX]);
+    const float2* rr = rows + (q * EY + ty0) * CGF_RP + tx;
+    for (int dy = 0; dy < 2 * rad; ++dy) S[q] = cadd(S[q], rr[dy * CGF_RP]);
   }
 #pragma unroll 1
   for (int k = 0; k < CGF_COL; ++k) {
     const int ty = ty0 + k, gy = y0 + ty;
 #pragma unroll
     for (int q = 0; q < CGF_Q; ++q)
-      S[q] = cadd(S[q], rows[(q * EY + ty + 2 * rad) * CGF_TX + tx]);
+      S[q] = cadd(S[q], rows[(q * EY + ty + 2 * rad) * CGF_RP + tx]);
     if (gy < M && gx < N) {
       const float n = trunc ? (float)(cgf_count(gy, M, rad) * cgf_count(gx, N, rad))
                             : (float)((2 * rad + 1) * (2 * rad + 1));
@@ -256,7 +260,7 @@ k_cgf_ab(const float* __restrict__ I, const float* __restrict__ p, int M, int N,
     }
     if (k + 1 < CGF_COL) {
 #pragma unroll
-      for (int q = 0; q < CGF_Q; ++q) S[q] = csub(S[q], rows[(q * EY + ty) * CGF_TX + tx]);
+      for (int q = 0; q < CGF_Q; ++q) S[q] = csub(S[q], rows[(q * EY + ty) * CGF_RP + tx]);
     }
   }
 }
@@ -282,9 +286,9 @@ k_cgf_out(const float* __restrict__ I, const float* __restrict__ ab, int M, int 
           int trunc_i, float* __restrict__ u) {
   extern __shared__ __align__(16) unsigned char cgf_sm[];
   const bool trunc = trunc_i != 0;
-  const int EX = CGF_TX + 2 * rad, EY = CGF_TY + 2 * rad;
-  float4* tile = reinterpret_cast<float4*>(cgf_sm);          // [EY][EX]
-  float4* rows = tile + EX * EY;                             // [2][EY][TX]: (hi pair, lo pair)
+  const int EY = CGF_TY + 2 * rad, TP = cgf_pitch(rad);
+  float4* tile = reinterpret_cast<float4*>(cgf_sm);  // [EY][TP]
+  float4* rows = tile + TP * EY;                     // [2][EY][CGF_RP]: (hi pair, lo pair)
   const size_t P = (size_t)M * N;
   const int x0 = blockIdx.x * CGF_TX, y0 = blockIdx.y * CGF_TY;
   cgf_stage(tile, ab, ab + P, ab + 2 * P, ab + 3 * P, make_float4(0.0f, 0.0f, 0.0f, 0.0f), M, N, y0,
@@ -292,8 +296,8 @@ k_cgf_out(const float* __restrict__ I, const float* __restrict__ ab, int M, int 
   __syncthreads();
   const float2 zero = make_float2(0.0f, 0.0f);
   for (int e = threadIdx.x; e < EY * (CGF_TX / CGF_ROW); e += blockDim.x) {
-    const int ty = e / (CGF_TX / CGF_ROW), tx = (e - ty * (CGF_TX / CGF_ROW)) * CGF_ROW;
-    const float4* in = tile + ty * EX + tx;
+    const int ty = e % EY, tx = (e / EY) * CGF_ROW;
+    const float4* in = tile + ty * TP + tx;
     CgfComp s;
     s.clear();
     auto add = [&](float4 v, float sg) {
@@ -307,7 +311,7 @@ k_cgf_out(const float* __restrict__ I, const float* __restrict__ ab, int M, int 
       add(in[k + 2 * rad], 1.0f);
 #pragma unroll
       for (int i = 0; i < 2; ++i)
-        rows[(i * EY + ty) * CGF_TX + tx + k] =
+        rows[(i * EY + ty) * CGF_RP + tx + k] =
             make_float4(s.hi[i].x, s.hi[i].y, s.lo[i].x, s.lo[i].y);
       if (k + 1 < CGF_ROW) add(in[k], -1.0f);
     }
@@ -320,7 +324,7 @@ k_cgf_out(const float* __restrict__ I, const float* __restrict__ ab, int M, int 
   auto add = [&](int ty, float sg) {
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
-      const float4 v = rows[(i * EY + ty) * CGF_TX + tx];
+      const float4 v = rows[(i * EY + ty) * CGF_RP + tx];
       s.add(i, make_float2(sg * v.x, sg * v.y), make_float2(sg * v.z, sg * v.w));
     }
   };
