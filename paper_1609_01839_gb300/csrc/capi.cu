@@ -495,7 +495,7 @@ cudaError_t record(gfdeconv_ctx* c, Plan& pl, cudaStream_t s, Timer* tm = nullpt
     }
     for (auto& cl : classes) {
       if (tm) tm->cur_cls = cl.class_id;
-      GFD_T(GFD_PHASE_SETUP, launch_embed_psf(cl, SEL_UI, s));
+      GFD_T(GFD_PHASE_SETUP, launch_embed_psf_rows(cl, s));
       // H and Y in double-float, rounded once (they fix the residual of Eq. 10-11)
       GFD_T(GFD_PHASE_SETUP, launch_fft2_r2c_df(cl, t.twdf, SEL_UI, SEL_H, s));
       GFD_T(GFD_PHASE_SETUP, launch_fft2_r2c_df(cl, t.twdf, SEL_Y, SEL_YS, s));

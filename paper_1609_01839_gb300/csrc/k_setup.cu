@@ -175,6 +175,21 @@ __global__ void k_embed_psf(ClassDesc cd, const ImgDesc* __restrict__ imgs, int 
   }
 }
 
+// The same for the rows that the PSF reaches only (launch_fft2_r2c_df reads no
+// others of them): rows (a - kh/2) mod M, a < min(kh, M).
+__global__ void k_embed_psf_rows(ClassDesc cd, const ImgDesc* __restrict__ imgs) {
+  const ImgDesc& d = imgs[cd.img0 + blockIdx.y];
+  const int M = cd.M, N = cd.N, rh = d.kh / 2, rw = d.kw / 2;
+  const int rows = d.kh < M ? d.kh : M;
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < rows * N; e += gridDim.x * blockDim.x) {
+    const int a0 = e / N, j = e - a0 * N;
+    float s = 0.0f;
+    for (int a = a0; a < d.kh; a += M)
+      for (int b = (j + rw) % N; b < d.kw; b += N) s += d.h[a * d.kw + b];
+    d.uI[(size_t)(((a0 - rh) % M + M) % M) * N + j] = s;
+  }
+}
+
 // Unpack column 0 of the packed H and Y into the bins (k, 0) and (k, N/2);
 // the DC bins take the FP64 sums (rounded once).
 __global__ void k_unpack_dc(ClassDesc cd, const ImgDesc* __restrict__ imgs, const ImgState* st) {
@@ -304,6 +319,13 @@ cudaError_t launch_embed_psf(const ClassLaunch& c, int dst, cudaStream_t s) {
   size_t nb = (total + 255) / 256;
   if (nb > 152 * 64) nb = 152 * 64;
   k_embed_psf<<<(unsigned)nb, 256, 0, s>>>(c.cd, c.imgs, dst);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_embed_psf_rows(const ClassLaunch& c, cudaStream_t s) {
+  int nb = (32 * c.cd.N + 255) / 256;  // PSFs of up to 32 rows in one sweep
+  if (nb > 256) nb = 256;
+  k_embed_psf_rows<<<dim3(nb, c.cd.n_img), 256, 0, s>>>(c.cd, c.imgs);
   return cudaGetLastError();
 }
 

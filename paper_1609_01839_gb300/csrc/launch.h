@@ -106,7 +106,8 @@ constexpr int ABSMAX_SCRATCH = 2 * ABSMAX_BLOCKS + 1;
 cudaError_t launch_plane_absmax(const ClassLaunch& c, unsigned int* scratch, cudaStream_t s);
 const void* some_kernel();  // any kernel of the library (its attributes)
 // Double-float 2-D real DFT of real plane src into spectrum plane dst
-// (SEL_H or SEL_YS); uses the S and Q_I planes as scratch.
+// (SEL_H or SEL_YS); uses the S and Q_I planes as scratch.  For dst = SEL_H the
+// rows beyond the PSF's are taken as zero and not read.
 cudaError_t launch_fft2_r2c_df(const ClassLaunch& c, const float4* twdf, int src, int dst,
                                cudaStream_t s);
 // Setup kernels.
@@ -114,6 +115,7 @@ cudaError_t launch_setup_stats(const ClassLaunch& c, cudaStream_t s);
 cudaError_t launch_init_u(const ClassLaunch& c, cudaStream_t s);
 cudaError_t launch_setup_init(const ClassLaunch& c, double rho_fixed, cudaStream_t s);
 cudaError_t launch_embed_psf(const ClassLaunch& c, int dst, cudaStream_t s);
+cudaError_t launch_embed_psf_rows(const ClassLaunch& c, cudaStream_t s);  // into u_I
 cudaError_t launch_unpack_dc(const ClassLaunch& c, cudaStream_t s);
 
 // Symmetric padding of an m x n plane to M x N, and the top-left crop back.
