@@ -449,12 +449,11 @@ cudaError_t build_plan(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs, int i
   } while (0)
 
 // Classes whose fallback passes of iteration k run as one launch: small
-// canvases, and few enough images that their clusters are resident together.
-// A pass over a canvas of 1024 x 1024 takes 8 blocks three times as long as the
-// ordinary pass, so there only the later iterations do, where most images need
-// none.
+// canvases.  A pass over a canvas of 1024 x 1024 takes 8 blocks three times as
+// long as the ordinary pass, so there only the later iterations do, where most
+// images need none.
 bool lambda_loop(const ClassLaunch& cl, int k) {
-  return cl.cd.M * cl.cd.N <= (k < 3 ? 1 : 4) * LAMBDA_LOOP_PIXELS && cl.cd.n_img <= 32;
+  return cl.cd.M * cl.cd.N <= (k < 3 ? 1 : 4) * LAMBDA_LOOP_PIXELS;
 }
 
 cudaError_t record(gfdeconv_ctx* c, Plan& pl, cudaStream_t s, Timer* tm = nullptr,
@@ -843,7 +842,7 @@ int gfdeconv_create(gfdeconv_ctx** out, int cuda_device, const gfdeconv_opts* op
   if (c->opts.lambda_rtol <= 0.0) c->opts.lambda_rtol = 1e-13;
   c->opts.tune_cache = nullptr;  // not retained
   c->tune = tune;
-  e = configure_kernels();
+  e = configure_kernels(c->opts.var_precision, c->opts.boundary);
   if (e != cudaSuccess) {
     delete c;
     return map_err(e);

@@ -885,16 +885,17 @@ cudaError_t launch_guided_filter(const ClassLaunch& c, int iter, int var_mode, i
   return cudaGetLastError();
 }
 
-cudaError_t configure_gf_kernel() {
-  const int modes[4] = {GFD_VAR_COMPENSATED, GFD_VAR_DOUBLE_FLOAT, GFD_VAR_FP64, GFD_VAR_FP32};
-  for (int mode : modes)
-    for (int b : {GFD_BOUNDARY_PERIODIC, GFD_BOUNDARY_TRUNCATED})
-      for (int rad = 0; rad <= GF_RMAX; ++rad) {
-        const cudaError_t e = cudaFuncSetAttribute(
-            (const void*)gf_kernel(mode, b, rad), cudaFuncAttributeMaxDynamicSharedMemorySize,
-            (int)(GFW_WARPS * gfw_ring_floats(rad) * sizeof(float)));
-        if (e != cudaSuccess) return e;
-      }
+// The kernels of one variance mode and boundary, a context's own: setting an
+// attribute loads its kernel.
+cudaError_t configure_gf_kernel(int var_mode, int boundary) {
+  for (int rad = 0; rad <= GF_RMAX; ++rad) {
+    const size_t bytes = GFW_WARPS * gfw_ring_floats(rad) * sizeof(float);
+    if (bytes <= DEFAULT_SMEM) continue;
+    const cudaError_t e = cudaFuncSetAttribute((const void*)gf_kernel(var_mode, boundary, rad),
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)bytes);
+    if (e != cudaSuccess) return e;
+  }
   return cudaSuccess;
 }
 

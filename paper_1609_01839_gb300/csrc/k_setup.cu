@@ -335,18 +335,18 @@ cudaError_t launch_unpack_dc(const ClassLaunch& c, cudaStream_t s) {
 }
 
 cudaError_t configure_fft_kernels();
-cudaError_t configure_gf_kernel();
+cudaError_t configure_gf_kernel(int var_mode, int boundary);
 cudaError_t configure_gfc_kernels();
 cudaError_t configure_adj_kernels();
 cudaError_t configure_df_kernels();
 
-cudaError_t configure_kernels() {
+cudaError_t configure_kernels(int var_mode, int boundary) {
   cudaError_t e = configure_fft_kernels();
   if (e != cudaSuccess) return e;
   if ((e = configure_df_kernels()) != cudaSuccess) return e;
   if ((e = configure_gfc_kernels()) != cudaSuccess) return e;
   if ((e = configure_adj_kernels()) != cudaSuccess) return e;
-  return configure_gf_kernel();
+  return configure_gf_kernel(var_mode, boundary);
 }
 
 }  // namespace gfd

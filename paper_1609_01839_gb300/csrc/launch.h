@@ -165,7 +165,10 @@ cudaError_t launch_adj_stats(const AdjDesc* descs, int n, int M, int N, cudaStre
 cudaError_t launch_adj_final(const AdjDesc* descs, int n, int M, int N, int max_psf,
                              cudaStream_t s);
 
-// Opt every kernel into large dynamic shared memory (once per process/device).
-cudaError_t configure_kernels();
+// Dynamic shared memory that a kernel may have without an attribute.
+constexpr size_t DEFAULT_SMEM = 48 * 1024;
+// Opt the kernels that a context of this variance mode and boundary can launch
+// into the dynamic shared memory beyond it that they need.
+cudaError_t configure_kernels(int var_mode, int boundary);
 
 }  // namespace gfd
