@@ -89,8 +89,10 @@ typedef struct {
   /* rho of the discrepancy target (Sec. 3.2): <= 0 selects Eq. 12, else a
    * fixed value in (0, 1]. */
   double rho;
-  /* 1 (default): capture each solve as a CUDA graph and replay it when the
-   * same batch (pointers, sizes, parameters) is solved again. */
+  /* 1 (default): capture each solve as a CUDA graph and replay it for the
+   * next one of the same canvas sizes, windows and iterations (in that order;
+   * pointers, PSFs, sigma and eps may differ).  Solves that ask for u_I or u_p,
+   * and solves from host buffers, replay for the same pointers only. */
   int use_graphs;
   /* Spectral passes of Eq. 11 launched per iteration after the one fused
    * into the forward transform (images whose root is resolved skip them) in
@@ -191,8 +193,9 @@ int gfdeconv_crop(gfdeconv_ctx* ctx, const float* u_canvas, int M, int N, float*
  * a_k = (Sigma_k + eps U)^-1 (mean(I p) - mu_k pbar_k) with Sigma_k the
  * window covariance of the 3 channels (Eq. 3 with a 3-vector slope),
  * b_k = pbar_k - a_k . mu_k (Eq. 4), u = abar . I + bbar (Eq. 5).  Window
- * statistics and the 3 x 3 solves in FP64; periodic or truncated windows as
- * gfdeconv_opts.boundary selects (var_precision does not apply). */
+ * statistics in exact split sums, the 3 x 3 solves in double-float; periodic or
+ * truncated windows as gfdeconv_opts.boundary selects (var_precision does not
+ * apply). */
 int gfdeconv_guidfilter_color(gfdeconv_ctx* ctx, const float* I, const float* p, int M, int N,
                               int w, double eps, float* u_out, void* stream);
 
@@ -222,9 +225,10 @@ int gfdeconv_fft2_r2c(gfdeconv_ctx* ctx, const float* x, int M, int N, float* X,
  * process (host threads may race on that first call safely): make that first
  * call outside any stream capture.  The cached address belongs to the
  * device's current context; after cudaDeviceReset on that device, create a
- * new gfdeconv context and do not use this entry point again in the process.  Nothing in the scratch has to start
- * at zero: every call writes the whole intermediate plane before reading it.  The scratch is shared by every call on a device, so
- * calls whose stream work overlaps (different streams, or different host
+ * new gfdeconv context and do not use this entry point again in the process.
+ * Nothing in the scratch has to start at zero: every call writes the whole
+ * intermediate plane before reading it.  The scratch is shared by every call
+ * on a device, so calls whose stream work overlaps (different streams, or different host
  * threads without ordering between them) race on it: order them on one stream
  * or synchronise between them.  ctx must be a live context (its twiddle table
  * is used; the context allocates nothing here either). */
@@ -290,7 +294,8 @@ int gfdeconv_tune_read(const char* path, int* chains, int* n_classes, int* shape
                        int max_classes);
 
 /* Tile shapes the context uses for an M x N canvas (tuned or built-in) and
- * its chain count; any output pointer may be NULL. */
+ * its chain count (an untuned solve of one canvas size of 2^26 pixels or more
+ * runs as one chain, of several sizes as two); any output pointer may be NULL. */
 int gfdeconv_tune_get(gfdeconv_ctx* ctx, int M, int N, int* col_threads, int* row_threads,
                       int* gf_rows, int* chains);
 

@@ -24,7 +24,7 @@
 // equations are eliminated in double-float (about 48 bits) and a, b rounded
 // once.  Pass 2's sums are compensated (an FP32 running sum plus the exact
 // error of every addition).  1024 x 1024, w = 9: 1111 us with FP64 sums and
-// solves, 137 us as it is, the same error against FP64 (2.5e-8).
+// solves, 131 us as it is, the same error against FP64 (2.5e-8).
 #include "common.cuh"
 #include "df.cuh"
 #include "launch.h"
