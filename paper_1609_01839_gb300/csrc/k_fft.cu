@@ -688,6 +688,9 @@ k_lambda_loop(ClassDesc cd, const ImgDesc* __restrict__ imgs, ImgState* st, int 
   ImgState* S = st + gi;
   // read by every block before the first cluster barrier, changed after it
   if (__ldcg(&S->need) == 0) return;
+  // The first block's shared memory is written below: it has to have started.
+  // (At the end no block touches another's memory after the last barrier.)
+  cl.sync();
   const ImgDesc& d = imgs[gi];
   const int pairs = cd.M * (cd.N / 2) / 2;
   double* part = cl.map_shared_rank(&s_part[0][0], 0) + rank * (KNODES + 1);
