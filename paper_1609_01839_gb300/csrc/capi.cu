@@ -22,6 +22,7 @@ using namespace gfd;
 namespace {
 
 constexpr int AUX_SLOTS = 8;
+constexpr int FILTER_SETS = 2 * AUX_SLOTS + 1;
 // Fallback lambda passes launched per iteration from the fourth iteration on.
 constexpr int LATE_LAMBDA_PASSES = 2;
 constexpr int CHAINS = GFD_CHAINS;
@@ -149,10 +150,16 @@ struct gfdeconv_ctx {
   bool have_plan = false;
   cudaStream_t last_stream = nullptr;
   long long last_launches = 0;
-  // per-image state and launch_plane_absmax's scratch of the utility calls,
-  // AUX_SLOTS of each in turn: calls in flight on several streams do not meet
+  // Per-image state and launch_plane_absmax's scratch of the filter calls, FILTER_SETS
+  // of each.  The first AUX_SLOTS streams that make such calls have one each
+  // (stream order is all they need); calls on any other stream take the next
+  // AUX_SLOTS in turn, each behind the set's last call by its event; calls that
+  // a caller captures share the last.
   ImgState* aux_st = nullptr;
   unsigned int* aux_max = nullptr;
+  unsigned long long aux_owner[AUX_SLOTS] = {};  // stream ids
+  int aux_owners = 0;
+  cudaEvent_t aux_done[AUX_SLOTS] = {};
   int aux_turn = 0;
   AuxSlot aux[AUX_SLOTS];
   int aux_next = 0;
@@ -623,13 +630,46 @@ cudaError_t aux_finish(AuxSlot* a, cudaStream_t s) {
   return cudaEventRecord(a->done, s);
 }
 
+// Whether the caller captures the stream into a graph of its own (events of
+// the context's other calls have no place there).
+bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+}
+
+// The set of state and scratch for a filter call on stream s, ordered behind the
+// set's last call; done: the event to record behind this one, or null.
+cudaError_t filter_set(gfdeconv_ctx* c, cudaStream_t s, int* set, cudaEvent_t* done) {
+  *done = nullptr;
+  if (capturing(s)) {
+    *set = FILTER_SETS - 1;
+    return cudaSuccess;
+  }
+  unsigned long long id = 0;  // unlike the handle, never given to another stream
+  GFD_CK(cudaStreamGetId(s, &id));
+  for (int i = 0; i < c->aux_owners; ++i)
+    if (c->aux_owner[i] == id) {
+      *set = i;
+      return cudaSuccess;
+    }
+  if (c->aux_owners < AUX_SLOTS) {
+    *set = c->aux_owners++;
+    c->aux_owner[*set] = id;
+    return cudaSuccess;
+  }
+  cudaEvent_t& ev = c->aux_done[c->aux_turn];
+  if (!ev) GFD_CK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+  GFD_CK(cudaStreamWaitEvent(s, ev, 0));
+  *set = AUX_SLOTS + c->aux_turn;
+  *done = ev;
+  c->aux_turn = (c->aux_turn + 1) % AUX_SLOTS;
+  return cudaSuccess;
+}
+
 // Marks the end of a solve for a later one on another stream (a launch that the
 // caller captures into a graph of its own is left alone, as before).
 cudaError_t record_done(gfdeconv_ctx* c, cudaStream_t s) {
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)
-    return cudaSuccess;
-  return cudaEventRecord(c->ev_done, s);
+  return capturing(s) ? cudaSuccess : cudaEventRecord(c->ev_done, s);
 }
 
 int solve_batched_dev(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs, int iters,
@@ -666,8 +706,7 @@ int solve_batched_dev(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs, int it
     // of a stream): the graph stays, only the descriptors are sent, in stream
     // order behind the last solve.  Not while the caller captures the stream:
     // the copy's source is this call's.
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
+    if (!capturing(s)) {
       Plan& pl = c->plan;
       for (int i = 0; i < n; ++i) {
         fill_desc(c, imgs[pl.order[i]], pl.h_imgs[i]);
@@ -875,10 +914,10 @@ int gfdeconv_create(gfdeconv_ctx** out, int cuda_device, const gfdeconv_opts* op
       (e = cudaMalloc(&c->d2, sizeof(float) * TAB_ENTRIES)) != cudaSuccess ||
       (e = cudaMemcpy(c->tw, tw.data(), sizeof(float2) * TAB_ENTRIES, cudaMemcpyHostToDevice)) != cudaSuccess ||
       (e = cudaMemcpy(c->d2, d2.data(), sizeof(float) * TAB_ENTRIES, cudaMemcpyHostToDevice)) != cudaSuccess ||
-      (e = cudaMalloc(&c->aux_st, AUX_SLOTS * sizeof(ImgState))) != cudaSuccess ||
-      (e = cudaMemset(c->aux_st, 0, AUX_SLOTS * sizeof(ImgState))) != cudaSuccess ||
-      (e = cudaMalloc(&c->aux_max, AUX_SLOTS * ABSMAX_SCRATCH * sizeof(unsigned int))) != cudaSuccess ||
-      (e = cudaMemset(c->aux_max, 0, AUX_SLOTS * ABSMAX_SCRATCH * sizeof(unsigned int))) != cudaSuccess ||
+      (e = cudaMalloc(&c->aux_st, FILTER_SETS * sizeof(ImgState))) != cudaSuccess ||
+      (e = cudaMemset(c->aux_st, 0, FILTER_SETS * sizeof(ImgState))) != cudaSuccess ||
+      (e = cudaMalloc(&c->aux_max, FILTER_SETS * ABSMAX_SCRATCH * sizeof(unsigned int))) != cudaSuccess ||
+      (e = cudaMemset(c->aux_max, 0, FILTER_SETS * ABSMAX_SCRATCH * sizeof(unsigned int))) != cudaSuccess ||
       (e = cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking)) != cudaSuccess ||
       (e = cudaEventCreateWithFlags(&c->ev_done, cudaEventDisableTiming)) != cudaSuccess ||
       (e = cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming)) != cudaSuccess) {
@@ -926,6 +965,8 @@ void gfdeconv_destroy(gfdeconv_ctx* c) {
   }
   if (c->ev_fork) cudaEventDestroy(c->ev_fork);
   if (c->ev_done) cudaEventDestroy(c->ev_done);
+  for (cudaEvent_t ev : c->aux_done)
+    if (ev) cudaEventDestroy(ev);
   delete c;
 }
 
@@ -1596,19 +1637,25 @@ int gfdeconv_guidfilter(gfdeconv_ctx* c, const float* I, const float* p, int M, 
   d.u = u_out;
   d.w = w;
   d.eps = eps;
-  const int turn = c->aux_turn;
-  c->aux_turn = (turn + 1) % AUX_SLOTS;
   ClassLaunch cl{};
   cl.cd = ClassDesc{M, N, 1, 0, N / 2};
   cl.one = &d;
-  cl.st = c->aux_st + turn;
+  cl.st = c->aux_st;
   cl.max_rad = (w - 1) / 2;
   cl.n_rad_groups = 1;
   cl.rad_groups[0] = RadGroup{0, 1, (w - 1) / 2};
-  if (c->opts.var_precision == GFD_VAR_COMPENSATED) {  // the split sums' bound
-    if ((e = launch_plane_absmax(cl, c->aux_max + turn * ABSMAX_SCRATCH, s)) != cudaSuccess) return map_err(e);
-  }
-  return map_err(launch_guided_filter(cl, -1, c->opts.var_precision, c->opts.boundary, s));
+  if (c->opts.var_precision != GFD_VAR_COMPENSATED)
+    return map_err(launch_guided_filter(cl, -1, c->opts.var_precision, c->opts.boundary, s));
+  // the split sums' bound needs a set of state and scratch
+  int set = 0;
+  cudaEvent_t done = nullptr;
+  if ((e = filter_set(c, s, &set, &done)) != cudaSuccess) return map_err(e);
+  cl.st = c->aux_st + set;
+  e = launch_plane_absmax(cl, c->aux_max + set * ABSMAX_SCRATCH, s);
+  if (e == cudaSuccess)
+    e = launch_guided_filter(cl, -1, c->opts.var_precision, c->opts.boundary, s);
+  if (e == cudaSuccess && done) e = cudaEventRecord(done, s);
+  return map_err(e);
 }
 
 int gfdeconv_pad_symmetric(gfdeconv_ctx* c, const float* y, int m, int n, float* y_canvas, int M,
