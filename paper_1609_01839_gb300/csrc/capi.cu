@@ -1711,7 +1711,7 @@ int gfdeconv_fft2_r2c(gfdeconv_ctx* c, const float* x, int M, int N, float* X, v
   ClassLaunch cl{};
   cl.cd = ClassDesc{M, N, 1, 0, N / 2};
   cl.one = &d;
-  cl.st = c->aux_st;
+  cl.st = nullptr;  // the plain passes keep no per-image state
   const Tables t{c->tw, c->d2, c->twdf};
   if ((e = launch_row_r2c(cl, t, SEL_U, SEL_S, false, s)) != cudaSuccess) return map_err(e);
   if ((e = launch_col_plain(cl, t, SEL_S, SEL_YS, false, s)) != cudaSuccess) return map_err(e);
@@ -1735,7 +1735,7 @@ int gfdeconv_fft2_c2r(gfdeconv_ctx* c, const float* X, int M, int N, float* x, v
   ClassLaunch cl{};
   cl.cd = ClassDesc{M, N, 1, 0, N / 2};
   cl.one = &d;
-  cl.st = c->aux_st;
+  cl.st = nullptr;  // the plain passes keep no per-image state
   const Tables t{c->tw, c->d2, c->twdf};
   if ((e = launch_col_plain(cl, t, SEL_QP, SEL_QI, true, s)) != cudaSuccess) return map_err(e);
   if ((e = launch_row_c2r(cl, t, SEL_QI, -1, SEL_UI, -1, 1.0f / ((float)M * (float)N), s)) !=

@@ -57,3 +57,24 @@ def test_captured_by_the_caller():
             assert torch.equal(alone, c.guidfilter(I, p, 7, 1e-3))
             torch.cuda.synchronize()
             assert torch.equal(alone, out)
+
+
+def test_transform_beside_a_filter_call():
+    """The inverse transform leaves the filter's bound of |I|, |p| alone."""
+    I, p = planes(2, 512, 512)
+    big = 1e9 * torch.rand(64, 64, device=DEV)
+    other = torch.cuda.Stream()
+    with gfd.Context(0) as c:
+        alone = c.guidfilter(I, p, 5, 1e-3)
+        X, x, out = c.fft2_r2c(big), torch.empty_like(big), torch.empty_like(I)
+        torch.cuda.synchronize()
+
+        def inverse():  # into a buffer of its own: the other stream writes it
+            assert gfd.lib.gfdeconv_fft2_c2r(c._h, X.data_ptr(), 64, 64, x.data_ptr(),
+                                             other.cuda_stream) == 0
+        for _ in range(100):
+            inverse()
+            c.guidfilter(I, p, 5, 1e-3, out=out)
+            inverse()
+            assert torch.equal(alone, out)
+        torch.cuda.synchronize()
