@@ -699,7 +699,8 @@ int solve_batched_dev(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs, int it
   }
   c->plan.copies = nullptr;
   std::vector<int> shape;
-  bool same = c->have_plan && c->plan.key == key;
+  // (a plan that gfdeconv_solve_batched_timed made has no graph yet)
+  bool same = c->have_plan && c->plan.key == key && (c->plan.exec || !c->opts.use_graphs);
   if (!same && !hc && c->opts.use_graphs) shape = plan_shape(n, imgs, iters);
   if (!same && !shape.empty() && c->have_plan && c->plan.exec && c->plan.shape == shape) {
     // Other buffers or parameters in a solve of the same shape (the next image
