@@ -91,8 +91,12 @@ typedef struct {
   double rho;
   /* 1 (default): capture each solve as a CUDA graph and replay it for the
    * next one of the same canvas sizes, windows and iterations (in that order;
-   * pointers, PSFs, sigma and eps may differ).  Solves that ask for u_I or u_p,
-   * and solves from host buffers, replay for the same pointers only. */
+   * pointers, PSFs, sigma and eps may differ), in stream order behind the last
+   * solve, whichever stream that ran on.  Solves that ask for u_I or u_p,
+   * and solves from host buffers, replay for the same pointers only.  0: direct
+   * launches, which a caller can capture into a graph of its own (that graph uses
+   * the context's workspace and descriptors: run it only while no other solve of
+   * the context does, and not after one of other buffers). */
   int use_graphs;
   /* Spectral passes of Eq. 11 launched per iteration after the one fused
    * into the forward transform (images whose root is resolved skip them) in

@@ -149,6 +149,7 @@ struct gfdeconv_ctx {
   Plan plan;
   bool have_plan = false;
   cudaStream_t last_stream = nullptr;
+  unsigned long long last_id = 0;  // its id: a handle may be given to another stream later
   long long last_launches = 0;
   // Per-image state and launch_plane_absmax's scratch of the filter calls, FILTER_SETS
   // of each.  The first AUX_SLOTS streams that make such calls have one each
@@ -666,10 +667,14 @@ cudaError_t filter_set(gfdeconv_ctx* c, cudaStream_t s, int* set, cudaEvent_t* d
   return cudaSuccess;
 }
 
-// Marks the end of a solve for a later one on another stream (a launch that the
-// caller captures into a graph of its own is left alone, as before).
-cudaError_t record_done(gfdeconv_ctx* c, cudaStream_t s) {
-  return capturing(s) ? cudaSuccess : cudaEventRecord(c->ev_done, s);
+// Puts stream s behind the context's last solve, which may have run on another
+// stream (workspace and descriptors are shared).
+cudaError_t after_last_solve(gfdeconv_ctx* c, cudaStream_t s) {
+  unsigned long long id = 0;
+  GFD_CK(cudaStreamGetId(s, &id));
+  if (id != c->last_id) GFD_CK(cudaStreamWaitEvent(s, c->ev_done, 0));
+  c->last_id = id;
+  return cudaSuccess;
 }
 
 int solve_batched_dev(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs, int iters,
@@ -698,6 +703,13 @@ int solve_batched_dev(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs, int it
     for (const auto& v : hc->out) put(v);
   }
   c->plan.copies = nullptr;
+  // (a solve that the caller captures, possible without graphs of the library's
+  // own, has no place in the order of the others)
+  const bool cap = capturing(s);
+  if (!cap) {
+    const cudaError_t e = after_last_solve(c, s);
+    if (e != cudaSuccess) return map_err(e);
+  }
   std::vector<int> shape;
   // (a plan that gfdeconv_solve_batched_timed made has no graph yet)
   bool same = c->have_plan && c->plan.key == key && (c->plan.exec || !c->opts.use_graphs);
@@ -705,19 +717,15 @@ int solve_batched_dev(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs, int it
   if (!same && !shape.empty() && c->have_plan && c->plan.exec && c->plan.shape == shape) {
     // Other buffers or parameters in a solve of the same shape (the next image
     // of a stream): the graph stays, only the descriptors are sent, in stream
-    // order behind the last solve.  Not while the caller captures the stream:
-    // the copy's source is this call's.
-    if (!capturing(s)) {
+    // order behind the last solve.
+    if (!cap) {
       Plan& pl = c->plan;
       for (int i = 0; i < n; ++i) {
         fill_desc(c, imgs[pl.order[i]], pl.h_imgs[i]);
         pl.user[i] = imgs[pl.order[i]];
       }
-      cudaError_t e = cudaSuccess;
-      if (s != c->last_stream) e = cudaStreamWaitEvent(s, c->ev_done, 0);
-      if (e == cudaSuccess)
-        e = cudaMemcpyAsync(c->d_imgs, pl.h_imgs.data(), sizeof(ImgDesc) * n, cudaMemcpyHostToDevice,
-                            s);
+      const cudaError_t e = cudaMemcpyAsync(c->d_imgs, pl.h_imgs.data(), sizeof(ImgDesc) * n,
+                                            cudaMemcpyHostToDevice, s);
       if (e != cudaSuccess) {
         drop_plan(c);
         return map_err(e);
@@ -752,12 +760,12 @@ int solve_batched_dev(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs, int it
   cudaError_t e;
   if (c->opts.use_graphs) {
     e = cudaGraphLaunch(c->plan.exec, s);
-    if (e == cudaSuccess && !c->plan.shape.empty()) e = record_done(c, s);
   } else {
     c->plan.copies = hc;
     e = record(c, c->plan, s);
     c->plan.copies = nullptr;
   }
+  if (e == cudaSuccess && !cap) e = cudaEventRecord(c->ev_done, s);
   c->last_stream = s;
   c->last_launches = c->plan.launches;
   return map_err(e);
@@ -1166,7 +1174,9 @@ int gfdeconv_solve_batched_timed(gfdeconv_ctx* c, int n, const gfdeconv_image* i
     c->have_plan = true;
   }
   Timer tm;
-  cudaError_t e = record(c, c->plan, s, &tm);
+  cudaError_t e = after_last_solve(c, s);
+  if (e == cudaSuccess) e = record(c, c->plan, s, &tm);
+  if (e == cudaSuccess) e = cudaEventRecord(c->ev_done, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return map_err(e);
   for (size_t i = 0; i < tm.used; ++i) {
