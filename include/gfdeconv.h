@@ -98,11 +98,10 @@ typedef struct {
    * the context's workspace and descriptors: run it only while no other solve of
    * the context does, and not after one of other buffers). */
   int use_graphs;
-  /* Spectral passes of Eq. 11 launched per iteration after the one fused
-   * into the forward transform (images whose root is resolved skip them) in
-   * iterations 0-2, whose brackets are wide; later iterations, whose bracket
-   * is centred on the extrapolated root, launch at most 2.  <= 0 selects 4,
-   * at most 16.  If an image's root is still bracketed after the last pass of
+  /* Spectral passes of Eq. 11 per iteration after the one fused into the
+   * forward transform (images whose root is resolved skip them).  <= 0 selects
+   * 4, at most 16; from the fourth iteration on at most 4 are taken, which
+   * resolve any root.  If an image's root is still bracketed after the last pass of
    * an iteration, GFD_STATUS_PASSES_EXHAUSTED is set. */
   int lambda_max_passes;
   /* Relative width of the final lambda bracket (the root search stops below

@@ -23,8 +23,11 @@ namespace {
 
 constexpr int AUX_SLOTS = 8;
 constexpr int FILTER_SETS = 2 * AUX_SLOTS + 1;
-// Fallback lambda passes launched per iteration from the fourth iteration on.
-constexpr int LATE_LAMBDA_PASSES = 2;
+// Most fallback lambda passes of an iteration from the fourth on.  Four resolve
+// any root: the bracket that a missed expansion leaves, the whole range beside
+// it, one of the range's 11 intervals (a ratio of up to 1e4), one of the
+// interval's (interpolated).
+constexpr int LATE_LAMBDA_PASSES = 4;
 constexpr int CHAINS = GFD_CHAINS;
 // A host <-> device copy that the host entry point asks a solve to issue.
 struct HostCopy {
@@ -304,6 +307,7 @@ void fill_desc(const gfdeconv_ctx* c, const gfdeconv_image& im, ImgDesc& d) {
   d.kh = im.kh;
   d.kw = im.kw;
   d.w = im.w;
+  d.max_pass = c->opts.lambda_max_passes;
   d.sigma = im.sigma;
   d.eps = im.eps;
   d.rho_fixed = c->opts.rho;
@@ -456,10 +460,11 @@ cudaError_t build_plan(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs, int i
     if (tm) GFD_CK(tm->end(s));                          \
   } while (0)
 
-// Classes whose fallback passes of iteration k run as one launch: small
+// Classes whose fallback passes of iteration k all run as one launch: small
 // canvases.  A pass over a canvas of 1024 x 1024 takes 8 blocks three times as
 // long as the ordinary pass, so there only the later iterations do, where most
-// images need none.
+// images need none.  On larger ones the later iterations' first pass is an ordinary
+// one and the others, hardly ever needed, are one launch.
 bool lambda_loop(const ClassLaunch& cl, int k) {
   return cl.cd.M * cl.cd.N <= (k < 3 ? 1 : 4) * LAMBDA_LOOP_PIXELS;
 }
@@ -526,7 +531,7 @@ cudaError_t record(gfdeconv_ctx* c, Plan& pl, cudaStream_t s, Timer* tm = nullpt
         L += 2;
       }
       // iterations 0-2 start from wide brackets; later ones from the
-      // extrapolated root, which the fused pass almost always resolves
+      // extrapolated root, which the fused pass mostly resolves
       const int npass = k < 3 ? passes : std::min(passes, LATE_LAMBDA_PASSES);
       for (auto& cl : classes)
         if (lambda_loop(cl, k)) {
@@ -536,9 +541,12 @@ cudaError_t record(gfdeconv_ctx* c, Plan& pl, cudaStream_t s, Timer* tm = nullpt
         }
       for (int p = 1; p <= npass; ++p)
         for (auto& cl : classes) {
-          if (lambda_loop(cl, k)) continue;
+          if (lambda_loop(cl, k) || (k >= 3 && p > 2)) continue;
           if (tm) tm->cur_cls = cl.class_id;
-          GFD_T(GFD_PHASE_LAMBDA_PASS, launch_lambda_pass(cl, k, p == npass, s));
+          if (k >= 3 && p == 2)
+            GFD_T(GFD_PHASE_LAMBDA_PASS, launch_lambda_loop(cl, k, npass - 1, s));
+          else
+            GFD_T(GFD_PHASE_LAMBDA_PASS, launch_lambda_pass(cl, k, p == npass, s));
           ++L;
         }
       for (auto& cl : classes) {

@@ -112,6 +112,7 @@ struct ImgState {
   unsigned int cta_done;   // items of the current spectral pass completed
   unsigned int gf_done;    // last-block-done counter (guided filter)
   int need;          // 1: lambda unresolved, a fallback pass must run
+  int max_pass;      // fallback passes that an iteration may take
   int status;        // ST_* bits
   int iter;          // iteration index of the pending outputs
   double rtol;       // relative width of lambda at which the root search stops
@@ -128,7 +129,8 @@ struct ImgDesc {
   double* lam_out;    // [iters] or null
   double* isnr_out;   // [iters] or null
   double* res_out;    // [iters] or null
-  int kh, kw, w, pad_;
+  int kh, kw, w;
+  int max_pass;       // fallback lambda passes that an iteration may take
   double sigma, eps, rho_fixed;
   double lam_rtol;    // relative width of lambda at which the root search stops
   // workspace planes (M*N/2 complex each)

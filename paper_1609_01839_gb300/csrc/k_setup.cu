@@ -153,6 +153,7 @@ __global__ void k_setup_init(ClassDesc cd, const ImgDesc* __restrict__ imgs, Img
   S->lam = NAN;
   S->need = 0;
   S->rtol = d.lam_rtol;
+  S->max_pass = d.max_pass;
   set_bracket(S, INITIAL_LO, INITIAL_HI);
 }
 

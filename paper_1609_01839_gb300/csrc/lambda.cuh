@@ -468,9 +468,11 @@ GFD_D void resolve_warp(ImgState* st, double lam, double prev, int iter, double*
 // tot[0..KMOM-1] are the sums N_k.  Every lane evaluates the series at a trial
 // point of its own in FP32, three rounds; two Newton steps with the series
 // in FP64 follow.  Sets lam to the root and returns true if it is accepted;
-// otherwise leaves the bracket of the next pass in (lo, hi).
-GFD_D bool moment_root_warp(const double* tot, double scale, float c, int lane, double& lam,
-                            float& lo, float& hi) {
+// otherwise leaves the bracket of the next pass in (lo, hi): up to a point that
+// the series has certainly past the root; without one a ratio of 3.95, narrow
+// enough to be interpolated, or (wide) the whole range on the root's side.
+GFD_D bool moment_root_warp(const double* tot, double scale, float c, float lam_up, bool wide,
+                            int lane, double& lam, float& lo, float& hi) {
   static_assert(KMOM == 8, "the series is evaluated by halves of four terms");
   const int nl = upd_lanes();
   const unsigned int mask = upd_mask();
@@ -555,6 +557,12 @@ GFD_D bool moment_root_warp(const double* tot, double scale, float c, int lane, 
   const float near = 0.99f * rb, far = past > 0.0f ? 1.01f * rp : 3.95f * near;
   lo = up ? c * near : c / far;
   hi = up ? c * far : c / near;
+  if (wide && past == 0.0f) {
+    if (up)
+      hi = fmaxf(lam_up, hi);
+    else
+      lo = (float)LAMBDA_LO;
+  }
   return false;
 }
 
@@ -568,7 +576,7 @@ __device__ __noinline__ static void lambda_update_warp(ImgState* st, const doubl
                               int lane) {
   // the state's fields are requested together: they come from L2, one trip
   const double invP = st->invP, T = st->T, invT = st->invT, prev = st->lam_prev;
-  const int mode = st->mode;
+  const int mode = st->mode, max_pass = st->max_pass;
   const float amax = (float)st->amax, node = lane < KNODES ? st->node[lane] : 0.0f;
   const double resinf = tot[KNODES] * invP;
   if (primary) {
@@ -600,7 +608,10 @@ __device__ __noinline__ static void lambda_update_warp(ImgState* st, const doubl
     }
     double lam;
     float lo, hi;
-    if (moment_root_warp(tot, invP * invT, c, lane, lam, lo, hi)) {
+    // lambda still jumps in iterations 3 and 4; two passes find a root far above
+    // c only if the first of them takes the whole range
+    const bool wide = max_pass == 2 && iter < 5;
+    if (moment_root_warp(tot, invP * invT, c, st->lam_up, wide, lane, lam, lo, hi)) {
       resolve_warp(st, lam, prev, iter, lam_out, lane);
       return;
     }

@@ -83,7 +83,7 @@ cudaError_t launch_col_fwd_lambda(const ClassLaunch& c, const Tables& t, int ite
 // Fallback lambda pass over the stored spectrum (exits early where resolved).
 cudaError_t launch_lambda_pass(const ClassLaunch& c, int iter, bool last_chance,
                                cudaStream_t s);
-// All fallback passes of an iteration (at most npass) in one launch, a cluster
+// Fallback passes of an iteration, the last npass of them, in one launch, a cluster
 // of blocks per image.
 constexpr int LAMBDA_LOOP_PIXELS = 512 * 512;
 cudaError_t launch_lambda_loop(const ClassLaunch& c, int iter, int npass, cudaStream_t s);
