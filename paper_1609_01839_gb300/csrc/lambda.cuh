@@ -630,8 +630,10 @@ __device__ __noinline__ static void lambda_update_warp(ImgState* st, const doubl
   const float hi = __shfl_sync(upd_mask(), xm, nk - 1);
   // a missed first bracket whose root is expected close to it
   const bool near = primary && iter == 2 && mode == MODE_CHEB;
-  // the second iteration's jump, past its first bracket: seldom far past it
-  const bool jump = primary && iter == 1;
+  // the second iteration's jump, past its first bracket: seldom far past it.  A
+  // root that is takes one pass more than from the whole range, four in all
+  // whatever it is: with fewer to go the whole range comes at once.
+  const bool jump = primary && iter == 1 && max_pass >= 4;
   bool open = true;
   if (!(g0 <= 0.0f)) {  // root below the bracket (or NaN)
     if (!isfinite(g0)) {
