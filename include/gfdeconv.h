@@ -196,9 +196,12 @@ int gfdeconv_crop(gfdeconv_ctx* ctx, const float* u_canvas, int M, int N, float*
  * a_k = (Sigma_k + eps U)^-1 (mean(I p) - mu_k pbar_k) with Sigma_k the
  * window covariance of the 3 channels (Eq. 3 with a 3-vector slope),
  * b_k = pbar_k - a_k . mu_k (Eq. 4), u = abar . I + bbar (Eq. 5).  Window
- * statistics in exact split sums, the 3 x 3 solves in double-float; periodic or
- * truncated windows as gfdeconv_opts.boundary selects (var_precision does not
- * apply). */
+ * statistics in exact split sums and the 3 x 3 solves in double-float where the
+ * values of a tile of 32 x 16 pixels and its surroundings suit that (within about
+ * [0, 1] for eps from 2e-5 on), in FP64 elsewhere (slower); a and b are kept in
+ * FP32.  A pixel that is not finite reaches the outputs within w - 1 pixels of it,
+ * whose windows hold it, and no others.  Periodic or truncated windows as
+ * gfdeconv_opts.boundary selects (var_precision does not apply). */
 int gfdeconv_guidfilter_color(gfdeconv_ctx* ctx, const float* I, const float* p, int M, int N,
                               int w, double eps, float* u_out, void* stream);
 
