@@ -121,6 +121,8 @@ struct SumIG {
   static constexpr int kSub = 1 << 30;
 };
 
+GFD_D bool is_finite(float v) { return fabsf(v) <= 3.402823466e38f; }  // false for NaN
+
 // The grids of one item: g and 1/g for (J, Q).
 struct IGGrid {
   float2 g, ig;
@@ -337,6 +339,19 @@ struct GfwCols {  // one accumulator per quantity and column
     const float q[4] = {x[0].y, x[1].y, x[2].y, x[3].y};
     col_update(V, j, q, sgn, G);
   }
+  // whether no column sum holds (or still holds, slid) a value that is not finite
+  GFD_D bool finite() const {
+    if constexpr (std::is_same<ACC, SumF64>::value) {
+      const double t = (V[2][0].v + V[2][1].v) + (V[2][2].v + V[2][3].v) + (V[3][0].v + V[3][1].v) +
+                       (V[3][2].v + V[3][3].v);
+      return t - t == 0.0;
+    } else if constexpr (std::is_same<ACC, SumDF>::value) {
+      return is_finite((V[2][0].lo + V[2][1].lo) + (V[2][2].lo + V[2][3].lo) +
+                       (V[3][0].lo + V[3][1].lo) + (V[3][2].lo + V[3][3].lo));
+    } else {
+      return true;  // re-formed every few rows
+    }
+  }
   template <class F>
   GFD_D void windows(const float (&n)[4], const float (&inv_n)[4], const IGGrid& G, F out) const {
     ACC S0[4], S1[4], S2[4], S3[4];
@@ -376,6 +391,10 @@ struct GfwCols<RAD, SumIG> {
       l01[k] = sgn > 0.0f ? cadd(l01[k], xl) : csub(l01[k], xl);
       l23[k] = __ffma2_rn(make_float2(sx, sx), xl, __ffma2_rn(make_float2(sl, sl), xh, l23[k]));
     }
+  }
+  GFD_D bool finite() const {
+    const float2 t = cadd(cadd(l23[0], l23[1]), cadd(l23[2], l23[3]));
+    return is_finite(t.x + t.y);
   }
   template <class F>
   GFD_D void windows(const float (&n)[4], const float (&inv_n)[4], const IGGrid& G, F out) const {
@@ -467,6 +486,8 @@ GFD_D void gfw_items(const ClassDesc& cd, const ImgDesc* __restrict__ imgs, ImgS
       const size_t c = (size_t)((y0 + H / 2) & (M - 1)) * N + ((x0 + WOUT / 2) & (N - 1));
       cI = __ldg(&I[c]);
       cP = __ldg(&P[c]);
+      if (!is_finite(cI)) cI = 0.0f;
+      if (!is_finite(cP)) cP = 0.0f;
     }
     const float eps = (float)d.eps;
     IGGrid G{};
@@ -543,7 +564,15 @@ GFD_D void gfw_items(const ClassDesc& cd, const ImgDesc* __restrict__ imgs, ImgS
         asm volatile("prefetch.global.L2 [%0];" ::"l"(I + off));
         asm volatile("prefetch.global.L2 [%0];" ::"l"(P + off));
       }
-      if (s % ACC::kSub == 0) {
+      bool direct = s % ACC::kSub == 0;
+      if (!direct) {
+        V.update(x, 1.0f, G);
+        V.update(old, -1.0f, G);
+        // A pixel that is not finite cannot be taken away again.  (Only planes of
+        // the caller's own can have one here and there.)
+        if (iter < 0 && !V.finite()) direct = true;
+      }
+      if (direct) {
         V.clear();
         int slot = s_cur;
 #pragma unroll(ACC::kSub < 1000 ? WIN : 1)
@@ -553,9 +582,6 @@ GFD_D void gfw_items(const ClassDesc& cd, const ImgDesc* __restrict__ imgs, ImgS
           V.update(y, 1.0f, G);
           slot = slot + 1 == RI ? 0 : slot + 1;
         }
-      } else {
-        V.update(x, 1.0f, G);
-        V.update(old, -1.0f, G);
       }
       ring_row(s_cur, old);
       // 2. row window sums -> a_k (Eq. 3), b_k (Eq. 4)

@@ -1,0 +1,63 @@
+"""A pixel that is not finite in a call of the guided filter: outputs more than w + 5
+pixels away (2 r = w - 1 by the windows, up to 3 more along a row and 3 down a
+column in either stage, where sums of a lane's four columns and of four rows are
+slid) are those of a finite pixel in its place.  Tolerance 1e-5 of the values' size: an
+infinite pixel takes the bound that the split sums' grid rests on, so that they
+fall back to plain FP32 sums (2^-24 times some tens of additions, over eps +
+variance of order 0.1)."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():  # pragma: no cover
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+import paper_1609_01839_gb300 as gfd  # noqa: E402
+
+DEV = torch.device("cuda:0")
+
+
+@pytest.mark.parametrize("mode", [gfd.VAR_COMPENSATED, gfd.VAR_FP64, gfd.VAR_DOUBLE_FLOAT])
+@pytest.mark.parametrize("value", [np.nan, np.inf])
+@pytest.mark.parametrize("plane", [0, 1])
+def test_stays_where_it_is(mode, value, plane):
+    M, N, w = 1024, 2048, 5
+    g = torch.Generator(device=DEV)
+    g.manual_seed(9)
+    planes = [torch.rand(M, N, generator=g, device=DEV) for _ in range(2)]
+    ii, jj = torch.arange(M, device=DEV)[:, None], torch.arange(N, device=DEV)[None, :]
+    with gfd.Context(0, var_precision=mode) as c:
+        want = c.guidfilter(*planes, w, 0.1)
+        far = torch.ones(M, N, dtype=torch.bool, device=DEV)
+        bad = [x.clone() for x in planes]
+        for y in range(0, M, 97):  # every row of an item, centres of items among them
+            for x in (y % 128, 60 + y, 1500 + y // 8):
+                bad[plane][y, x % N] = value
+                dy, dx = (ii - y).abs(), (jj - x % N).abs()
+                far &= ~((torch.minimum(dy, M - dy) <= w + 5) & (torch.minimum(dx, N - dx) <= w + 5))
+        got = c.guidfilter(*bad, w, 0.1)
+    assert float(far.float().mean()) > 0.9
+    assert float((got - want).abs()[far].max()) < 1e-5  # (false for NaN)
+    assert not bool(torch.isfinite(got[~torch.isfinite(bad[plane])]).any())
+
+
+@pytest.mark.parametrize("mode", [gfd.VAR_COMPENSATED, gfd.VAR_FP64, gfd.VAR_DOUBLE_FLOAT])
+def test_at_every_place_of_an_item(mode):
+    """The centre of an item is its reference: no place may matter."""
+    M = N = 128
+    g = torch.Generator(device=DEV)
+    g.manual_seed(10)
+    I, p = (torch.rand(M, N, generator=g, device=DEV) for _ in range(2))
+    with gfd.Context(0, var_precision=mode) as c:
+        want = c.guidfilter(I, p, 3, 0.1)
+        for y in range(0, M, 5):
+            for x in (0, 1, 59, 60, 61, 62, 127):
+                J = I.clone()
+                J[y, x] = float("nan")
+                got = c.guidfilter(J, p, 3, 0.1)
+                dy = (torch.arange(M, device=DEV)[:, None] - y).abs()
+                dx = (torch.arange(N, device=DEV)[None, :] - x).abs()
+                far = ~((torch.minimum(dy, M - dy) <= 8) & (torch.minimum(dx, N - dx) <= 8))
+                assert float((got - want).abs()[far].max()) < 1e-5, (y, x)
