@@ -302,8 +302,8 @@ int gfdeconv_tune_read(const char* path, int* chains, int* n_classes, int* shape
                        int max_classes);
 
 /* Tile shapes the context uses for an M x N canvas (tuned or built-in) and
- * its chain count (an untuned solve of one canvas size of 2^26 pixels or more
- * runs as one chain, of several sizes as two); any output pointer may be NULL. */
+ * its chain count (untuned: 4, and 1 to 3 for solves of 2^24 pixels or more); any
+ * output pointer may be NULL. */
 int gfdeconv_tune_get(gfdeconv_ctx* ctx, int M, int N, int* col_threads, int* row_threads,
                       int* gf_rows, int* chains);
 

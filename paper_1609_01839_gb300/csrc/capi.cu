@@ -321,16 +321,36 @@ void drop_plan(gfdeconv_ctx* c) {
 }
 
 // Chains of an untuned solve.  Concurrent chains fill the tails of each other's
-// kernels; where a kernel runs for many waves they only cut its launches into
-// pieces.  Whole solves with 1, 2 and 4 chains: 4 images of 4096^2 58.4, 60.0,
-// 63.3 ms; 256 uneven images (107 Mpixel, three sizes) 40.0, 37.5, 38.6; 64
-// (27 Mpixel) 12.7, 11.3, 10.9.  (With host copies the chains also spread
-// the transfers: four there.)
+// kernels and overlap one's setup and lambda passes with another's transforms; each
+// chain more also cuts every launch into smaller pieces.  How much there is to fill goes
+// with the batch's pixels (waves per launch) and with the groups of one size and
+// window that have launches of their own.  ms with 1, 2, 3, 4 chains, 10 iterations
+// (*: 30), three windows in turn or, on the right, one:
+//   128 Mpixel   8 x 4096^2* 95.4 96.0 97.6 99.7   |  99.9 102.5 105.0 104.7
+//                128 x 1024^2 33.0 31.3 31.9 32.1  |  33.7 32.6 33.2 33.6
+//    64 Mpixel   4 x 4096^2*  50.0 47.6 48.8 49.8  |  51.5 52.1 52.0 54.4
+//                16 x 2048^2* 44.0 44.2 44.1 45.4  |  45.6 46.7 47.3 47.8
+//                64 x 1024^2  17.1 15.8 16.2 16.5  |  17.5 16.5 17.0 17.2
+//                256 x 512^2  17.8 16.5 16.7 16.9  |  18.1 16.8 17.2 17.2
+//                1024 x 256^2 23.3 20.1 19.9 20.1  |  23.6 21.0 20.8 20.7
+//    32 Mpixel   32 x 1024^2  9.25 8.40 8.44 8.70  |  9.23 8.46 8.83 9.15
+//                512 x 256^2  12.2 10.2 9.99 10.4  |  12.1 10.4 10.6 10.7
+//    24 Mpixel   64 uneven    9.03 8.15 7.63 8.01
+//    16 Mpixel   16 x 1024^2  5.31 4.67 4.61 4.80  |  5.05 4.65 4.78 4.98
+//     8 Mpixel   8 x 1024^2   3.19 2.84 2.64 2.61
+//     1 Mpixel   4 x 512^2    1.04 0.92 0.91 0.82
+// One chain wins only where all of a launch's many waves are of one kind and its images
+// large.  (With host copies the chains also spread the transfers: four there.)
 int default_chains(const std::vector<ClassLaunch>& classes) {
   long long px = 0;
-  for (const ClassLaunch& cl : classes) px += (long long)cl.cd.M * cl.cd.N * cl.cd.n_img;
-  if (px < (1LL << 26)) return CHAINS;
-  return classes.size() == 1 ? 1 : 2;
+  int groups = 0;
+  for (const ClassLaunch& cl : classes) {
+    px += (long long)cl.cd.M * cl.cd.N * cl.cd.n_img;
+    groups += cl.n_rad_groups;
+  }
+  if (px < (1LL << 24)) return CHAINS;
+  if (px < (1LL << 26)) return groups == 1 ? 2 : 3;
+  return groups == 1 && classes[0].cd.M * classes[0].cd.N >= (1 << 22) ? 1 : 2;
 }
 
 cudaError_t build_plan(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs, int iters,
