@@ -279,9 +279,11 @@ int gfdeconv_solve_batched_timed(gfdeconv_ctx* ctx, int n, const gfdeconv_image*
  * overwritten) on `stream` with event pairs around every launch, for each
  * candidate of one tile shape at a time:
  *   col_threads in {64, 128, 256}: threads per column-pass block, which fixes
- *     the tile width of the spectra (4096-row canvases always use 512);
+ *     the tile width of the spectra (canvases of 2048 rows and more and solves of
+ *     at most 2^20 pixels of a size have one width only);
  *   row_threads in {64, 128, 256}: threads per row-pass block (rows per item);
- *   gf_rows in {16, 32, 64}: output rows per guided-filter item;
+ *   gf_rows in {16, 32, 64, 128}: most output rows of a guided-filter item (launches
+ *     that they would leave few items for take fewer);
  * keeping per canvas size the fastest over the phases the shape affects, then
  * times graph replays of the solve with 1 to 4 concurrent chains.  The
  * result applies to the context's later solves and, if `path` is not NULL
@@ -302,8 +304,8 @@ int gfdeconv_tune_read(const char* path, int* chains, int* n_classes, int* shape
                        int max_classes);
 
 /* Tile shapes the context uses for an M x N canvas (tuned or built-in) and
- * its chain count (untuned: 4, and 1 to 3 for solves of 2^24 pixels or more); any
- * output pointer may be NULL. */
+ * its chain count (untuned: the last solve's, 4 before the first; it goes with the
+ * solve's pixels, sizes and windows); any output pointer may be NULL. */
 int gfdeconv_tune_get(gfdeconv_ctx* ctx, int M, int N, int* col_threads, int* row_threads,
                       int* gf_rows, int* chains);
 

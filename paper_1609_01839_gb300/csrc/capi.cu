@@ -806,7 +806,7 @@ int solve_batched_dev(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs, int it
 bool valid_tune(const ClassTune& t) {
   auto p2 = [](int v, int lo, int hi) { return v >= lo && v <= hi && (v & (v - 1)) == 0; };
   return p2(t.M, 8, 4096) && p2(t.N, 8, 4096) && p2(t.col_threads, 32, 256) &&
-         p2(t.row_threads, 32, 256) && p2(t.gf_rows, 16, 64);
+         p2(t.row_threads, 32, 256) && p2(t.gf_rows, 16, DEF_GF_ROWS);
 }
 
 bool load_tune(const char* path, TuneTable* out) {
@@ -1083,7 +1083,7 @@ int gfdeconv_autotune(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs, int it
         GFD_PHASE_ROW_INV}},
       {&ClassTune::row_threads, {64, 128, 256},
        {GFD_PHASE_ROW_FWD, GFD_PHASE_COL_FWD_LAMBDA, GFD_PHASE_ROW_INV}},
-      {&ClassTune::gf_rows, {16, 32, 64}, {GFD_PHASE_GUIDED_FILTER}}};
+      {&ClassTune::gf_rows, {16, 32, 64, 128}, {GFD_PHASE_GUIDED_FILTER}}};
   for (const Axis& ax : axes) {
     std::vector<double> best(sizes.size(), 1e300);
     std::vector<int> pick(sizes.size(), 0);
@@ -1108,7 +1108,9 @@ int gfdeconv_autotune(gfdeconv_ctx* c, int n, const gfdeconv_image* imgs, int it
     }
     for (size_t ci = 0; ci < sizes.size(); ++ci) {
       ClassTune t = cur.get(sizes[ci].first, sizes[ci].second);
-      t.*(ax.field) = pick[ci];
+      // the short column passes have a tile width of their own: nothing to choose
+      const bool fixed = ax.field == &ClassTune::col_threads && c->plan.classes[ci].short_cols;
+      t.*(ax.field) = fixed ? saved.get(t.M, t.N).col_threads : pick[ci];
       cur.set(t);
     }
   }
@@ -1174,7 +1176,8 @@ int gfdeconv_tune_get(gfdeconv_ctx* c, int M, int N, int* col_threads, int* row_
   if (col_threads) *col_threads = t.col_threads;
   if (row_threads) *row_threads = t.row_threads;
   if (gf_rows) *gf_rows = t.gf_rows;
-  if (chains) *chains = c->tune.chains;
+  // untuned, the count goes with the solve: the last one's
+  if (chains) *chains = c->tune.tuned_chains || !c->have_plan ? c->tune.chains : c->plan.nparts;
   return GFD_OK;
 }
 

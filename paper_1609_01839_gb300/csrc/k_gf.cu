@@ -899,8 +899,8 @@ cudaError_t launch_guided_filter(const ClassLaunch& c, int iter, int var_mode, i
     const int div = c.grid_div > 1 ? c.grid_div : 1;
     const int blocks = (per_sm * gf_sm_count() + div - 1) / div;
     const int strips = (cd.N + gfw_wout(rg.rad) - 1) / gfw_wout(rg.rad);
-    // the default leaves the choice to the rule; a tuned shape bounds it
-    const int hmax = c.gf_rows > 0 && c.gf_rows != DEF_GF_ROWS ? c.gf_rows : 2 * DEF_GF_ROWS;
+    // the tile shape bounds the rule's choice
+    const int hmax = c.gf_rows > 0 ? c.gf_rows : DEF_GF_ROWS;
     const int H = gfw_rows(cd.M, hmax, rg.rad, cd.n_img, strips, blocks * W,
                            (4 * gf_sm_count() + div - 1) / div);
     const int n_items = cd.n_img * strips * ((cd.M + H - 1) / H);

@@ -24,7 +24,7 @@ enum PlaneSel : int {
 // tile width; rows per guided-filter item), chosen by gfdeconv_autotune.
 constexpr int DEF_ROW_THREADS = 256;
 constexpr int DEF_COL_THREADS = 256;
-constexpr int DEF_GF_ROWS = 64;
+constexpr int DEF_GF_ROWS = 128;
 
 // Most pixels of a class (all its images) that take the short column passes.
 constexpr long long SHORT_PIXELS = 1 << 20;
@@ -51,7 +51,7 @@ struct ClassLaunch {
   RadGroup rad_groups[9];
   int grid_div;         // persistent grids use 1/grid_div of the resident slots (0 = 1)
   int row_threads;      // threads per row-pass block (0 = DEF_ROW_THREADS)
-  int gf_rows;          // largest rows per guided-filter item (0 = DEF_GF_ROWS)
+  int gf_rows;          // most rows of a guided-filter item (0 = DEF_GF_ROWS)
   int class_id;         // index of the class in its plan (instrumentation)
   bool short_cols;      // small problem: the short column passes (and their tile width)
 };
