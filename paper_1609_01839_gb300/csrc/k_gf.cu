@@ -753,9 +753,9 @@ k_plane_absmax(const float* __restrict__ I, const float* __restrict__ p, int P4,
   __shared__ bool s_last;
   const float4* I4 = reinterpret_cast<const float4*>(I);
   const float4* p4 = reinterpret_cast<const float4*>(p);
-  auto top = [](float m, float4 v) {
-    return fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
-  };
+  // (values that are not finite have no part in it: fmaxf passes over NaN)
+  auto top1 = [](float m, float v) { return is_finite(v) ? fmaxf(m, fabsf(v)) : m; };
+  auto top = [&](float m, float4 v) { return top1(top1(top1(top1(m, v.x), v.y), v.z), v.w); };
   float mi = 0.0f, mp = 0.0f;
   const int step = gridDim.x * blockDim.x;
   int i = blockIdx.x * blockDim.x + threadIdx.x;

@@ -1,9 +1,8 @@
 """A pixel that is not finite in a call of the guided filter: outputs more than w + 5
 pixels away (2 r = w - 1 by the windows, up to 3 more along a row and 3 down a
 column in either stage, where sums of a lane's four columns and of four rows are
-slid) are those of a finite pixel in its place.  Tolerance 1e-5 of the values' size: an
-infinite pixel takes the bound that the split sums' grid rests on, so that they
-fall back to plain FP32 sums (2^-24 times some tens of additions, over eps +
+slid) are those of a finite pixel in its place.  Tolerance 1e-5 of the values' size: what
+plain FP32 sums would reach (2^-24 times some tens of additions, over eps +
 variance of order 0.1)."""
 import numpy as np
 import pytest
@@ -61,3 +60,29 @@ def test_at_every_place_of_an_item(mode):
                 dx = (torch.arange(N, device=DEV)[None, :] - x).abs()
                 far = ~((torch.minimum(dy, M - dy) <= 8) & (torch.minimum(dx, N - dx) <= 8))
                 assert float((got - want).abs()[far].max()) < 1e-5, (y, x)
+
+
+@pytest.mark.parametrize("boundary", [gfd.BOUNDARY_PERIODIC, gfd.BOUNDARY_TRUNCATED])
+def test_infinite_pixels_leave_the_grid(boundary):
+    """The grid of the split sums rests on the finite pixels: away from infinite ones
+    the sums are as good as without them.  Nearly flat planes much smaller than one, eps
+    far below what plain FP32 sums of the deviations resolve; measured against FP64
+    sums, with room for the sums that are formed again from the ring of rows."""
+    M, N, w = 256, 512, 9
+    g = torch.Generator(device=DEV)
+    g.manual_seed(12)
+    ramp = torch.linspace(0.0, 0.1, M, device=DEV)[:, None] * torch.ones(M, N, device=DEV)
+    I, p = (ramp + 1e-3 * torch.rand(M, N, generator=g, device=DEV) for _ in range(2))
+    J, q = I.clone(), p.clone()
+    J[100, 200], q[180, 400] = float("inf"), float("-inf")
+    dy = torch.arange(M, device=DEV)[:, None]
+    dx = torch.arange(N, device=DEV)[None, :]
+    far = torch.ones(M, N, dtype=torch.bool, device=DEV)
+    for y, x in ((100, 200), (180, 400)):
+        far &= ((dy - y).abs() > w + 5) | ((dx - x).abs() > w + 5)
+    with gfd.Context(0, var_precision=gfd.VAR_FP64, boundary=boundary) as c:
+        want = c.guidfilter(I, p, w, 1e-7)
+    with gfd.Context(0, boundary=boundary) as c:
+        alone = (c.guidfilter(I, p, w, 1e-7) - want).abs()[far].max()
+        beside = (c.guidfilter(J, q, w, 1e-7) - want).abs()[far].max()
+    assert float(beside) <= 4 * float(alone)
