@@ -1305,10 +1305,13 @@ static void cfg_col_width(cudaError_t& e) {
   if (e == cudaSuccess) e = allow_smem(k_col_fwd_lambda<M, BT>);
   if (e == cudaSuccess) e = allow_smem(k_col_solve_inv<M, BT>);
 }
+// Each width that GFD_COL_WIDTHS has for M once: 4096 / M (16 at most), halved down
+// to 2; one kernel for all widths below 256 rows.
 template <int M>
 static cudaError_t cfg_col_fused() {
   cudaError_t e = cudaSuccess;
-  for (int B = 2; B <= 16; B *= 2) GFD_COL_WIDTHS(cfg_col_width, M, B, e);
+  constexpr int top = M >= 2048 || M < 256 ? 2 : 4096 / M;
+  for (int B = 2; B <= top; B *= 2) GFD_COL_WIDTHS(cfg_col_width, M, B, e);
   return e;
 }
 
