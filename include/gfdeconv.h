@@ -176,7 +176,9 @@ int gfdeconv_solve_batched_host(gfdeconv_ctx* ctx, int n, const gfdeconv_image* 
 /* u = guidfilter(I, p, w, eps) (Sec. 2, Eq. 3-5) with periodic windows:
  * I guidance, p filtering input, all M*N device buffers.  A pixel that is not
  * finite makes its own output and may make those within w + 5 pixels not finite
- * (periodic windows; GFD_VAR_FP32 sums too); outputs further away keep their values. */
+ * (periodic windows; GFD_VAR_FP32 sums too); outputs further away keep their values.
+ * Calls may be in flight on any number of streams; of the calls that the caller
+ * captures into graphs of its own, up to eight at a time (in the order of capture). */
 int gfdeconv_guidfilter(gfdeconv_ctx* ctx, const float* I, const float* p, int M, int N,
                         int w, double eps, float* u_out, void* stream);
 

@@ -22,7 +22,7 @@ using namespace gfd;
 namespace {
 
 constexpr int AUX_SLOTS = 8;
-constexpr int FILTER_SETS = 2 * AUX_SLOTS + 1;
+constexpr int FILTER_SETS = 3 * AUX_SLOTS;
 // Most fallback lambda passes of an iteration from the fourth on.  Four resolve
 // any root: the bracket that a missed expansion leaves, the whole range beside
 // it, one of the range's 11 intervals (a ratio of up to 1e4), one of the
@@ -158,13 +158,13 @@ struct gfdeconv_ctx {
   // of each.  The first AUX_SLOTS streams that make such calls have one each
   // (stream order is all they need); calls on any other stream take the next
   // AUX_SLOTS in turn, each behind the set's last call by its event; calls that
-  // a caller captures share the last.
+  // a caller captures take the last AUX_SLOTS in turn (nothing orders the replays).
   ImgState* aux_st = nullptr;
   unsigned int* aux_max = nullptr;
   unsigned long long aux_owner[AUX_SLOTS] = {};  // stream ids
   int aux_owners = 0;
   cudaEvent_t aux_done[AUX_SLOTS] = {};
-  int aux_turn = 0;
+  int aux_turn = 0, aux_cap_turn = 0;
   AuxSlot aux[AUX_SLOTS];
   int aux_next = 0;
   char* stage = nullptr;
@@ -671,7 +671,8 @@ bool capturing(cudaStream_t s) {
 cudaError_t filter_set(gfdeconv_ctx* c, cudaStream_t s, int* set, cudaEvent_t* done) {
   *done = nullptr;
   if (capturing(s)) {
-    *set = FILTER_SETS - 1;
+    *set = 2 * AUX_SLOTS + c->aux_cap_turn;
+    c->aux_cap_turn = (c->aux_cap_turn + 1) % AUX_SLOTS;
     return cudaSuccess;
   }
   unsigned long long id = 0;  // unlike the handle, never given to another stream

@@ -78,3 +78,35 @@ def test_transform_beside_a_filter_call():
             inverse()
             assert torch.equal(alone, out)
         torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("branches", [1, 2])
+def test_captured_calls_at_once(branches):
+    """Graphs of the caller's with a filter call in each branch, replayed on streams
+    of their own: up to eight captured calls of a context may be in flight."""
+    inputs = [planes(i, *((1024, 2048), (512, 512))[i % 2]) for i in range(8)]
+    streams = [torch.cuda.Stream() for _ in range(8 // branches)]
+    with gfd.Context(0) as c:
+        alone = [c.guidfilter(I, p, 5, 1e-3) for I, p in inputs]
+        outs = [torch.empty_like(I) for I, _ in inputs]
+        torch.cuda.synchronize()
+        graphs = []
+        for q in range(len(streams)):
+            g, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+            with torch.cuda.graph(g):
+                main = torch.cuda.current_stream()
+                side.wait_stream(main)
+                for k, s in zip(range(branches), (main, side)):
+                    i = q * branches + k
+                    c.guidfilter(*inputs[i], 5, 1e-3, stream=s, out=outs[i])
+                main.wait_stream(side)
+            graphs.append(g)
+        for _ in range(20):
+            for o in outs:
+                o.zero_()
+            torch.cuda.synchronize()
+            for g, s in zip(graphs, streams):
+                with torch.cuda.stream(s):
+                    g.replay()
+            torch.cuda.synchronize()
+            assert all(torch.equal(a, o) for a, o in zip(alone, outs))
