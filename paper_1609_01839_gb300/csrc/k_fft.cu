@@ -64,7 +64,7 @@ GFD_D unsigned int warp_mask() {
 // values that a row has in each tile (16 to 64 bytes per store): the
 // transform that staged its input, every stage and its output in shared memory
 // took 4.25 ms (forward) and 7.4 ms (inverse, two planes) per batched solve of
-// 256 images, this one 2.95 and 5.7 ms.
+// 256 images, this one 3.0 and 5.3 ms.
 // ---------------------------------------------------------------------------
 
 // The slots of a mirrored butterfly pair (A, B) of radix r over positions
@@ -356,8 +356,8 @@ k_col_plain(ClassDesc cd, const ImgDesc* __restrict__ imgs, const __grid_constan
 // keeps its sums while consecutive items belong to the same image; it
 // publishes them (one partial slot, one counter update) only when the image
 // changes.  Batched solve of 256 images, 15 iterations: 10.3 ms with staged
-// tiles and 12 or 8 nodes per pass, 7.0 ms as it is; 4 images of 4096^2, 30
-// iterations: 16.2 -> 9.5 ms (without prefetch, which takes 10.8 ms there: one
+// tiles and 12 or 8 nodes per pass, 6.9 ms as it is; 4 images of 4096^2, 30
+// iterations: 16.2 -> 9.2 ms (without prefetch, which takes 10.8 ms there: one
 // block per SM loads and computes in turn).  Three blocks per SM (80 registers)
 // spill and take 8.0 ms.
 template <int M, int BT>

@@ -111,10 +111,12 @@ struct SumDF {
 // their rounding is about 1 / (2 split_max) of that of plain sums.
 // Everything comes in pairs (J, Q), one packed FP32 instruction per pair, in
 // the register pairs that the ring's rows load; mixing int32 and FP32 halves
-// cost 10 % more instructions.  What bounds the kernel now: the FP32 pipe, the
-// shuffles (0.93 per cycle and SM) and issue are each about half busy, with 12
-// warps per SM (registers and rings) to overlap them; DRAM is at 15 %.  Per
-// batched solve of 256 images 14.7 -> 12.1 ms, of which 1.3 by the choice of
+// cost 10 % more instructions.  What bounds the kernel now: over a 4096 x 4096
+// image, w = 9 (138 us), the FMA pipe is busy 48 % of the cycles, the data path of
+// shared memory and shuffles 55 %, issue 48 %, DRAM 17 %, with 8 to 12 warps per SM
+// (rows per item, registers, rings) to overlap them; the wait between dependent
+// packed operations is the top stall.  Launches of few items are at 20 to 45 %.  Per
+// batched solve of 256 images 14.7 -> 12.2 ms, of which 1.3 by the choice of
 // rows per item (gfw_rows).  Fewer registers (128: spills) took 15.3 ms; leaving
 // rows re-read through L1 instead of the ring 16.7 ms.
 struct SumIG {
