@@ -36,10 +36,11 @@
 // / 4096 and the covariances about 6e-11 R R'.  Held against the rounding of u,
 // 2^-24 s with s a low estimate of |p| in the tile, and against eps, that is small
 // enough where R_p <= 256 s, R_I R_p <= 2^14 sqrt(eps) s and R_I^2 <= 2^16 eps
-// (images of [0, 1] down to eps = 2e-5).  Tiles beyond (bright pixels in a dark
-// neighbourhood, tiny eps), tiles with values that are not finite or whose
-// squares leave FP32's range, and offsets that leave the grid too few bits are
-// summed and solved in FP64 (cgf_ab_exact) at that kernel's price.
+// (images of [0, 1] down to eps = 2e-5).  A nearly flat plane's range counts as
+// |v| / (256 (2r+1)) at least, which keeps |v| below 2^20 grid steps.  Tiles beyond
+// (bright pixels in a dark neighbourhood, tiny eps) and tiles with values that are
+// not finite or whose squares leave FP32's range are summed and solved in FP64
+// (cgf_ab_exact) at that kernel's price.
 #include "common.cuh"
 #include "df.cuh"
 #include "launch.h"
@@ -307,6 +308,7 @@ k_cgf_ab(const float* __restrict__ I, const float* __restrict__ p, int M, int N,
   CgfGrid G[4];
   {
     const float inv = 1.0f / (float)(4096 / (2 * rad + 1) - 2);
+    const float flat = 1.0f / (float)(256 * (2 * rad + 1));
     const float cs[4] = {c.x, c.y, c.z, c.w};
     float top = 0.0f, low = s_max[4][0], mean = 0.0f;
 #pragma unroll
@@ -320,6 +322,9 @@ k_cgf_ab(const float* __restrict__ I, const float* __restrict__ p, int M, int N,
           mean += s_max[4][w] / (float)(CGF_THREADS / 32);
         }
       }
+      // |v| <= 2^20 g: a nearly flat plane takes the coarser grid of a larger range
+      // (one tile of 2048 in FP64, clipped at 1 but for a pixel, held up its call by 5 us)
+      if (b > 0.0f) b = fmaxf(b, (fabsf(cs[q]) + b) * flat);
       int e = 0;
       float f = 0.5f;
       if (b > 0.0f) f = frexpf(b * inv, &e);
@@ -333,7 +338,7 @@ k_cgf_ab(const float* __restrict__ I, const float* __restrict__ p, int M, int N,
         const float sc = fmaxf(low, mean * 0.015625f);
         fast = fast && b <= 256.0f * sc && top * b <= 16384.0f * sqrtf(eps.x) * sc;
       }
-      fast = fast && (b == 0.0f || (b >= 1e-25f && fabsf(cs[q]) + b <= 1048576.0f * G[q].g));
+      fast = fast && (b == 0.0f || b >= 1e-25f);
     }
     fast = fast && top * top <= 65536.0f * eps.x;
   }

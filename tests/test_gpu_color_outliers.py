@@ -134,3 +134,24 @@ def test_two_levels(eps, low):
     I = (I + np.where(edge, 0.9, low)).astype(np.float32)
     p = (abs(p) + np.where(edge, 0.8, low)).astype(np.float32)
     check(I, p, 9, eps)
+
+
+@pytest.mark.parametrize("w", [1, 3, 9, 17])
+@pytest.mark.parametrize("level", [1.0, 1000.0])
+@pytest.mark.parametrize("spread", [2.0 ** -23, 1e-6, 1e-4, 3e-3])
+def test_nearly_flat_planes(w, level, spread):
+    """Planes that hardly move about a value far from zero (clipped highlights), some or
+    all of them: the grid is then as coarse as the value asks for."""
+    I, p = inputs(31, top=level)
+    rng = np.random.default_rng(32)
+    near = lambda: (level * (1 - spread * rng.random(p.shape))).astype(np.float32)  # noqa: E731
+    for flat in ([2], [0, 1, 2, 3]):
+        J, q = I.copy(), p.copy()
+        for k in flat:
+            if k < 3:
+                J[k] = near()
+            else:
+                q = near()
+        eps = 1e-3 * level ** 2
+        u, tol = reference(J, q, w, eps)
+        assert (np.abs(gpu(J, q, w, eps) - u) <= tol).all(), flat
