@@ -20,15 +20,15 @@
 //
 // Arithmetic.  FP64 runs at 1.5 operations per cycle and SM on this part (70
 // cycles latency), so ordinary tiles use none per pixel.  Pass 1 splits each value on
-// a grid of the tile, v = c + g m + l with c a pixel of the tile and |m| <=
-// 4096 / (2r+1), as the grey-scale filter does (l is formed from v and c
+// a grid of the tile, v = c + g m + l with c the grid's point next to a pixel of the
+// tile and |m| <= 4096 / (2r+1), as the grey-scale filter does (l is formed from v and c
 // themselves, not from their rounded difference): the sums of m and of the
 // products m m' are exact in FP32, those of the remainders' parts are small,
 // and n S_mm' - S_m S_m' is formed exactly as a double-float.  The normal
 // equations are eliminated in double-float (about 48 bits) and a, b rounded
 // once.  Pass 2's sums are compensated (an FP32 running sum plus the exact
 // error of every addition).  1024 x 1024, w = 9: 1111 us with FP64 sums and
-// solves, 136 us as it is, the same error against FP64 (2.5e-8); 131 us with slid
+// solves, 135 us as it is, the same error against FP64 (2.5e-8); 128 us with slid
 // sums of rounded deviations and no look at the tile, which spread what is not
 // finite and lost dark pixels' digits beside bright ones.
 //
@@ -98,9 +98,10 @@ GFD_D void cgf_stage(float4* s, const float* p0, const float* p1, const float* p
   }
 }
 
-// One plane's split: v - c = g m + l.  mc, lc: the centre's own (whole) split.
+// One plane's split: v - c = g m + l, c = g mc the reference (on the grid, so that
+// |l| <= g / 2).
 struct CgfGrid {
-  float g, ig, mc, lc;
+  float g, ig, mc;
 };
 constexpr float CGF_MAGIC = 12582912.0f;  // rounds |t| < 2^22 to an integer
 
@@ -129,7 +130,6 @@ struct CgfSums {
     for (int c = 0; c < 4; ++c) {
       cgf_split(vs[c], G[c].g, G[c].ig, m[c], xl[c]);
       m[c] -= G[c].mc;
-      xl[c] -= G[c].lc;
       xh[c] = m[c] * G[c].g;
       x[c] = xh[c] + xl[c];
       out(c, h[c] + m[c], l[c] + xl[c]);
@@ -309,7 +309,7 @@ k_cgf_ab(const float* __restrict__ I, const float* __restrict__ p, int M, int N,
   {
     const float inv = 1.0f / (float)(4096 / (2 * rad + 1) - 2);
     const float flat = 1.0f / (float)(256 * (2 * rad + 1));
-    const float cs[4] = {c.x, c.y, c.z, c.w};
+    float cs[4] = {c.x, c.y, c.z, c.w};
     float top = 0.0f, low = s_max[4][0], mean = 0.0f;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -322,16 +322,18 @@ k_cgf_ab(const float* __restrict__ I, const float* __restrict__ p, int M, int N,
           mean += s_max[4][w] / (float)(CGF_THREADS / 32);
         }
       }
-      // |v| <= 2^20 g: a nearly flat plane takes the coarser grid of a larger range
-      // (one tile of 2048 in FP64, clipped at 1 but for a pixel, held up its call by 5 us)
-      if (b > 0.0f) b = fmaxf(b, (fabsf(cs[q]) + b) * flat);
+      // |v| <= 2^20 g: a nearly flat plane takes the coarser grid of a larger range (in
+      // FP64 such planes, highlights clipped at 1, took 908 us instead of 123)
+      b = fmaxf(b, (fabsf(cs[q]) + b) * flat);
       int e = 0;
       float f = 0.5f;
       if (b > 0.0f) f = frexpf(b * inv, &e);
       if (e < -100) e = -100;
       G[q].g = ldexpf(ceilf(8.0f * f) * 0.125f, e);  // 3-bit mantissa: g m is exact
       G[q].ig = 1.0f / G[q].g;
-      cgf_split(cs[q], G[q].g, G[q].ig, G[q].mc, G[q].lc);
+      float lc;
+      cgf_split(cs[q], G[q].g, G[q].ig, G[q].mc, lc);
+      cs[q] -= lc;  // (exact, as |c| <= 2^20 g)
       if (q < 3) {
         top = fmaxf(top, b);
       } else {  // the lowest of the warps' means (a few bright pixels do not raise it)
@@ -341,16 +343,19 @@ k_cgf_ab(const float* __restrict__ I, const float* __restrict__ p, int M, int N,
       fast = fast && (b == 0.0f || b >= 1e-25f);
     }
     fast = fast && top * top <= 65536.0f * eps.x;
+    c = make_float4(cs[0], cs[1], cs[2], cs[3]);
+  }
+  // pixels outside the canvas of truncated windows count nothing: no deviation, or zero
+  if (trunc && (x0 < rad || y0 < rad || x0 + CGF_TX + rad > N || y0 + CGF_TY + rad > M)) {
+    const float4 none = fast ? c : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    for (int e = threadIdx.x; e < EX * EY; e += blockDim.x) {
+      const int ty = e / EX, tx = e - ty * EX;
+      if (cgf_wrap(y0 - rad + ty, M, true) < 0 || cgf_wrap(x0 - rad + tx, N, true) < 0)
+        tile[ty * TP + tx] = none;
+    }
+    __syncthreads();
   }
   if (!fast) {  // the same for the whole block
-    if (trunc) {  // out-of-canvas pixels count nothing
-      for (int e = threadIdx.x; e < EX * EY; e += blockDim.x) {
-        const int ty = e / EX, tx = e - ty * EX;
-        if (cgf_wrap(y0 - rad + ty, M, true) < 0 || cgf_wrap(x0 - rad + tx, N, true) < 0)
-          tile[ty * TP + tx] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      }
-      __syncthreads();
-    }
     cgf_ab_exact(tile, reinterpret_cast<double*>(rows), M, N, rad, eps_d, trunc, x0, y0, ab);
     return;
   }

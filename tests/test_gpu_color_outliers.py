@@ -155,3 +155,16 @@ def test_nearly_flat_planes(w, level, spread):
         eps = 1e-3 * level ** 2
         u, tol = reference(J, q, w, eps)
         assert (np.abs(gpu(J, q, w, eps) - u) <= tol).all(), flat
+
+
+@pytest.mark.parametrize("seed", [41, 42])
+def test_black_and_grey_fields(seed):
+    """A grey image in three channels (a matrix singular but for eps), black fields beside
+    bright ones, eps at the end of the split's range (R^2 = 2^16 eps): the remainders
+    are half a grid step at most, so that the black fields keep the tolerance."""
+    rng = np.random.default_rng(seed)
+    i, j = np.mgrid[:64, :64]
+    g = np.where((i // 13 + j // 17) % 2 == 0, 0.6, 0.0) + 1e-3 * rng.standard_normal((64, 64))
+    I = np.stack([np.clip(g, 0, 1).astype(np.float32)] * 3)
+    p = (I[0] + 0.03 * rng.standard_normal((64, 64))).astype(np.float32)
+    check(I, p, 9, 1e-5)
